@@ -11,126 +11,11 @@
 #include <cmath>
 
 #include "../../include/kafila_gemm.h"
-#include "prefill.cuh"
+#include "prefill_tc.cuh"
 
 namespace kfl {
 
-// ---------------------------------------------------------------------------- tcgen05 / TMA
 namespace {
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Tensor-memory allocation by one whole warp; the base address is written to shared memory.
-__device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-
-// Shared-memory matrix descriptor of a K-major operand in the 128-byte swizzled layout: rows of
-// 128 bytes (64 bf16 of K), groups of 8 rows 1024 bytes apart (the stride byte offset); the
-// leading byte offset is unused in this layout (1 by convention); descriptor version 1; swizzle
-// mode 2 (128 bytes).  A slice of 16 K values starts 32 bytes further within the row.
-__device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
-// Instruction descriptor of kind::f16: fp32 accumulator (bits 4-5 = 1), A and B both bf16 (bits
-// 7-9 and 10-12 = 1) or both fp16 (0), both K-major (bits 15, 16 = 0), N >> 3 in bits 17-22,
-// M >> 4 in bits 24-28.
-__host__ __device__ constexpr uint32_t idesc_kind_f16(int m, int n, bool bf16) {
-  return (1u << 4) | ((bf16 ? 1u : 0u) << 7) | ((bf16 ? 1u : 0u) << 10) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(m >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t da, uint64_t db, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Arrive on an mbarrier of this CTA once every MMA this thread issued before has completed.
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-
-// 32 consecutive fp32 columns of this thread's tensor-memory lane (warp w reads lanes 32 w ..).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
-      : "memory");
-}
-
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, int c3,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-      "[%6];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-      : "memory");
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  return (uint32_t)f32_to_bf16_rne(lo) | ((uint32_t)f32_to_bf16_rne(hi) << 16);
-}
-
-// x as two bf16 terms: hi = bf16(x), lo = bf16(x - hi) (the difference is exact in fp32).
-__device__ __forceinline__ void split_bf16(float x, uint16_t &hi, uint16_t &lo) {
-  hi = f32_to_bf16_rne(x);
-  lo = f32_to_bf16_rne(x - bf16_to_f32(hi));
-}
-// The same with fp16 terms (about 2^-22 relative left; |x| must stay below 65504).
-__device__ __forceinline__ void split_f16(float x, uint16_t &hi, uint16_t &lo) {
-  hi = f32_to_f16_rn(x);
-  lo = f32_to_f16_rn(x - f16_to_f32(hi));
-}
-__device__ __forceinline__ void split_term(float x, uint16_t &hi, uint16_t &lo, int f16) {
-  if (f16)
-    split_f16(x, hi, lo);
-  else
-    split_bf16(x, hi, lo);
-}
-// Two values as packed pairs of their hi and lo terms.  fp16 terms of a value that fp16 cannot
-// hold (|x| >= 65520 rounds to infinity, or not finite) set ERR_F16_RANGE in *err.
-__device__ __forceinline__ void split_pack(float x0, float x1, uint32_t &hi, uint32_t &lo, int f16 = 0,
-                                           unsigned *err = nullptr) {
-  if (f16 && err && !(fabsf(x0) < 65520.f && fabsf(x1) < 65520.f)) atomicOr(err, ERR_F16_RANGE);
-  uint16_t h0, l0, h1, l1;
-  split_term(x0, h0, l0, f16);
-  split_term(x1, h1, l1, f16);
-  hi = (uint32_t)h0 | ((uint32_t)h1 << 16);
-  lo = (uint32_t)l0 | ((uint32_t)l1 << 16);
-}
 
 // ---------------------------------------------------------------------------- GEMM epilogues
 // Thread = one token t of the tile (its tensor-memory lane); v[j] = Y[t][n + j], j < 32.
@@ -249,6 +134,16 @@ __device__ __forceinline__ void epilogue32(const PrefillEpiParams &ep, int t, in
   }
 }
 
+// The MMAs of one K block of 64 (a 128-byte swizzled row): 16 K values at a time, both terms of X
+// against the same W slice.  A slice starts 32 bytes (2 in the descriptor's units) after the one before.
+__device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, bool accumulate) {
+#pragma unroll
+  for (int k = 0; k < PG_K / 16; ++k) {
+    mma_bf16_ss(d, da + 2 * k, db + 2 * k, idesc, accumulate || k > 0);
+    mma_bf16_ss(d, da + (PG_A_BYTES >> 4) + 2 * k, db + 2 * k, idesc, 1);
+  }
+}
+
 // ---------------------------------------------------------------------------- GEMM kernel
 // Split-K: the launch is a cluster of ep.splits (2, 4 or 8) CTAs per output tile (blockIdx.z =
 // rank); unsplit GEMMs run prefill_gemm_persistent.
@@ -256,11 +151,12 @@ template <int MODE>
 __global__ void __launch_bounds__(PG_THREADS, 1)
     prefill_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_a2,
                         const __grid_constant__ CUtensorMap tm_b, int n_kblocks, PrefillEpiParams ep) {
+  pdl_launch_dependents();
   static_assert(MODE != PE_ARGMAX, "the argmax partials are per whole tile: lm_head is never split");
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t s_full[PG_STAGES], s_empty[PG_STAGES], s_accum;
   __shared__ uint32_t s_tmem;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const int t0 = blockIdx.x * PG_M, n0 = blockIdx.y * PG_N;
   // split-K: split blockIdx.z of ep.splits takes K blocks [kb0, kb1)
   const int kb0 = (int)((long long)blockIdx.z * n_kblocks / ep.splits);
@@ -285,9 +181,11 @@ __global__ void __launch_bounds__(PG_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
+  pdl_wait();
 
   if (threadIdx.x == 0) {
     // ---- TMA producer
+    asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
     int issued[PG_STAGES] = {};
     bool ok = true;
     for (int j = 0; j < nkb; ++j) {
@@ -311,27 +209,25 @@ __global__ void __launch_bounds__(PG_THREADS, 1)
       for (int s = 0; s < PG_STAGES; ++s)
         if (issued[s] > 0) mbar_wait(smem_addr(&s_full[s]), (issued[s] - 1) & 1);
     }
-  } else if (threadIdx.x == 32) {
-    // ---- MMA issuer
+  } else if (warp == 1) {
+    // ---- MMA issuer (the whole warp, one elected lane issuing)
     // A and B always share one type: both bf16, or (int4 stages) both fp16
     const uint32_t idesc = ep.f16 ? idesc_kind_f16(PG_M, PG_N, false) : idesc_kind_f16(PG_M, PG_N, true);
     for (int j = 0; j < nkb; ++j) {
       const int s = j % PG_STAGES;
-      if (!mbar_wait(smem_addr(&s_full[s]), (j / PG_STAGES) & 1)) {
-        atomicOr(ep.err, ERR_TIMEOUT);
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_addr(&s_full[s]), (j / PG_STAGES) & 1))) {
+        if (lane == 0) atomicOr(ep.err, ERR_TIMEOUT);
         break;
       }
       tc_fence_after();
-      const uint32_t a = sa + s * 2 * PG_A_BYTES, b = sb + s * PG_B_BYTES;
-#pragma unroll
-      for (int k = 0; k < PG_K / 16; ++k) {
-        const uint64_t db = sdesc_k_sw128(b + 32 * k);
-        mma_bf16_ss(tmem, sdesc_k_sw128(a + 32 * k), db, idesc, (j | k) != 0);
-        mma_bf16_ss(tmem, sdesc_k_sw128(a + PG_A_BYTES + 32 * k), db, idesc, 1);
+      const uint64_t da = sdesc_k_sw128(sa + s * 2 * PG_A_BYTES), db = sdesc_k_sw128(sb + s * PG_B_BYTES);
+      if (elect_one()) {
+        mma_kblock(tmem, da, db, idesc, j != 0);
+        mma_commit(smem_addr(&s_empty[s]));  // the stage is free once these MMAs have read it
       }
-      mma_commit(smem_addr(&s_empty[s]));  // the stage is free once these MMAs have read it
+      __syncwarp();
     }
-    mma_commit(smem_addr(&s_accum));  // the accumulator is complete (or, after a timeout, idle)
+    if (elect_one()) mma_commit(smem_addr(&s_accum));  // the accumulator is complete (or, after a timeout, idle)
   }
   __syncwarp();
 
@@ -420,7 +316,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
   __shared__ __align__(8) uint64_t s_full[PG_STAGES], s_empty[PG_STAGES], s_acc_full[2], s_acc_empty[2], s_drain;
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const int t_tiles = (ep.T + PG_M - 1) / PG_M, n_tiles = (ep.N + PG_N - 1) / PG_N;
   const int tiles = t_tiles * n_tiles;
   const uint32_t raw = smem_addr(smem_raw);
@@ -446,9 +342,12 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   volatile int *abort_flag = &s_abort;
+  pdl_launch_dependents();
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
+      asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
       // ---- TMA producer: k-block it of the CTA's sequence uses stage it % S
       int issued[PG_STAGES] = {};
       long long it = 0;
@@ -479,47 +378,41 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- MMA issuer: tile i of this CTA accumulates into TMEM columns (i % 2) * PG_N
-      const uint32_t idesc = ep.f16 ? idesc_kind_f16(PG_M, PG_N, false) : idesc_kind_f16(PG_M, PG_N, true);
-      long long it = 0;
-      int i = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++i) {
-        const int buf = i & 1;
-        if (i >= 2 && !mbar_wait(smem_addr(&s_acc_empty[buf]), ((i >> 1) - 1) & 1)) {
-          ok = false;
-          break;
-        }
+    // ---- MMA issuer (the whole warp, one elected lane issuing): tile i of this CTA accumulates
+    // into TMEM columns (i % 2) * PG_N
+    const uint32_t idesc = ep.f16 ? idesc_kind_f16(PG_M, PG_N, false) : idesc_kind_f16(PG_M, PG_N, true);
+    int s = 0, i = 0;
+    uint32_t use = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++i) {
+      const int buf = i & 1;
+      if (i >= 2) ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&s_acc_empty[buf]), ((i >> 1) - 1) & 1));
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d = tmem + (uint32_t)(buf * PG_N);
+      for (int kb = 0; kb < n_kblocks; ++kb) {
+        ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_full[s]), use & 1));
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(buf * PG_N);
-        for (int kb = 0; kb < n_kblocks; ++kb, ++it) {
-          const int s = (int)(it % PG_STAGES);
-          if (*abort_flag || !mbar_wait(smem_addr(&s_full[s]), (uint32_t)(it / PG_STAGES) & 1)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a = sa + s * 2 * PG_A_BYTES, b = sb + s * PG_B_BYTES;
-#pragma unroll
-          for (int k = 0; k < PG_K / 16; ++k) {
-            const uint64_t db = sdesc_k_sw128(b + 32 * k);
-            mma_bf16_ss(d, sdesc_k_sw128(a + 32 * k), db, idesc, (kb | k) != 0);
-            mma_bf16_ss(d, sdesc_k_sw128(a + PG_A_BYTES + 32 * k), db, idesc, 1);
-          }
+        const uint64_t da = sdesc_k_sw128(sa + s * 2 * PG_A_BYTES), db = sdesc_k_sw128(sb + s * PG_B_BYTES);
+        if (elect_one()) {
+          mma_kblock(d, da, db, idesc, kb != 0);
           mma_commit(smem_addr(&s_empty[s]));
         }
-        if (ok) mma_commit(smem_addr(&s_acc_full[buf]));
+        __syncwarp();
+        if (++s == PG_STAGES) s = 0, ++use;
       }
-      if (!ok) {
-        *abort_flag = 1;
-        atomicOr(ep.err, ERR_TIMEOUT);
-      }
-      // every MMA issued has completed before TMEM can be freed
-      mma_commit(smem_addr(&s_drain));
-      mbar_wait(smem_addr(&s_drain), 0);
+      if (ok && elect_one()) mma_commit(smem_addr(&s_acc_full[buf]));
+      __syncwarp();
     }
+    if (!ok && lane == 0) {
+      *abort_flag = 1;
+      atomicOr(ep.err, ERR_TIMEOUT);
+    }
+    // every MMA issued has completed before TMEM can be freed
+    if (elect_one()) mma_commit(smem_addr(&s_drain));
     __syncwarp();
+    mbar_wait(smem_addr(&s_drain), 0);
   } else {
     // ---- epilogue warps 2..5: TMEM lanes 32 q .. 32 q + 31 (q = warp % 4) are tokens t0 + 32 q + lane
     const int q = warp & 3, row = 32 * q + lane;
@@ -629,6 +522,8 @@ template <int HD>
 __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnParams p) {
   using L = PaLayout<HD>;
   extern __shared__ __align__(16) uint8_t sm[];
+  pdl_launch_dependents();
+  pdl_wait();
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int g = lane / 4, c = lane % 4;
   // the longest blocks (latest tokens) first
@@ -773,8 +668,11 @@ __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnPar
 // holds the same position.
 __global__ void prefill_input_kernel(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                      const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                     int max_ctx, unsigned *err) {
+                                     int max_ctx, unsigned *tickets, int n_tickets, unsigned *err) {
   const int t = blockIdx.x;
+  pdl_launch_dependents();
+  // the narrow GEMMs' tickets, in case a pass that gave up left some
+  for (int j = t * blockDim.x + threadIdx.x; j < n_tickets; j += gridDim.x * blockDim.x) tickets[j] = 0;
   __shared__ int s_bad;
   if (threadIdx.x == 0) s_bad = 0;
   __syncthreads();
@@ -804,6 +702,8 @@ __global__ void prefill_input_kernel(const int *ids, const float *hidden_in, con
 __global__ void prefill_rmsnorm_kernel(const float *h, int ldh, int d, const float *g, float eps, uint16_t *x,
                                        uint16_t *x_lo, int ldx, int f16, unsigned *err) {
   const int t = blockIdx.x, d4 = d / 4;
+  pdl_launch_dependents();
+  pdl_wait();
   const float4 *row = reinterpret_cast<const float4 *>(h + (size_t)t * ldh);
   float ss = 0.f;
   for (int i = threadIdx.x; i < d4; i += blockDim.x) {
@@ -882,6 +782,8 @@ __global__ void split_rows_kernel(const float *x, int K, int ldx, uint16_t *hi, 
 // one warp per token (each lane scans every 32nd tile, then the warp keeps the largest value and,
 // among equal values, the lowest index).
 __global__ void prefill_argmax_kernel(const float *amax, const int *aidx, int n_tiles, int T, int *next_ids) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32;
   if (t >= T) return;  // uniform per warp
   float best = -INFINITY;
@@ -939,20 +841,50 @@ int encode_act_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int 
              : -1;
 }
 
+int encode_terms_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int ld, int terms, size_t term_stride,
+                     int box_rows) {
+  auto fn = encode_fn();
+  if (!fn || ld % 8 != 0 || term_stride % 8 != 0 || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return -1;
+  const cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)terms};
+  const cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)term_stride * 2};
+  const cuuint32_t box[3] = {PG_K, (cuuint32_t)box_rows, (cuuint32_t)terms};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<uint16_t *>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? 0
+             : -1;
+}
+
 // Weight tiles [n_rb][n_kt][RB][KT] bf16 as a 4-D tensor (column, row, K tile, row block):
-// boxes of 64 columns x RB rows x 1 K tile x PG_N / RB row blocks; row blocks >= n_rb read as zero.
-int encode_tiles_map(CUtensorMap *map, const uint8_t *tiles, int n_kt, int n_rb) {
+// boxes of 64 columns x RB rows x 1 K tile x box_rb row blocks; row blocks >= n_rb read as zero.
+int encode_tiles_map(CUtensorMap *map, const uint8_t *tiles, int n_kt, int n_rb, int box_rb) {
   auto fn = encode_fn();
   if (!fn) return -1;
   const cuuint64_t dims[4] = {(cuuint64_t)KT, (cuuint64_t)RB, (cuuint64_t)n_kt, (cuuint64_t)n_rb};
   const cuuint64_t strides[3] = {(cuuint64_t)KT * 2, (cuuint64_t)TILE_BYTES, (cuuint64_t)TILE_BYTES * n_kt};
-  const cuuint32_t box[4] = {PG_K, RB, 1, PG_N / RB};
+  const cuuint32_t box[4] = {PG_K, RB, 1, (cuuint32_t)box_rb};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<uint8_t *>(tiles), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
              ? 0
              : -1;
+}
+
+// Launches a kernel that waits for the kernel before it only where it needs its results.
+template <typename... P, typename... A>
+static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  pdl_attribute(attr[0]);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 template <int MODE>
@@ -973,19 +905,20 @@ static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, cons
   cfg.blockDim = dim3(PG_THREADS);
   cfg.dynamicSmemBytes = PG_SMEM;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 1;
-  attr[0].val.clusterDim.y = 1;
+  cudaLaunchAttribute attr[2];
+  pdl_attribute(attr[0]);
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 1;
+  attr[1].val.clusterDim.y = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   PrefillEpiParams e = ep;
   if constexpr (MODE != PE_ARGMAX) {
     // the largest split count not above the chosen one whose cluster fits on the device
     static int fits[9] = {};  // 0 unknown, 1 yes, -1 no
     while (e.splits > 1) {
       if (fits[e.splits] == 0) {
-        attr[0].val.clusterDim.z = e.splits;
+        attr[1].val.clusterDim.z = e.splits;
         cfg.gridDim = dim3(1, 1, e.splits);
         int n = 0;
         fits[e.splits] =
@@ -997,7 +930,7 @@ static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, cons
     }
     if (e.splits > 1) {
       cfg.gridDim = dim3((e.T + PG_M - 1) / PG_M, (e.N + PG_N - 1) / PG_N, e.splits);
-      attr[0].val.clusterDim.z = e.splits;
+      attr[1].val.clusterDim.z = e.splits;
       return cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<MODE>, a, a2, b, 2 * n_kt, e);
     }
   }
@@ -1012,7 +945,7 @@ static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, cons
   const long long tiles = (long long)((e.T + PG_M - 1) / PG_M) * ((e.N + PG_N - 1) / PG_N);
   cfg.gridDim = dim3((unsigned)std::min<long long>(tiles, n_sm));
   cfg.blockDim = dim3(PP_THREADS);
-  cfg.numAttrs = 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, prefill_gemm_persistent<MODE>, a, a2, b, 2 * n_kt, e);
 }
 
@@ -1060,8 +993,7 @@ static cudaError_t launch_attn_hd(const PrefillAttnParams &p, cudaStream_t s) {
     attr = true;
   }
   const dim3 grid((p.T + PA_ROWS - 1) / PA_ROWS, p.n_heads);
-  prefill_attn_kernel<HD><<<grid, PA_THREADS, bytes, s>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(prefill_attn_kernel<HD>, grid, PA_THREADS, bytes, s, p);
 }
 
 cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, cudaStream_t s) {
@@ -1071,16 +1003,15 @@ cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, cudaStr
 
 cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                  const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                 int max_ctx, unsigned *err, cudaStream_t s) {
+                                 int max_ctx, unsigned *tickets, int n_tickets, unsigned *err, cudaStream_t s) {
   prefill_input_kernel<<<T, 256, 0, s>>>(ids, hidden_in, positions_in, T, embed, vocab, d, ldh, h, positions,
-                                         max_ctx, err);
+                                         max_ctx, tickets, n_tickets, err);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const float *g, float eps, uint16_t *x,
                                    uint16_t *x_lo, int ldx, int f16, unsigned *err, cudaStream_t s) {
-  prefill_rmsnorm_kernel<<<T, 256, 0, s>>>(h, ldh, d, g, eps, x, x_lo, ldx, f16, err);
-  return cudaGetLastError();
+  return launch_pdl(prefill_rmsnorm_kernel, dim3(T), 256, 0, s, h, ldh, d, g, eps, x, x_lo, ldx, f16, err);
 }
 
 cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, cudaStream_t s) {
@@ -1096,8 +1027,7 @@ cudaError_t launch_split_bf16(const float *x, int T, int K, int ldx, uint16_t *h
 
 cudaError_t launch_prefill_argmax(const float *amax, const int *aidx, int n_tiles, int T, int *next_ids,
                                   cudaStream_t s) {
-  prefill_argmax_kernel<<<(T + 3) / 4, 128, 0, s>>>(amax, aidx, n_tiles, T, next_ids);
-  return cudaGetLastError();
+  return launch_pdl(prefill_argmax_kernel, dim3((T + 3) / 4), 128, 0, s, amax, aidx, n_tiles, T, next_ids);
 }
 
 }  // namespace kfl
@@ -1116,25 +1046,31 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     cudaGetLastError();
     return KFL_ERR_CUDA;
   }
-  const int splits = prefill_splits(T, N, n_kt, n_sm);
+  // few tokens: the few-token kernel, which needs room for partial sums and tickets too
+  const bool narrow = T <= NW_MAX_TP;
+  const int rows = (T + 7) / 8 * 8, n_tickets = narrow_max_tiles(N);
+  const size_t tile_bytes = (size_t)n_rb * n_kt * TILE_BYTES, x_bytes = (size_t)rows * ld * 2;
+  const size_t ws_bytes = narrow ? narrow_ws_bytes(n_sm, T) + (size_t)n_tickets * 4 : 0;
   void *mem = nullptr;
-  const size_t tile_bytes = (size_t)n_rb * n_kt * TILE_BYTES, x_bytes = (size_t)T * ld * 2;
-  if (cudaMalloc(&mem, tile_bytes + 2 * x_bytes + 16) != cudaSuccess) {
+  if (cudaMalloc(&mem, tile_bytes + 2 * x_bytes + ws_bytes + 16) != cudaSuccess) {
     cudaGetLastError();
     return KFL_ERR_OOM;
   }
   uint8_t *tiles = static_cast<uint8_t *>(mem);
   uint16_t *xhi = reinterpret_cast<uint16_t *>(tiles + tile_bytes);
-  uint16_t *xlo = xhi + (size_t)T * ld;
-  unsigned *err = reinterpret_cast<unsigned *>(xlo + (size_t)T * ld);
+  uint16_t *xlo = xhi + (size_t)rows * ld;
+  float *partial = reinterpret_cast<float *>(xlo + (size_t)rows * ld);
+  unsigned *err = reinterpret_cast<unsigned *>(reinterpret_cast<uint8_t *>(partial) + (narrow ? narrow_ws_bytes(n_sm, T) : 0));
   int rc = KFL_OK;
   CUtensorMap mh, ml, mb;
-  if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess ||
+  if (cudaMemsetAsync(err, 0, 16 + (narrow ? (size_t)n_tickets * 4 : 0), s) != cudaSuccess ||
       launch_split_bf16(x, T, K, ldx, xhi, xlo, ld, s) != cudaSuccess ||
       launch_repack_bf16(w, N, K, nullptr, N, n_rb, n_kt, tiles, s) != cudaSuccess) {
     rc = KFL_ERR_CUDA;
-  } else if (encode_act_map(&mh, xhi, K, T, ld) || encode_act_map(&ml, xlo, K, T, ld) ||
-             encode_tiles_map(&mb, tiles, n_kt, n_rb)) {
+  } else if (narrow ? encode_terms_map(&mh, xhi, K, T, ld, 2, (size_t)rows * ld, narrow_tp(T, 2)) ||
+                          encode_tiles_map(&mb, tiles, n_kt, n_rb, 128 / RB)
+                    : encode_act_map(&mh, xhi, K, T, ld) || encode_act_map(&ml, xlo, K, T, ld) ||
+                          encode_tiles_map(&mb, tiles, n_kt, n_rb, PG_N / RB)) {
     rc = KFL_ERR_CUDA;
   } else {
     PrefillEpiParams e = {};
@@ -1143,9 +1079,16 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     e.out = y;
     e.ldo = ldy;
     e.err = err;
-    e.splits = splits;
     unsigned h_err = 0;
-    if (launch_prefill_gemm(PE_STORE, mh, ml, mb, n_kt, e, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess ||
+    cudaError_t ce;
+    if (narrow) {
+      const NarrowWorkspace ws = {partial, err + 4, n_sm};
+      ce = launch_prefill_narrow(PE_STORE, mb, mh, K, 2, ws, e, s);
+    } else {
+      e.splits = prefill_splits(T, N, n_kt, n_sm);
+      ce = launch_prefill_gemm(PE_STORE, mh, ml, mb, n_kt, e, s);
+    }
+    if (ce != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess ||
         cudaMemcpy(&h_err, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
       rc = KFL_ERR_CUDA;
     else if (h_err & ERR_TIMEOUT)

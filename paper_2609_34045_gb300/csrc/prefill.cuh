@@ -45,8 +45,10 @@ struct PrefillEpiParams {
   float *out;              // PE_STORE / PE_RESID: fp32 [T][ldo]
   int ldo;
   uint16_t *out16;         // PE_SWIGLU: hi term, bf16 [T][ldo16] (N / 2 columns); PE_QKV: q, bf16 [T][ldo16]
-  uint16_t *out16lo;       // PE_SWIGLU: lo term, same layout
+  uint16_t *out16lo;       // PE_SWIGLU: lo term, same layout (out16 + term_stride)
   int ldo16;
+  int terms;               // PE_SWIGLU: terms stored, term_stride elements apart
+  size_t term_stride;
   // PE_QKV: rows [0, qdim) q, [qdim, qdim + kvdim) k (pairs (i, i + hd/2) adjacent per head, as
   // the weights were loaded), then v in natural order; K/V stored at the token's position of
   // KV slot `slot` of this layer's caches [max_batch][Hkv][max_ctx][hd]
@@ -77,9 +79,34 @@ struct PrefillAttnParams {
   unsigned *err;           // ERR_F16_RANGE if an fp16 output term cannot hold its value
 };
 
+// ---- the prefill GEMM of few tokens (prefill_narrow.cu): weight rows as M, the tokens' terms
+// side by side as N, split stream-K over one CTA per SM
+constexpr int NW_MAX_TP = 128;            // tokens of a tile (two terms: 256 MMA columns)
+constexpr int NW_W_BYTES = 128 * 64 * 2;  // a 128-row weight slice of 64 K
+struct NarrowWorkspace {
+  float *partial;     // narrow_ws_bytes
+  unsigned *tickets;  // at least narrow_max_tiles(N) per tile of tokens, zero before the first launch
+  int n_sm;
+};
+size_t narrow_ws_bytes(int n_sm, int T);  // for passes of up to T tokens
+int narrow_max_tiles(int N);
+int narrow_tp(int T, int terms);  // tokens of a tile
+// w: encode_tiles_map with 2 row blocks per box; x: encode_terms_map with narrow_tp rows per box.
+cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensorMap &x, int K, int terms,
+                                  const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s);
+
 // Host side (prefill.cu).
 int encode_act_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int ld);
-int encode_tiles_map(CUtensorMap *map, const uint8_t *tiles, int n_kt, int n_rb);
+// The terms of activation rows [term][rows][K] (row stride ld, term stride term_stride elements):
+// boxes of 64 columns x box_rows rows x every term.
+int encode_terms_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int ld, int terms, size_t term_stride,
+                     int box_rows);
+int encode_tiles_map(CUtensorMap *map, const uint8_t *tiles, int n_kt, int n_rb, int box_rb);
+// The launch attribute of a kernel that waits (griddepcontrol.wait) for the kernel before it.
+inline void pdl_attribute(cudaLaunchAttribute &a) {
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+}
 // Splits of K (1, 2, 4 or 8) for a GEMM of T tokens x N rows (n_kt K tiles) on n_sm SMs: the
 // count that minimises an estimate of waves x work per CTA.
 int prefill_splits(int T, int N, int n_kt, int n_sm);
@@ -88,7 +115,7 @@ cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a_hi, const CUtenso
 cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, cudaStream_t s);
 cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                  const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                 int max_ctx, unsigned *err, cudaStream_t s);
+                                 int max_ctx, unsigned *tickets, int n_tickets, unsigned *err, cudaStream_t s);
 cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const float *g, float eps, uint16_t *x,
                                    uint16_t *x_lo, int ldx, int f16, unsigned *err, cudaStream_t s);
 // int4 group-64 tiles [n_rb][n_kt][TILE4_BYTES] -> fp16 tiles [n_rb][2 n_kt][RB][KT] of code x scale.

@@ -264,7 +264,9 @@ struct kfl_stage {
   int pf_cap = 0;
   float *pf_h = nullptr;
   uint16_t *pf_q = nullptr;
-  uint16_t *pf_x[2] = {}, *pf_o[2] = {}, *pf_a[2] = {};  // GEMM inputs as hi and lo bf16 terms
+  uint16_t *pf_x = nullptr, *pf_o = nullptr, *pf_a = nullptr;  // GEMM inputs as terms [term][token][ld]
+  NarrowWorkspace pf_nw = {};  // the few-token GEMM's partial sums and tickets
+  int pf_n_tickets = 0, pf_amax_cols = 0;
   int *pf_pos = nullptr, *pf_aidx = nullptr;
   float *pf_amax = nullptr;
   std::vector<void *> pf_allocs;
@@ -272,6 +274,7 @@ struct kfl_stage {
   // lm_head.  int4 stages: one map per matrix kind [j] (then lm_head) over pf_w16, the fp16 tiles
   // of the matrix being multiplied (dequantized just before its GEMM)
   std::vector<CUtensorMap> pf_maps;  // int4: [buffer * 5 + kind]
+  std::vector<CUtensorMap> pf_maps_nw;  // bf16 stages: the same tiles in the few-token GEMM's boxes
   std::vector<CUtensorMap> kv_maps;  // attention clusters: layer l's K cache [2 l] and V cache [2 l + 1]
   uint16_t *pf_w16[2] = {};
   // int4: matrix g + 1 of a pass is dequantized on pf_side into buffer (g + 1) % 2 while GEMM g
@@ -809,16 +812,21 @@ int ensure_prefill(kfl_stage *st, int tokens) {
       st->pf_allocs.push_back(*p);
       return true;
     };
-    const int n_tiles = (P.V + PG_N - 1) / PG_N;
-    bool ok = get((void **)&st->pf_h, (size_t)cap * P.ldh * 4) && get((void **)&st->pf_q, (size_t)cap * pf_ld(P.qdim) * 2);
-    for (int j = 0; j < 2; ++j)
-      ok = ok && get((void **)&st->pf_x[j], (size_t)cap * pf_ld(P.d) * 2) &&
-           get((void **)&st->pf_o[j], (size_t)cap * pf_ld(P.qdim) * 2) &&
-           get((void **)&st->pf_a[j], (size_t)cap * pf_ld(P.F) * 2);
-    if (!ok || !get((void **)&st->pf_pos, (size_t)cap * 4) ||
-        !get((void **)&st->pf_amax, (size_t)cap * n_tiles * 4) ||
-        !get((void **)&st->pf_aidx, (size_t)cap * n_tiles * 4))
-      return KFL_ERR_OOM;
+    bool ok = get((void **)&st->pf_h, (size_t)cap * P.ldh * 4) && get((void **)&st->pf_q, (size_t)cap * pf_ld(P.qdim) * 2) &&
+              get((void **)&st->pf_x, (size_t)2 * cap * pf_ld(P.d) * 2) &&
+              get((void **)&st->pf_o, (size_t)2 * cap * pf_ld(P.qdim) * 2) &&
+              get((void **)&st->pf_a, (size_t)2 * cap * pf_ld(P.F) * 2) && get((void **)&st->pf_pos, (size_t)cap * 4);
+    // argmax partials: per 256-column tile, or (up to NW_MAX_TP tokens) per 32 rows
+    const size_t am = std::max((size_t)cap * ((P.V + PG_N - 1) / PG_N),
+                               (size_t)std::min(cap, NW_MAX_TP) * narrow_max_tiles(P.V) * 4);
+    ok = ok && get((void **)&st->pf_amax, am * 4) && get((void **)&st->pf_aidx, am * 4);
+    int most = std::max(std::max(P.qkv.N, P.o.N), std::max(P.gu.N, P.down.N));
+    if (st->flags & KFL_LOGITS_OUT) most = std::max(most, P.V);
+    st->pf_n_tickets = narrow_max_tiles(most);
+    st->pf_nw.n_sm = P.n_sm;
+    ok = ok && get((void **)&st->pf_nw.partial, narrow_ws_bytes(P.n_sm, cap)) &&
+         get((void **)&st->pf_nw.tickets, (size_t)st->pf_n_tickets * 4);
+    if (!ok) return KFL_ERR_OOM;
     st->pf_cap = cap;
   }
   if (st->pf_maps.empty() && st->cfg.weight_fmt == KFL_INT4_G64) {
@@ -850,21 +858,25 @@ int ensure_prefill(kfl_stage *st, int tokens) {
     for (int b = 0; b < 2; ++b)
       for (int j = 0; j < n_kinds; ++j)
         if (encode_tiles_map(&maps[b * 5 + j], reinterpret_cast<const uint8_t *>(st->pf_w16[b]), 2 * kinds[j]->n_kt,
-                             kinds[j]->n_rb))
+                             kinds[j]->n_rb, PG_N / RB))
           return KFL_ERR_CUDA;
     st->pf_maps = std::move(maps);
   }
   if (st->pf_maps.empty()) {
-    std::vector<CUtensorMap> maps(4 * P.nl + 1);
+    std::vector<CUtensorMap> maps(4 * P.nl + 1), narrow(4 * P.nl + 1);
+    auto encode = [&](int i, const Mat &m) {
+      return encode_tiles_map(&maps[i], m.tiles, m.n_kt, m.n_rb, PG_N / RB) ||
+             encode_tiles_map(&narrow[i], m.tiles, m.n_kt, m.n_rb, 128 / RB);
+    };
     for (int l = 0; l < P.nl; ++l) {
       const LayerDev &L = st->layers[l];
       const Mat *m[4] = {&L.qkv, &L.o, &L.gu, &L.down};
       for (int j = 0; j < 4; ++j)
-        if (encode_tiles_map(&maps[4 * l + j], m[j]->tiles, m[j]->n_kt, m[j]->n_rb)) return KFL_ERR_CUDA;
+        if (encode(4 * l + j, *m[j])) return KFL_ERR_CUDA;
     }
-    if ((st->flags & KFL_LOGITS_OUT) && encode_tiles_map(&maps[4 * P.nl], st->lm.tiles, st->lm.n_kt, st->lm.n_rb))
-      return KFL_ERR_CUDA;
+    if ((st->flags & KFL_LOGITS_OUT) && encode(4 * P.nl, st->lm)) return KFL_ERR_CUDA;
     st->pf_maps = std::move(maps);
+    st->pf_maps_nw = std::move(narrow);
   }
   return KFL_OK;
 }
@@ -903,6 +915,9 @@ cudaError_t pf_dequant(kfl_stage *st, int g) {
   return err;
 }
 
+// Whether a pass of n tokens runs on the few-token GEMM.
+bool pf_narrow(const kfl_stage *st, int n) { return st->cfg.weight_fmt == KFL_BF16 && n <= NW_MAX_TP; }
+
 // int4: start of a pass on stream s: both buffers free once s's earlier work is done; the first
 // matrix is dequantized.
 cudaError_t pf_pass_begin(kfl_stage *st, cudaStream_t s) {
@@ -914,16 +929,47 @@ cudaError_t pf_pass_begin(kfl_stage *st, cudaStream_t s) {
   return err;
 }
 
-// One prefill GEMM with matrix j of block l (j = 4: lm_head) and the split count chosen for its
-// shape.  int4 stages read the matrix's fp16 copy, dequantized ahead on the side stream (the
-// next one is started before this GEMM, so dequantization overlaps the products).
-cudaError_t pf_gemm(kfl_stage *st, int mode, const CUtensorMap &a, const CUtensorMap &a2, int l, int j,
-                    PrefillEpiParams e, cudaStream_t s) {
+// A GEMM input of one pass: its terms [term][n rows][ld], and the maps that the GEMMs read it through.
+struct PfInput {
+  uint16_t *base = nullptr;
+  int K = 0, ld = 0, n = 0, terms = 0;
+  size_t stride = 0;  // elements from term to term
+  CUtensorMap term[2];  // tiles of PG_M tokens, a map per term
+  CUtensorMap all;      // narrow tiles, every term in a box
+  int encode(uint16_t *p, int K_, int n_, int terms_, bool narrow) {
+    base = p;
+    K = K_;
+    n = n_;
+    terms = terms_;
+    ld = pf_ld(K);
+    stride = (size_t)round_up(n, 8) * ld;
+    if (narrow) return encode_terms_map(&all, base, K, n, ld, terms, stride, narrow_tp(n, terms));
+    for (int j = 0; j < 2; ++j)
+      if (encode_act_map(&term[j], base + j * stride, K, n, ld)) return -1;
+    return 0;
+  }
+};
+
+// One prefill GEMM with matrix j of block l (j = 4: lm_head).  bf16 stages run passes of up to
+// NW_MAX_TP tokens on the few-token kernel, longer ones (and int4 stages) on 128-token tiles with
+// the split count chosen for the shape.  int4 stages read the matrix's fp16 copy, dequantized ahead on
+// the side stream (the next one is started before this GEMM, so dequantization overlaps the products).
+cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, PrefillEpiParams e, cudaStream_t s) {
   const Mat &m = pf_mat(st, l, j);
   const bool i4 = st->cfg.weight_fmt == KFL_INT4_G64;
   int n_kt = m.n_kt;
   const CUtensorMap *b;
   const int g = st->pf_seq++;
+  e.T = x.n;
+  e.terms = x.terms;
+  e.f16 = i4 ? 1 : 0;
+  if (mode == PE_ARGMAX) {
+    e.amax = st->pf_amax;
+    e.aidx = st->pf_aidx;
+    e.n_tiles = st->pf_amax_cols;
+  }
+  if (pf_narrow(st, x.n))
+    return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], x.all, m.K, x.terms, st->pf_nw, e, s);
   if (i4) {
     cudaError_t err = pf_dequant(st, g + 1);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, st->pf_deq[g % 2], 0);
@@ -933,9 +979,8 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const CUtensorMap &a, const CUtenso
   } else {
     b = &st->pf_maps[j == 4 ? 4 * st->P.nl : 4 * l + j];
   }
-  e.f16 = i4 ? 1 : 0;
   e.splits = mode == PE_ARGMAX ? 1 : prefill_splits(e.T, e.N, n_kt, st->P.n_sm);
-  cudaError_t err = launch_prefill_gemm(mode, a, a2, *b, n_kt, e, s);
+  cudaError_t err = launch_prefill_gemm(mode, x.term[0], x.term[1], *b, n_kt, e, s);
   if (err == cudaSuccess && i4) err = cudaEventRecord(st->pf_used[g % 2], s);
   return err;
 }
@@ -951,26 +996,34 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
   if (rc != KFL_OK) return rc;
   const bool embed = (st->flags & KFL_EMBED_IN) != 0;
   const int i4 = st->cfg.weight_fmt == KFL_INT4_G64 ? 1 : 0;
-  const int ldx = pf_ld(P.d), ldq = pf_ld(P.qdim), lda = pf_ld(P.F);
+  const int ldq = pf_ld(P.qdim), lda = pf_ld(P.F);
   const float eps = st->cfg.rms_eps;
   for (int t0 = 0; t0 < T; t0 += st->pf_cap) {
     const int n = std::min(st->pf_cap, T - t0);
+    const bool narrow = pf_narrow(st, n);
     CK(launch_prefill_input(ids ? ids + t0 : nullptr, hidden_in ? hidden_in + (size_t)t0 * P.d : nullptr,
                             positions + t0, n, embed ? st->embed : nullptr, P.V, P.d, P.ldh, st->pf_h, st->pf_pos,
-                            st->cfg.max_ctx, st->err, s));
+                            st->cfg.max_ctx, st->pf_nw.tickets, st->pf_n_tickets, st->err, s));
     CK(pf_pass_begin(st, s));
-    CUtensorMap mx[2], mo[2], ma[2];
-    for (int j = 0; j < 2; ++j)
-      if (encode_act_map(&mx[j], st->pf_x[j], P.d, n, ldx) || encode_act_map(&mo[j], st->pf_o[j], P.qdim, n, ldq) ||
-          encode_act_map(&ma[j], st->pf_a[j], P.F, n, lda))
-        return KFL_ERR_CUDA;
+    PfInput x, o, a;
+    if (x.encode(st->pf_x, P.d, n, 2, narrow) || o.encode(st->pf_o, P.qdim, n, 2, narrow) ||
+        a.encode(st->pf_a, P.F, n, 2, narrow))
+      return KFL_ERR_CUDA;
+    st->pf_amax_cols = narrow ? narrow_max_tiles(P.V) * 4 : (P.V + PG_N - 1) / PG_N;
+    auto norm = [&](const float *g) {
+      return launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, g, eps, x.base, x.base + x.stride, x.ld, i4, st->err, s);
+    };
+    PrefillEpiParams r = {};  // O and down: into the residual stream
+    r.err = st->err;
+    r.N = P.d;
+    r.out = st->pf_h;
+    r.ldo = P.ldh;
     for (int l = 0; l < P.nl; ++l) {
       const LayerDev &L = st->layers[l];
       uint16_t *kcl = st->kc + (size_t)l * P.kv_elems_per_layer;
       uint16_t *vcl = st->vc + (size_t)l * P.kv_elems_per_layer;
-      CK(launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, L.g_attn, eps, st->pf_x[0], st->pf_x[1], ldx, i4, st->err, s));
+      CK(norm(L.g_attn));
       PrefillEpiParams e = {};
-      e.T = n;
       e.err = st->err;
       e.N = L.qkv.N;
       e.out16 = st->pf_q;
@@ -986,54 +1039,44 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       e.max_ctx = st->cfg.max_ctx;
       e.rope_cos = st->rope_cos;
       e.rope_sin = st->rope_sin;
-      CK(pf_gemm(st, PE_QKV, mx[0], mx[1], l, 0, e, s));
-      PrefillAttnParams a = {};
-      a.q = st->pf_q;
-      a.ldq = ldq;
-      a.o = st->pf_o[0];
-      a.o_lo = st->pf_o[1];
-      a.ldo = ldq;
-      a.f16 = i4;
-      a.kcache = kcl;
-      a.vcache = vcl;
-      a.positions = st->pf_pos;
-      a.slot = user;
-      a.T = n;
-      a.n_heads = P.hq;
-      a.n_kv_heads = P.hkv;
-      a.max_ctx = st->cfg.max_ctx;
-      a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)P.hd));
-      a.err = st->err;
-      CK(launch_prefill_attention(a, P.hd, s));
-      PrefillEpiParams r = {};
-      r.T = n;
-      r.err = st->err;
-      r.N = P.d;
-      r.out = st->pf_h;
-      r.ldo = P.ldh;
-      CK(pf_gemm(st, PE_RESID, mo[0], mo[1], l, 1, r, s));
-      CK(launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, L.g_ffn, eps, st->pf_x[0], st->pf_x[1], ldx, i4, st->err, s));
+      CK(pf_gemm(st, PE_QKV, x, l, 0, e, s));
+      PrefillAttnParams t = {};
+      t.q = st->pf_q;
+      t.ldq = ldq;
+      t.o = o.base;
+      t.o_lo = o.base + o.stride;
+      t.ldo = o.ld;
+      t.f16 = i4;
+      t.kcache = kcl;
+      t.vcache = vcl;
+      t.positions = st->pf_pos;
+      t.slot = user;
+      t.T = n;
+      t.n_heads = P.hq;
+      t.n_kv_heads = P.hkv;
+      t.max_ctx = st->cfg.max_ctx;
+      t.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)P.hd));
+      t.err = st->err;
+      CK(launch_prefill_attention(t, P.hd, s));
+      CK(pf_gemm(st, PE_RESID, o, l, 1, r, s));
+      CK(norm(L.g_ffn));
       PrefillEpiParams g = {};
-      g.T = n;
       g.err = st->err;
       g.N = 2 * P.F;
-      g.out16 = st->pf_a[0];
-      g.out16lo = st->pf_a[1];
+      g.out16 = a.base;
+      g.out16lo = a.base + a.stride;
+      g.term_stride = a.stride;
       g.ldo16 = lda;
-      CK(pf_gemm(st, PE_SWIGLU, mx[0], mx[1], l, 2, g, s));
-      CK(pf_gemm(st, PE_RESID, ma[0], ma[1], l, 3, r, s));
+      CK(pf_gemm(st, PE_SWIGLU, x, l, 2, g, s));
+      CK(pf_gemm(st, PE_RESID, a, l, 3, r, s));
     }
     if (st->flags & KFL_LOGITS_OUT) {
-      CK(launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, st->g_final, eps, st->pf_x[0], st->pf_x[1], ldx, i4, st->err, s));
+      CK(norm(st->g_final));
       PrefillEpiParams z = {};
-      z.T = n;
       z.err = st->err;
       z.N = P.V;
-      z.amax = st->pf_amax;
-      z.aidx = st->pf_aidx;
-      z.n_tiles = (P.V + PG_N - 1) / PG_N;
-      CK(pf_gemm(st, PE_ARGMAX, mx[0], mx[1], -1, 4, z, s));
-      CK(launch_prefill_argmax(st->pf_amax, st->pf_aidx, z.n_tiles, n, next_ids + t0, s));
+      CK(pf_gemm(st, PE_ARGMAX, x, -1, 4, z, s));
+      CK(launch_prefill_argmax(st->pf_amax, st->pf_aidx, st->pf_amax_cols, n, next_ids + t0, s));
     }
     if (hidden_out)
       CK(cudaMemcpy2DAsync(hidden_out + (size_t)t0 * P.d, (size_t)P.d * 4, st->pf_h, (size_t)P.ldh * 4,
