@@ -668,11 +668,9 @@ __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnPar
 // holds the same position.
 __global__ void prefill_input_kernel(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                      const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                     int max_ctx, unsigned *tickets, int n_tickets, unsigned *err) {
+                                     int max_ctx, unsigned *err) {
   const int t = blockIdx.x;
   pdl_launch_dependents();
-  // the narrow GEMMs' tickets, in case a pass that gave up left some
-  for (int j = t * blockDim.x + threadIdx.x; j < n_tickets; j += gridDim.x * blockDim.x) tickets[j] = 0;
   __shared__ int s_bad;
   if (threadIdx.x == 0) s_bad = 0;
   __syncthreads();
@@ -1003,9 +1001,9 @@ cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, cudaStr
 
 cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                  const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                 int max_ctx, unsigned *tickets, int n_tickets, unsigned *err, cudaStream_t s) {
+                                 int max_ctx, unsigned *err, cudaStream_t s) {
   prefill_input_kernel<<<T, 256, 0, s>>>(ids, hidden_in, positions_in, T, embed, vocab, d, ldh, h, positions,
-                                         max_ctx, tickets, n_tickets, err);
+                                         max_ctx, err);
   return cudaGetLastError();
 }
 
@@ -1046,11 +1044,11 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     cudaGetLastError();
     return KFL_ERR_CUDA;
   }
-  // few tokens: the few-token kernel, which needs room for partial sums and tickets too
+  // few tokens: the few-token kernel, which needs room for partial sums too
   const bool narrow = T <= NW_MAX_TP;
-  const int rows = (T + 7) / 8 * 8, n_tickets = narrow_max_tiles(N);
+  const int rows = (T + 7) / 8 * 8;
   const size_t tile_bytes = (size_t)n_rb * n_kt * TILE_BYTES, x_bytes = (size_t)rows * ld * 2;
-  const size_t ws_bytes = narrow ? narrow_ws_bytes(n_sm, T) + (size_t)n_tickets * 4 : 0;
+  const size_t ws_bytes = narrow ? narrow_ws_bytes(n_sm, T) : 0;
   void *mem = nullptr;
   if (cudaMalloc(&mem, tile_bytes + 2 * x_bytes + ws_bytes + 16) != cudaSuccess) {
     cudaGetLastError();
@@ -1060,10 +1058,10 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
   uint16_t *xhi = reinterpret_cast<uint16_t *>(tiles + tile_bytes);
   uint16_t *xlo = xhi + (size_t)rows * ld;
   float *partial = reinterpret_cast<float *>(xlo + (size_t)rows * ld);
-  unsigned *err = reinterpret_cast<unsigned *>(reinterpret_cast<uint8_t *>(partial) + (narrow ? narrow_ws_bytes(n_sm, T) : 0));
+  unsigned *err = reinterpret_cast<unsigned *>(reinterpret_cast<uint8_t *>(partial) + ws_bytes);
   int rc = KFL_OK;
   CUtensorMap mh, ml, mb;
-  if (cudaMemsetAsync(err, 0, 16 + (narrow ? (size_t)n_tickets * 4 : 0), s) != cudaSuccess ||
+  if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess ||
       launch_split_bf16(x, T, K, ldx, xhi, xlo, ld, s) != cudaSuccess ||
       launch_repack_bf16(w, N, K, nullptr, N, n_rb, n_kt, tiles, s) != cudaSuccess) {
     rc = KFL_ERR_CUDA;
@@ -1082,7 +1080,7 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     unsigned h_err = 0;
     cudaError_t ce;
     if (narrow) {
-      const NarrowWorkspace ws = {partial, err + 4, n_sm};
+      const NarrowWorkspace ws = {partial, n_sm};
       ce = launch_prefill_narrow(PE_STORE, mb, mh, K, 2, ws, e, s);
     } else {
       e.splits = prefill_splits(T, N, n_kt, n_sm);

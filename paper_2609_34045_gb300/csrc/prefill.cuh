@@ -82,18 +82,21 @@ struct PrefillAttnParams {
 // ---- the prefill GEMM of few tokens (prefill_narrow.cu): weight rows as M, the tokens' terms
 // side by side as N, split stream-K over one CTA per SM
 constexpr int NW_MAX_TP = 128;            // tokens of a tile (two terms: 256 MMA columns)
+constexpr int N4_MAX_TOKENS = 1024;      // int4 stages: passes of up to this many tokens decode in the GEMM
 constexpr int NW_W_BYTES = 128 * 64 * 2;  // a 128-row weight slice of 64 K
 struct NarrowWorkspace {
-  float *partial;     // narrow_ws_bytes
-  unsigned *tickets;  // at least narrow_max_tiles(N) per tile of tokens, zero before the first launch
+  float *partial;  // narrow_ws_bytes
   int n_sm;
 };
 size_t narrow_ws_bytes(int n_sm, int T);  // for passes of up to T tokens
-int narrow_max_tiles(int N);
+int narrow_argmax_slots(int N);  // PE_ARGMAX: partial maxima per token (n_tiles of PrefillEpiParams)
 int narrow_tp(int T, int terms);  // tokens of a tile
 // w: encode_tiles_map with 2 row blocks per box; x: encode_terms_map with narrow_tp rows per box.
 cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensorMap &x, int K, int terms,
                                   const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s);
+// The same over int4 tiles [n_rb][n_kt][TILE4_BYTES], decoded in the kernel (fp16 terms).
+cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int n_kt, const CUtensorMap &x, int K,
+                                   int terms, const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s);
 
 // Host side (prefill.cu).
 int encode_act_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int ld);
@@ -115,7 +118,7 @@ cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a_hi, const CUtenso
 cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, cudaStream_t s);
 cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                  const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                 int max_ctx, unsigned *tickets, int n_tickets, unsigned *err, cudaStream_t s);
+                                 int max_ctx, unsigned *err, cudaStream_t s);
 cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const float *g, float eps, uint16_t *x,
                                    uint16_t *x_lo, int ldx, int f16, unsigned *err, cudaStream_t s);
 // int4 group-64 tiles [n_rb][n_kt][TILE4_BYTES] -> fp16 tiles [n_rb][2 n_kt][RB][KT] of code x scale.

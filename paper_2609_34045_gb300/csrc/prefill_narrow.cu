@@ -7,16 +7,15 @@
 // the HBM bandwidth about 750).  So every SM streams an equal share of the matrix, whatever its
 // shape: the K blocks of all row tiles form one sequence, CTA c takes the contiguous range
 // [c U / G, (c + 1) U / G) of it, and a row tile that several CTAs share is summed from their
-// partial sums in CTA order by the last of them to arrive (no CTA ever waits for another).
+// partial sums in CTA order by a small kernel behind it (narrow_reduce_kernel).
 // The tokens' terms share each MMA: 128 weight rows x (terms x tokens) columns, so a token count
 // of 16 costs an eighth of the 128-token tile of prefill_gemm_persistent, and the epilogue's lanes
 // hold consecutive output columns of one token.
 //
-// Measured (7B-shaped block, 43 tokens): the gate/up loop streams its 272 MB in 36 us (7.0 TB/s
-// after the first ring fill); a GEMM takes 17 (Q/K/V), 28 (down) and 45 us (gate/up) from its first
-// CTA to its last, of which 4 to 8 us are the shared tiles' sums and epilogues at the end; clusters
-// of up to 8 CTAs per 128-token tile, reducing through distributed shared memory, took 51, 39 and
-// 58 us (four blocks with everything between: 954 -> 697 us).
+// Measured (7B-shaped blocks, 43 tokens): the gate/up loop streams its 272 MB in 36 us (7.0 TB/s
+// after the first ring fill).  Clusters of up to 8 CTAs per 128-token tile, reducing through
+// distributed shared memory, took 51 us for Q/K/V, 39 for O and down on average and 58 for gate/up
+// (four blocks with everything between: 954 us, now 614).
 #include <algorithm>
 #include <type_traits>
 
@@ -29,8 +28,9 @@ namespace {
 constexpr int NW_WARPS = 10;             // TMA, MMA, 8 epilogue warps
 constexpr int NW_THREADS = NW_WARPS * 32;
 constexpr int NW_EPI_THREADS = 256;
+constexpr int NW_EPI_WARP = 2;            // the first epilogue warp
 constexpr int NW_MAX_STAGES = 12;
-constexpr int NW_SMEM = 224 * 1024;      // ring + alignment slack
+constexpr int NW_RING = 226 * 1024;      // shared memory of the rings: a block's 227 KiB less the barriers' KiB
 
 struct NarrowParams {
   int n_kb;         // K blocks of 64
@@ -41,9 +41,14 @@ struct NarrowParams {
   int acc_cols;     // TMEM columns of one 128-row accumulator (tp * terms rounded up to 32)
   int bufs;         // accumulators: 1 or 2
   int tmem_cols;
-  float *ws;        // partial sums: [G][2][mb][tp][128]
-  unsigned *tickets;  // [n_tiles], zero between launches
+  float *ws;        // partial sums (narrow_partial)
 };
+
+// Where (in float4, plus the row) CTA c's partial of its slot holds the sums of 128-row block m and token
+// group gr: [c][slot][m][gr][4 x 4 tokens][128 rows].
+__device__ __forceinline__ size_t narrow_partial(int c, int slot, int m, int gr, int mb, int tp) {
+  return (((size_t)c * 2 + slot) * mb * (tp / 16) + (size_t)m * (tp / 16) + gr) * (4 * 128);
+}
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -54,20 +59,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// Whether `ok` holds on all n threads that meet at named barrier id.
-__device__ __forceinline__ bool named_bar_and(int id, int n, bool ok) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %3, 0;\n\t"
-      "barrier.cta.red.and.pred p, %1, %2, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r)
-      : "r"(id), "r"(n), "r"((uint32_t)ok)
-      : "memory");
-  return r != 0;
-}
 
 // The epilogue of 16 tokens t0 .. t0 + 15 of output row n (this lane's; the warp's lanes hold 32
 // consecutive rows starting at a multiple of 32): load() fetches what it needs besides the sums, all
@@ -172,6 +163,115 @@ struct NarrowEpilogue {
   }
 };
 
+// The epilogue warps' part of a CTA with range [u0, u1) of the U units: every segment's sums, from its
+// accumulator to the outputs or, where CTAs share the tile, to the partial sums (narrow_reduce_kernel).
+template <int MODE, int MB>
+__device__ __forceinline__ void narrow_epilogue_warps(const NarrowParams &p, const PrefillEpiParams &ep, uint32_t tmem,
+                                                      long long u0, long long u1, uint64_t *s_acc_full,
+                                                      uint64_t *s_acc_empty, volatile int *abort_flag) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  // ---- epilogue warps: TMEM lanes 32 q .. (q = warp % 4) are 32 consecutive rows of the tile;
+  // the two warps of a quadrant take alternate groups of 16 tokens
+  pdl_wait();  // h, the partial sums and the outputs may still be in use by the previous kernel
+  const int q = warp & 3, grp = (warp - NW_EPI_WARP) >> 2, row = 32 * q + lane;
+  const int groups = p.tp / 16;
+  int seg = 0;
+  for (long long u = u0; u < u1; ++seg) {
+    const int tile = (int)(u / p.n_kb);
+    const long long t_lo = (long long)tile * p.n_kb, t_hi = t_lo + p.n_kb, end = min(u1, t_hi);
+    const int buf = p.bufs == 2 ? seg & 1 : 0;
+    const bool ready = __all_sync(
+        0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_acc_full[buf]), (uint32_t)(p.bufs == 2 ? seg >> 1 : seg) & 1));
+    if (!ready) {
+      if (lane == 0) {
+        *abort_flag = 1;
+        atomicOr(ep.err, ERR_TIMEOUT);
+      }
+      break;
+    }
+    tc_fence_after();
+    const bool whole = u == t_lo && end == t_hi;
+    const int r_tile = tile / p.t_tiles, tt0 = (tile % p.t_tiles) * p.tp;
+    for (int m = 0; m < MB; ++m) {
+      const int n = (r_tile * MB + m) * 128 + row;
+      for (int gr = grp; gr < groups; gr += 2) {
+        const int t0 = tt0 + gr * 16;
+        if (t0 >= ep.T) break;
+        NarrowEpilogue<MODE> e;
+        if (whole) e.load(ep, n, t0, lane);
+        const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((buf * MB + m) * p.acc_cols + gr * 16);
+        uint32_t r0[16], r1[16], r2[16];
+        tmem_ld16(ta, r0);
+        tmem_ld16(ta + p.tp, r1);
+        if (p.terms == 3) tmem_ld16(ta + 2 * p.tp, r2);
+        tmem_wait_ld();
+        float v[16];
+        // the smaller terms first
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float lo = p.terms == 3 ? __uint_as_float(r1[j]) + __uint_as_float(r2[j]) : __uint_as_float(r1[j]);
+          v[j] = __uint_as_float(r0[j]) + lo;
+        }
+        if (whole) {
+          e.store(ep, n, t0, v, lane, (r_tile * MB + m) * 4 + q);
+        } else {
+          // this CTA's slot 0: the range starts inside the tile; slot 1: it ends inside
+          float4 *w = reinterpret_cast<float4 *>(p.ws) +
+                      narrow_partial(blockIdx.x, u > t_lo ? 0 : 1, m, gr, MB, p.tp) + row;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) w[j * 128] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        }
+      }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_addr(&s_acc_empty[buf]));
+    u = end;
+  }
+}
+
+// The tiles that several CTAs share: their partial sums, added in CTA order, and the epilogue.  One
+// block per 128 rows x 16 tokens, so that the sums (up to 70 KB a CTA of the GEMM) are read by the
+// whole GPU at once: summed by the last CTA to arrive at a tile, inside the GEMM, they cost 4 to 8 us
+// at 43 tokens and 20 to 50 us at 100, of a tail in which most SMs were idle.
+template <int MODE>
+__global__ void __launch_bounds__(128) narrow_reduce_kernel(NarrowParams p, int mb, int gemm_ctas, PrefillEpiParams ep) {
+  pdl_launch_dependents();
+  const int groups = p.tp / 16, gr = blockIdx.x % groups, m = blockIdx.x / groups % mb, tile = blockIdx.x / groups / mb;
+  const int q = threadIdx.x / 32, lane = threadIdx.x % 32, row = threadIdx.x;
+  const long long U = (long long)p.n_tiles * p.n_kb, G = gemm_ctas, t_lo = (long long)tile * p.n_kb;
+  const int r_tile = tile / p.t_tiles, t0 = (tile % p.t_tiles) * p.tp + gr * 16;
+  // the CTAs whose ranges meet the tile; every one but the first starts inside it
+  const int first = (int)(((t_lo + 1) * G - 1) / U), last = (int)(((t_lo + p.n_kb) * G - 1) / U);
+  const int slot0 = first * U / G > t_lo ? 0 : 1;
+  pdl_wait();
+  if (first == last || t0 >= ep.T) return;
+  const int n = (r_tile * mb + m) * 128 + row;
+  const float4 *ws = reinterpret_cast<const float4 *>(p.ws) + row;
+  NarrowEpilogue<MODE> e;
+  e.load(ep, n, t0, lane);
+  float v[16] = {};
+  for (int c = first; c <= last; c += 4) {
+    float4 x[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 *w = ws + narrow_partial(c + i, c + i == first ? slot0 : 0, m, gr, mb, p.tp);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[i][j] = c + i <= last ? __ldcg(w + j * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        v[4 * j] += x[i][j].x;
+        v[4 * j + 1] += x[i][j].y;
+        v[4 * j + 2] += x[i][j].z;
+        v[4 * j + 3] += x[i][j].w;
+      }
+  }
+  e.store(ep, n, t0, v, lane, (r_tile * mb + m) * 4 + q);
+}
+
 // MB: 128-row blocks per tile, 1 or 2.
 template <int MODE, int MB>
 __global__ void __launch_bounds__(NW_THREADS, 1)
@@ -180,7 +280,7 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t s_full[NW_MAX_STAGES], s_empty[NW_MAX_STAGES], s_acc_full[2], s_acc_empty[2], s_drain;
   __shared__ uint32_t s_tmem;
-  __shared__ int s_abort, s_last;
+  __shared__ int s_abort;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const uint32_t ring = (smem_addr(smem_raw) + 1023u) & ~1023u;
   const long long U = (long long)p.n_tiles * p.n_kb, G = gridDim.x;
@@ -211,61 +311,65 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
   pdl_launch_dependents();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---- TMA producer: the i-th K block of the CTA's range uses stage i % S.  Weights do not
-      // depend on the previous kernel: the first round of them is under way before the wait on it
-      const uint64_t pol = policy_evict_first();
-      const uint32_t bytes = x_off + (uint32_t)p.tp * p.terms * 128u;
-      // the ring position and the (tile, K block) of the next weight and token loads
-      struct At {
-        int s, use, kb, r, t;  // stage, its use, K block, row tile, token tile
-      };
-      const int tile0 = (int)(u0 / p.n_kb);
-      At w = {0, 0, (int)(u0 % p.n_kb), tile0 / p.t_tiles, tile0 % p.t_tiles}, x = w;
-      auto next = [&](At &a) {
-        if (++a.s == p.stages) a.s = 0, ++a.use;
-        if (++a.kb == p.n_kb) {
-          a.kb = 0;
-          if (++a.t == p.t_tiles) a.t = 0, ++a.r;
-        }
-      };
-      auto weights = [&]() {
-        const uint32_t full = smem_addr(&s_full[w.s]), dst = ring + w.s * p.stage_bytes;
+    // ---- TMA producer (the whole warp, one elected lane issuing): the i-th K block of the CTA's range
+    // uses stage i % S.  Weights do not depend on the previous kernel: the first round of them is
+    // under way before the wait on it
+    const uint64_t pol = policy_evict_first();
+    const uint32_t bytes = x_off + (uint32_t)p.tp * p.terms * 128u;
+    // the ring position and the (tile, K block) of the next weight and token loads
+    struct At {
+      int s, use, kb, r, t;  // stage, its use, K block, row tile, token tile
+    };
+    const int tile0 = (int)(u0 / p.n_kb);
+    At w = {0, 0, (int)(u0 % p.n_kb), tile0 / p.t_tiles, tile0 % p.t_tiles}, x = w;
+    auto next = [&](At &a) {
+      if (++a.s == p.stages) a.s = 0, ++a.use;
+      if (++a.kb == p.n_kb) {
+        a.kb = 0;
+        if (++a.t == p.t_tiles) a.t = 0, ++a.r;
+      }
+    };
+    auto weights = [&]() {
+      const uint32_t full = smem_addr(&s_full[w.s]), dst = ring + w.s * p.stage_bytes;
+      if (elect_one()) {
         mbar_arrive_expect_tx(full, bytes);
+#pragma unroll
         for (int m = 0; m < MB; ++m)
           tma_load_4d_hint(dst + m * NW_W_BYTES, &tm_w, (w.kb & 1) * 64, 0, w.kb >> 1, (w.r * MB + m) * (128 / RB),
                            full, pol);
-        next(w);
-      };
-      auto tokens = [&]() {
-        tma_load_3d(ring + x.s * p.stage_bytes + x_off, &tm_x, x.kb * 64, x.t * p.tp, 0, smem_addr(&s_full[x.s]));
-        next(x);
-      };
-      const int total = (int)(u1 - u0), lead = min(total, p.stages);
-      for (int i = 0; i < lead; ++i) weights();
-      pdl_wait();
-      asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
-      for (int i = 0; i < lead; ++i) tokens();
-      bool ok = true;
-      for (int i = lead; i < total; ++i) {
-        if (*abort_flag || !mbar_wait(smem_addr(&s_empty[w.s]), (uint32_t)(w.use - 1) & 1)) {
-          ok = false;
-          break;
-        }
-        weights();
-        tokens();
       }
-      if (!ok) {
+      __syncwarp();
+      next(w);
+    };
+    auto tokens = [&]() {
+      if (elect_one())
+        tma_load_3d(ring + x.s * p.stage_bytes + x_off, &tm_x, x.kb * 64, x.t * p.tp, 0, smem_addr(&s_full[x.s]));
+      __syncwarp();
+      next(x);
+    };
+    const int total = (int)(u1 - u0), lead = min(total, p.stages);
+    for (int i = 0; i < lead; ++i) weights();
+    pdl_wait();
+    asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
+    for (int i = 0; i < lead; ++i) tokens();
+    bool ok = true;
+    for (int i = lead; i < total; ++i) {
+      ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_empty[w.s]), (uint32_t)(w.use - 1) & 1));
+      if (!ok) break;
+      weights();
+      tokens();
+    }
+    if (!ok) {
+      if (lane == 0) {
         *abort_flag = 1;
         atomicOr(ep.err, ERR_TIMEOUT);
-        // let the copies in flight land: stage s was last filled in its use number w.use - (s >= w.s)
-        for (int s = 0; s < p.stages; ++s) {
-          const int last = w.use - (s >= w.s ? 1 : 0);
-          if (last >= 0) mbar_wait(smem_addr(&s_full[s]), (uint32_t)last & 1);
-        }
+      }
+      // let the copies in flight land: stage s was last filled in its use number w.use - (s >= w.s)
+      for (int s = 0; s < p.stages; ++s) {
+        const int last = w.use - (s >= w.s ? 1 : 0);
+        if (last >= 0) mbar_wait(smem_addr(&s_full[s]), (uint32_t)last & 1);
       }
     }
-    __syncwarp();
   } else if (warp == 1) {
     // ---- MMA issuer (the whole warp, one elected lane issuing): segment i of the range (one row
     // tile's share) accumulates into buffer i % bufs
@@ -291,10 +395,12 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
         const uint32_t a = ring + s * p.stage_bytes;
         const uint64_t da = sdesc_k_sw128(a), db = sdesc_k_sw128(a + x_off);
         if (elect_one()) {
+          // one accumulator after the other: at N = 256 an MMA takes 128 cycles behind one on the same
+          // accumulator, 150 behind one on another
 #pragma unroll
-          for (int k = 0; k < 4; ++k)  // 16 K values further: 32 bytes, 2 in the descriptor's units
+          for (int m = 0; m < MB; ++m)
 #pragma unroll
-            for (int m = 0; m < MB; ++m)
+            for (int k = 0; k < 4; ++k)  // 16 K values further: 32 bytes, 2 in the descriptor's units
               mma_bf16_ss(d + m * p.acc_cols, da + m * (NW_W_BYTES >> 4) + 2 * k, db + 2 * k, idesc, (i | k) != 0);
           mma_commit(smem_addr(&s_empty[s]));
         }
@@ -312,112 +418,344 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
     __syncwarp();
     mbar_wait(smem_addr(&s_drain), 0);
   } else {
-    // ---- epilogue warps: TMEM lanes 32 q .. (q = warp % 4) are 32 consecutive rows of the tile;
-    // the two warps of a quadrant take alternate groups of 16 tokens
-    pdl_wait();  // h, the partial sums and the outputs may still be in use by the previous kernel
-    const int q = warp & 3, grp = (warp - 2) >> 2, row = 32 * q + lane;
-    const int groups = p.tp / 16;
-    const size_t part = (size_t)MB * p.tp * 128;  // floats of one partial
-    int seg = 0;
-    for (long long u = u0; u < u1; ++seg) {
-      const int tile = (int)(u / p.n_kb);
-      const long long t_lo = (long long)tile * p.n_kb, t_hi = t_lo + p.n_kb, end = min(u1, t_hi);
-      const int buf = p.bufs == 2 ? seg & 1 : 0;
-      const bool ready = named_bar_and(
-          1, NW_EPI_THREADS,
-          !*abort_flag && mbar_wait(smem_addr(&s_acc_full[buf]), (uint32_t)(p.bufs == 2 ? seg >> 1 : seg) & 1));
-      if (!ready) {
-        if (lane == 0) {
-          *abort_flag = 1;
-          atomicOr(ep.err, ERR_TIMEOUT);
+    narrow_epilogue_warps<MODE, MB>(p, ep, tmem, u0, u1, s_acc_full, s_acc_empty, abort_flag);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem, p.tmem_cols);
+  }
+}
+
+// ---------------------------------------------------------------------------- int4 weights
+// The same product with int4 weights decoded on the way: a K unit is half an int4 tile (128 columns)
+// of the tile's 256 rows, whose codes and scales (17 KiB, four row blocks) arrive by bulk copies;
+// eight converter warps turn each 64-column half into the swizzled fp16 A operand of the MMAs (code x
+// scale rounded to fp16, as dequant_int4_f16_kernel rounds it), while the tokens' slices arrive by TMA
+// beside it.  Reads of HBM are the int4 bytes alone: dequantizing a matrix to an fp16 copy first
+// costs 4.5 times its bytes (0.53 read, 2 written and 2 read again).
+// 256 rows to a tile: a token slice (up to 32 KiB) is read from L2 once per 16 KiB of fp16 weights of
+// two 128-row blocks, and each converter warp has two independent 16-row groups in hand.
+// Measured, one 72B-shaped block: 1206 -> 261 us at 16 tokens, 1228 -> 359 at 100, 2188 -> 1298 at 512 and
+// 2939 -> 2468 at 900, against fp16 copies made ahead on a second stream (745 us of a block's time
+// whatever the prompt).  Bound by the converters at few tokens and by the MMAs from about 100.
+constexpr int N4_CONV_WARPS = 8;
+constexpr int N4_CONV_WARP = 10;  // the first converter warp
+constexpr int N4_THREADS = (N4_CONV_WARP + N4_CONV_WARPS) * 32;
+constexpr int N4_A_BYTES = 2 * NW_W_BYTES;                                   // 256 rows x 64 fp16
+constexpr int N4_RB_BYTES = TILE4_CODE_BYTES / 2 + TILE4_SCALE_BYTES / 2;    // one row block's half tile
+constexpr int N4_CODE_BYTES = 4 * N4_RB_BYTES;
+constexpr int N4_MAX_CODE_STAGES = 8, N4_MAX_A_STAGES = 3, N4_MAX_X_STAGES = 6;
+
+// The rings of a CTA: code stages, operand (A) stages and token stages.
+struct Narrow4Params {
+  const uint8_t *tiles;
+  int n_rb, n_kt;
+  int c_stages, a_stages, x_stages, x_bytes;
+};
+
+
+__device__ __forceinline__ void stsm_x4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2),
+               "r"(r3)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t hmul2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t hfma2(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t r;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+
+// The eight codes of an A-fragment word as exact fp16 pairs: rows gid and gid + 8 of columns 2 tig,
+// 2 tig + 1 (c0, c1) and of columns 2 tig + 8, 2 tig + 9 (c2, c3).  The nibbles, top bit flipped, become
+// 1024 + u or 1024 + 16 u (u = code + 8).
+__device__ __forceinline__ void decode_word(uint32_t w, uint32_t &c0, uint32_t &c1, uint32_t &c2, uint32_t &c3) {
+  const uint32_t w8 = w >> 8;
+  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c0) : "r"(w), "r"(0x000F000Fu), "r"(0x64086408u));
+  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c1) : "r"(w8), "r"(0x000F000Fu), "r"(0x64086408u));
+  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c2) : "r"(w), "r"(0x00F000F0u), "r"(0x64806480u));
+  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c3) : "r"(w8), "r"(0x00F000F0u), "r"(0x64806480u));
+  c0 = hfma2(c0, 0x3C003C00u, 0xE408E408u);  // - 1032
+  c1 = hfma2(c1, 0x3C003C00u, 0xE408E408u);
+  c2 = hfma2(c2, 0x2C002C00u, 0xD480D480u);  // / 16 - 72
+  c3 = hfma2(c3, 0x2C002C00u, 0xD480D480u);
+}
+
+// fp16 pair of codes times an fp32 scale, rounded once.
+__device__ __forceinline__ uint32_t scale_pair_f32(uint32_t c, float sc) {
+  return (uint32_t)f32_to_f16_rn(f16_to_f32((uint16_t)c) * sc) |
+         ((uint32_t)f32_to_f16_rn(f16_to_f32((uint16_t)(c >> 16)) * sc) << 16);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(N4_THREADS, 1)
+    prefill_narrow4_kernel(const Narrow4Params r, const __grid_constant__ CUtensorMap tm_x, NarrowParams p,
+                           PrefillEpiParams ep) {
+  constexpr int MB = 2;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t s_cfull[N4_MAX_CODE_STAGES], s_cempty[N4_MAX_CODE_STAGES], s_xfull[N4_MAX_X_STAGES],
+      s_xempty[N4_MAX_X_STAGES], s_afull[N4_MAX_A_STAGES], s_aempty[N4_MAX_A_STAGES], s_acc_full[2], s_acc_empty[2],
+      s_drain;
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
+  const uint32_t a_ring = (smem_addr(smem_raw) + 1023u) & ~1023u;
+  const uint32_t x_ring = a_ring + r.a_stages * N4_A_BYTES;
+  const uint32_t codes = x_ring + r.x_stages * r.x_bytes;  // [code stage][row block][codes, scales]
+  const long long U = (long long)p.n_tiles * p.n_kb, G = gridDim.x;
+  const long long u0 = blockIdx.x * U / G, u1 = (blockIdx.x + 1) * U / G;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < r.c_stages; ++s) {
+      mbar_init(smem_addr(&s_cfull[s]), 1);
+      mbar_init(smem_addr(&s_cempty[s]), N4_CONV_WARPS);
+    }
+    for (int s = 0; s < r.a_stages; ++s) {
+      mbar_init(smem_addr(&s_afull[s]), N4_CONV_WARPS);
+      mbar_init(smem_addr(&s_aempty[s]), 1);
+    }
+    for (int s = 0; s < r.x_stages; ++s) {
+      mbar_init(smem_addr(&s_xfull[s]), 1);
+      mbar_init(smem_addr(&s_xempty[s]), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_addr(&s_acc_full[b]), 1);
+      mbar_init(smem_addr(&s_acc_empty[b]), NW_EPI_THREADS / 32);
+    }
+    mbar_init(smem_addr(&s_drain), 1);
+    s_abort = 0;
+    fence_mbar_init();
+  }
+  __syncwarp();
+  if (warp == 0) tmem_alloc(smem_addr(&s_tmem), p.tmem_cols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_tmem;
+  volatile int *abort_flag = &s_abort;
+  pdl_launch_dependents();
+
+  if (warp == 0) {
+    // ---- producer (the whole warp, one elected lane issuing): units' codes as the code ring frees,
+    // their two token slices as the token ring does
+    const uint64_t pol = p.t_tiles == 1 ? policy_evict_first() : policy_evict_normal();
+    struct At {
+      int kb, r, t;  // K unit, row tile, token tile
+    };
+    const int tile0 = (int)(u0 / p.n_kb);
+    At w = {(int)(u0 % p.n_kb), tile0 / p.t_tiles, tile0 % p.t_tiles}, x = w;
+    auto next = [&](At &a) {
+      if (++a.kb == p.n_kb) {
+        a.kb = 0;
+        if (++a.t == p.t_tiles) a.t = 0, ++a.r;
+      }
+    };
+    const int total = (int)(u1 - u0);
+    int cs = 0, cuse = 0, xs = 0, xuse = 0, c_done = 0, x_done = 0, half = 0;
+    auto issue_codes = [&]() {
+      const uint32_t full = smem_addr(&s_cfull[cs]), dst = codes + cs * N4_CODE_BYTES;
+      if (elect_one()) {
+        mbar_arrive_expect_tx(full, N4_CODE_BYTES);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          // row blocks past the end repeat the last: their rows are beyond N and never stored
+          const int rb = min(w.r * 4 + b, r.n_rb - 1);
+          const uint8_t *t = r.tiles + ((size_t)rb * r.n_kt + (w.kb >> 1)) * TILE4_BYTES;
+          bulk_g2s(dst + b * N4_RB_BYTES, t + (w.kb & 1) * (TILE4_CODE_BYTES / 2), TILE4_CODE_BYTES / 2, full, pol);
+          bulk_g2s(dst + b * N4_RB_BYTES + TILE4_CODE_BYTES / 2,
+                   t + TILE4_CODE_BYTES + (w.kb & 1) * (TILE4_SCALE_BYTES / 2), TILE4_SCALE_BYTES / 2, full, pol);
         }
+      }
+      __syncwarp();
+      next(w);
+      ++c_done;
+      if (++cs == r.c_stages) cs = 0, ++cuse;
+    };
+    auto issue_tokens = [&]() {
+      const uint32_t full = smem_addr(&s_xfull[xs]);
+      if (elect_one()) {
+        mbar_arrive_expect_tx(full, r.x_bytes);
+        tma_load_3d(x_ring + xs * r.x_bytes, &tm_x, x.kb * 128 + half * 64, x.t * p.tp, 0, full);
+      }
+      __syncwarp();
+      if (half) next(x);
+      half ^= 1;
+      ++x_done;
+      if (++xs == r.x_stages) xs = 0, ++xuse;
+    };
+    while (c_done < min(total, r.c_stages)) issue_codes();
+    pdl_wait();
+    asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
+    while (x_done < min(2 * total, r.x_stages)) issue_tokens();
+    bool ok = true;
+    // whichever ring has room goes first; one of them always will, or a wait elsewhere gives up
+    for (uint32_t idle = 0; x_done < 2 * total || c_done < total;) {
+      bool did = false;
+      if (c_done < total && __any_sync(0xffffffffu, mbar_test_wait(smem_addr(&s_cempty[cs]), (uint32_t)(cuse - 1) & 1))) {
+        issue_codes();
+        did = true;
+      }
+      if (x_done < 2 * total && __any_sync(0xffffffffu, mbar_test_wait(smem_addr(&s_xempty[xs]), (uint32_t)(xuse - 1) & 1))) {
+        issue_tokens();
+        did = true;
+      }
+      idle = did ? 0 : idle + 1;
+      if (__any_sync(0xffffffffu, *abort_flag != 0) || idle > WAIT_LIMIT) {
+        ok = false;
         break;
       }
-      tc_fence_after();
-      const bool whole = u == t_lo && end == t_hi;
-      const int r_tile = tile / p.t_tiles, tt0 = (tile % p.t_tiles) * p.tp;
-      for (int m = 0; m < MB; ++m) {
-        const int n = (r_tile * MB + m) * 128 + row;
-        for (int gr = grp; gr < groups; gr += 2) {
-          const int t0 = tt0 + gr * 16;
-          if (t0 >= ep.T) break;
-          NarrowEpilogue<MODE> e;
-          if (whole) e.load(ep, n, t0, lane);
-          const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((buf * MB + m) * p.acc_cols + gr * 16);
-          uint32_t r0[16], r1[16], r2[16];
-          tmem_ld16(ta, r0);
-          tmem_ld16(ta + p.tp, r1);
-          if (p.terms == 3) tmem_ld16(ta + 2 * p.tp, r2);
-          tmem_wait_ld();
-          float v[16];
-          // the smaller terms first
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float lo = p.terms == 3 ? __uint_as_float(r1[j]) + __uint_as_float(r2[j]) : __uint_as_float(r1[j]);
-            v[j] = __uint_as_float(r0[j]) + lo;
-          }
-          if (whole) {
-            e.store(ep, n, t0, v, lane, (r_tile * MB + m) * 4 + q);
-          } else {
-            // this CTA's slot 0: the range starts inside the tile; slot 1: it ends inside
-            float4 *w = reinterpret_cast<float4 *>(p.ws + ((size_t)blockIdx.x * 2 + (u > t_lo ? 0 : 1)) * part) +
-                        (size_t)(m * groups + gr) * 4 * 128 + row;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) w[j * 128] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-          }
-        }
+      if (idle >= WAIT_FAST_SPINS) __nanosleep(64);
+    }
+    if (!ok) {
+      if (lane == 0) {
+        *abort_flag = 1;
+        atomicOr(ep.err, ERR_TIMEOUT);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_addr(&s_acc_empty[buf]));
-      if (!whole) {
-        // the CTAs that share the tile are first .. last; the last to take the ticket sums their
-        // partials in CTA order, four partials (256 bytes a thread) in flight
-        const int first = (int)(((t_lo + 1) * G - 1) / U), last = (int)((t_hi * G - 1) / U);
-        const int slot0 = first * U / G > t_lo ? 0 : 1;  // of CTA `first`; the others start inside the tile
-        named_bar_sync(1, NW_EPI_THREADS);
-        if (threadIdx.x == 64) {
-          const unsigned old = atom_add_acq_rel(p.tickets + tile, 1u);
-          s_last = old == (unsigned)(last - first);
-          if (s_last) p.tickets[tile] = 0;
+      for (int s = 0; s < r.c_stages; ++s) {
+        const int last = cuse - (s >= cs ? 1 : 0);
+        if (last >= 0) mbar_wait(smem_addr(&s_cfull[s]), (uint32_t)last & 1);
+      }
+      for (int s = 0; s < r.x_stages; ++s) {
+        const int last = xuse - (s >= xs ? 1 : 0);
+        if (last >= 0) mbar_wait(smem_addr(&s_xfull[s]), (uint32_t)last & 1);
+      }
+    }
+  } else if (warp == 1) {
+    // ---- MMA issuer, as in prefill_narrow_kernel; a unit is two stages
+    const uint32_t idesc = idesc_kind_f16(128, p.tp * p.terms, false);
+    int as = 0, xs = 0, left = (int)(u1 - u0), n = p.n_kb - (int)(u0 % p.n_kb);
+    uint32_t ause = 0, xuse = 0;
+    bool ok = true;
+    for (int seg = 0; left > 0 && ok; ++seg, n = p.n_kb) {
+      n = min(n, left);
+      left -= n;
+      const int buf = p.bufs == 2 ? seg & 1 : 0;
+      if (seg >= p.bufs) {
+        const uint32_t back = (uint32_t)(p.bufs == 2 ? (seg >> 1) - 1 : seg - 1);
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&s_acc_empty[buf]), back & 1));
+        if (!ok) break;
+      }
+      tc_fence_after();
+      const uint32_t d = tmem + (uint32_t)(buf * MB * p.acc_cols);
+      for (int i = 0; i < 2 * n; ++i) {
+        ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_xfull[xs]), xuse & 1) &&
+                                         mbar_wait(smem_addr(&s_afull[as]), ause & 1));
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t da = sdesc_k_sw128(a_ring + as * N4_A_BYTES), db = sdesc_k_sw128(x_ring + xs * r.x_bytes);
+        if (elect_one()) {
+#pragma unroll
+          for (int m = 0; m < MB; ++m)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              mma_bf16_ss(d + m * p.acc_cols, da + m * (NW_W_BYTES >> 4) + 2 * k, db + 2 * k, idesc, (i | k) != 0);
+          mma_commit(smem_addr(&s_aempty[as]));
+          mma_commit(smem_addr(&s_xempty[xs]));
         }
-        named_bar_sync(1, NW_EPI_THREADS);
-        if (s_last) {
-          for (int m = 0; m < MB; ++m) {
-            const int n = (r_tile * MB + m) * 128 + row;
-            for (int gr = grp; gr < groups; gr += 2) {
-              const int t0 = tt0 + gr * 16;
-              if (t0 >= ep.T) break;
-              const float4 *at = reinterpret_cast<const float4 *>(p.ws) + (size_t)(m * groups + gr) * 4 * 128 + row;
-              NarrowEpilogue<MODE> e;
-              e.load(ep, n, t0, lane);
-              float v[16] = {};
-              for (int c = first; c <= last; c += 4) {
-                float4 x[4][4];
+        __syncwarp();
+        if (++as == r.a_stages) as = 0, ++ause;
+        if (++xs == r.x_stages) xs = 0, ++xuse;
+      }
+      if (ok && elect_one()) mma_commit(smem_addr(&s_acc_full[buf]));
+      __syncwarp();
+    }
+    if (!ok && lane == 0) {
+      *abort_flag = 1;
+      atomicOr(ep.err, ERR_TIMEOUT);
+    }
+    if (elect_one()) mma_commit(smem_addr(&s_drain));  // every MMA issued has completed before TMEM is freed
+    __syncwarp();
+    mbar_wait(smem_addr(&s_drain), 0);
+  } else if (warp < N4_CONV_WARP) {
+    narrow_epilogue_warps<MODE, MB>(p, ep, tmem, u0, u1, s_acc_full, s_acc_empty, abort_flag);
+  } else {
+    // ---- converters: warp w decodes 16-row groups (row block b, r16) = (w / 4 and w / 4 + 2, w % 4)
+    const int cw = warp - N4_CONV_WARP, r16 = cw & 3, gid = lane >> 2;
+    // where this lane's stmatrix row goes: matrices 0..3 are rows 0-7 and 8-15 of columns 0-7, then of
+    // columns 8-15 of each 16-column step j; 16-byte chunks of a 128-byte row XOR the row (mod 8)
+    const int mrow = (lane & 7) + ((lane >> 3) & 1) * 8, mcol = lane >> 4;
+    uint32_t off[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  const float4 *w = at + ((size_t)(c + i) * 2 + (c + i == first ? slot0 : 0)) * (part / 4);
+    for (int j = 0; j < 4; ++j) off[j] = (uint32_t)((r16 * 16 + mrow) * 128 + (((2 * j + mcol) ^ (lane & 7)) << 4));
+    int cs = 0, s = 0;
+    uint32_t cuse = 0, use = 0;
+    const int total = (int)(u1 - u0);
+    bool ok = true;
+    for (int i = 0; i < total && ok; ++i) {
+      ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_cfull[cs]), cuse & 1));
+      if (!ok) break;
+      // the unit's codes and scales of this warp's rows: [half][group]
+      const uint32_t src = codes + cs * N4_CODE_BYTES + (cw >> 2) * N4_RB_BYTES;
+      uint4 w[2][2];
+      uint32_t sc[2][2];
+      bool exact = true;
 #pragma unroll
-                  for (int j = 0; j < 4; ++j)
-                    x[i][j] = c + i <= last ? __ldcg(w + j * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+      for (int half = 0; half < 2; ++half)
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+        for (int g = 0; g < 2; ++g) {
+          const uint32_t blk = src + 2 * g * N4_RB_BYTES;
+          uint4 &v = w[half][g];
+          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                       : "r"(blk + r16 * 1024 + half * 512 + lane * 16));
+          asm volatile("ld.shared.u32 %0, [%1];"
+                       : "=r"(sc[half][g])
+                       : "r"(blk + TILE4_CODE_BYTES / 2 + (((half * 8 + gid) * 4 + r16) * 4)));
+        }
+      // a bf16 scale that fp16 holds exactly: the fp16 product of code and scale is rounded as the
+      // fp32 product would be; others (below 2^-14, or too large) go through fp32
 #pragma unroll
-                  for (int j = 0; j < 4; ++j) {
-                    v[4 * j] += x[i][j].x;
-                    v[4 * j + 1] += x[i][j].y;
-                    v[4 * j + 2] += x[i][j].z;
-                    v[4 * j + 3] += x[i][j].w;
-                  }
-              }
-              e.store(ep, n, t0, v, lane, (r_tile * MB + m) * 4 + q);
+      for (int half = 0; half < 2; ++half)
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const float s0 = bf16_lo(sc[half][g]), s1 = bf16_hi(sc[half][g]);
+          exact = exact && f16_to_f32(f32_to_f16_rn(s0)) == s0 && f16_to_f32(f32_to_f16_rn(s1)) == s1;
+        }
+      exact = __all_sync(0xffffffffu, exact);
+      if (lane == 0) mbar_arrive(smem_addr(&s_cempty[cs]));
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        ok = ok && (use == 0 || __all_sync(0xffffffffu, mbar_wait(smem_addr(&s_aempty[s]), (use - 1) & 1)));
+        if (!ok) break;
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          // row block b = cw / 4 + 2 g: rows 64 (b % 2) of 128-row block b / 2
+          const uint32_t dst = a_ring + s * N4_A_BYTES + g * NW_W_BYTES + (cw >> 2) * (64 * 128);
+          const float s0 = bf16_lo(sc[half][g]), s1 = bf16_hi(sc[half][g]);
+          const uint32_t words[4] = {w[half][g].x, w[half][g].y, w[half][g].z, w[half][g].w};
+          if (exact) {
+            const uint32_t p0 = f32_to_f16_rn(s0) * 0x10001u, p1 = f32_to_f16_rn(s1) * 0x10001u;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              uint32_t c0, c1, c2, c3;
+              decode_word(words[j], c0, c1, c2, c3);
+              stsm_x4(dst + off[j], hmul2(c0, p0), hmul2(c1, p1), hmul2(c2, p0), hmul2(c3, p1));
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              uint32_t c0, c1, c2, c3;
+              decode_word(words[j], c0, c1, c2, c3);
+              stsm_x4(dst + off[j], scale_pair_f32(c0, s0), scale_pair_f32(c1, s1), scale_pair_f32(c2, s0),
+                      scale_pair_f32(c3, s1));
             }
           }
         }
-        named_bar_sync(1, NW_EPI_THREADS);  // s_last is read by all before the next segment writes it
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stores, before the MMAs read them
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_addr(&s_afull[s]));
+        if (++s == r.a_stages) s = 0, ++use;
       }
-      u = end;
+      if (++cs == r.c_stages) cs = 0, ++cuse;
+    }
+    if (!ok && lane == 0) {
+      *abort_flag = 1;
+      atomicOr(ep.err, ERR_TIMEOUT);
     }
   }
   tc_fence_before();
@@ -434,32 +772,54 @@ size_t narrow_ws_bytes(int n_sm, int T) {
   // two slots per CTA of 256 rows x tp tokens
   return (size_t)n_sm * 2 * 256 * std::min(NW_MAX_TP, (T + 15) / 16 * 16) * sizeof(float);
 }
-int narrow_max_tiles(int N) { return (N + 127) / 128; }
+int narrow_argmax_slots(int N) { return (N + 127) / 128 * 4; }
 
-template <int MODE, int MB>
-static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x, const NarrowParams &p, int grid,
-                                      const PrefillEpiParams &ep, cudaStream_t s) {
-  static bool set = false;
-  if (!set) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(prefill_narrow_kernel<MODE, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, NW_SMEM);
-    if (e != cudaSuccess) return e;
-    set = true;
-  }
+// Opts a kernel in to a block's whole shared memory; returns its dynamic part (the rings start on
+// the KiB boundary after the kernel's own barriers), or -1.
+static int ring_smem(const void *kernel) {
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, kernel) != cudaSuccess || a.sharedSizeBytes > 1024) return -1;
+  const int dyn = NW_RING + 1024 - (int)a.sharedSizeBytes;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) == cudaSuccess ? dyn : -1;
+}
+
+template <int MODE>
+static cudaError_t launch_narrow_reduce(const NarrowParams &p, int mb, int grid, const PrefillEpiParams &ep,
+                                        cudaStream_t s) {
+  if (p.n_tiles % grid == 0) return cudaSuccess;  // every range is whole tiles
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(NW_THREADS);
-  cfg.dynamicSmemBytes = NW_SMEM;
+  cfg.gridDim = dim3((unsigned)(p.n_tiles * mb * (p.tp / 16)));
+  cfg.blockDim = dim3(128);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   pdl_attribute(attr[0]);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, prefill_narrow_kernel<MODE, MB>, w, x, p, ep);
+  return cudaLaunchKernelEx(&cfg, narrow_reduce_kernel<MODE>, p, mb, grid, ep);
+}
+
+template <int MODE, int MB>
+static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x, const NarrowParams &p, int grid,
+                                      const PrefillEpiParams &ep, cudaStream_t s) {
+  static const int smem = ring_smem(reinterpret_cast<const void *>(prefill_narrow_kernel<MODE, MB>));
+  if (smem < 0) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(NW_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  pdl_attribute(attr[0]);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_narrow_kernel<MODE, MB>, w, x, p, ep);
+  return e == cudaSuccess ? launch_narrow_reduce<MODE>(p, MB, grid, ep, s) : e;
 }
 
 int narrow_tp(int T, int terms) {
-  return std::min((T + 15) / 16 * 16, terms == 2 ? NW_MAX_TP : 80);  // terms * tp <= 256 MMA columns
+  const int most = terms == 2 ? NW_MAX_TP : 80;  // terms * tp <= 256 MMA columns
+  const int tiles = (T + most - 1) / most;
+  return ((T + tiles - 1) / tiles + 15) / 16 * 16;
 }
 
 cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensorMap &x, int K, int terms,
@@ -469,7 +829,6 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensor
   p.terms = terms;
   p.tp = narrow_tp(ep.T, terms);
   p.t_tiles = (ep.T + p.tp - 1) / p.tp;
-  if (mode == PE_ARGMAX && p.t_tiles != 1) return cudaErrorInvalidValue;
   const int cols = p.tp * terms;
   // wide tiles of many rows share their tokens' slices between two 128-row blocks: the slices (2 x
   // 16 KiB of terms at 128 tokens) then cost no more L2 reads than the weights
@@ -481,9 +840,8 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensor
   p.tmem_cols = 32;
   while (p.tmem_cols < p.bufs * mb * p.acc_cols) p.tmem_cols *= 2;
   p.stage_bytes = mb * NW_W_BYTES + cols * 128;
-  p.stages = std::min(NW_MAX_STAGES, (NW_SMEM - 1024) / p.stage_bytes);
+  p.stages = std::min(NW_MAX_STAGES, NW_RING / p.stage_bytes);
   p.ws = ws.partial;
-  p.tickets = ws.tickets;
   // at least four K blocks per CTA: finer splits cost more in partial sums than they stream sooner
   const long long U = (long long)p.n_tiles * p.n_kb;
   const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min<long long>(p.n_tiles, ws.n_sm), U / 4));
@@ -493,6 +851,60 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensor
   };
   switch (mode) {
     case PE_STORE: return go(std::integral_constant<int, PE_STORE>());
+    case PE_RESID: return go(std::integral_constant<int, PE_RESID>());
+    case PE_SWIGLU: return go(std::integral_constant<int, PE_SWIGLU>());
+    case PE_QKV: return go(std::integral_constant<int, PE_QKV>());
+    case PE_ARGMAX: return go(std::integral_constant<int, PE_ARGMAX>());
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int MODE>
+static cudaError_t launch_narrow4_mode(const Narrow4Params &r, const CUtensorMap &x, const NarrowParams &p, int grid,
+                                       const PrefillEpiParams &ep, cudaStream_t s) {
+  static const int smem = ring_smem(reinterpret_cast<const void *>(prefill_narrow4_kernel<MODE>));
+  if (smem < 0) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(N4_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  pdl_attribute(attr[0]);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_narrow4_kernel<MODE>, r, x, p, ep);
+  return e == cudaSuccess ? launch_narrow_reduce<MODE>(p, 2, grid, ep, s) : e;
+}
+
+cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int n_kt, const CUtensorMap &x, int K,
+                                   int terms, const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
+  if (ep.T <= 0 || ep.N <= 0) return cudaSuccess;
+  NarrowParams p = {};
+  p.terms = terms;
+  p.tp = narrow_tp(ep.T, terms);
+  p.t_tiles = (ep.T + p.tp - 1) / p.tp;
+  const int cols = p.tp * terms;
+  p.n_kb = (K + 127) / 128;
+  p.n_tiles = (ep.N + 255) / 256 * p.t_tiles;
+  p.acc_cols = (cols + 31) / 32 * 32;
+  p.bufs = 4 * p.acc_cols <= 512 ? 2 : 1;
+  p.tmem_cols = 32;
+  while (p.tmem_cols < p.bufs * 2 * p.acc_cols) p.tmem_cols *= 2;
+  // three code stages at least (70 KiB ahead of the converters with what they hold), then the token ring
+  // (slices come from L2: about a microsecond), then more codes
+  Narrow4Params r = {tiles, n_rb, n_kt, 0, 0, 0, cols * 128};
+  r.a_stages = r.x_bytes <= 16384 ? 3 : 2;
+  r.x_stages = std::min(N4_MAX_X_STAGES, (NW_RING - r.a_stages * N4_A_BYTES - 3 * N4_CODE_BYTES) / r.x_bytes);
+  r.c_stages = std::min(N4_MAX_CODE_STAGES, (NW_RING - r.a_stages * N4_A_BYTES - r.x_stages * r.x_bytes) / N4_CODE_BYTES);
+  p.ws = ws.partial;
+  // at least two units (2 x 128 columns) per CTA, as prefill_narrow_kernel's four K blocks of 64
+  const long long U = (long long)p.n_tiles * p.n_kb;
+  const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min<long long>(p.n_tiles, ws.n_sm), U / 2));
+  auto go = [&](auto m) {
+    return launch_narrow4_mode<decltype(m)::value>(r, x, p, grid, ep, s);
+  };
+  switch (mode) {
     case PE_RESID: return go(std::integral_constant<int, PE_RESID>());
     case PE_SWIGLU: return go(std::integral_constant<int, PE_SWIGLU>());
     case PE_QKV: return go(std::integral_constant<int, PE_QKV>());

@@ -265,8 +265,8 @@ struct kfl_stage {
   float *pf_h = nullptr;
   uint16_t *pf_q = nullptr;
   uint16_t *pf_x = nullptr, *pf_o = nullptr, *pf_a = nullptr;  // GEMM inputs as terms [term][token][ld]
-  NarrowWorkspace pf_nw = {};  // the few-token GEMM's partial sums and tickets
-  int pf_n_tickets = 0, pf_amax_cols = 0;
+  NarrowWorkspace pf_nw = {};  // the few-token GEMM's partial sums
+  int pf_amax_cols = 0;
   int *pf_pos = nullptr, *pf_aidx = nullptr;
   float *pf_amax = nullptr;
   std::vector<void *> pf_allocs;
@@ -796,10 +796,15 @@ constexpr int PF_PASS = 2048;  // tokens per pass of the dense prefill
 
 int pf_ld(int n) { return round_up(n, 64); }
 
+// Whether a pass of n tokens runs on the few-token GEMM.
+bool pf_narrow(const kfl_stage *st, int n) {
+  return n <= (st->cfg.weight_fmt == KFL_BF16 ? NW_MAX_TP : env_int("KFL_N4_MAX", N4_MAX_TOKENS));
+}
+
 // Workspace for passes of up to `tokens` tokens (grown, never shrunk) and the weight maps.
 int ensure_prefill(kfl_stage *st, int tokens) {
   const Plan &P = st->P;
-  const int cap = std::min(PF_PASS, round_up(tokens, PG_M));
+  const int cap = std::min(PF_PASS, round_up(tokens, PG_M)), first = std::min(PF_PASS, tokens);
   if (cap > st->pf_cap) {
     for (void *p : st->pf_allocs) cudaFree(p);
     st->pf_allocs.clear();
@@ -816,20 +821,18 @@ int ensure_prefill(kfl_stage *st, int tokens) {
               get((void **)&st->pf_x, (size_t)2 * cap * pf_ld(P.d) * 2) &&
               get((void **)&st->pf_o, (size_t)2 * cap * pf_ld(P.qdim) * 2) &&
               get((void **)&st->pf_a, (size_t)2 * cap * pf_ld(P.F) * 2) && get((void **)&st->pf_pos, (size_t)cap * 4);
-    // argmax partials: per 256-column tile, or (up to NW_MAX_TP tokens) per 32 rows
-    const size_t am = std::max((size_t)cap * ((P.V + PG_N - 1) / PG_N),
-                               (size_t)std::min(cap, NW_MAX_TP) * narrow_max_tiles(P.V) * 4);
-    ok = ok && get((void **)&st->pf_amax, am * 4) && get((void **)&st->pf_aidx, am * 4);
-    int most = std::max(std::max(P.qkv.N, P.o.N), std::max(P.gu.N, P.down.N));
-    if (st->flags & KFL_LOGITS_OUT) most = std::max(most, P.V);
-    st->pf_n_tickets = narrow_max_tiles(most);
+    // argmax partials: per 256-column tile, or (passes on the few-token GEMM) per 32 rows
+    if (st->flags & KFL_LOGITS_OUT) {
+      const int narrow = std::min(cap, st->cfg.weight_fmt == KFL_BF16 ? NW_MAX_TP : N4_MAX_TOKENS);
+      const size_t am = std::max((size_t)cap * ((P.V + PG_N - 1) / PG_N), (size_t)narrow * narrow_argmax_slots(P.V));
+      ok = ok && get((void **)&st->pf_amax, am * 4) && get((void **)&st->pf_aidx, am * 4);
+    }
     st->pf_nw.n_sm = P.n_sm;
-    ok = ok && get((void **)&st->pf_nw.partial, narrow_ws_bytes(P.n_sm, cap)) &&
-         get((void **)&st->pf_nw.tickets, (size_t)st->pf_n_tickets * 4);
+    ok = ok && get((void **)&st->pf_nw.partial, narrow_ws_bytes(P.n_sm, cap));
     if (!ok) return KFL_ERR_OOM;
     st->pf_cap = cap;
   }
-  if (st->pf_maps.empty() && st->cfg.weight_fmt == KFL_INT4_G64) {
+  if (st->pf_maps.empty() && st->cfg.weight_fmt == KFL_INT4_G64 && !pf_narrow(st, first)) {
     // the fp16 scratch holds the largest matrix; its maps are per matrix kind
     const Mat *kinds[5] = {&P.qkv, &P.o, &P.gu, &P.down, &P.lm};
     const int n_kinds = (st->flags & KFL_LOGITS_OUT) ? 5 : 4;
@@ -862,7 +865,7 @@ int ensure_prefill(kfl_stage *st, int tokens) {
           return KFL_ERR_CUDA;
     st->pf_maps = std::move(maps);
   }
-  if (st->pf_maps.empty()) {
+  if (st->pf_maps.empty() && st->cfg.weight_fmt == KFL_BF16) {
     std::vector<CUtensorMap> maps(4 * P.nl + 1), narrow(4 * P.nl + 1);
     auto encode = [&](int i, const Mat &m) {
       return encode_tiles_map(&maps[i], m.tiles, m.n_kt, m.n_rb, PG_N / RB) ||
@@ -915,9 +918,6 @@ cudaError_t pf_dequant(kfl_stage *st, int g) {
   return err;
 }
 
-// Whether a pass of n tokens runs on the few-token GEMM.
-bool pf_narrow(const kfl_stage *st, int n) { return st->cfg.weight_fmt == KFL_BF16 && n <= NW_MAX_TP; }
-
 // int4: start of a pass on stream s: both buffers free once s's earlier work is done; the first
 // matrix is dequantized.
 cudaError_t pf_pass_begin(kfl_stage *st, cudaStream_t s) {
@@ -968,6 +968,8 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
     e.aidx = st->pf_aidx;
     e.n_tiles = st->pf_amax_cols;
   }
+  if (pf_narrow(st, x.n) && i4)
+    return launch_prefill_narrow4(mode, m.tiles, m.n_rb, m.n_kt, x.all, m.K, x.terms, st->pf_nw, e, s);
   if (pf_narrow(st, x.n))
     return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], x.all, m.K, x.terms, st->pf_nw, e, s);
   if (i4) {
@@ -1003,13 +1005,13 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
     const bool narrow = pf_narrow(st, n);
     CK(launch_prefill_input(ids ? ids + t0 : nullptr, hidden_in ? hidden_in + (size_t)t0 * P.d : nullptr,
                             positions + t0, n, embed ? st->embed : nullptr, P.V, P.d, P.ldh, st->pf_h, st->pf_pos,
-                            st->cfg.max_ctx, st->pf_nw.tickets, st->pf_n_tickets, st->err, s));
-    CK(pf_pass_begin(st, s));
+                            st->cfg.max_ctx, st->err, s));
+    if (!narrow) CK(pf_pass_begin(st, s));
     PfInput x, o, a;
     if (x.encode(st->pf_x, P.d, n, 2, narrow) || o.encode(st->pf_o, P.qdim, n, 2, narrow) ||
         a.encode(st->pf_a, P.F, n, 2, narrow))
       return KFL_ERR_CUDA;
-    st->pf_amax_cols = narrow ? narrow_max_tiles(P.V) * 4 : (P.V + PG_N - 1) / PG_N;
+    st->pf_amax_cols = narrow ? narrow_argmax_slots(P.V) : (P.V + PG_N - 1) / PG_N;
     auto norm = [&](const float *g) {
       return launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, g, eps, x.base, x.base + x.stride, x.ld, i4, st->err, s);
     };

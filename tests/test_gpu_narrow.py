@@ -1,6 +1,7 @@
 """GPU parity of the prefill's few-token matrix product (stream-K over the SMs, weight rows as the MMA's
 rows) at the edges of its tiles: token groups of 16 up to 128, row tiles of 128 and (many rows, more
-than 64 tokens) 256, one K block of 64 up to several per CTA, with ragged tails.
+than 64 tokens) 256, one K block of 64 up to several per CTA, with ragged tails; and its int4 form,
+which decodes the weights on the way (256-row tiles, K units of 128).
 
 The plain product against fp64: x carried to about 2^-16 relative by its two terms, fp32
 accumulation, so each element within 1e-4 of its row's RMS plus 2^-14 relative (the bar of the
@@ -12,9 +13,11 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from gpu_helpers import Pair, ensure_built
 from paper_2609_34045_gb300 import stage as K
-from test_gpu_parity import RAGGED, RAGGED128
+from paper_2609_34045_gb300 import workload as wl
+from test_gpu_parity import RAGGED, RAGGED128, RAGGED_INT4
 from test_gpu_prefill import _prefill
 
 pytestmark = pytest.mark.gpu
@@ -46,11 +49,43 @@ def test_product_matches_fp64(T, Kd, N):
 
 
 @pytest.mark.parametrize("model,n", [(RAGGED, 16), (RAGGED, 65), (RAGGED, 128), (RAGGED128, 33),
-                                     (dataclasses.replace(RAGGED, vocab=30000), 70)])
+                                     (dataclasses.replace(RAGGED, vocab=30000), 70), (RAGGED_INT4, 16),
+                                     (RAGGED_INT4, 65), (RAGGED_INT4, 100), (RAGGED_INT4, 129)])
 def test_prefill_matches_the_oracle(model, n, monkeypatch):
+    # (the bar holds the attention's bf16 q and softmax weights too: at d_model 448, ffn 1024 they alone
+    # give 1.02e-2 to 3.3e-2 of the RMS over three seeds, the same to 2e-6 with the 128-token tiles)
     monkeypatch.setenv("KFL_PREFILL_DENSE_MIN", "1")
     p = Pair(model, 0, 2, K.KFL_IS_HEAD, 2, (5, 30), 192, seed=43, max_batch=2)
     for _ in range(2):
         _prefill(p, 1, 30, n, 43, True)
     p.compare_kv()
     p.close()
+
+
+def test_int4_scales_below_the_fp16_normals():
+    """Scales that fp16 cannot hold exactly (2^-14 and below, bf16 significands) take the fp32 product
+    of code and scale.  The down projection's are set to 2^-16 and below: fp16 weights of 2^-24
+    resolution then carry about 2^-9 relative, averaged over 704 products, so the block's
+    contribution stays within 1e-2 of its RMS."""
+    m, n, seed = RAGGED_INT4, 40, 47
+    w = wl.layer_weights(m, 0, seed)
+    words, scales = w["wd"]
+    w["wv"] = (np.zeros_like(w["wv"][0]), w["wv"][1])  # attention adds nothing
+    w["wd"] = (words, wl.f32_to_bf16_bits(wl.bf16_bits_to_f32(scales) * np.float32(2.0 ** -9)))
+    st = K.kfl_stage_create(K.model_cfg(m, 64, 1), 0, 1, 0)
+    K.kfl_stage_load_layer(st, 0, w, on_device=False)
+    ora = oracle.OracleStage(m, 0, 1, False, False, 1, 64)
+    ora.load_layer(0, w)
+    hidden = wl.hidden_in(m, 0, n, seed) * np.float32(2.0 ** -8)
+    pos = np.arange(n, dtype=np.int32)
+    ref = ora.prefill(0, pos, hidden_in=hidden)["hidden_out"]
+    out = torch.zeros(n, m.d_model, device="cuda")
+    K.kfl_stage_prefill(st, None, torch.tensor(hidden, device="cuda"), torch.tensor(pos, device="cuda"), 0, n, out, None,
+                        torch.cuda.current_stream().cuda_stream)
+    assert K.kfl_stage_status(st) == 0
+    got = out.cpu().numpy()
+    # the block's contribution alone (the sum with the hidden states is fp32: exact to 1e-7 of them)
+    delta = ref - hidden
+    rms = np.sqrt(np.mean(delta * delta, axis=1, keepdims=True))
+    assert np.all(np.abs(got - hidden - delta) <= 1e-2 * rms)
+    K.kfl_stage_destroy(st)
