@@ -58,7 +58,7 @@ extern "C" {
  * lim(i); section V-D, admission).  qk_norm: 0, or 1 for Qwen3-family blocks (the models served
  * in section VI): each head of q and of k is RMS-normalised over head_dim with its own gain (the
  * layer's q_norm, k_norm; epsilon rms_eps) before RoPE.  A qk_norm stage runs one kernel per
- * phase (KFL_PERSISTENT is ignored) and prefills through decode steps. */
+ * phase (KFL_PERSISTENT is ignored). */
 typedef struct {
   int n_layers_total, d_model, n_heads, n_kv_heads, head_dim, ffn, vocab;
   float rms_eps, rope_theta;
@@ -159,11 +159,14 @@ int kfl_stage_decode_users(kfl_stage *st, const int32_t *token_ids, const float 
  * one decode step, Section VI, instrumentation paragraph).  From KFL_PREFILL_DENSE_MIN tokens
  * (environment, default 16) the prompt runs densely: passes of up to 2048 tokens through
  * tensor-core matrix products (tcgen05) and causal attention, each activation carried as two
- * 16-bit terms (bf16 with bf16 weights; fp16 with int4 weights, dequantized to fp16 tiles in
- * device memory the stage allocates at its first dense prefill).  Shorter prompts, and every
- * prompt of a qk_norm stage, go as steps of up to max_batch rows, in order, every row of a step
- * addressing the user's slot (the decode step's kernels).  Enqueued on cuda_stream, returns
- * without waiting.
+ * 16-bit terms (bf16 with bf16 weights; fp16 with int4 weights, decoded in the products or, for
+ * passes of more than 1024 tokens, dequantized to fp16 tiles first; the workspace is allocated at
+ * the stage's first dense prefill).  bf16 stages run a qk_norm stage's prompts, and prompts that
+ * are shorter (while KFL_PREFILL_DENSE_MIN is not set) but longer than one step, densely at the
+ * decode steps' precision (three bf16 terms per activation).  Other prompts, and those while a
+ * capture, trace or profile is on or for which no workspace can be allocated, go as steps of up
+ * to max_batch rows, in order, every row of a step addressing the user's slot (the decode step's
+ * kernels).  Enqueued on cuda_stream, returns without waiting.
  *   token_ids  device int32[n_tokens] (KFL_EMBED_IN), else ignored
  *   hidden_in  device fp32[n_tokens][d_model] (without KFL_EMBED_IN)
  *   positions  device int32[n_tokens]: token t's position, distinct, normally start + t; the

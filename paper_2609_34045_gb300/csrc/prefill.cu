@@ -101,6 +101,22 @@ __device__ __forceinline__ void epilogue32(const PrefillEpiParams &ep, int t, in
       } else {
         dst = ep.kcache + (((size_t)ep.slot * ep.hkv + head) * ep.max_ctx + pos) * ep.hd;
       }
+      if (is_q && ep.out) {  // q in fp32
+        float *q1 = ep.out + (size_t)t * ep.ldo + (size_t)head * ep.hd + i0, *q2 = q1 + half;
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) {
+          float y1[4], y2[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float a1 = v[2 * (i + j)], a2 = v[2 * (i + j) + 1];
+            y1[j] = a1 * c[i + j] - a2 * sv[i + j];
+            y2[j] = a2 * c[i + j] + a1 * sv[i + j];
+          }
+          *reinterpret_cast<float4 *>(q1 + i) = make_float4(y1[0], y1[1], y1[2], y1[3]);
+          *reinterpret_cast<float4 *>(q2 + i) = make_float4(y2[0], y2[1], y2[2], y2[3]);
+        }
+        return;
+      }
       // rotated first halves -> dst[i0 ..], second halves -> dst[i0 + hd/2 ..]: 32 bytes each
       uint32_t w1[8], w2[8];
 #pragma unroll
@@ -462,9 +478,21 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
 // user's cache rows [0, position]: S = Q K^T and O = P V on bf16 m16n8k16 MMAs, softmax online
 // over key blocks of 64 rows double-buffered in shared memory (rows padded by 16 bytes so the
 // matrix loads are free of bank conflicts).
+//
+// A short prompt has few such blocks (28 at 43 tokens and 28 heads) while its keys may be many: the
+// key blocks are then split over a cluster of up to 8 CTAs, whose (m, l, O) meet in distributed
+// shared memory in rank order (43 tokens at 700: a serial chain of 12 key blocks, 31 us, on 28 of
+// 152 SMs before).
+//
+// PRECISE: q is fp32 and enters, like the softmax weights, as a bf16 pair (rounded + rest, about 2^-17),
+// as in the decode step's attention; the output has p.terms terms.  Twice the MMAs: taken for passes of up
+// to 512 tokens and wherever the GEMMs run on few-token tiles (7B-shaped, 43 tokens at 700: the block's
+// error against 64 bits 5.2e-4 -> 1.8e-5, the four-block pass 615 -> 564 us with the split; 500
+// tokens 1.2e-3 -> 1.7e-4 for 1% of the pass).
 
 constexpr int PA_ROWS = 64;
 constexpr int PA_THREADS = 128;
+constexpr int PA_MAX_SPLIT = 8;  // CTAs of a key-split cluster
 
 __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                          uint32_t b0, uint32_t b1) {
@@ -500,8 +528,32 @@ struct PaLayout {
   static constexpr int K_OFF = TILE;          // 2 buffers
   static constexpr int V_OFF = 3 * TILE;      // 2 buffers
   static constexpr int POS_OFF = 5 * TILE;    // int [64]
-  static constexpr int BYTES = POS_OFF + PA_ROWS * 4;
+  static constexpr int ML_OFF = POS_OFF + PA_ROWS * 4;  // float (m, l) [64]
+  static constexpr int BYTES = ML_OFF + PA_ROWS * 8;
+  // after the key loop, where K and V were: this CTA's O [64][O_LD] for its cluster
+  static constexpr int O_LD = HD + 4;
+  static_assert(PA_ROWS * O_LD * 4 <= 4 * TILE, "O fits where K and V were");
 };
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+
+// Two values as packed pairs of bf16 (rounded) and of what rounding left (bf16 again).
+__device__ __forceinline__ void pair_bf16(float x0, float x1, uint32_t &hi, uint32_t &lo) {
+  hi = pack_bf16(x0, x1);
+  lo = pack_bf16(x0 - bf16_lo(hi), x1 - bf16_hi(hi));
+}
 
 // Rows [r0, r0 + 64) of a [rows][HD] bf16 matrix (row stride ld elements) into a padded tile;
 // rows at or above `limit` are zero.
@@ -518,7 +570,19 @@ __device__ __forceinline__ void pa_load_tile(uint8_t *tile, const uint16_t *src,
   }
 }
 
-template <int HD>
+// Two consecutive output elements as the O projection's input terms.
+__device__ __forceinline__ void store_terms(const PrefillAttnParams &p, size_t at, float x0, float x1) {
+  uint32_t hi, lo;
+  split_pack(x0, x1, hi, lo, p.f16, p.err);
+  *reinterpret_cast<uint32_t *>(p.o + at) = hi;
+  *reinterpret_cast<uint32_t *>(p.o + p.term_stride + at) = lo;
+  if (p.terms == 3) {  // bf16 terms: what the first two leave
+    const float r0 = x0 - bf16_lo(hi) - bf16_lo(lo), r1 = x1 - bf16_hi(hi) - bf16_hi(lo);
+    *reinterpret_cast<uint32_t *>(p.o + 2 * p.term_stride + at) = pack_bf16(r0, r1);
+  }
+}
+
+template <int HD, bool PRECISE>
 __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnParams p) {
   using L = PaLayout<HD>;
   extern __shared__ __align__(16) uint8_t sm[];
@@ -529,37 +593,50 @@ __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnPar
   // the longest blocks (latest tokens) first
   const int qb = gridDim.x - 1 - blockIdx.x;
   const int h = blockIdx.y, kvh = h / (p.n_heads / p.n_kv_heads);
+  const int rank = blockIdx.z, n_split = gridDim.z;
   const int t0 = qb * PA_ROWS;
   int *s_pos = reinterpret_cast<int *>(sm + L::POS_OFF);
   if (threadIdx.x < PA_ROWS) s_pos[threadIdx.x] = t0 + threadIdx.x < p.T ? p.positions[t0 + threadIdx.x] : -1;
-  pa_load_tile<HD>(sm + L::Q_OFF, p.q + h * HD, p.ldq, t0, p.T);
+  if constexpr (!PRECISE) pa_load_tile<HD>(sm + L::Q_OFF, p.q + h * HD, p.ldq, t0, p.T);
   cp_async_commit();
   __syncthreads();
   int max_pos = -1;
   for (int i = 0; i < PA_ROWS; ++i) max_pos = max(max_pos, s_pos[i]);
-  const int n_kb = (max_pos + PA_ROWS) / PA_ROWS;  // key blocks covering [0, max_pos]
+  const int n_all = (max_pos + PA_ROWS) / PA_ROWS;  // key blocks covering [0, max_pos]
+  const int kb0 = rank * n_all / n_split, n_kb = (rank + 1) * n_all / n_split;  // this CTA's: [kb0, n_kb)
   const int kv_limit = min(max_pos + 1, p.max_ctx);
   const size_t head_base = ((size_t)p.slot * p.n_kv_heads + kvh) * p.max_ctx * HD;
   const uint16_t *kg = p.kcache + head_base, *vg = p.vcache + head_base;
-  if (n_kb > 0) {
-    pa_load_tile<HD>(sm + L::K_OFF, kg, HD, 0, kv_limit);
-    pa_load_tile<HD>(sm + L::V_OFF, vg, HD, 0, kv_limit);
+  if (kb0 < n_kb) {
+    pa_load_tile<HD>(sm + L::K_OFF, kg, HD, kb0 * PA_ROWS, kv_limit);
+    pa_load_tile<HD>(sm + L::V_OFF, vg, HD, kb0 * PA_ROWS, kv_limit);
   }
   cp_async_commit();
   const int qp0 = s_pos[16 * warp + g], qp1 = s_pos[16 * warp + g + 8];
+  // Q fragments of this warp's 16 rows
+  uint32_t qf[HD / 16][4], ql[PRECISE ? HD / 16 : 1][4];
+  if constexpr (PRECISE) {
+    const int ra = t0 + 16 * warp + g, rb = ra + 8;
+    const float *qa = p.q32 + (size_t)min(ra, p.T - 1) * p.ldq + h * HD, *qr = p.q32 + (size_t)min(rb, p.T - 1) * p.ldq + h * HD;
+#pragma unroll
+    for (int kk = 0; kk < HD / 16; ++kk)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {  // rows g, g + 8; columns 2c, 2c + 1 then + 8
+        const float2 v = *reinterpret_cast<const float2 *>((j & 1 ? qr : qa) + kk * 16 + 2 * c + (j & 2 ? 8 : 0));
+        pair_bf16(v.x, v.y, qf[kk][j], ql[kk][j]);
+      }
+  }
   cp_async_wait_all();
   __syncthreads();
-  // Q fragments of this warp's 16 rows
-  uint32_t qf[HD / 16][4];
-  {
+  if constexpr (!PRECISE) {
     const uint32_t qbase = smem_addr(sm + L::Q_OFF) + (16 * warp + (lane % 16)) * L::ROW + (lane / 16) * 16;
 #pragma unroll
     for (int kk = 0; kk < HD / 16; ++kk) ldsm_x4(qf[kk][0], qf[kk][1], qf[kk][2], qf[kk][3], qbase + kk * 32);
   }
   float oacc[HD / 8][4] = {};
   float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
-  for (int kb = 0; kb < n_kb; ++kb) {
-    const int buf = kb & 1;
+  for (int kb = kb0; kb < n_kb; ++kb) {
+    const int buf = (kb - kb0) & 1;
     if (kb + 1 < n_kb) {  // the next block loads while this one is used
       pa_load_tile<HD>(sm + L::K_OFF + (buf ^ 1) * L::TILE, kg, HD, (kb + 1) * PA_ROWS, kv_limit);
       pa_load_tile<HD>(sm + L::V_OFF + (buf ^ 1) * L::TILE, vg, HD, (kb + 1) * PA_ROWS, kv_limit);
@@ -578,6 +655,10 @@ __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnPar
         ldsm_x4(b0, b1, b2, b3, kbase + (nt * 8 + (lane % 8)) * L::ROW + kk * 32 + (lane / 8) * 16);
         mma16816(s[nt], qf[kk][0], qf[kk][1], qf[kk][2], qf[kk][3], b0, b1);
         mma16816(s[nt], qf[kk + 1][0], qf[kk + 1][1], qf[kk + 1][2], qf[kk + 1][3], b2, b3);
+        if constexpr (PRECISE) {
+          mma16816(s[nt], ql[kk][0], ql[kk][1], ql[kk][2], ql[kk][3], b0, b1);
+          mma16816(s[nt], ql[kk + 1][0], ql[kk + 1][1], ql[kk + 1][2], ql[kk + 1][3], b2, b3);
+        }
       }
     }
     // scale, causal mask, online softmax (rows g and g + 8 of the warp)
@@ -614,51 +695,123 @@ __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnPar
     }
     l0 = l0 * corr0 + rs0;
     l1 = l1 * corr1 + rs1;
+    // O = O corr + P V: 4 key steps of 16; V fragments by transposed matrix loads
+    const uint32_t vlane = vbase + ((lane % 8) + ((lane / 8) & 1) * 8) * L::ROW + (lane / 16) * 16;
+    if constexpr (PRECISE) {
+      // a block's products from zero, added to O in fp32: tensor-core accumulation truncates, and over
+      // thousands of keys that would show (see prefill_narrow_kernel)
+      uint32_t a[4][4], e[4][4];
 #pragma unroll
-    for (int dt = 0; dt < HD / 8; ++dt) {
-      oacc[dt][0] *= corr0;
-      oacc[dt][1] *= corr0;
-      oacc[dt][2] *= corr1;
-      oacc[dt][3] *= corr1;
-    }
-    // O += P V: 4 key steps of 16; V fragments by transposed matrix loads
+      for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t a0 = pack_bf16(s[2 * j][0], s[2 * j][1]), a1 = pack_bf16(s[2 * j][2], s[2 * j][3]);
-      const uint32_t a2 = pack_bf16(s[2 * j + 1][0], s[2 * j + 1][1]), a3 = pack_bf16(s[2 * j + 1][2], s[2 * j + 1][3]);
+        for (int i = 0; i < 4; ++i) pair_bf16(s[2 * j + i / 2][2 * (i & 1)], s[2 * j + i / 2][2 * (i & 1) + 1], a[j][i], e[j][i]);
 #pragma unroll
       for (int dt = 0; dt < HD / 8; dt += 2) {
-        uint32_t b0, b1, b2, b3;
-        ldsm_x4_t(b0, b1, b2, b3,
-                  vbase + (j * 16 + (lane % 8) + ((lane / 8) & 1) * 8) * L::ROW + (dt + lane / 16) * 16);
-        mma16816(oacc[dt], a0, a1, a2, a3, b0, b1);
-        mma16816(oacc[dt + 1], a0, a1, a2, a3, b2, b3);
+        float y[2][4] = {};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          uint32_t b0, b1, b2, b3;
+          ldsm_x4_t(b0, b1, b2, b3, vlane + j * 16 * L::ROW + dt * 16);
+          mma16816(y[0], e[j][0], e[j][1], e[j][2], e[j][3], b0, b1);
+          mma16816(y[1], e[j][0], e[j][1], e[j][2], e[j][3], b2, b3);
+          mma16816(y[0], a[j][0], a[j][1], a[j][2], a[j][3], b0, b1);
+          mma16816(y[1], a[j][0], a[j][1], a[j][2], a[j][3], b2, b3);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          oacc[dt + i][0] = oacc[dt + i][0] * corr0 + y[i][0];
+          oacc[dt + i][1] = oacc[dt + i][1] * corr0 + y[i][1];
+          oacc[dt + i][2] = oacc[dt + i][2] * corr1 + y[i][2];
+          oacc[dt + i][3] = oacc[dt + i][3] * corr1 + y[i][3];
+        }
+      }
+    } else {
+#pragma unroll
+      for (int dt = 0; dt < HD / 8; ++dt) {
+        oacc[dt][0] *= corr0;
+        oacc[dt][1] *= corr0;
+        oacc[dt][2] *= corr1;
+        oacc[dt][3] *= corr1;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t a0 = pack_bf16(s[2 * j][0], s[2 * j][1]), a1 = pack_bf16(s[2 * j][2], s[2 * j][3]);
+        const uint32_t a2 = pack_bf16(s[2 * j + 1][0], s[2 * j + 1][1]), a3 = pack_bf16(s[2 * j + 1][2], s[2 * j + 1][3]);
+#pragma unroll
+        for (int dt = 0; dt < HD / 8; dt += 2) {
+          uint32_t b0, b1, b2, b3;
+          ldsm_x4_t(b0, b1, b2, b3, vlane + j * 16 * L::ROW + dt * 16);
+          mma16816(oacc[dt], a0, a1, a2, a3, b0, b1);
+          mma16816(oacc[dt + 1], a0, a1, a2, a3, b2, b3);
+        }
       }
     }
     cp_async_wait_all();
     __syncthreads();
   }
-  // row sums over the quad, normalize, store bf16
+  // row sums over the quad
   l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
   l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
   l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
   l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
+  if (n_split > 1) {
+    // this CTA's state for the cluster; every warp is past its last key block (the loop ends in a barrier)
+    float *so = reinterpret_cast<float *>(sm + L::K_OFF);
+    float2 *sml = reinterpret_cast<float2 *>(sm + L::ML_OFF);
+    const int r = 16 * warp + g;
+#pragma unroll
+    for (int dt = 0; dt < HD / 8; ++dt) {
+      *reinterpret_cast<float2 *>(so + r * L::O_LD + dt * 8 + 2 * c) = make_float2(oacc[dt][0], oacc[dt][1]);
+      *reinterpret_cast<float2 *>(so + (r + 8) * L::O_LD + dt * 8 + 2 * c) = make_float2(oacc[dt][2], oacc[dt][3]);
+    }
+    if (c == 0) {
+      sml[r] = make_float2(m0, l0);
+      sml[r + 8] = make_float2(m1, l1);
+    }
+    cluster_sync_all();
+    // rank k merges rows [k 64 / n, (k + 1) 64 / n), four columns per thread and step
+    const int rows = PA_ROWS / n_split;
+    for (int e = threadIdx.x; e < rows * (HD / 4); e += PA_THREADS) {
+      const int row = rank * rows + e / (HD / 4), col = e % (HD / 4) * 4, t = t0 + row;
+      float2 ml[PA_MAX_SPLIT];
+      float4 o[PA_MAX_SPLIT];
+#pragma unroll
+      for (int k = 0; k < PA_MAX_SPLIT; ++k)
+        if (k < n_split) {
+          ml[k] = ld_cluster_f2(map_to_rank(smem_addr(sml + row), k));
+          o[k] = ld_cluster_f4(map_to_rank(smem_addr(so + row * L::O_LD + col), k));
+        }
+      float m = -INFINITY;
+#pragma unroll
+      for (int k = 0; k < PA_MAX_SPLIT; ++k)
+        if (k < n_split) m = fmaxf(m, ml[k].x);
+      float l = 0.f, y[4] = {};
+#pragma unroll
+      for (int k = 0; k < PA_MAX_SPLIT; ++k)
+        if (k < n_split && ml[k].x > -INFINITY) {
+          const float w = exp2f(ml[k].x - m);
+          l += ml[k].y * w;
+          y[0] += o[k].x * w;
+          y[1] += o[k].y * w;
+          y[2] += o[k].z * w;
+          y[3] += o[k].w * w;
+        }
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      if (t < p.T) {
+        store_terms(p, (size_t)t * p.ldo + h * HD + col, y[0] * inv, y[1] * inv);
+        store_terms(p, (size_t)t * p.ldo + h * HD + col + 2, y[2] * inv, y[3] * inv);
+      }
+    }
+    cluster_sync_all();  // no CTA leaves while others read its shared memory
+    return;
+  }
   const float inv0 = l0 > 0.f ? 1.f / l0 : 0.f, inv1 = l1 > 0.f ? 1.f / l1 : 0.f;
   const int ta = t0 + 16 * warp + g, tb = ta + 8;
 #pragma unroll
   for (int dt = 0; dt < HD / 8; ++dt) {
     const int col = h * HD + dt * 8 + 2 * c;
-    uint32_t hi, lo;
-    if (ta < p.T) {
-      split_pack(oacc[dt][0] * inv0, oacc[dt][1] * inv0, hi, lo, p.f16, p.err);
-      *reinterpret_cast<uint32_t *>(p.o + (size_t)ta * p.ldo + col) = hi;
-      *reinterpret_cast<uint32_t *>(p.o_lo + (size_t)ta * p.ldo + col) = lo;
-    }
-    if (tb < p.T) {
-      split_pack(oacc[dt][2] * inv1, oacc[dt][3] * inv1, hi, lo, p.f16, p.err);
-      *reinterpret_cast<uint32_t *>(p.o + (size_t)tb * p.ldo + col) = hi;
-      *reinterpret_cast<uint32_t *>(p.o_lo + (size_t)tb * p.ldo + col) = lo;
-    }
+    if (ta < p.T) store_terms(p, (size_t)ta * p.ldo + col, oacc[dt][0] * inv0, oacc[dt][1] * inv0);
+    if (tb < p.T) store_terms(p, (size_t)tb * p.ldo + col, oacc[dt][2] * inv1, oacc[dt][3] * inv1);
   }
 }
 
@@ -668,9 +821,10 @@ __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnPar
 // holds the same position.
 __global__ void prefill_input_kernel(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                      const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                     int max_ctx, unsigned *err) {
+                                     int max_ctx, int user, int *slots, unsigned *err) {
   const int t = blockIdx.x;
   pdl_launch_dependents();
+  if (slots && threadIdx.x == 0) slots[t] = user;
   __shared__ int s_bad;
   if (threadIdx.x == 0) s_bad = 0;
   __syncthreads();
@@ -695,10 +849,16 @@ __global__ void prefill_input_kernel(const int *ids, const float *hidden_in, con
     h[(size_t)t * ldh + i] = embed ? bf16_to_f32(embed[(size_t)id * d + i]) : hidden_in[(size_t)t * d + i];
 }
 
-// x[t] = h[t] / rms(h[t]) * g as hi and lo 16-bit terms, one block per token, four elements per
+// What rounding leaves out of the fp32 product a * b * c (to first order).
+__device__ __forceinline__ float product3_rest(float a, float b, float c) {
+  const float p = a * b;
+  return fmaf(fmaf(a, b, -p), c, fmaf(p, c, -(p * c)));
+}
+
+// x[t] = h[t] / rms(h[t]) * g as two or three 16-bit terms (term_stride elements apart), one block per token, four elements per
 // thread step (d a multiple of 8; h, g and x rows 16-byte aligned).
 __global__ void prefill_rmsnorm_kernel(const float *h, int ldh, int d, const float *g, float eps, uint16_t *x,
-                                       uint16_t *x_lo, int ldx, int f16, unsigned *err) {
+                                       size_t term_stride, int terms, int ldx, int f16, unsigned *err) {
   const int t = blockIdx.x, d4 = d / 4;
   pdl_launch_dependents();
   pdl_wait();
@@ -718,16 +878,23 @@ __global__ void prefill_rmsnorm_kernel(const float *h, int ldh, int d, const flo
     if (threadIdx.x == 0) red[0] = v;
   }
   __syncthreads();
-  const float inv = rsqrtf(red[0] / d + eps);
+  const float inv = 1.0f / sqrtf(red[0] / d + eps);
   const float4 *g4 = reinterpret_cast<const float4 *>(g);
-  uint2 *xh = reinterpret_cast<uint2 *>(x + (size_t)t * ldx), *xl = reinterpret_cast<uint2 *>(x_lo + (size_t)t * ldx);
+  uint2 *xh = reinterpret_cast<uint2 *>(x + (size_t)t * ldx), *xl = reinterpret_cast<uint2 *>(x + term_stride + (size_t)t * ldx);
+  uint2 *xr = reinterpret_cast<uint2 *>(x + 2 * term_stride + (size_t)t * ldx);
   for (int i = threadIdx.x; i < d4; i += blockDim.x) {
     const float4 v = row[i], gg = g4[i];
     uint2 hi, lo;
-    split_pack(v.x * inv * gg.x, v.y * inv * gg.y, hi.x, lo.x, f16, err);
-    split_pack(v.z * inv * gg.z, v.w * inv * gg.w, hi.y, lo.y, f16, err);
+    const float y0 = v.x * inv * gg.x, y1 = v.y * inv * gg.y, y2 = v.z * inv * gg.z, y3 = v.w * inv * gg.w;
+    split_pack(y0, y1, hi.x, lo.x, f16, err);
+    split_pack(y2, y3, hi.y, lo.y, f16, err);
     xh[i] = hi;
     xl[i] = lo;
+    if (terms == 3)  // bf16 terms: what the first two, and the products' roundings, leave
+      xr[i] = make_uint2(pack_bf16(y0 - bf16_lo(hi.x) - bf16_lo(lo.x) + product3_rest(v.x, inv, gg.x),
+                                   y1 - bf16_hi(hi.x) - bf16_hi(lo.x) + product3_rest(v.y, inv, gg.y)),
+                         pack_bf16(y2 - bf16_lo(hi.y) - bf16_lo(lo.y) + product3_rest(v.z, inv, gg.z),
+                                   y3 - bf16_hi(hi.y) - bf16_hi(lo.y) + product3_rest(v.w, inv, gg.w)));
   }
 }
 
@@ -981,35 +1148,52 @@ cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a, const CUtensorMa
   }
 }
 
-template <int HD>
-static cudaError_t launch_attn_hd(const PrefillAttnParams &p, cudaStream_t s) {
+template <int HD, bool PRECISE>
+static cudaError_t launch_attn_hd(const PrefillAttnParams &p, int n_sm, cudaStream_t s) {
   static bool attr = false;
   const int bytes = PaLayout<HD>::BYTES;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_attn_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaFuncSetAttribute(prefill_attn_kernel<HD, PRECISE>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  const dim3 grid((p.T + PA_ROWS - 1) / PA_ROWS, p.n_heads);
-  return launch_pdl(prefill_attn_kernel<HD>, grid, PA_THREADS, bytes, s, p);
+  // split the keys until about two CTAs per SM (as many as fit) have work
+  const int blocks = (p.T + PA_ROWS - 1) / PA_ROWS * p.n_heads;
+  int split = 1;
+  while (split < PA_MAX_SPLIT && blocks * split * 2 <= 2 * n_sm) split *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((p.T + PA_ROWS - 1) / PA_ROWS, p.n_heads, split);
+  cfg.blockDim = dim3(PA_THREADS);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  pdl_attribute(at[0]);
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 1;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = split;
+  cfg.attrs = at;
+  cfg.numAttrs = split > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, prefill_attn_kernel<HD, PRECISE>, p);
 }
 
-cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, cudaStream_t s) {
+cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, int n_sm, cudaStream_t s) {
   if (p.T <= 0) return cudaSuccess;
-  return hd == 128 ? launch_attn_hd<128>(p, s) : launch_attn_hd<64>(p, s);
+  if (p.q32) return hd == 128 ? launch_attn_hd<128, true>(p, n_sm, s) : launch_attn_hd<64, true>(p, n_sm, s);
+  return hd == 128 ? launch_attn_hd<128, false>(p, n_sm, s) : launch_attn_hd<64, false>(p, n_sm, s);
 }
 
 cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                  const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                 int max_ctx, unsigned *err, cudaStream_t s) {
+                                 int max_ctx, int user, int *slots, unsigned *err, cudaStream_t s) {
   prefill_input_kernel<<<T, 256, 0, s>>>(ids, hidden_in, positions_in, T, embed, vocab, d, ldh, h, positions,
-                                         max_ctx, err);
+                                         max_ctx, user, slots, err);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const float *g, float eps, uint16_t *x,
-                                   uint16_t *x_lo, int ldx, int f16, unsigned *err, cudaStream_t s) {
-  return launch_pdl(prefill_rmsnorm_kernel, dim3(T), 256, 0, s, h, ldh, d, g, eps, x, x_lo, ldx, f16, err);
+                                   size_t term_stride, int terms, int ldx, int f16, unsigned *err, cudaStream_t s) {
+  return launch_pdl(prefill_rmsnorm_kernel, dim3(T), 256, 0, s, h, ldh, d, g, eps, x, term_stride, terms, ldx, f16, err);
 }
 
 cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, cudaStream_t s) {

@@ -49,7 +49,7 @@ struct PrefillEpiParams {
   int ldo16;
   int terms;               // PE_SWIGLU: terms stored, term_stride elements apart
   size_t term_stride;
-  // PE_QKV: rows [0, qdim) q, [qdim, qdim + kvdim) k (pairs (i, i + hd/2) adjacent per head, as
+  // PE_QKV (out not NULL: q in fp32 to out [T][ldo] instead of out16): rows [0, qdim) q, [qdim, qdim + kvdim) k (pairs (i, i + hd/2) adjacent per head, as
   // the weights were loaded), then v in natural order; K/V stored at the token's position of
   // KV slot `slot` of this layer's caches [max_batch][Hkv][max_ctx][hd]
   uint16_t *kcache, *vcache;
@@ -69,9 +69,11 @@ struct PrefillEpiParams {
 
 struct PrefillAttnParams {
   const uint16_t *q;       // [T][ldq] bf16, RoPE applied, heads in natural order
+  const float *q32;        // not NULL: q in fp32 instead, carried (like the softmax weights) as bf16 pairs
   int ldq;
-  uint16_t *o, *o_lo;      // [T][ldo]: the output as hi and lo terms (fp16 if f16, else bf16)
-  int ldo, f16;
+  uint16_t *o;             // [T][ldo]: the output as 2 or 3 terms, term_stride apart (fp16 if f16, else bf16)
+  int ldo, f16, terms;
+  size_t term_stride;
   const uint16_t *kcache, *vcache;  // this layer's [max_batch][Hkv][max_ctx][hd]
   const int *positions;    // [T], -1: refused (output 0)
   int slot, T, n_heads, n_kv_heads, max_ctx;
@@ -115,12 +117,12 @@ inline void pdl_attribute(cudaLaunchAttribute &a) {
 int prefill_splits(int T, int N, int n_kt, int n_sm);
 cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a_hi, const CUtensorMap &a_lo, const CUtensorMap &b,
                                 int n_kt, const PrefillEpiParams &ep, cudaStream_t s);
-cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, cudaStream_t s);
+cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, int n_sm, cudaStream_t s);
 cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                  const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,
-                                 int max_ctx, unsigned *err, cudaStream_t s);
+                                 int max_ctx, int user, int *slots, unsigned *err, cudaStream_t s);
 cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const float *g, float eps, uint16_t *x,
-                                   uint16_t *x_lo, int ldx, int f16, unsigned *err, cudaStream_t s);
+                                   size_t term_stride, int terms, int ldx, int f16, unsigned *err, cudaStream_t s);
 // int4 group-64 tiles [n_rb][n_kt][TILE4_BYTES] -> fp16 tiles [n_rb][2 n_kt][RB][KT] of code x scale.
 cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, cudaStream_t s);
 cudaError_t launch_split_bf16(const float *x, int T, int K, int ldx, uint16_t *hi, uint16_t *lo, int ld,

@@ -28,6 +28,8 @@ namespace {
 constexpr int NW_WARPS = 10;             // TMA, MMA, 8 epilogue warps
 constexpr int NW_THREADS = NW_WARPS * 32;
 constexpr int NW_EPI_THREADS = 256;
+constexpr int NW_DRAIN_TP = 80;          // tokens of a tile of three terms
+constexpr int NW_DRAIN_KB = 2;           // K blocks per drained accumulator
 constexpr int NW_EPI_WARP = 2;            // the first epilogue warp
 constexpr int NW_MAX_STAGES = 12;
 constexpr int NW_RING = 226 * 1024;      // shared memory of the rings: a block's 227 KiB less the barriers' KiB
@@ -40,6 +42,7 @@ struct NarrowParams {
   int stages, stage_bytes;
   int acc_cols;     // TMEM columns of one 128-row accumulator (tp * terms rounded up to 32)
   int bufs;         // accumulators: 1 or 2
+  int chunk;        // K blocks that one accumulator takes before the epilogue warps add it up (DRAIN; else all)
   int tmem_cols;
   float *ws;        // partial sums (narrow_partial)
 };
@@ -124,13 +127,18 @@ struct NarrowEpilogue {
         // rows (2 i, 2 i + 1) of a head are its RoPE pair (i, i + hd / 2)
         const bool odd = lane & 1, is_q = n - lane < ep.qdim;
         const int r0 = is_q ? n : n - ep.qdim, head = r0 / ep.hd, i = (r0 % ep.hd) / 2, at = odd ? i + ep.hd / 2 : i;
+        float *q32 = is_q && ep.out ? ep.out + (size_t)t0 * ep.ldo + (size_t)head * ep.hd + at : nullptr;
         uint16_t *base = is_q ? ep.out16 + (size_t)t0 * ep.ldo16 + (size_t)head * ep.hd + at
                               : ep.kcache + ((size_t)ep.slot * ep.hkv + head) * ep.max_ctx * ep.hd + at;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const float other = __shfl_xor_sync(0xffffffffu, v[j], 1);
           const float y = odd ? v[j] * a[j] + other * b[j] : v[j] * a[j] - other * b[j];
-          if (pos[j] >= 0 && row_ok) base[is_q ? (size_t)j * ep.ldo16 : (size_t)pos[j] * ep.hd] = f32_to_bf16_rne(y);
+          if (q32) {
+            if (pos[j] >= 0 && row_ok) q32[(size_t)j * ep.ldo] = y;
+          } else if (pos[j] >= 0 && row_ok) {
+            base[is_q ? (size_t)j * ep.ldo16 : (size_t)pos[j] * ep.hd] = f32_to_bf16_rne(y);
+          }
         }
       } else {
         const int r0 = n - ep.qdim - ep.kvdim;
@@ -165,10 +173,11 @@ struct NarrowEpilogue {
 
 // The epilogue warps' part of a CTA with range [u0, u1) of the U units: every segment's sums, from its
 // accumulator to the outputs or, where CTAs share the tile, to the partial sums (narrow_reduce_kernel).
-template <int MODE, int MB>
+template <int MODE, int MB, bool DRAIN>
 __device__ __forceinline__ void narrow_epilogue_warps(const NarrowParams &p, const PrefillEpiParams &ep, uint32_t tmem,
                                                       long long u0, long long u1, uint64_t *s_acc_full,
                                                       uint64_t *s_acc_empty, volatile int *abort_flag) {
+  static_assert(!DRAIN || MB == 1, "a drained tile's sums fit the registers");
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   // ---- epilogue warps: TMEM lanes 32 q .. (q = warp % 4) are 32 consecutive rows of the tile;
   // the two warps of a quadrant take alternate groups of 16 tokens
@@ -176,56 +185,95 @@ __device__ __forceinline__ void narrow_epilogue_warps(const NarrowParams &p, con
   const int q = warp & 3, grp = (warp - NW_EPI_WARP) >> 2, row = 32 * q + lane;
   const int groups = p.tp / 16;
   int seg = 0;
-  for (long long u = u0; u < u1; ++seg) {
-    const int tile = (int)(u / p.n_kb);
-    const long long t_lo = (long long)tile * p.n_kb, t_hi = t_lo + p.n_kb, end = min(u1, t_hi);
-    const int buf = p.bufs == 2 ? seg & 1 : 0;
-    const bool ready = __all_sync(
-        0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_acc_full[buf]), (uint32_t)(p.bufs == 2 ? seg >> 1 : seg) & 1));
-    if (!ready) {
-      if (lane == 0) {
-        *abort_flag = 1;
-        atomicOr(ep.err, ERR_TIMEOUT);
-      }
-      break;
+  // accumulator number `seg` (a segment, or a chunk of one) is complete; false: given up
+  auto wait_acc = [&]() {
+    const uint32_t bar = smem_addr(&s_acc_full[p.bufs == 2 ? seg & 1 : 0]);
+    const bool ready =
+        __all_sync(0xffffffffu, !*abort_flag && mbar_wait(bar, (uint32_t)(p.bufs == 2 ? seg >> 1 : seg) & 1));
+    if (!ready && lane == 0) {
+      *abort_flag = 1;
+      atomicOr(ep.err, ERR_TIMEOUT);
     }
     tc_fence_after();
-    const bool whole = u == t_lo && end == t_hi;
-    const int r_tile = tile / p.t_tiles, tt0 = (tile % p.t_tiles) * p.tp;
-    for (int m = 0; m < MB; ++m) {
-      const int n = (r_tile * MB + m) * 128 + row;
-      for (int gr = grp; gr < groups; gr += 2) {
-        const int t0 = tt0 + gr * 16;
-        if (t0 >= ep.T) break;
-        NarrowEpilogue<MODE> e;
-        if (whole) e.load(ep, n, t0, lane);
-        const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((buf * MB + m) * p.acc_cols + gr * 16);
-        uint32_t r0[16], r1[16], r2[16];
-        tmem_ld16(ta, r0);
-        tmem_ld16(ta + p.tp, r1);
-        if (p.terms == 3) tmem_ld16(ta + 2 * p.tp, r2);
-        tmem_wait_ld();
-        float v[16];
-        // the smaller terms first
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float lo = p.terms == 3 ? __uint_as_float(r1[j]) + __uint_as_float(r2[j]) : __uint_as_float(r1[j]);
-          v[j] = __uint_as_float(r0[j]) + lo;
-        }
-        if (whole) {
-          e.store(ep, n, t0, v, lane, (r_tile * MB + m) * 4 + q);
-        } else {
-          // this CTA's slot 0: the range starts inside the tile; slot 1: it ends inside
-          float4 *w = reinterpret_cast<float4 *>(p.ws) +
-                      narrow_partial(blockIdx.x, u > t_lo ? 0 : 1, m, gr, MB, p.tp) + row;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) w[j * 128] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-        }
-      }
-    }
+    return ready;
+  };
+  auto release_acc = [&]() {
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(smem_addr(&s_acc_empty[buf]));
+    if (lane == 0) mbar_arrive(smem_addr(&s_acc_empty[p.bufs == 2 ? seg & 1 : 0]));
+    ++seg;
+  };
+  // 16 tokens' sums of the accumulator, the smaller terms first
+  auto read_acc = [&](int m, int gr, float(&v)[16]) {
+    const int buf = p.bufs == 2 ? seg & 1 : 0;
+    const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((buf * MB + m) * p.acc_cols + gr * 16);
+    uint32_t r0[16], r1[16], r2[16];
+    tmem_ld16(ta, r0);
+    tmem_ld16(ta + p.tp, r1);
+    if (p.terms == 3) tmem_ld16(ta + 2 * p.tp, r2);
+    tmem_wait_ld();
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const float lo = p.terms == 3 ? __uint_as_float(r1[j]) + __uint_as_float(r2[j]) : __uint_as_float(r1[j]);
+      v[j] = __uint_as_float(r0[j]) + lo;
+    }
+  };
+  for (long long u = u0; u < u1;) {
+    const int tile = (int)(u / p.n_kb);
+    const long long t_lo = (long long)tile * p.n_kb, t_hi = t_lo + p.n_kb, end = min(u1, t_hi);
+    const bool whole = u == t_lo && end == t_hi;
+    const int r_tile = tile / p.t_tiles, tt0 = (tile % p.t_tiles) * p.tp;
+    auto finish = [&](int m, int gr, const float(&v)[16], const NarrowEpilogue<MODE> &e) {
+      const int n = (r_tile * MB + m) * 128 + row;
+      if (whole) {
+        e.store(ep, n, tt0 + gr * 16, v, lane, (r_tile * MB + m) * 4 + q);
+      } else {
+        // this CTA's slot 0: the range starts inside the tile; slot 1: it ends inside
+        float4 *w = reinterpret_cast<float4 *>(p.ws) + narrow_partial(blockIdx.x, u > t_lo ? 0 : 1, m, gr, MB, p.tp) + row;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j * 128] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+      }
+    };
+    if constexpr (DRAIN) {
+      constexpr int OWN = (NW_DRAIN_TP / 16 + 1) / 2;  // groups of this warp
+      float sum[OWN][16] = {};
+      for (int left = (int)(end - u); left > 0; left -= p.chunk) {
+        if (!wait_acc()) return;
+#pragma unroll
+        for (int k = 0; k < OWN; ++k) {
+          const int gr = grp + 2 * k;
+          if (gr < groups) {
+            float v[16];
+            read_acc(0, gr, v);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) sum[k][j] += v[j];
+          }
+        }
+        release_acc();
+      }
+#pragma unroll
+      for (int k = 0; k < OWN; ++k) {
+        const int gr = grp + 2 * k, t0 = tt0 + gr * 16;
+        if (gr < groups && t0 < ep.T) {
+          NarrowEpilogue<MODE> e;
+          if (whole) e.load(ep, r_tile * 128 + row, t0, lane);
+          finish(0, gr, sum[k], e);
+        }
+      }
+    } else {
+      if (!wait_acc()) return;
+      for (int m = 0; m < MB; ++m)
+        for (int gr = grp; gr < groups; gr += 2) {
+          const int t0 = tt0 + gr * 16;
+          if (t0 >= ep.T) break;
+          NarrowEpilogue<MODE> e;
+          if (whole) e.load(ep, (r_tile * MB + m) * 128 + row, t0, lane);
+          float v[16];
+          read_acc(m, gr, v);
+          finish(m, gr, v, e);
+        }
+      release_acc();
+    }
     u = end;
   }
 }
@@ -272,8 +320,15 @@ __global__ void __launch_bounds__(128) narrow_reduce_kernel(NarrowParams p, int 
   e.store(ep, n, t0, v, lane, (r_tile * mb + m) * 4 + q);
 }
 
-// MB: 128-row blocks per tile, 1 or 2.
-template <int MODE, int MB>
+// MB: 128-row blocks per tile, 1 or 2.  DRAIN (MB 1, two accumulators): each accumulator takes only
+// p.chunk K blocks, and the epilogue warps add the chunks up in registers.  A tensor-core accumulation
+// truncates: about 3e-8 of the sum per 16 K values, always towards zero, so 224 of them (K = 3584) put
+// the products of three-term activations at 5e-6, an order above the fp32 FMAs of a decode step;
+// chunks of 128 K values leave 2.5e-7.
+// Measured on 7B-shaped QK-norm prompts: of 512,000 K and as many V elements of a block, 67 and 54 land
+// beside the bf16 that 64 bits round to (84 and 82 as decode steps; 2,400 with two terms, undrained);
+// 200 tokens, two blocks: 11,690 us as decode steps, 798 drained, 677 undrained.
+template <int MODE, int MB, bool DRAIN>
 __global__ void __launch_bounds__(NW_THREADS, 1)
     prefill_narrow_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                           NarrowParams p, PrefillEpiParams ep) {
@@ -314,7 +369,8 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
     // ---- TMA producer (the whole warp, one elected lane issuing): the i-th K block of the CTA's range
     // uses stage i % S.  Weights do not depend on the previous kernel: the first round of them is
     // under way before the wait on it
-    const uint64_t pol = policy_evict_first();
+    // weights that another token tile reads again stay in L2
+    const uint64_t pol = p.t_tiles == 1 ? policy_evict_first() : policy_evict_normal();
     const uint32_t bytes = x_off + (uint32_t)p.tp * p.terms * 128u;
     // the ring position and the (tile, K block) of the next weight and token loads
     struct At {
@@ -372,14 +428,15 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
     }
   } else if (warp == 1) {
     // ---- MMA issuer (the whole warp, one elected lane issuing): segment i of the range (one row
-    // tile's share) accumulates into buffer i % bufs
+    // tile's share, or with DRAIN a chunk of it) accumulates into buffer i % bufs
     const uint32_t idesc = idesc_kind_f16(128, p.tp * p.terms, !ep.f16);
-    int s = 0, left = (int)(u1 - u0), n = p.n_kb - (int)(u0 % p.n_kb);
+    int s = 0, left = (int)(u1 - u0), kb = (int)(u0 % p.n_kb);
     uint32_t use = 0;
     bool ok = true;
-    for (int seg = 0; left > 0 && ok; ++seg, n = p.n_kb) {
-      n = min(n, left);
+    for (int seg = 0; left > 0 && ok; ++seg) {
+      const int n = min(min(p.n_kb - kb, left), DRAIN ? p.chunk : p.n_kb);
       left -= n;
+      kb = kb + n == p.n_kb ? 0 : kb + n;
       const int buf = p.bufs == 2 ? seg & 1 : 0;
       if (seg >= p.bufs) {
         const uint32_t back = (uint32_t)(p.bufs == 2 ? (seg >> 1) - 1 : seg - 1);
@@ -418,7 +475,7 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
     __syncwarp();
     mbar_wait(smem_addr(&s_drain), 0);
   } else {
-    narrow_epilogue_warps<MODE, MB>(p, ep, tmem, u0, u1, s_acc_full, s_acc_empty, abort_flag);
+    narrow_epilogue_warps<MODE, MB, DRAIN>(p, ep, tmem, u0, u1, s_acc_full, s_acc_empty, abort_flag);
   }
   tc_fence_before();
   __syncthreads();
@@ -672,7 +729,7 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
     __syncwarp();
     mbar_wait(smem_addr(&s_drain), 0);
   } else if (warp < N4_CONV_WARP) {
-    narrow_epilogue_warps<MODE, MB>(p, ep, tmem, u0, u1, s_acc_full, s_acc_empty, abort_flag);
+    narrow_epilogue_warps<MODE, MB, false>(p, ep, tmem, u0, u1, s_acc_full, s_acc_empty, abort_flag);
   } else {
     // ---- converters: warp w decodes 16-row groups (row block b, r16) = (w / 4 and w / 4 + 2, w % 4)
     const int cw = warp - N4_CONV_WARP, r16 = cw & 3, gid = lane >> 2;
@@ -798,10 +855,10 @@ static cudaError_t launch_narrow_reduce(const NarrowParams &p, int mb, int grid,
   return cudaLaunchKernelEx(&cfg, narrow_reduce_kernel<MODE>, p, mb, grid, ep);
 }
 
-template <int MODE, int MB>
+template <int MODE, int MB, bool DRAIN>
 static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x, const NarrowParams &p, int grid,
                                       const PrefillEpiParams &ep, cudaStream_t s) {
-  static const int smem = ring_smem(reinterpret_cast<const void *>(prefill_narrow_kernel<MODE, MB>));
+  static const int smem = ring_smem(reinterpret_cast<const void *>(prefill_narrow_kernel<MODE, MB, DRAIN>));
   if (smem < 0) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
@@ -812,12 +869,12 @@ static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x
   pdl_attribute(attr[0]);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_narrow_kernel<MODE, MB>, w, x, p, ep);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_narrow_kernel<MODE, MB, DRAIN>, w, x, p, ep);
   return e == cudaSuccess ? launch_narrow_reduce<MODE>(p, MB, grid, ep, s) : e;
 }
 
 int narrow_tp(int T, int terms) {
-  const int most = terms == 2 ? NW_MAX_TP : 80;  // terms * tp <= 256 MMA columns
+  const int most = terms == 2 ? NW_MAX_TP : NW_DRAIN_TP;  // terms * tp <= 256 MMA columns
   const int tiles = (T + most - 1) / most;
   return ((T + tiles - 1) / tiles + 15) / 16 * 16;
 }
@@ -832,7 +889,9 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensor
   const int cols = p.tp * terms;
   // wide tiles of many rows share their tokens' slices between two 128-row blocks: the slices (2 x
   // 16 KiB of terms at 128 tokens) then cost no more L2 reads than the weights
-  const int mb = cols > 128 && (ep.N + 255) / 256 * p.t_tiles >= ws.n_sm * 3 / 4 ? 2 : 1;
+  // Q/K/V: K and V are rounded to bf16 next, and every error before that moves some across a rounding
+  p.chunk = mode == PE_QKV || mode == PE_STORE ? 1 : NW_DRAIN_KB;
+  const int mb = terms == 2 && cols > 128 && (ep.N + 255) / 256 * p.t_tiles >= ws.n_sm * 3 / 4 ? 2 : 1;
   p.n_kb = (K + 63) / 64;
   p.n_tiles = (ep.N + 128 * mb - 1) / (128 * mb) * p.t_tiles;
   p.acc_cols = (cols + 31) / 32 * 32;
@@ -847,7 +906,9 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensor
   const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min<long long>(p.n_tiles, ws.n_sm), U / 4));
   auto go = [&](auto m) {
     constexpr int MODE = decltype(m)::value;
-    return mb == 2 ? launch_narrow_mode<MODE, 2>(w, x, p, grid, ep, s) : launch_narrow_mode<MODE, 1>(w, x, p, grid, ep, s);
+    if (terms == 3) return launch_narrow_mode<MODE, 1, true>(w, x, p, grid, ep, s);
+    return mb == 2 ? launch_narrow_mode<MODE, 2, false>(w, x, p, grid, ep, s)
+                   : launch_narrow_mode<MODE, 1, false>(w, x, p, grid, ep, s);
   };
   switch (mode) {
     case PE_STORE: return go(std::integral_constant<int, PE_STORE>());

@@ -267,7 +267,8 @@ struct kfl_stage {
   uint16_t *pf_x = nullptr, *pf_o = nullptr, *pf_a = nullptr;  // GEMM inputs as terms [term][token][ld]
   NarrowWorkspace pf_nw = {};  // the few-token GEMM's partial sums
   int pf_amax_cols = 0;
-  int *pf_pos = nullptr, *pf_aidx = nullptr;
+  int *pf_pos = nullptr, *pf_slots = nullptr, *pf_aidx = nullptr;
+  float *pf_raw = nullptr;  // QK-norm stages: the Q/K/V projection before the norm and RoPE [token][ld_raw]
   float *pf_amax = nullptr;
   std::vector<void *> pf_allocs;
   // bf16 stages: the maps of every layer's weight tiles [4 l + j] (Q/K/V, O, gate/up, down), then
@@ -792,12 +793,15 @@ int run_step(kfl_stage *st, const int32_t *ids, const float *hidden_in, const in
 }
 
 // ---- dense prefill (bf16 weights) ---------------------------------------------------------
-constexpr int PF_PASS = 2048;  // tokens per pass of the dense prefill
+constexpr int PF_PASS = 2048;        // tokens per pass of the dense prefill
+constexpr int PF_PAIR_TOKENS = 512;  // passes of up to this many tokens carry q and the softmax weights as pairs
 
 int pf_ld(int n) { return round_up(n, 64); }
 
-// Whether a pass of n tokens runs on the few-token GEMM.
-bool pf_narrow(const kfl_stage *st, int n) {
+// Whether a pass of n tokens runs on the few-token GEMM: few tokens, or three terms per activation,
+// which the 128-token tiles do not take.
+bool pf_narrow(const kfl_stage *st, int n, bool precise = false) {
+  if (precise) return true;
   return n <= (st->cfg.weight_fmt == KFL_BF16 ? NW_MAX_TP : env_int("KFL_N4_MAX", N4_MAX_TOKENS));
 }
 
@@ -817,13 +821,18 @@ int ensure_prefill(kfl_stage *st, int tokens) {
       st->pf_allocs.push_back(*p);
       return true;
     };
-    bool ok = get((void **)&st->pf_h, (size_t)cap * P.ldh * 4) && get((void **)&st->pf_q, (size_t)cap * pf_ld(P.qdim) * 2) &&
-              get((void **)&st->pf_x, (size_t)2 * cap * pf_ld(P.d) * 2) &&
-              get((void **)&st->pf_o, (size_t)2 * cap * pf_ld(P.qdim) * 2) &&
-              get((void **)&st->pf_a, (size_t)2 * cap * pf_ld(P.F) * 2) && get((void **)&st->pf_pos, (size_t)cap * 4);
+    // two terms per input, and q in bf16; QK-norm stages three, and q in fp32 (so do passes of fewer
+    // than 16 tokens, which need less than the room of 128 with two)
+    const size_t rows = (size_t)cap * (st->cfg.qk_norm ? 3 : 2);
+    bool ok = get((void **)&st->pf_h, (size_t)cap * P.ldh * 4) && get((void **)&st->pf_q, rows * pf_ld(P.qdim) * 2) &&
+              get((void **)&st->pf_x, rows * pf_ld(P.d) * 2) && get((void **)&st->pf_o, rows * pf_ld(P.qdim) * 2) &&
+              get((void **)&st->pf_a, rows * pf_ld(P.F) * 2) && get((void **)&st->pf_pos, (size_t)cap * 4) &&
+              get((void **)&st->pf_slots, (size_t)cap * 4);
+    if (st->cfg.qk_norm) ok = ok && get((void **)&st->pf_raw, (size_t)cap * P.ld_raw * 4);
     // argmax partials: per 256-column tile, or (passes on the few-token GEMM) per 32 rows
     if (st->flags & KFL_LOGITS_OUT) {
-      const int narrow = std::min(cap, st->cfg.weight_fmt == KFL_BF16 ? NW_MAX_TP : N4_MAX_TOKENS);
+      const int most = st->cfg.weight_fmt != KFL_BF16 ? N4_MAX_TOKENS : st->cfg.qk_norm ? PF_PASS : NW_MAX_TP;
+      const int narrow = std::min(cap, most);
       const size_t am = std::max((size_t)cap * ((P.V + PG_N - 1) / PG_N), (size_t)narrow * narrow_argmax_slots(P.V));
       ok = ok && get((void **)&st->pf_amax, am * 4) && get((void **)&st->pf_aidx, am * 4);
     }
@@ -968,9 +977,9 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
     e.aidx = st->pf_aidx;
     e.n_tiles = st->pf_amax_cols;
   }
-  if (pf_narrow(st, x.n) && i4)
+  if (i4 && pf_narrow(st, x.n))
     return launch_prefill_narrow4(mode, m.tiles, m.n_rb, m.n_kt, x.all, m.K, x.terms, st->pf_nw, e, s);
-  if (pf_narrow(st, x.n))
+  if (!i4 && pf_narrow(st, x.n, x.terms == 3))
     return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], x.all, m.K, x.terms, st->pf_nw, e, s);
   if (i4) {
     cudaError_t err = pf_dequant(st, g + 1);
@@ -991,8 +1000,11 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
 // K/V appended to the user's slot) -> causal attention over the slot -> O GEMM + residual ->
 // RMSNorm -> gate/up GEMM (SwiGLU) -> down GEMM + residual; the head: final RMSNorm -> lm_head GEMM
 // with the greedy argmax.
+//
+// precise: every activation in three bf16 terms (24 bits) and, in attention, q and the softmax weights
+// in two, as a decode step's attention has them: the precision of the decode steps.
 int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in, const int32_t *positions, int user,
-                      int T, float *hidden_out, int32_t *next_ids, cudaStream_t s) {
+                      int T, float *hidden_out, int32_t *next_ids, bool precise, cudaStream_t s) {
   const Plan &P = st->P;
   int rc = ensure_prefill(st, T);
   if (rc != KFL_OK) return rc;
@@ -1002,18 +1014,19 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
   const float eps = st->cfg.rms_eps;
   for (int t0 = 0; t0 < T; t0 += st->pf_cap) {
     const int n = std::min(st->pf_cap, T - t0);
-    const bool narrow = pf_narrow(st, n);
+    const bool narrow = pf_narrow(st, n, precise);
+    const int terms = precise ? 3 : 2;
     CK(launch_prefill_input(ids ? ids + t0 : nullptr, hidden_in ? hidden_in + (size_t)t0 * P.d : nullptr,
                             positions + t0, n, embed ? st->embed : nullptr, P.V, P.d, P.ldh, st->pf_h, st->pf_pos,
-                            st->cfg.max_ctx, st->err, s));
+                            st->cfg.max_ctx, user, st->pf_slots, st->err, s));
     if (!narrow) CK(pf_pass_begin(st, s));
     PfInput x, o, a;
-    if (x.encode(st->pf_x, P.d, n, 2, narrow) || o.encode(st->pf_o, P.qdim, n, 2, narrow) ||
-        a.encode(st->pf_a, P.F, n, 2, narrow))
+    if (x.encode(st->pf_x, P.d, n, terms, narrow) || o.encode(st->pf_o, P.qdim, n, terms, narrow) ||
+        a.encode(st->pf_a, P.F, n, terms, narrow))
       return KFL_ERR_CUDA;
     st->pf_amax_cols = narrow ? narrow_argmax_slots(P.V) : (P.V + PG_N - 1) / PG_N;
     auto norm = [&](const float *g) {
-      return launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, g, eps, x.base, x.base + x.stride, x.ld, i4, st->err, s);
+      return launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, g, eps, x.base, x.stride, terms, x.ld, i4, st->err, s);
     };
     PrefillEpiParams r = {};  // O and down: into the residual stream
     r.err = st->err;
@@ -1041,12 +1054,47 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       e.max_ctx = st->cfg.max_ctx;
       e.rope_cos = st->rope_cos;
       e.rope_sin = st->rope_sin;
-      CK(pf_gemm(st, PE_QKV, x, l, 0, e, s));
+      // q in fp32, and q and the softmax weights as bf16 pairs in attention, wherever attention is
+      // bound by latency rather than by its MMAs (which this doubles)
+      float *q32 = narrow || n <= PF_PAIR_TOKENS ? reinterpret_cast<float *>(st->pf_q) : nullptr;
+      if (st->cfg.qk_norm) {
+        PrefillEpiParams raw = {};
+        raw.err = st->err;
+        raw.N = L.qkv.N;
+        raw.out = st->pf_raw;
+        raw.ldo = P.ld_raw;
+        CK(pf_gemm(st, PE_STORE, x, l, 0, raw, s));
+        QkNormParams qn = {};
+        qn.raw = st->pf_raw;
+        qn.ld_raw = P.ld_raw;
+        qn.g_q = L.g_q;
+        qn.g_k = L.g_k;
+        qn.q = q32;
+        qn.kcache = kcl;
+        qn.vcache = vcl;
+        qn.positions = st->pf_pos;
+        qn.slots = st->pf_slots;
+        qn.rope_cos = st->rope_cos;
+        qn.rope_sin = st->rope_sin;
+        qn.batch = n;
+        qn.n_heads = P.hq;
+        qn.n_kv_heads = P.hkv;
+        qn.head_dim = P.hd;
+        qn.max_ctx = st->cfg.max_ctx;
+        qn.eps = eps;
+        CK(launch_qknorm(qn, s, true));
+      } else {
+        e.out = q32;
+        e.ldo = P.qdim;
+        CK(pf_gemm(st, PE_QKV, x, l, 0, e, s));
+      }
       PrefillAttnParams t = {};
       t.q = st->pf_q;
-      t.ldq = ldq;
+      t.q32 = q32;
+      t.ldq = q32 ? P.qdim : ldq;
       t.o = o.base;
-      t.o_lo = o.base + o.stride;
+      t.term_stride = o.stride;
+      t.terms = terms;
       t.ldo = o.ld;
       t.f16 = i4;
       t.kcache = kcl;
@@ -1059,7 +1107,7 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       t.max_ctx = st->cfg.max_ctx;
       t.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)P.hd));
       t.err = st->err;
-      CK(launch_prefill_attention(t, P.hd, s));
+      CK(launch_prefill_attention(t, P.hd, P.n_sm, s));
       CK(pf_gemm(st, PE_RESID, o, l, 1, r, s));
       CK(norm(L.g_ffn));
       PrefillEpiParams g = {};
@@ -1085,6 +1133,26 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
                            (size_t)P.d * 4, n, cudaMemcpyDeviceToDevice, s));
   }
   return KFL_OK;
+}
+
+// Whether a prompt that would else go as decode steps runs densely, at their precision (bf16 weights:
+// the int4 path's fp16 terms have a range that the decode steps' scaled ones do not).  Decode steps
+// stay where their kernels are observed (capture, trace, profile) and where the workspace is missing and
+// cannot be made: no memory, or s is being captured.
+bool prefill_precise(kfl_stage *st, int n_tokens, int dense_min, cudaStream_t s) {
+  if (st->cfg.weight_fmt != KFL_BF16 || st->capture || st->trace || st->profile) return false;
+  // a QK-norm stage's prompts from dense_min on; others too short for it (unless its line was moved)
+  // that would take more than one decode step
+  if (st->cfg.qk_norm ? n_tokens < dense_min : n_tokens <= st->cfg.max_batch || std::getenv("KFL_PREFILL_DENSE_MIN"))
+    return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const int need = std::min(PF_PASS, round_up(n_tokens, PG_M));
+  if (cap != cudaStreamCaptureStatusNone) return st->pf_cap >= need && !st->pf_maps.empty();
+  return ensure_prefill(st, n_tokens) == KFL_OK;
 }
 
 // host or device source -> device pointer (a temporary copy for host sources)
@@ -1500,10 +1568,12 @@ extern "C" int kfl_stage_prefill(kfl_stage *st, const int32_t *token_ids, const 
   if (!st->loaded()) return KFL_ERR_STATE;
   CK(cudaSetDevice(st->dev));
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  // the dense path from KFL_PREFILL_DENSE_MIN tokens on (default 16); QK-norm stages take the
-  // decode-step path (the dense path has no QK-norm epilogue)
-  if (n_tokens >= env_int("KFL_PREFILL_DENSE_MIN", 16) && !st->cfg.qk_norm)
-    return run_prefill_dense(st, token_ids, hidden_in, positions, user, n_tokens, hidden_out, next_ids, s);
+  // the dense path from KFL_PREFILL_DENSE_MIN tokens on (default 16)
+  const int dense_min = env_int("KFL_PREFILL_DENSE_MIN", 16);
+  if (n_tokens >= dense_min && !st->cfg.qk_norm)
+    return run_prefill_dense(st, token_ids, hidden_in, positions, user, n_tokens, hidden_out, next_ids, false, s);
+  if (prefill_precise(st, n_tokens, dense_min, s))
+    return run_prefill_dense(st, token_ids, hidden_in, positions, user, n_tokens, hidden_out, next_ids, true, s);
   const int d = st->P.d;
   // else the prompt in chunks of max_batch consecutive tokens: each chunk is one decode step whose
   // rows all address the user's KV slot, so a token attends to the chunk's earlier tokens too

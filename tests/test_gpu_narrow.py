@@ -89,3 +89,32 @@ def test_int4_scales_below_the_fp16_normals():
     rms = np.sqrt(np.mean(delta * delta, axis=1, keepdims=True))
     assert np.all(np.abs(got - hidden - delta) <= 1e-2 * rms)
     K.kfl_stage_destroy(st)
+
+
+@pytest.mark.parametrize("model,n,start,max_batch", [
+    (RAGGED, 5, 30, 4), (RAGGED, 15, 100, 1), (RAGGED128, 9, 7, 4),
+    (dataclasses.replace(RAGGED, qk_norm=True), 17, 30, 2),
+    (dataclasses.replace(RAGGED128, qk_norm=True), 165, 300, 4)])  # three token tiles, keys split over a cluster
+def test_dense_at_decode_precision(model, n, start, max_batch, monkeypatch):
+    """Prompts that run densely in place of decode steps (QK-norm stages; others longer than one step but
+    shorter than 16 tokens): the oracle's bar, and the decode steps' results.  Both sides carry
+    activations to 2^-22 or better and q and the softmax weights to 2^-17, so they differ where a
+    K or V element lands on the other side of a bf16 rounding (2^-8 of it): a few of the elements
+    that a row attends to, 1e-3 of its RMS at most (the bar allows ten times that)."""
+    monkeypatch.delenv("KFL_PREFILL_DENSE_MIN", raising=False)
+    p = Pair(model, 0, 2, 0, 2, (5, start), 512, seed=53, max_batch=max(2, max_batch))
+    K.kfl_stage_debug_capture(p.st, None)  # observed stages keep the decode steps
+    _prefill(p, 1, start, n, 53, False)
+    p.compare_kv()
+    hidden = torch.tensor(wl.hidden_in(model, 3, n, 53), dtype=torch.float32, device="cuda")
+    pos = torch.arange(start, start + n, dtype=torch.int32, device="cuda")
+    out = [torch.zeros(n, model.d_model, device="cuda") for _ in range(2)]
+    for o, line in zip(out, (None, str(1 << 30))):
+        if line:
+            monkeypatch.setenv("KFL_PREFILL_DENSE_MIN", line)
+        K.kfl_stage_prefill(p.st, None, hidden, pos, 1, n, o, None, torch.cuda.current_stream().cuda_stream)
+    assert K.kfl_stage_status(p.st) == 0
+    dense, steps = (o.cpu().numpy().astype(np.float64) for o in out)
+    rms = np.sqrt(np.mean(steps * steps, axis=1, keepdims=True))
+    assert np.all(np.abs(dense - steps) <= 1e-3 * rms)
+    p.close()

@@ -81,7 +81,7 @@ CASES = [
     ("hd128-200", RAGGED128, 0, 2, K.KFL_IS_HEAD, (0, 100, 7), 1, 200, 320),
     ("int4-head", RAGGED_INT4, 0, 2, K.KFL_IS_HEAD, (9, 70, 131), 1, 7, 192),
     ("int4-head-260", RAGGED_INT4, 0, 2, K.KFL_IS_HEAD, (9, 70, 131), 2, 260, 448),
-    # QK-norm stages prefill through decode steps whatever the prompt length
+    # QK-norm (dense: three terms per activation, the norm and RoPE in a kernel of their own)
     ("qknorm-head-40", dataclasses.replace(RAGGED, qk_norm=True), 0, 3, K.KFL_IS_HEAD, (5, 30, 70), 1, 40, 192),
 ]
 
