@@ -161,180 +161,33 @@ __device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t da, uint64_t db,
 }
 
 // ---------------------------------------------------------------------------- GEMM kernel
-// Split-K: the launch is a cluster of ep.splits (2, 4 or 8) CTAs per output tile (blockIdx.z =
-// rank); unsplit GEMMs run prefill_gemm_persistent.
-template <int MODE>
-__global__ void __launch_bounds__(PG_THREADS, 1)
-    prefill_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_a2,
-                        const __grid_constant__ CUtensorMap tm_b, int n_kblocks, PrefillEpiParams ep) {
-  pdl_launch_dependents();
-  static_assert(MODE != PE_ARGMAX, "the argmax partials are per whole tile: lm_head is never split");
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t s_full[PG_STAGES], s_empty[PG_STAGES], s_accum;
-  __shared__ uint32_t s_tmem;
-  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
-  const int t0 = blockIdx.x * PG_M, n0 = blockIdx.y * PG_N;
-  // split-K: split blockIdx.z of ep.splits takes K blocks [kb0, kb1)
-  const int kb0 = (int)((long long)blockIdx.z * n_kblocks / ep.splits);
-  const int kb1 = (int)((long long)(blockIdx.z + 1) * n_kblocks / ep.splits);
-  const int nkb = kb1 - kb0;
-  // the swizzled tiles start on a 1024-byte boundary
-  const uint32_t raw = smem_addr(smem_raw);
-  const uint32_t sa = (raw + 1023u) & ~1023u;      // [stage][hi, lo] activation tiles
-  const uint32_t sb = sa + PG_STAGES * 2 * PG_A_BYTES;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < PG_STAGES; ++s) {
-      mbar_init(smem_addr(&s_full[s]), 1);
-      mbar_init(smem_addr(&s_empty[s]), 1);
-    }
-    mbar_init(smem_addr(&s_accum), 1);
-    fence_mbar_init();
-  }
-  __syncwarp();
-  if (warp == 0) tmem_alloc(smem_addr(&s_tmem), PG_TMEM_COLS);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = s_tmem;
-  pdl_wait();
-
-  if (threadIdx.x == 0) {
-    // ---- TMA producer
-    asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
-    int issued[PG_STAGES] = {};
-    bool ok = true;
-    for (int j = 0; j < nkb; ++j) {
-      const int s = j % PG_STAGES, kb = kb0 + j;
-      const uint32_t use = j / PG_STAGES;
-      if (use > 0 && !mbar_wait(smem_addr(&s_empty[s]), (use - 1) & 1)) {
-        ok = false;
-        break;
-      }
-      const uint32_t full = smem_addr(&s_full[s]);
-      mbar_arrive_expect_tx(full, 2 * PG_A_BYTES + PG_B_BYTES);
-      tma_load_2d(sa + s * 2 * PG_A_BYTES, &tm_a, kb * PG_K, t0, full);
-      tma_load_2d(sa + s * 2 * PG_A_BYTES + PG_A_BYTES, &tm_a2, kb * PG_K, t0, full);
-      // weight tiles: (column within the K tile, row within the row block, K tile, row block)
-      tma_load_4d(sb + s * PG_B_BYTES, &tm_b, (kb & 1) * PG_K, 0, kb >> 1, n0 / RB, full);
-      ++issued[s];
-    }
-    if (!ok) {
-      atomicOr(ep.err, ERR_TIMEOUT);
-      // let the copies in flight land before the CTA's shared memory is released
-      for (int s = 0; s < PG_STAGES; ++s)
-        if (issued[s] > 0) mbar_wait(smem_addr(&s_full[s]), (issued[s] - 1) & 1);
-    }
-  } else if (warp == 1) {
-    // ---- MMA issuer (the whole warp, one elected lane issuing)
-    // A and B always share one type: both bf16, or (int4 stages) both fp16
-    const uint32_t idesc = ep.f16 ? idesc_kind_f16(PG_M, PG_N, false) : idesc_kind_f16(PG_M, PG_N, true);
-    for (int j = 0; j < nkb; ++j) {
-      const int s = j % PG_STAGES;
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_addr(&s_full[s]), (j / PG_STAGES) & 1))) {
-        if (lane == 0) atomicOr(ep.err, ERR_TIMEOUT);
-        break;
-      }
-      tc_fence_after();
-      const uint64_t da = sdesc_k_sw128(sa + s * 2 * PG_A_BYTES), db = sdesc_k_sw128(sb + s * PG_B_BYTES);
-      if (elect_one()) {
-        mma_kblock(tmem, da, db, idesc, j != 0);
-        mma_commit(smem_addr(&s_empty[s]));  // the stage is free once these MMAs have read it
-      }
-      __syncwarp();
-    }
-    if (elect_one()) mma_commit(smem_addr(&s_accum));  // the accumulator is complete (or, after a timeout, idle)
-  }
-  __syncwarp();
-
-  // ---- epilogue: warp w holds tokens t0 + 32 w + lane
-  // block-uniform: the split path synchronises the whole block
-  const bool ready = __syncthreads_and(mbar_wait(smem_addr(&s_accum), 0)) != 0;
-  if (!ready && threadIdx.x == 0) atomicOr(ep.err, ERR_TIMEOUT);
-  tc_fence_after();
-  const int row = warp * 32 + lane, t = t0 + row;
-  EpiState<MODE> st;
-  {
-    // split-K over a cluster of S = ep.splits CTAs (rank = blockIdx.z).  Column chunk c (32
-    // columns) of the tile belongs to rank c / (8 / S).  Every CTA pushes each chunk of its fp32
-    // accumulator into the owner's shared memory (posted remote stores; the pipeline buffers are
-    // idle now), at [own rank][row][chunk within the owner's share]; after the cluster barrier
-    // each owner sums its chunks over the ranks in rank order (deterministic) from its own shared
-    // memory and runs the epilogue.  The first barrier keeps a CTA from writing into a peer whose
-    // pipeline still uses that memory.  Both barriers are reached by every CTA, whatever its
-    // pipeline did.
-    const int S = ep.splits, per = (PG_N / 32) / S, ld = per * 32 + 4;
-    float *red = reinterpret_cast<float *>(smem_raw + (sa - raw));  // [S][PG_M][ld]
-    cluster_sync_all();
-    if (ready) {
-      for (int c = 0; c < PG_N / 32; ++c) {
-        if (n0 + 32 * c >= ep.N) break;
-        uint32_t r[32];
-        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + 32 * c, r);
-        const int owner = c / per;
-        const uint32_t dst = map_to_rank(smem_addr(red + ((size_t)blockIdx.z * PG_M + row) * ld + (c % per) * 32),
-                                         owner);
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          st_cluster_f4(dst + 16 * j, make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                                  __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3])));
-      }
-    }
-    cluster_sync_all();
-    if (ready) {
-      for (int cc = 0; cc < per; ++cc) {
-        const int n = n0 + 32 * (blockIdx.z * per + cc);
-        if (n >= ep.N) break;
-        float acc[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = 0.f;
-        for (int q = 0; q < S; ++q) {
-          const float4 *src = reinterpret_cast<const float4 *>(red + ((size_t)q * PG_M + row) * ld + cc * 32);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float4 v4 = src[j];
-            acc[4 * j] += v4.x;
-            acc[4 * j + 1] += v4.y;
-            acc[4 * j + 2] += v4.z;
-            acc[4 * j + 3] += v4.w;
-          }
-        }
-        uint32_t r[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(acc[j]);
-        if (t < ep.T) epilogue32<MODE>(ep, t, n, r, st);
-      }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    tc_fence_after();
-    tmem_dealloc(tmem, PG_TMEM_COLS);
-  }
-}
-
-// ---------------------------------------------------------------------------- persistent GEMM
-// The unsplit GEMM as a persistent kernel: one CTA per SM takes tiles c, c + grid, ...  The TMA
-// ring runs on across tile boundaries, and two accumulators (all 512 TMEM columns) let the MMAs of
-// the next tile proceed while four epilogue warps drain the previous one.  Warp 0 lane 0 issues
-// TMA, warp 1 lane 0 issues MMAs, warps 2-5 run the epilogue (warp w reads TMEM lanes
-// 32 (w % 4) ..).  Every wait is bounded; a CTA that gives up sets ERR_TIMEOUT, lets its copies
-// and MMAs in flight complete (bounded), frees its TMEM and returns.
+// One CTA per SM walks its share of the tiles (TileShare).  The TMA ring runs on across tile
+// boundaries, and two accumulators (all 512 TMEM columns) let the MMAs of the next tile proceed while
+// four epilogue warps drain the previous one.  Warp 0 issues TMA, warp 1 MMAs, warps 2-5 run the
+// epilogue (warp w reads TMEM lanes 32 (w % 4) ..).  Every wait is bounded; a CTA that gives up sets
+// ERR_TIMEOUT, lets its copies and MMAs in flight complete (bounded), frees its TMEM and returns.
+//
+// Bound by the tensor pipe (two terms against every weight).  Splitting K over clusters of 2 to 8 CTAs,
+// as this did where the tiles fill the last round badly, cost 7 to 39 us a round of CTAs in cluster
+// launch and distributed shared memory: the down projection of 500 tokens (56 tiles) took 173 us, now
+// 85 with the kernel that sums its parts.  Two 7B-shaped blocks: 931 -> 815 us at 500 tokens, 2620 -> 1951 at
+// 1500, 2608 at 2048 as before (its tiles fill their rounds).
 constexpr int PP_THREADS = 192;
 constexpr int PP_TMEM_COLS = 2 * PG_N;
+
+// Where (in float4, plus the token row) a partial holds columns 4 j .. of the tile.
+__device__ __forceinline__ size_t wide_partial(int part, int j) { return ((size_t)part * (PG_N / 4) + j) * PG_M; }
 
 template <int MODE>
 __global__ void __launch_bounds__(PP_THREADS, 1)
     prefill_gemm_persistent(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_a2,
-                            const __grid_constant__ CUtensorMap tm_b, int n_kblocks, PrefillEpiParams ep) {
+                            const __grid_constant__ CUtensorMap tm_b, TileShare share, float *ws, PrefillEpiParams ep) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t s_full[PG_STAGES], s_empty[PG_STAGES], s_acc_full[2], s_acc_empty[2], s_drain;
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
-  const int t_tiles = (ep.T + PG_M - 1) / PG_M, n_tiles = (ep.N + PG_N - 1) / PG_N;
-  const int tiles = t_tiles * n_tiles;
+  const int t_tiles = (ep.T + PG_M - 1) / PG_M;
   const uint32_t raw = smem_addr(smem_raw);
   const uint32_t sa = (raw + 1023u) & ~1023u;  // [stage][hi, lo] activation tiles
   const uint32_t sb = sa + PG_STAGES * 2 * PG_A_BYTES;
@@ -362,57 +215,59 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
   pdl_wait();
 
   if (warp == 0) {
-    if (lane == 0) {
-      asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
-      // ---- TMA producer: k-block it of the CTA's sequence uses stage it % S
-      int issued[PG_STAGES] = {};
-      long long it = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-        const int t0 = (tile % t_tiles) * PG_M, n0 = (tile / t_tiles) * PG_N;
-        for (int kb = 0; kb < n_kblocks; ++kb, ++it) {
-          const int s = (int)(it % PG_STAGES);
-          const uint32_t use = (uint32_t)(it / PG_STAGES);
-          if (*abort_flag || (use > 0 && !mbar_wait(smem_addr(&s_empty[s]), (use - 1) & 1))) {
-            ok = false;
-            break;
-          }
-          const uint32_t full = smem_addr(&s_full[s]);
+    // ---- TMA producer (the whole warp, one elected lane issuing)
+    asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
+    int s = 0, use = 0;
+    bool ok = true;
+    for (TileWalk w(share); ok && w.next();) {
+      const int t0 = (w.tile % t_tiles) * PG_M, n0 = (w.tile / t_tiles) * PG_N;
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+        ok = __all_sync(0xffffffffu,
+                        !*abort_flag && (use == 0 || mbar_wait(smem_addr(&s_empty[s]), (uint32_t)(use - 1) & 1)));
+        if (!ok) break;
+        const uint32_t full = smem_addr(&s_full[s]);
+        if (elect_one()) {
           mbar_arrive_expect_tx(full, 2 * PG_A_BYTES + PG_B_BYTES);
           tma_load_2d(sa + s * 2 * PG_A_BYTES, &tm_a, kb * PG_K, t0, full);
           tma_load_2d(sa + s * 2 * PG_A_BYTES + PG_A_BYTES, &tm_a2, kb * PG_K, t0, full);
+          // weight tiles: (column within the K tile, row within the row block, K tile, row block)
           tma_load_4d(sb + s * PG_B_BYTES, &tm_b, (kb & 1) * PG_K, 0, kb >> 1, n0 / RB, full);
-          ++issued[s];
         }
-      }
-      if (!ok) {
-        *abort_flag = 1;
-        atomicOr(ep.err, ERR_TIMEOUT);
-        for (int s = 0; s < PG_STAGES; ++s)
-          if (issued[s] > 0) mbar_wait(smem_addr(&s_full[s]), (issued[s] - 1) & 1);
+        __syncwarp();
+        if (++s == PG_STAGES) s = 0, ++use;
       }
     }
-    __syncwarp();
+    if (!ok) {
+      if (lane == 0) {
+        *abort_flag = 1;
+        atomicOr(ep.err, ERR_TIMEOUT);
+      }
+      // let the copies in flight land before the CTA's shared memory is released
+      for (int i = 0; i < PG_STAGES; ++i) {
+        const int last = use - (i >= s ? 1 : 0);
+        if (last >= 0) mbar_wait(smem_addr(&s_full[i]), (uint32_t)last & 1);
+      }
+    }
   } else if (warp == 1) {
-    // ---- MMA issuer (the whole warp, one elected lane issuing): tile i of this CTA accumulates
+    // ---- MMA issuer (the whole warp, one elected lane issuing): segment i of this CTA accumulates
     // into TMEM columns (i % 2) * PG_N
     const uint32_t idesc = ep.f16 ? idesc_kind_f16(PG_M, PG_N, false) : idesc_kind_f16(PG_M, PG_N, true);
     int s = 0, i = 0;
     uint32_t use = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++i) {
+    for (TileWalk w(share); ok && w.next(); ++i) {
       const int buf = i & 1;
       if (i >= 2) ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&s_acc_empty[buf]), ((i >> 1) - 1) & 1));
       if (!ok) break;
       tc_fence_after();
       const uint32_t d = tmem + (uint32_t)(buf * PG_N);
-      for (int kb = 0; kb < n_kblocks; ++kb) {
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
         ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_full[s]), use & 1));
         if (!ok) break;
         tc_fence_after();
         const uint64_t da = sdesc_k_sw128(sa + s * 2 * PG_A_BYTES), db = sdesc_k_sw128(sb + s * PG_B_BYTES);
         if (elect_one()) {
-          mma_kblock(d, da, db, idesc, kb != 0);
+          mma_kblock(d, da, db, idesc, kb != w.kb0);
           mma_commit(smem_addr(&s_empty[s]));
         }
         __syncwarp();
@@ -433,7 +288,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     // ---- epilogue warps 2..5: TMEM lanes 32 q .. 32 q + 31 (q = warp % 4) are tokens t0 + 32 q + lane
     const int q = warp & 3, row = 32 * q + lane;
     int i = 0;
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++i) {
+    for (TileWalk w(share); w.next(); ++i) {
       const int buf = i & 1;
       const bool ready = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_acc_full[buf]), (i >> 1) & 1));
       if (!ready) {
@@ -444,18 +299,26 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
         break;
       }
       tc_fence_after();
-      const int t_tile = tile % t_tiles, n_tile = tile / t_tiles;
-      const int t = t_tile * PG_M + row, n0 = n_tile * PG_N;
+      const int n_tile = w.tile / t_tiles, t = (w.tile % t_tiles) * PG_M + row, n0 = n_tile * PG_N;
+      const bool whole = w.whole();
       EpiState<MODE> st;
       for (int c = 0; c < PG_N / 32; ++c) {
         const int n = n0 + 32 * c;
         if (n >= ep.N) break;  // uniform across the warp
         uint32_t r[32];
         tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * PG_N + 32 * c), r);
-        if (t < ep.T) epilogue32<MODE>(ep, t, n, r, st);
+        if (whole) {
+          if (t < ep.T) epilogue32<MODE>(ep, t, n, r, st);
+        } else {
+          float4 *at = reinterpret_cast<float4 *>(ws) + wide_partial(w.part, 8 * c) + row;
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            at[j * PG_M] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                                       __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
+        }
       }
       if constexpr (MODE == PE_ARGMAX) {
-        if (t < ep.T) {
+        if (whole && t < ep.T) {
           ep.amax[(size_t)t * ep.n_tiles + n_tile] = st.best;
           ep.aidx[(size_t)t * ep.n_tiles + n_tile] = st.bidx;
         }
@@ -470,6 +333,52 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
   if (warp == 0) {
     tc_fence_after();
     tmem_dealloc(tmem, PP_TMEM_COLS);
+  }
+}
+
+// The tiles that several CTAs share: their partial sums, added in K order, and the epilogue.  One
+// block (thread = token) per tile and 32 columns (PE_ARGMAX: per tile, whose maximum it keeps).
+template <int MODE>
+__global__ void __launch_bounds__(PG_M) wide_reduce_kernel(TileShare share, int gemm_ctas, const float *ws,
+                                                            PrefillEpiParams ep) {
+  pdl_launch_dependents();
+  constexpr int CHUNKS = PG_N / 32, PER = MODE == PE_ARGMAX ? CHUNKS : 1;
+  const int sk = blockIdx.x / (CHUNKS / PER), c0 = blockIdx.x % (CHUNKS / PER) * PER;
+  const int t_tiles = (ep.T + PG_M - 1) / PG_M, tile = share.waves * gemm_ctas + sk;
+  const TileParts parts(share, sk, gemm_ctas);
+  const int n_tile = tile / t_tiles, t = (tile % t_tiles) * PG_M + threadIdx.x;
+  pdl_wait();
+  if (parts.n == 1 || t >= ep.T) return;
+  EpiState<MODE> st;
+  for (int c = c0; c < c0 + PER && n_tile * PG_N + 32 * c < ep.N; ++c) {
+    float v[32] = {};
+    for (int k = 0; k < parts.n; k += 2) {
+      float4 x[2][8];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float4 *at =
+            reinterpret_cast<const float4 *>(ws) + wide_partial(parts.part(k + i), 8 * c) + threadIdx.x;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[i][j] = k + i < parts.n ? __ldcg(at + j * PG_M) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          v[4 * j] += x[i][j].x;
+          v[4 * j + 1] += x[i][j].y;
+          v[4 * j + 2] += x[i][j].z;
+          v[4 * j + 3] += x[i][j].w;
+        }
+    }
+    uint32_t r[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(v[j]);
+    epilogue32<MODE>(ep, t, n_tile * PG_N + 32 * c, r, st);
+  }
+  if constexpr (MODE == PE_ARGMAX) {
+    ep.amax[(size_t)t * ep.n_tiles + n_tile] = st.best;
+    ep.aidx[(size_t)t * ep.n_tiles + n_tile] = st.bidx;
   }
 }
 
@@ -898,41 +807,46 @@ __global__ void prefill_rmsnorm_kernel(const float *h, int ldh, int d, const flo
   }
 }
 
-// One thread per 8 consecutive outputs of one row (16 bytes): the int4 tile stores the nibble of
-// (row rb*64 + r16*16 + gid + 8 ((i >> 1) & 1), column kt*256 + 128 h + 16 (4 q + j) + 2 tig +
-// 8 (i & 1) + ((i >> 2) & 1)) as nibble i of word j + 4 lane + 128 q + 256 r16 + 1024 h
-// (lane = 4 gid + tig), and the row's group scales after the codes; so the 8 columns
-// 16 m + 8 e .. + 7 of a row come from lanes tig = 0..3, nibbles i with i & 1 = e.
-__global__ void dequant_int4_f16_kernel(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst) {
-  const long long total = (long long)n_rb * n_kt * RB * (KT4 / 8);
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int c8 = (int)(e % (KT4 / 8));      // 8-column chunk within the int4 tile (0..31)
-    const long long rt = e / (KT4 / 8);
-    const int r = (int)(rt % RB);              // row within the row block
-    const long long t = rt / RB;               // int4 tile index rb * n_kt + kt
-    const int col0 = c8 * 8;                   // 0..248
-    const int h = col0 >> 7, m = (col0 >> 4) & 7, ebit = (col0 >> 3) & 1;
-    const int q = m >> 2, j = m & 3, r16 = r >> 4, gid = r & 7, rhalf = (r >> 3) & 1;
-    const uint8_t *tile = tiles4 + (size_t)t * TILE4_BYTES;
-    const uint32_t *words = reinterpret_cast<const uint32_t *>(tile);
-    const float sc = bf16_to_f32(reinterpret_cast<const uint16_t *>(tile + TILE4_CODE_BYTES)[tile4_scale_index(r, col0 >> 6)]);
-    uint16_t out[8];
+// Half an int4 tile (64 rows x 128 columns) to its fp16 tile, code x scale rounded once (decode_word,
+// scale_pair): warp r16 decodes 16 rows, in the fragment order of the codes, into shared memory by
+// matrix stores, and the block writes the 16 KiB tile out in 16-byte pieces.  Bound by HBM: 0.53 bytes
+// read and 2 written per weight.  (One thread per 8 outputs, gathering the codes word by word and
+// rounding each product on its own, ran at 2.9 TB/s: a 72B-shaped block of 900 tokens 2940 -> 2389 us.)
+constexpr int DQ_ROW = KT * 2 + 16;  // bytes per staged row: eight rows' pieces fall on distinct banks
+__global__ void __launch_bounds__(128) dequant_int4_f16_kernel(const uint8_t *tiles4, int n_tiles, uint16_t *dst) {
+  __shared__ __align__(16) uint8_t stage[RB * DQ_ROW];
+  const int r16 = threadIdx.x / 32, lane = threadIdx.x % 32, gid = lane >> 2;
+  // matrices 0..3 of a 16-column step: rows 0-7 and 8-15 of its first 8 columns, then of its last 8
+  const uint32_t st = smem_addr(stage) + (r16 * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * DQ_ROW + (lane >> 4) * 16;
+  for (int h = blockIdx.x; h < 2 * n_tiles; h += gridDim.x) {
+    const uint8_t *tile = tiles4 + (size_t)(h >> 1) * TILE4_BYTES;
+    uint4 w[2];
+    uint32_t sc[2];
 #pragma unroll
-    for (int tig = 0; tig < 4; ++tig) {
-      const uint32_t w = words[j + 4 * (4 * gid + tig) + 128 * q + 256 * r16 + 1024 * h];
+    for (int q = 0; q < 2; ++q) {
+      w[q] = __ldcs(reinterpret_cast<const uint4 *>(tile + (h & 1) * 4096 + r16 * 1024 + q * 512) + lane);
+      sc[q] = *reinterpret_cast<const uint32_t *>(tile + TILE4_CODE_BYTES +
+                                                  2 * tile4_scale_index(r16 * 16 + gid, 2 * (h & 1) + q));
+    }
+    __syncthreads();  // the stage is free
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const int i = ebit | (rhalf << 1) | (b << 2);
-        const int nib = (int)((w >> (4 * i)) & 0xFu);
-        out[2 * tig + b] = f32_to_f16_rn((float)(nib >= 8 ? nib - 16 : nib) * sc);
+    for (int q = 0; q < 2; ++q) {
+      const ScalePair sp(sc[q]);
+      const bool exact = __all_sync(0xffffffffu, sp.exact());
+      const uint32_t words[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        uint32_t c0, c1, c2, c3;
+        decode_word(words[j], c0, c1, c2, c3);
+        sp.apply(exact, c0, c1, c2, c3);
+        stsm_x4(st + q * 128 + j * 32, c0, c1, c2, c3);
       }
     }
-    // fp16 tile (rb, 2 kt + h): row r, columns (col0 & 127) ..
-    const long long rb = t / n_kt, kt = t % n_kt;
-    uint16_t *d = dst + ((size_t)(rb * 2 * n_kt + 2 * kt + h) * RB + r) * KT + (col0 & 127);
-    *reinterpret_cast<uint4 *>(d) = make_uint4(out[0] | (uint32_t)out[1] << 16, out[2] | (uint32_t)out[3] << 16,
-                                               out[4] | (uint32_t)out[5] << 16, out[6] | (uint32_t)out[7] << 16);
+    __syncthreads();
+    uint4 *out = reinterpret_cast<uint4 *>(dst + (size_t)h * RB * KT);  // fp16 tile (rb, 2 kt + half)
+#pragma unroll
+    for (int e = threadIdx.x; e < RB * KT / 8; e += 128)
+      __stcs(out + e, *reinterpret_cast<const uint4 *>(stage + (e / (KT / 8)) * DQ_ROW + (e % (KT / 8)) * 16));
   }
 }
 
@@ -1053,97 +967,36 @@ static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int threads, size
 }
 
 template <int MODE>
-static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b, int n_kt,
-                               const PrefillEpiParams &ep, cudaStream_t s) {
+static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b, int n_kb,
+                               const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
   static bool smem_set = false;
   if (!smem_set) {
     cudaError_t e = cudaFuncSetAttribute(prefill_gemm_persistent<MODE>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
-    if constexpr (MODE != PE_ARGMAX)
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(prefill_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)PG_SMEM);
     if (e != cudaSuccess) return e;
     smem_set = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(PG_THREADS);
-  cfg.dynamicSmemBytes = PG_SMEM;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[2];
-  pdl_attribute(attr[0]);
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = 1;
-  attr[1].val.clusterDim.y = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  PrefillEpiParams e = ep;
-  if constexpr (MODE != PE_ARGMAX) {
-    // the largest split count not above the chosen one whose cluster fits on the device
-    static int fits[9] = {};  // 0 unknown, 1 yes, -1 no
-    while (e.splits > 1) {
-      if (fits[e.splits] == 0) {
-        attr[1].val.clusterDim.z = e.splits;
-        cfg.gridDim = dim3(1, 1, e.splits);
-        int n = 0;
-        fits[e.splits] =
-            cudaOccupancyMaxActiveClusters(&n, prefill_gemm_kernel<MODE>, &cfg) == cudaSuccess && n > 0 ? 1 : -1;
-        cudaGetLastError();
-      }
-      if (fits[e.splits] > 0) break;
-      e.splits /= 2;
-    }
-    if (e.splits > 1) {
-      cfg.gridDim = dim3((e.T + PG_M - 1) / PG_M, (e.N + PG_N - 1) / PG_N, e.splits);
-      attr[1].val.clusterDim.z = e.splits;
-      return cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<MODE>, a, a2, b, 2 * n_kt, e);
-    }
-  }
-  // one persistent CTA per SM (fewer if there are fewer tiles)
-  static int n_sm = 0;
-  if (!n_sm) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return cudaErrorInvalidDevice;
-  }
-  const long long tiles = (long long)((e.T + PG_M - 1) / PG_M) * ((e.N + PG_N - 1) / PG_N);
-  cfg.gridDim = dim3((unsigned)std::min<long long>(tiles, n_sm));
-  cfg.blockDim = dim3(PP_THREADS);
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, prefill_gemm_persistent<MODE>, a, a2, b, 2 * n_kt, e);
+  // one persistent CTA per SM (fewer if there are not four K blocks for each)
+  const int tiles = (ep.T + PG_M - 1) / PG_M * ((ep.N + PG_N - 1) / PG_N);
+  const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min(tiles, ws.n_sm), (long long)tiles * n_kb / 4));
+  const TileShare share = share_tiles(tiles, n_kb, grid, false, NW_PARTS);
+  cudaError_t e = launch_pdl(prefill_gemm_persistent<MODE>, dim3(grid), PP_THREADS, PG_SMEM, s, a, a2, b, share, ws.partial, ep);
+  if (e == cudaSuccess && share.cut())
+    e = launch_pdl(wide_reduce_kernel<MODE>, dim3(share.tail * (MODE == PE_ARGMAX ? 1 : PG_N / 32)), PG_M, 0, s, share,
+                   grid, ws.partial, ep);
+  return e;
 }
 
-int prefill_splits(int T, int N, int n_kt, int n_sm) {
-  const long long base = (long long)((T + PG_M - 1) / PG_M) * ((N + PG_N - 1) / PG_N);
-  const int n_kb = 2 * n_kt;
-  // waves x (K blocks per split + a fixed cost per CTA of about 6 K blocks: pipeline fill and
-  // epilogue; 1.5 more for the cluster reduction), over the split counts 1, 2, 4, 8 that keep
-  // at least 4 K blocks each
-  int best = 1;
-  double best_t = 1e30;
-  for (int S = 1; S <= 8 && n_kb / S >= 4; S *= 2) {
-    const double waves = (double)((base * S + n_sm - 1) / n_sm);
-    const double t = waves * ((double)n_kb / S + 6.0 + (S > 1 ? 1.5 : 0.0));
-    if (t < best_t - 1e-9) {
-      best_t = t;
-      best = S;
-    }
-  }
-  return best;
-}
-
-cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b,
-                                int n_kt, const PrefillEpiParams &ep, cudaStream_t s) {
+cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b, int K,
+                                const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
   if (ep.T <= 0 || ep.N <= 0) return cudaSuccess;
-  if (ep.splits != 1 && ep.splits != 2 && ep.splits != 4 && ep.splits != 8) return cudaErrorInvalidValue;
-  if (mode == PE_ARGMAX && ep.splits != 1) return cudaErrorInvalidValue;  // partial maxima are per tile
+  const int n_kb = (K + PG_K - 1) / PG_K;
   switch (mode) {
-    case PE_STORE: return launch_mode<PE_STORE>(a, a2, b, n_kt, ep, s);
-    case PE_RESID: return launch_mode<PE_RESID>(a, a2, b, n_kt, ep, s);
-    case PE_SWIGLU: return launch_mode<PE_SWIGLU>(a, a2, b, n_kt, ep, s);
-    case PE_QKV: return launch_mode<PE_QKV>(a, a2, b, n_kt, ep, s);
-    case PE_ARGMAX: return launch_mode<PE_ARGMAX>(a, a2, b, n_kt, ep, s);
+    case PE_STORE: return launch_mode<PE_STORE>(a, a2, b, n_kb, ws, ep, s);
+    case PE_RESID: return launch_mode<PE_RESID>(a, a2, b, n_kb, ws, ep, s);
+    case PE_SWIGLU: return launch_mode<PE_SWIGLU>(a, a2, b, n_kb, ws, ep, s);
+    case PE_QKV: return launch_mode<PE_QKV>(a, a2, b, n_kb, ws, ep, s);
+    case PE_ARGMAX: return launch_mode<PE_ARGMAX>(a, a2, b, n_kb, ws, ep, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1197,7 +1050,7 @@ cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const 
 }
 
 cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, cudaStream_t s) {
-  dequant_int4_f16_kernel<<<8 * 152, 256, 0, s>>>(tiles4, n_rb, n_kt, dst);
+  dequant_int4_f16_kernel<<<8 * 152, 128, 0, s>>>(tiles4, n_rb * n_kt, dst);
   return cudaGetLastError();
 }
 
@@ -1228,11 +1081,11 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     cudaGetLastError();
     return KFL_ERR_CUDA;
   }
-  // few tokens: the few-token kernel, which needs room for partial sums too
+  // few tokens: the few-token kernel
   const bool narrow = T <= NW_MAX_TP;
   const int rows = (T + 7) / 8 * 8;
   const size_t tile_bytes = (size_t)n_rb * n_kt * TILE_BYTES, x_bytes = (size_t)rows * ld * 2;
-  const size_t ws_bytes = narrow ? narrow_ws_bytes(n_sm, T) : 0;
+  const size_t ws_bytes = narrow_ws_bytes(n_sm, T);
   void *mem = nullptr;
   if (cudaMalloc(&mem, tile_bytes + 2 * x_bytes + ws_bytes + 16) != cudaSuccess) {
     cudaGetLastError();
@@ -1263,13 +1116,9 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     e.err = err;
     unsigned h_err = 0;
     cudaError_t ce;
-    if (narrow) {
-      const NarrowWorkspace ws = {partial, n_sm};
-      ce = launch_prefill_narrow(PE_STORE, mb, mh, K, 2, ws, e, s);
-    } else {
-      e.splits = prefill_splits(T, N, n_kt, n_sm);
-      ce = launch_prefill_gemm(PE_STORE, mh, ml, mb, n_kt, e, s);
-    }
+    const NarrowWorkspace ws = {partial, n_sm};
+    ce = narrow ? launch_prefill_narrow(PE_STORE, mb, mh, K, 2, ws, e, s)
+                : launch_prefill_gemm(PE_STORE, mh, ml, mb, K, ws, e, s);
     if (ce != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess ||
         cudaMemcpy(&h_err, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
       rc = KFL_ERR_CUDA;

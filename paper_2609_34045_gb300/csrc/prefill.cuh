@@ -14,9 +14,8 @@ namespace kfl {
 // decode path's fp32 activations; W is bf16 as stored (int4 stages: fp16 tiles dequantized from
 // the int4 ones, with fp16 terms of X).  An output tile is PG_M tokens x PG_N weight rows,
 // computed with tcgen05.mma (M = PG_M, N = PG_N, K = 16 per instruction; each K slice once with
-// Xhi and once with Xlo against the same W slice), the fp32 accumulator in tensor memory: by a
-// persistent CTA per SM with two accumulators (prefill_gemm_persistent), or, split over K, by a
-// cluster of 2, 4 or 8 CTAs that reduce through distributed shared memory (prefill_gemm_kernel).  Operands reach shared memory by TMA with the 128-byte swizzle, PG_K = 64 bf16 (one
+// Xhi and once with Xlo against the same W slice), the fp32 accumulator in tensor memory, by a
+// persistent CTA per SM with two accumulators (prefill_gemm_persistent).  Operands reach shared memory by TMA with the 128-byte swizzle, PG_K = 64 bf16 (one
 // swizzle row) per pipeline stage: Xhi and Xlo through 2-D maps of the activation rows, W through
 // a 4-D map of the decode path's weight tiles [N/RB][K/KT][RB][KT] (one box = PG_N / RB row
 // blocks x 64 columns of one K tile), so the prefill streams the weights from where the decode
@@ -27,8 +26,6 @@ constexpr int PG_K = 64;
 constexpr int PG_STAGES = 3;
 constexpr int PG_A_BYTES = PG_M * PG_K * 2;  // 16 KiB per term
 constexpr int PG_B_BYTES = PG_N * PG_K * 2;  // 32 KiB
-constexpr int PG_THREADS = 128;              // split kernel: TMA (thread 0), MMA (thread 32); all: epilogue
-constexpr int PG_TMEM_COLS = PG_N;           // split kernel: fp32 accumulator columns
 constexpr size_t PG_SMEM = (size_t)PG_STAGES * (2 * PG_A_BYTES + PG_B_BYTES) + 1024;  // + alignment slack
 
 enum PrefillEpi : int {
@@ -60,9 +57,6 @@ struct PrefillEpiParams {
   float *amax;
   int *aidx;
   int n_tiles;
-  // split-K: 1, 2, 4 or 8 CTAs per output tile, launched as a cluster that reduces through
-  // distributed shared memory (PE_ARGMAX: 1)
-  int splits;
   unsigned *err;           // ERR_TIMEOUT if a pipeline wait gave up; ERR_F16_RANGE (PE_SWIGLU, fp16
                            // terms) if a value is beyond the fp16 range
 };
@@ -84,7 +78,8 @@ struct PrefillAttnParams {
 // ---- the prefill GEMM of few tokens (prefill_narrow.cu): weight rows as M, the tokens' terms
 // side by side as N, split stream-K over one CTA per SM
 constexpr int NW_MAX_TP = 128;            // tokens of a tile (two terms: 256 MMA columns)
-constexpr int N4_MAX_TOKENS = 1024;      // int4 stages: passes of up to this many tokens decode in the GEMM
+constexpr int NW_PARTS = 3;               // partial sums per CTA in a GEMM's workspace
+constexpr int N4_MAX_TOKENS = 512;       // int4 stages: passes of up to this many tokens decode in the GEMM
 constexpr int NW_W_BYTES = 128 * 64 * 2;  // a 128-row weight slice of 64 K
 struct NarrowWorkspace {
   float *partial;  // narrow_ws_bytes
@@ -112,11 +107,8 @@ inline void pdl_attribute(cudaLaunchAttribute &a) {
   a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   a.val.programmaticStreamSerializationAllowed = 1;
 }
-// Splits of K (1, 2, 4 or 8) for a GEMM of T tokens x N rows (n_kt K tiles) on n_sm SMs: the
-// count that minimises an estimate of waves x work per CTA.
-int prefill_splits(int T, int N, int n_kt, int n_sm);
-cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a_hi, const CUtensorMap &a_lo, const CUtensorMap &b,
-                                int n_kt, const PrefillEpiParams &ep, cudaStream_t s);
+cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a_hi, const CUtensorMap &a_lo, const CUtensorMap &b, int K,
+                                const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s);
 cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, int n_sm, cudaStream_t s);
 cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const int *positions_in, int T,
                                  const uint16_t *embed, int vocab, int d, int ldh, float *h, int *positions,

@@ -5,9 +5,8 @@
 // Up to 128 tokens the product is bound by the weights' stream from HBM (2 T flops per weight
 // byte and term: at T = 128 the MMAs of a 16 KiB weight slice take about 512 cycles, its share of
 // the HBM bandwidth about 750).  So every SM streams an equal share of the matrix, whatever its
-// shape: the K blocks of all row tiles form one sequence, CTA c takes the contiguous range
-// [c U / G, (c + 1) U / G) of it, and a row tile that several CTAs share is summed from their
-// partial sums in CTA order by a small kernel behind it (narrow_reduce_kernel).
+// shape (TileShare), and a row tile that several CTAs share is summed from their partial sums in CTA
+// order by a small kernel behind it (narrow_reduce_kernel).
 // The tokens' terms share each MMA: 128 weight rows x (terms x tokens) columns, so a token count
 // of 16 costs an eighth of the 128-token tile of prefill_gemm_persistent, and the epilogue's lanes
 // hold consecutive output columns of one token.
@@ -35,8 +34,7 @@ constexpr int NW_MAX_STAGES = 12;
 constexpr int NW_RING = 226 * 1024;      // shared memory of the rings: a block's 227 KiB less the barriers' KiB
 
 struct NarrowParams {
-  int n_kb;         // K blocks of 64
-  int n_tiles;      // row tiles (of 128 mb rows) x token tiles
+  TileShare share;  // of row tiles (of 128 mb rows) x token tiles, in K blocks of 64 (int4: units of 128)
   int t_tiles;
   int tp, terms;    // tokens of a tile (a multiple of 16), terms per token: tp * terms columns
   int stages, stage_bytes;
@@ -47,10 +45,10 @@ struct NarrowParams {
   float *ws;        // partial sums (narrow_partial)
 };
 
-// Where (in float4, plus the row) CTA c's partial of its slot holds the sums of 128-row block m and token
-// group gr: [c][slot][m][gr][4 x 4 tokens][128 rows].
-__device__ __forceinline__ size_t narrow_partial(int c, int slot, int m, int gr, int mb, int tp) {
-  return (((size_t)c * 2 + slot) * mb * (tp / 16) + (size_t)m * (tp / 16) + gr) * (4 * 128);
+// Where (in float4, plus the row) a partial holds the sums of 128-row block m and token group gr:
+// [part][m][gr][4 x 4 tokens][128 rows].
+__device__ __forceinline__ size_t narrow_partial(int part, int m, int gr, int mb, int tp) {
+  return ((size_t)part * mb * (tp / 16) + (size_t)m * (tp / 16) + gr) * (4 * 128);
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
@@ -171,12 +169,12 @@ struct NarrowEpilogue {
   }
 };
 
-// The epilogue warps' part of a CTA with range [u0, u1) of the U units: every segment's sums, from its
+// The epilogue warps' part of a CTA: every segment's sums, from its
 // accumulator to the outputs or, where CTAs share the tile, to the partial sums (narrow_reduce_kernel).
 template <int MODE, int MB, bool DRAIN>
 __device__ __forceinline__ void narrow_epilogue_warps(const NarrowParams &p, const PrefillEpiParams &ep, uint32_t tmem,
-                                                      long long u0, long long u1, uint64_t *s_acc_full,
-                                                      uint64_t *s_acc_empty, volatile int *abort_flag) {
+                                                      uint64_t *s_acc_full, uint64_t *s_acc_empty,
+                                                      volatile int *abort_flag) {
   static_assert(!DRAIN || MB == 1, "a drained tile's sums fit the registers");
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   // ---- epilogue warps: TMEM lanes 32 q .. (q = warp % 4) are 32 consecutive rows of the tile;
@@ -218,26 +216,23 @@ __device__ __forceinline__ void narrow_epilogue_warps(const NarrowParams &p, con
       v[j] = __uint_as_float(r0[j]) + lo;
     }
   };
-  for (long long u = u0; u < u1;) {
-    const int tile = (int)(u / p.n_kb);
-    const long long t_lo = (long long)tile * p.n_kb, t_hi = t_lo + p.n_kb, end = min(u1, t_hi);
-    const bool whole = u == t_lo && end == t_hi;
-    const int r_tile = tile / p.t_tiles, tt0 = (tile % p.t_tiles) * p.tp;
+  for (TileWalk w(p.share); w.next();) {
+    const bool whole = w.whole();
+    const int r_tile = w.tile / p.t_tiles, tt0 = (w.tile % p.t_tiles) * p.tp;
     auto finish = [&](int m, int gr, const float(&v)[16], const NarrowEpilogue<MODE> &e) {
       const int n = (r_tile * MB + m) * 128 + row;
       if (whole) {
         e.store(ep, n, tt0 + gr * 16, v, lane, (r_tile * MB + m) * 4 + q);
       } else {
-        // this CTA's slot 0: the range starts inside the tile; slot 1: it ends inside
-        float4 *w = reinterpret_cast<float4 *>(p.ws) + narrow_partial(blockIdx.x, u > t_lo ? 0 : 1, m, gr, MB, p.tp) + row;
+        float4 *at = reinterpret_cast<float4 *>(p.ws) + narrow_partial(w.part, m, gr, MB, p.tp) + row;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) w[j * 128] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        for (int j = 0; j < 4; ++j) at[j * 128] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
       }
     };
     if constexpr (DRAIN) {
       constexpr int OWN = (NW_DRAIN_TP / 16 + 1) / 2;  // groups of this warp
       float sum[OWN][16] = {};
-      for (int left = (int)(end - u); left > 0; left -= p.chunk) {
+      for (int left = w.kb1 - w.kb0; left > 0; left -= p.chunk) {
         if (!wait_acc()) return;
 #pragma unroll
         for (int k = 0; k < OWN; ++k) {
@@ -274,38 +269,35 @@ __device__ __forceinline__ void narrow_epilogue_warps(const NarrowParams &p, con
         }
       release_acc();
     }
-    u = end;
   }
 }
 
-// The tiles that several CTAs share: their partial sums, added in CTA order, and the epilogue.  One
+// The tiles that several CTAs share: their partial sums, added in K order, and the epilogue.  One
 // block per 128 rows x 16 tokens, so that the sums (up to 70 KB a CTA of the GEMM) are read by the
 // whole GPU at once: summed by the last CTA to arrive at a tile, inside the GEMM, they cost 4 to 8 us
 // at 43 tokens and 20 to 50 us at 100, of a tail in which most SMs were idle.
 template <int MODE>
 __global__ void __launch_bounds__(128) narrow_reduce_kernel(NarrowParams p, int mb, int gemm_ctas, PrefillEpiParams ep) {
   pdl_launch_dependents();
-  const int groups = p.tp / 16, gr = blockIdx.x % groups, m = blockIdx.x / groups % mb, tile = blockIdx.x / groups / mb;
+  const int groups = p.tp / 16, gr = blockIdx.x % groups, m = blockIdx.x / groups % mb, sk = blockIdx.x / groups / mb;
   const int q = threadIdx.x / 32, lane = threadIdx.x % 32, row = threadIdx.x;
-  const long long U = (long long)p.n_tiles * p.n_kb, G = gemm_ctas, t_lo = (long long)tile * p.n_kb;
+  const int tile = p.share.waves * gemm_ctas + sk;
   const int r_tile = tile / p.t_tiles, t0 = (tile % p.t_tiles) * p.tp + gr * 16;
-  // the CTAs whose ranges meet the tile; every one but the first starts inside it
-  const int first = (int)(((t_lo + 1) * G - 1) / U), last = (int)(((t_lo + p.n_kb) * G - 1) / U);
-  const int slot0 = first * U / G > t_lo ? 0 : 1;
+  const TileParts parts(p.share, sk, gemm_ctas);
   pdl_wait();
-  if (first == last || t0 >= ep.T) return;
+  if (parts.n == 1 || t0 >= ep.T) return;
   const int n = (r_tile * mb + m) * 128 + row;
   const float4 *ws = reinterpret_cast<const float4 *>(p.ws) + row;
   NarrowEpilogue<MODE> e;
   e.load(ep, n, t0, lane);
   float v[16] = {};
-  for (int c = first; c <= last; c += 4) {
+  for (int k = 0; k < parts.n; k += 4) {
     float4 x[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const float4 *w = ws + narrow_partial(c + i, c + i == first ? slot0 : 0, m, gr, mb, p.tp);
+      const float4 *w = ws + narrow_partial(parts.part(k + i), m, gr, mb, p.tp);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[i][j] = c + i <= last ? __ldcg(w + j * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int j = 0; j < 4; ++j) x[i][j] = k + i < parts.n ? __ldcg(w + j * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -319,6 +311,24 @@ __global__ void __launch_bounds__(128) narrow_reduce_kernel(NarrowParams p, int 
   }
   e.store(ep, n, t0, v, lane, (r_tile * mb + m) * 4 + q);
 }
+
+// A producer's place in its CTA's segments: the K block it loads next, of row tile r_tile and the tokens
+// from t0 (worked out once a segment).
+struct NarrowAt {
+  TileWalk w;
+  int kb, r_tile, t0;
+  bool more;
+  __device__ __forceinline__ explicit NarrowAt(const NarrowParams &p) : w(p.share) { seek(p); }
+  __device__ __forceinline__ void seek(const NarrowParams &p) {
+    more = w.next();
+    kb = more ? w.kb0 : 0;
+    r_tile = more ? w.tile / p.t_tiles : 0;
+    t0 = more ? (w.tile - r_tile * p.t_tiles) * p.tp : 0;
+  }
+  __device__ __forceinline__ void next(const NarrowParams &p) {
+    if (++kb == w.kb1) seek(p);
+  }
+};
 
 // MB: 128-row blocks per tile, 1 or 2.  DRAIN (MB 1, two accumulators): each accumulator takes only
 // p.chunk K blocks, and the epilogue warps add the chunks up in registers.  A tensor-core accumulation
@@ -338,8 +348,6 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
   __shared__ int s_abort;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const uint32_t ring = (smem_addr(smem_raw) + 1023u) & ~1023u;
-  const long long U = (long long)p.n_tiles * p.n_kb, G = gridDim.x;
-  const long long u0 = blockIdx.x * U / G, u1 = (blockIdx.x + 1) * U / G;
   const uint32_t x_off = (uint32_t)MB * NW_W_BYTES;
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -372,45 +380,35 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
     // weights that another token tile reads again stay in L2
     const uint64_t pol = p.t_tiles == 1 ? policy_evict_first() : policy_evict_normal();
     const uint32_t bytes = x_off + (uint32_t)p.tp * p.terms * 128u;
-    // the ring position and the (tile, K block) of the next weight and token loads
-    struct At {
-      int s, use, kb, r, t;  // stage, its use, K block, row tile, token tile
-    };
-    const int tile0 = (int)(u0 / p.n_kb);
-    At w = {0, 0, (int)(u0 % p.n_kb), tile0 / p.t_tiles, tile0 % p.t_tiles}, x = w;
-    auto next = [&](At &a) {
-      if (++a.s == p.stages) a.s = 0, ++a.use;
-      if (++a.kb == p.n_kb) {
-        a.kb = 0;
-        if (++a.t == p.t_tiles) a.t = 0, ++a.r;
-      }
-    };
+    NarrowAt w(p), x(p);  // where the next weight and the next token loads are
+    int ws = 0, wuse = 0, xs = 0, xuse = 0;
     auto weights = [&]() {
-      const uint32_t full = smem_addr(&s_full[w.s]), dst = ring + w.s * p.stage_bytes;
+      const uint32_t full = smem_addr(&s_full[ws]), dst = ring + ws * p.stage_bytes;
       if (elect_one()) {
         mbar_arrive_expect_tx(full, bytes);
 #pragma unroll
         for (int m = 0; m < MB; ++m)
-          tma_load_4d_hint(dst + m * NW_W_BYTES, &tm_w, (w.kb & 1) * 64, 0, w.kb >> 1, (w.r * MB + m) * (128 / RB),
-                           full, pol);
+          tma_load_4d_hint(dst + m * NW_W_BYTES, &tm_w, (w.kb & 1) * 64, 0, w.kb >> 1,
+                           (w.r_tile * MB + m) * (128 / RB), full, pol);
       }
       __syncwarp();
-      next(w);
+      w.next(p);
+      if (++ws == p.stages) ws = 0, ++wuse;
     };
     auto tokens = [&]() {
       if (elect_one())
-        tma_load_3d(ring + x.s * p.stage_bytes + x_off, &tm_x, x.kb * 64, x.t * p.tp, 0, smem_addr(&s_full[x.s]));
+        tma_load_3d(ring + xs * p.stage_bytes + x_off, &tm_x, x.kb * 64, x.t0, 0, smem_addr(&s_full[xs]));
       __syncwarp();
-      next(x);
+      x.next(p);
+      if (++xs == p.stages) xs = 0, ++xuse;
     };
-    const int total = (int)(u1 - u0), lead = min(total, p.stages);
-    for (int i = 0; i < lead; ++i) weights();
+    while (w.more && wuse == 0) weights();
     pdl_wait();
     asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
-    for (int i = 0; i < lead; ++i) tokens();
+    while (x.more && xuse == 0) tokens();
     bool ok = true;
-    for (int i = lead; i < total; ++i) {
-      ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_empty[w.s]), (uint32_t)(w.use - 1) & 1));
+    while (w.more) {
+      ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_empty[ws]), (uint32_t)(wuse - 1) & 1));
       if (!ok) break;
       weights();
       tokens();
@@ -420,9 +418,9 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
         *abort_flag = 1;
         atomicOr(ep.err, ERR_TIMEOUT);
       }
-      // let the copies in flight land: stage s was last filled in its use number w.use - (s >= w.s)
+      // let the copies in flight land: stage s was last filled in its use number wuse - (s >= ws)
       for (int s = 0; s < p.stages; ++s) {
-        const int last = w.use - (s >= w.s ? 1 : 0);
+        const int last = wuse - (s >= ws ? 1 : 0);
         if (last >= 0) mbar_wait(smem_addr(&s_full[s]), (uint32_t)last & 1);
       }
     }
@@ -430,13 +428,17 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
     // ---- MMA issuer (the whole warp, one elected lane issuing): segment i of the range (one row
     // tile's share, or with DRAIN a chunk of it) accumulates into buffer i % bufs
     const uint32_t idesc = idesc_kind_f16(128, p.tp * p.terms, !ep.f16);
-    int s = 0, left = (int)(u1 - u0), kb = (int)(u0 % p.n_kb);
+    TileWalk w(p.share);
+    int s = 0, left = 0;  // K blocks of the segment not yet issued
     uint32_t use = 0;
     bool ok = true;
-    for (int seg = 0; left > 0 && ok; ++seg) {
-      const int n = min(min(p.n_kb - kb, left), DRAIN ? p.chunk : p.n_kb);
+    for (int seg = 0; ok; ++seg) {
+      if (left == 0) {
+        if (!w.next()) break;
+        left = w.kb1 - w.kb0;
+      }
+      const int n = DRAIN ? min(left, p.chunk) : left;
       left -= n;
-      kb = kb + n == p.n_kb ? 0 : kb + n;
       const int buf = p.bufs == 2 ? seg & 1 : 0;
       if (seg >= p.bufs) {
         const uint32_t back = (uint32_t)(p.bufs == 2 ? (seg >> 1) - 1 : seg - 1);
@@ -475,7 +477,7 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
     __syncwarp();
     mbar_wait(smem_addr(&s_drain), 0);
   } else {
-    narrow_epilogue_warps<MODE, MB, DRAIN>(p, ep, tmem, u0, u1, s_acc_full, s_acc_empty, abort_flag);
+    narrow_epilogue_warps<MODE, MB, DRAIN>(p, ep, tmem, s_acc_full, s_acc_empty, abort_flag);
   }
   tc_fence_before();
   __syncthreads();
@@ -494,9 +496,9 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
 // costs 4.5 times its bytes (0.53 read, 2 written and 2 read again).
 // 256 rows to a tile: a token slice (up to 32 KiB) is read from L2 once per 16 KiB of fp16 weights of
 // two 128-row blocks, and each converter warp has two independent 16-row groups in hand.
-// Measured, one 72B-shaped block: 1206 -> 261 us at 16 tokens, 1228 -> 359 at 100, 2188 -> 1298 at 512 and
-// 2939 -> 2468 at 900, against fp16 copies made ahead on a second stream (745 us of a block's time
-// whatever the prompt).  Bound by the converters at few tokens and by the MMAs from about 100.
+// Measured, one 72B-shaped block: 261 us at 16 tokens, 359 at 100 and 1389 at 512, against 1207, 1228 and
+// 2188 with fp16 copies made ahead on a second stream (1517 at 512 with their faster kernel of today,
+// which takes over from there).  Bound by the converters at few tokens and by the MMAs from about 100.
 constexpr int N4_CONV_WARPS = 8;
 constexpr int N4_CONV_WARP = 10;  // the first converter warp
 constexpr int N4_THREADS = (N4_CONV_WARP + N4_CONV_WARPS) * 32;
@@ -513,43 +515,6 @@ struct Narrow4Params {
 };
 
 
-__device__ __forceinline__ void stsm_x4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
-  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2),
-               "r"(r3)
-               : "memory");
-}
-__device__ __forceinline__ uint32_t hmul2(uint32_t a, uint32_t b) {
-  uint32_t r;
-  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-  return r;
-}
-__device__ __forceinline__ uint32_t hfma2(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t r;
-  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
-  return r;
-}
-
-// The eight codes of an A-fragment word as exact fp16 pairs: rows gid and gid + 8 of columns 2 tig,
-// 2 tig + 1 (c0, c1) and of columns 2 tig + 8, 2 tig + 9 (c2, c3).  The nibbles, top bit flipped, become
-// 1024 + u or 1024 + 16 u (u = code + 8).
-__device__ __forceinline__ void decode_word(uint32_t w, uint32_t &c0, uint32_t &c1, uint32_t &c2, uint32_t &c3) {
-  const uint32_t w8 = w >> 8;
-  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c0) : "r"(w), "r"(0x000F000Fu), "r"(0x64086408u));
-  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c1) : "r"(w8), "r"(0x000F000Fu), "r"(0x64086408u));
-  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c2) : "r"(w), "r"(0x00F000F0u), "r"(0x64806480u));
-  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c3) : "r"(w8), "r"(0x00F000F0u), "r"(0x64806480u));
-  c0 = hfma2(c0, 0x3C003C00u, 0xE408E408u);  // - 1032
-  c1 = hfma2(c1, 0x3C003C00u, 0xE408E408u);
-  c2 = hfma2(c2, 0x2C002C00u, 0xD480D480u);  // / 16 - 72
-  c3 = hfma2(c3, 0x2C002C00u, 0xD480D480u);
-}
-
-// fp16 pair of codes times an fp32 scale, rounded once.
-__device__ __forceinline__ uint32_t scale_pair_f32(uint32_t c, float sc) {
-  return (uint32_t)f32_to_f16_rn(f16_to_f32((uint16_t)c) * sc) |
-         ((uint32_t)f32_to_f16_rn(f16_to_f32((uint16_t)(c >> 16)) * sc) << 16);
-}
-
 template <int MODE>
 __global__ void __launch_bounds__(N4_THREADS, 1)
     prefill_narrow4_kernel(const Narrow4Params r, const __grid_constant__ CUtensorMap tm_x, NarrowParams p,
@@ -565,8 +530,6 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
   const uint32_t a_ring = (smem_addr(smem_raw) + 1023u) & ~1023u;
   const uint32_t x_ring = a_ring + r.a_stages * N4_A_BYTES;
   const uint32_t codes = x_ring + r.x_stages * r.x_bytes;  // [code stage][row block][codes, scales]
-  const long long U = (long long)p.n_tiles * p.n_kb, G = gridDim.x;
-  const long long u0 = blockIdx.x * U / G, u1 = (blockIdx.x + 1) * U / G;
   if (threadIdx.x == 0) {
     for (int s = 0; s < r.c_stages; ++s) {
       mbar_init(smem_addr(&s_cfull[s]), 1);
@@ -601,19 +564,8 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
     // ---- producer (the whole warp, one elected lane issuing): units' codes as the code ring frees,
     // their two token slices as the token ring does
     const uint64_t pol = p.t_tiles == 1 ? policy_evict_first() : policy_evict_normal();
-    struct At {
-      int kb, r, t;  // K unit, row tile, token tile
-    };
-    const int tile0 = (int)(u0 / p.n_kb);
-    At w = {(int)(u0 % p.n_kb), tile0 / p.t_tiles, tile0 % p.t_tiles}, x = w;
-    auto next = [&](At &a) {
-      if (++a.kb == p.n_kb) {
-        a.kb = 0;
-        if (++a.t == p.t_tiles) a.t = 0, ++a.r;
-      }
-    };
-    const int total = (int)(u1 - u0);
-    int cs = 0, cuse = 0, xs = 0, xuse = 0, c_done = 0, x_done = 0, half = 0;
+    NarrowAt w(p), x(p);  // where the next codes and the next token slices are
+    int cs = 0, cuse = 0, xs = 0, xuse = 0, half = 0;
     auto issue_codes = [&]() {
       const uint32_t full = smem_addr(&s_cfull[cs]), dst = codes + cs * N4_CODE_BYTES;
       if (elect_one()) {
@@ -621,7 +573,7 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
           // row blocks past the end repeat the last: their rows are beyond N and never stored
-          const int rb = min(w.r * 4 + b, r.n_rb - 1);
+          const int rb = min(w.r_tile * 4 + b, r.n_rb - 1);
           const uint8_t *t = r.tiles + ((size_t)rb * r.n_kt + (w.kb >> 1)) * TILE4_BYTES;
           bulk_g2s(dst + b * N4_RB_BYTES, t + (w.kb & 1) * (TILE4_CODE_BYTES / 2), TILE4_CODE_BYTES / 2, full, pol);
           bulk_g2s(dst + b * N4_RB_BYTES + TILE4_CODE_BYTES / 2,
@@ -629,35 +581,33 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
         }
       }
       __syncwarp();
-      next(w);
-      ++c_done;
+      w.next(p);
       if (++cs == r.c_stages) cs = 0, ++cuse;
     };
     auto issue_tokens = [&]() {
       const uint32_t full = smem_addr(&s_xfull[xs]);
       if (elect_one()) {
         mbar_arrive_expect_tx(full, r.x_bytes);
-        tma_load_3d(x_ring + xs * r.x_bytes, &tm_x, x.kb * 128 + half * 64, x.t * p.tp, 0, full);
+        tma_load_3d(x_ring + xs * r.x_bytes, &tm_x, x.kb * 128 + half * 64, x.t0, 0, full);
       }
       __syncwarp();
-      if (half) next(x);
+      if (half) x.next(p);
       half ^= 1;
-      ++x_done;
       if (++xs == r.x_stages) xs = 0, ++xuse;
     };
-    while (c_done < min(total, r.c_stages)) issue_codes();
+    while (w.more && cuse == 0) issue_codes();
     pdl_wait();
     asm volatile("fence.proxy.async;" ::: "memory");  // the previous kernel's stores, before TMA reads them
-    while (x_done < min(2 * total, r.x_stages)) issue_tokens();
+    while (x.more && xuse == 0) issue_tokens();
     bool ok = true;
     // whichever ring has room goes first; one of them always will, or a wait elsewhere gives up
-    for (uint32_t idle = 0; x_done < 2 * total || c_done < total;) {
+    for (uint32_t idle = 0; x.more || w.more;) {
       bool did = false;
-      if (c_done < total && __any_sync(0xffffffffu, mbar_test_wait(smem_addr(&s_cempty[cs]), (uint32_t)(cuse - 1) & 1))) {
+      if (w.more && __any_sync(0xffffffffu, mbar_test_wait(smem_addr(&s_cempty[cs]), (uint32_t)(cuse - 1) & 1))) {
         issue_codes();
         did = true;
       }
-      if (x_done < 2 * total && __any_sync(0xffffffffu, mbar_test_wait(smem_addr(&s_xempty[xs]), (uint32_t)(xuse - 1) & 1))) {
+      if (x.more && __any_sync(0xffffffffu, mbar_test_wait(smem_addr(&s_xempty[xs]), (uint32_t)(xuse - 1) & 1))) {
         issue_tokens();
         did = true;
       }
@@ -685,12 +635,12 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
   } else if (warp == 1) {
     // ---- MMA issuer, as in prefill_narrow_kernel; a unit is two stages
     const uint32_t idesc = idesc_kind_f16(128, p.tp * p.terms, false);
-    int as = 0, xs = 0, left = (int)(u1 - u0), n = p.n_kb - (int)(u0 % p.n_kb);
+    TileWalk w(p.share);
+    int as = 0, xs = 0;
     uint32_t ause = 0, xuse = 0;
     bool ok = true;
-    for (int seg = 0; left > 0 && ok; ++seg, n = p.n_kb) {
-      n = min(n, left);
-      left -= n;
+    for (int seg = 0; ok && w.next(); ++seg) {
+      const int n = w.kb1 - w.kb0;
       const int buf = p.bufs == 2 ? seg & 1 : 0;
       if (seg >= p.bufs) {
         const uint32_t back = (uint32_t)(p.bufs == 2 ? (seg >> 1) - 1 : seg - 1);
@@ -729,7 +679,7 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
     __syncwarp();
     mbar_wait(smem_addr(&s_drain), 0);
   } else if (warp < N4_CONV_WARP) {
-    narrow_epilogue_warps<MODE, MB, false>(p, ep, tmem, u0, u1, s_acc_full, s_acc_empty, abort_flag);
+    narrow_epilogue_warps<MODE, MB, false>(p, ep, tmem, s_acc_full, s_acc_empty, abort_flag);
   } else {
     // ---- converters: warp w decodes 16-row groups (row block b, r16) = (w / 4 and w / 4 + 2, w % 4)
     const int cw = warp - N4_CONV_WARP, r16 = cw & 3, gid = lane >> 2;
@@ -741,7 +691,8 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
     for (int j = 0; j < 4; ++j) off[j] = (uint32_t)((r16 * 16 + mrow) * 128 + (((2 * j + mcol) ^ (lane & 7)) << 4));
     int cs = 0, s = 0;
     uint32_t cuse = 0, use = 0;
-    const int total = (int)(u1 - u0);
+    int total = 0;  // the CTA's units
+    for (TileWalk w(p.share); w.next();) total += w.kb1 - w.kb0;
     bool ok = true;
     for (int i = 0; i < total && ok; ++i) {
       ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_cfull[cs]), cuse & 1));
@@ -764,15 +715,10 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
                        : "=r"(sc[half][g])
                        : "r"(blk + TILE4_CODE_BYTES / 2 + (((half * 8 + gid) * 4 + r16) * 4)));
         }
-      // a bf16 scale that fp16 holds exactly: the fp16 product of code and scale is rounded as the
-      // fp32 product would be; others (below 2^-14, or too large) go through fp32
 #pragma unroll
       for (int half = 0; half < 2; ++half)
 #pragma unroll
-        for (int g = 0; g < 2; ++g) {
-          const float s0 = bf16_lo(sc[half][g]), s1 = bf16_hi(sc[half][g]);
-          exact = exact && f16_to_f32(f32_to_f16_rn(s0)) == s0 && f16_to_f32(f32_to_f16_rn(s1)) == s1;
-        }
+        for (int g = 0; g < 2; ++g) exact = exact && ScalePair(sc[half][g]).exact();
       exact = __all_sync(0xffffffffu, exact);
       if (lane == 0) mbar_arrive(smem_addr(&s_cempty[cs]));
 #pragma unroll
@@ -783,24 +729,14 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
         for (int g = 0; g < 2; ++g) {
           // row block b = cw / 4 + 2 g: rows 64 (b % 2) of 128-row block b / 2
           const uint32_t dst = a_ring + s * N4_A_BYTES + g * NW_W_BYTES + (cw >> 2) * (64 * 128);
-          const float s0 = bf16_lo(sc[half][g]), s1 = bf16_hi(sc[half][g]);
+          const ScalePair sp(sc[half][g]);
           const uint32_t words[4] = {w[half][g].x, w[half][g].y, w[half][g].z, w[half][g].w};
-          if (exact) {
-            const uint32_t p0 = f32_to_f16_rn(s0) * 0x10001u, p1 = f32_to_f16_rn(s1) * 0x10001u;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              uint32_t c0, c1, c2, c3;
-              decode_word(words[j], c0, c1, c2, c3);
-              stsm_x4(dst + off[j], hmul2(c0, p0), hmul2(c1, p1), hmul2(c2, p0), hmul2(c3, p1));
-            }
-          } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              uint32_t c0, c1, c2, c3;
-              decode_word(words[j], c0, c1, c2, c3);
-              stsm_x4(dst + off[j], scale_pair_f32(c0, s0), scale_pair_f32(c1, s1), scale_pair_f32(c2, s0),
-                      scale_pair_f32(c3, s1));
-            }
+          for (int j = 0; j < 4; ++j) {
+            uint32_t c0, c1, c2, c3;
+            decode_word(words[j], c0, c1, c2, c3);
+            sp.apply(exact, c0, c1, c2, c3);
+            stsm_x4(dst + off[j], c0, c1, c2, c3);
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stores, before the MMAs read them
@@ -826,8 +762,8 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
 }  // namespace
 
 size_t narrow_ws_bytes(int n_sm, int T) {
-  // two slots per CTA of 256 rows x tp tokens
-  return (size_t)n_sm * 2 * 256 * std::min(NW_MAX_TP, (T + 15) / 16 * 16) * sizeof(float);
+  // NW_PARTS partials per CTA of 256 rows x tp tokens
+  return (size_t)n_sm * NW_PARTS * 256 * std::min(NW_MAX_TP, (T + 15) / 16 * 16) * sizeof(float);
 }
 int narrow_argmax_slots(int N) { return (N + 127) / 128 * 4; }
 
@@ -843,9 +779,9 @@ static int ring_smem(const void *kernel) {
 template <int MODE>
 static cudaError_t launch_narrow_reduce(const NarrowParams &p, int mb, int grid, const PrefillEpiParams &ep,
                                         cudaStream_t s) {
-  if (p.n_tiles % grid == 0) return cudaSuccess;  // every range is whole tiles
+  if (!p.share.cut()) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(p.n_tiles * mb * (p.tp / 16)));
+  cfg.gridDim = dim3((unsigned)(p.share.tail * mb * (p.tp / 16)));
   cfg.blockDim = dim3(128);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -892,8 +828,7 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensor
   // Q/K/V: K and V are rounded to bf16 next, and every error before that moves some across a rounding
   p.chunk = mode == PE_QKV || mode == PE_STORE ? 1 : NW_DRAIN_KB;
   const int mb = terms == 2 && cols > 128 && (ep.N + 255) / 256 * p.t_tiles >= ws.n_sm * 3 / 4 ? 2 : 1;
-  p.n_kb = (K + 63) / 64;
-  p.n_tiles = (ep.N + 128 * mb - 1) / (128 * mb) * p.t_tiles;
+  const int n_kb = (K + 63) / 64, n_tiles = (ep.N + 128 * mb - 1) / (128 * mb) * p.t_tiles;
   p.acc_cols = (cols + 31) / 32 * 32;
   p.bufs = 2 * mb * p.acc_cols <= 512 ? 2 : 1;
   p.tmem_cols = 32;
@@ -902,8 +837,9 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensor
   p.stages = std::min(NW_MAX_STAGES, NW_RING / p.stage_bytes);
   p.ws = ws.partial;
   // at least four K blocks per CTA: finer splits cost more in partial sums than they stream sooner
-  const long long U = (long long)p.n_tiles * p.n_kb;
-  const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min<long long>(p.n_tiles, ws.n_sm), U / 4));
+  const long long U = (long long)n_tiles * n_kb;
+  const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min<long long>(n_tiles, ws.n_sm), U / 4));
+  p.share = share_tiles(n_tiles, n_kb, grid, p.t_tiles == 1, NW_PARTS);
   auto go = [&](auto m) {
     constexpr int MODE = decltype(m)::value;
     if (terms == 3) return launch_narrow_mode<MODE, 1, true>(w, x, p, grid, ep, s);
@@ -946,8 +882,7 @@ cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int
   p.tp = narrow_tp(ep.T, terms);
   p.t_tiles = (ep.T + p.tp - 1) / p.tp;
   const int cols = p.tp * terms;
-  p.n_kb = (K + 127) / 128;
-  p.n_tiles = (ep.N + 255) / 256 * p.t_tiles;
+  const int n_kb = (K + 127) / 128, n_tiles = (ep.N + 255) / 256 * p.t_tiles;
   p.acc_cols = (cols + 31) / 32 * 32;
   p.bufs = 4 * p.acc_cols <= 512 ? 2 : 1;
   p.tmem_cols = 32;
@@ -960,8 +895,9 @@ cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int
   r.c_stages = std::min(N4_MAX_CODE_STAGES, (NW_RING - r.a_stages * N4_A_BYTES - r.x_stages * r.x_bytes) / N4_CODE_BYTES);
   p.ws = ws.partial;
   // at least two units (2 x 128 columns) per CTA, as prefill_narrow_kernel's four K blocks of 64
-  const long long U = (long long)p.n_tiles * p.n_kb;
-  const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min<long long>(p.n_tiles, ws.n_sm), U / 2));
+  const long long U = (long long)n_tiles * n_kb;
+  const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min<long long>(n_tiles, ws.n_sm), U / 2));
+  p.share = share_tiles(n_tiles, n_kb, grid, p.t_tiles == 1, NW_PARTS);
   auto go = [&](auto m) {
     return launch_narrow4_mode<decltype(m)::value>(r, x, p, grid, ep, s);
   };

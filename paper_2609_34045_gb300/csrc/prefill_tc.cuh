@@ -150,6 +150,158 @@ __device__ __forceinline__ void split_terms(float x, uint16_t (&t)[3], int terms
     t[2] = f16 ? f32_to_f16_rn(r) : f32_to_bf16_rne(r);
   }
 }
+// ---- int4 weights as fp16 MMA operands
+__device__ __forceinline__ void stsm_x4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2),
+               "r"(r3)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t hmul2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t hfma2(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t r;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+
+// The eight codes of an A-fragment word as exact fp16 pairs: rows gid and gid + 8 of columns 2 tig,
+// 2 tig + 1 (c0, c1) and of columns 2 tig + 8, 2 tig + 9 (c2, c3).  The nibbles, top bit flipped, become
+// 1024 + u or 1024 + 16 u (u = code + 8).
+__device__ __forceinline__ void decode_word(uint32_t w, uint32_t &c0, uint32_t &c1, uint32_t &c2, uint32_t &c3) {
+  const uint32_t w8 = w >> 8;
+  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c0) : "r"(w), "r"(0x000F000Fu), "r"(0x64086408u));
+  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c1) : "r"(w8), "r"(0x000F000Fu), "r"(0x64086408u));
+  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c2) : "r"(w), "r"(0x00F000F0u), "r"(0x64806480u));
+  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c3) : "r"(w8), "r"(0x00F000F0u), "r"(0x64806480u));
+  c0 = hfma2(c0, 0x3C003C00u, 0xE408E408u);  // - 1032
+  c1 = hfma2(c1, 0x3C003C00u, 0xE408E408u);
+  c2 = hfma2(c2, 0x2C002C00u, 0xD480D480u);  // / 16 - 72
+  c3 = hfma2(c3, 0x2C002C00u, 0xD480D480u);
+}
+
+// fp16 pair of codes times an fp32 scale, rounded once.
+__device__ __forceinline__ uint32_t scale_pair_f32(uint32_t c, float sc) {
+  return (uint32_t)f32_to_f16_rn(f16_to_f32((uint16_t)c) * sc) |
+         ((uint32_t)f32_to_f16_rn(f16_to_f32((uint16_t)(c >> 16)) * sc) << 16);
+}
+
+// The bf16 scales of rows gid and gid + 8 of a weight group, applied to decode_word's codes.
+struct ScalePair {
+  float s0, s1;
+  uint32_t p0, p1;
+  __device__ __forceinline__ explicit ScalePair(uint32_t sc) : s0(bf16_lo(sc)), s1(bf16_hi(sc)) {
+    p0 = f32_to_f16_rn(s0) * 0x10001u;
+    p1 = f32_to_f16_rn(s1) * 0x10001u;
+  }
+  // scales that fp16 holds exactly: the fp16 product of code and scale is rounded as the fp32 product
+  // would be; others (below 2^-14, or too large) go through fp32
+  __device__ __forceinline__ bool exact() const {
+    return f16_to_f32((uint16_t)p0) == s0 && f16_to_f32((uint16_t)p1) == s1;
+  }
+  __device__ __forceinline__ void apply(bool exact, uint32_t &c0, uint32_t &c1, uint32_t &c2, uint32_t &c3) const {
+    if (exact) {
+      c0 = hmul2(c0, p0), c1 = hmul2(c1, p1), c2 = hmul2(c2, p0), c3 = hmul2(c3, p1);
+    } else {
+      c0 = scale_pair_f32(c0, s0), c1 = scale_pair_f32(c1, s1);
+      c2 = scale_pair_f32(c2, s0), c3 = scale_pair_f32(c3, s1);
+    }
+  }
+};
+
+// How the CTAs of a GEMM share its output tiles (each n_kb K blocks long).  Whole tiles first, tile
+// c + i G to CTA c, for `waves` rounds: the CTAs at work together then read few weight rows and few
+// tokens, at the same K, from L2.  The `tail` tiles left over would leave SMs idle in a last round:
+//  - splits = 0 (one token tile: the weights pass through L2 once, whatever the order): as one
+//    sequence of K blocks of which CTA c takes [c U / G, (c + 1) U / G), an equal share to the block; the
+//    last whole round joins it, so that no tile is cut more than about twice more than it must be;
+//  - splits = S: every tail tile's K in S parts, part p of all tiles before part p + 1 of any, so that
+//    CTAs at work together still read the same K (the sequence had each at a K of its own: 2048
+//    tokens' down projection, 290 MB of weights and tokens, went from 201 to 281 us).
+// A cut tile is summed from its partial sums, in K order, by a kernel behind the GEMM.
+struct TileShare {
+  int n_kb, waves, tail, splits;
+  bool cut() const { return tail > 0 && splits != 1; }
+};
+// parts_per_cta: how many partial sums per CTA the workspace holds (2 for the sequence).
+inline TileShare share_tiles(int tiles, int n_kb, int grid, bool sequence, int parts_per_cta) {
+  TileShare s = {n_kb, tiles / grid, tiles % grid, 1};
+  if (s.tail == 0) return s;
+  // (the device's arithmetic on the sequence is 32-bit: a 64-bit division is a microsecond's start)
+  if (sequence && (long long)(tiles % grid + grid) * n_kb * grid < (1ll << 31)) {
+    s.splits = 0;
+    if (s.waves > 0) --s.waves, s.tail += grid;
+    return s;
+  }
+  // in K blocks' time: rounds of parts, a few blocks' worth of ring refill per round, and for cut tiles
+  // the kernel that sums them (its launch, and 256 KB written and read per part)
+  double best = 1e30;
+  for (int S = 1; S <= 8 && S * 4 <= n_kb && (S == 1 || S * s.tail <= parts_per_cta * grid); ++S) {
+    const int rounds = (s.tail * S + grid - 1) / grid;
+    const double t = rounds * ((n_kb + S - 1) / S + 2.0) + (S > 1 ? 10.0 + s.tail * S / 12.0 : 0.0);
+    if (t < best) best = t, s.splits = S;
+  }
+  return s;
+}
+// One CTA's segments in order: K blocks [kb0, kb1) of `tile`; `part`: its place among the partial sums.
+struct TileWalk {
+  TileShare s;
+  int i, tile, kb0, kb1, part;
+  unsigned u, u1;
+  __device__ __forceinline__ explicit TileWalk(const TileShare &share) : s(share), i(0) {
+    const unsigned U = s.splits == 0 ? s.tail * s.n_kb : 0;
+    u = blockIdx.x * U / gridDim.x;
+    u1 = (blockIdx.x + 1) * U / gridDim.x;
+  }
+  __device__ __forceinline__ bool next() {
+    if (i < s.waves) {
+      tile = blockIdx.x + i * gridDim.x;
+      kb0 = 0;
+      kb1 = s.n_kb;
+    } else if (s.splits > 0) {
+      part = blockIdx.x + (i - s.waves) * gridDim.x;
+      if (part >= s.tail * s.splits) return false;
+      const int sp = part / s.tail;
+      tile = s.waves * gridDim.x + part - sp * s.tail;
+      kb0 = sp * s.n_kb / s.splits;
+      kb1 = (sp + 1) * s.n_kb / s.splits;
+    } else {
+      if (u >= u1) return false;
+      const unsigned t = u / (unsigned)s.n_kb;
+      tile = s.waves * gridDim.x + t;
+      kb0 = (int)(u - t * s.n_kb);
+      kb1 = min(s.n_kb, kb0 + (int)(u1 - u));
+      part = blockIdx.x * 2 + (kb0 > 0 ? 0 : 1);
+      u += kb1 - kb0;
+    }
+    ++i;
+    return true;
+  }
+  __device__ __forceinline__ bool whole() const { return kb0 == 0 && kb1 == s.n_kb; }
+};
+// The partial sums of tail tile k, in K order.
+struct TileParts {
+  int n, at, step, rest;  // part i: i == 0 ? at : rest + i * step
+  __device__ __forceinline__ TileParts(const TileShare &s, int k, int grid) {
+    if (s.splits > 0) {
+      n = s.splits;
+      at = rest = k;
+      step = s.tail;
+    } else {
+      // the CTAs first .. last meet the tile; every one but the first starts inside it
+      const unsigned U = s.tail * s.n_kb, G = grid, lo = k * s.n_kb;
+      const int first = (int)(((lo + 1) * G - 1) / U), last = (int)(((lo + s.n_kb) * G - 1) / U);
+      n = last - first + 1;
+      at = first * 2 + (first * U / G > lo ? 0 : 1);
+      rest = first * 2;
+      step = 2;
+    }
+  }
+  __device__ __forceinline__ int part(int i) const { return i == 0 ? at : rest + i * step; }
+};
+
 // Two values as packed pairs of their hi and lo terms.  fp16 terms of a value that fp16 cannot
 // hold (|x| >= 65520 rounds to infinity, or not finite) set ERR_F16_RANGE in *err.
 __device__ __forceinline__ void split_pack(float x0, float x1, uint32_t &hi, uint32_t &lo, int f16 = 0,

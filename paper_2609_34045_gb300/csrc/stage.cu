@@ -798,12 +798,19 @@ constexpr int PF_PAIR_TOKENS = 512;  // passes of up to this many tokens carry q
 
 int pf_ld(int n) { return round_up(n, 64); }
 
-// Whether a pass of n tokens runs on the few-token GEMM: few tokens, or three terms per activation,
-// which the 128-token tiles do not take.
-bool pf_narrow(const kfl_stage *st, int n, bool precise = false) {
-  if (precise) return true;
-  return n <= (st->cfg.weight_fmt == KFL_BF16 ? NW_MAX_TP : env_int("KFL_N4_MAX", N4_MAX_TOKENS));
+// The most tokens that a pass on the few-token GEMM takes (with two terms; passes with three always take
+// it: the 128-token tiles do not).  bf16: 128, one token tile; two tiles and up are faster at 128
+// tokens x 256 rows (one 7B-shaped block: 240 us at 128 tokens either way, 408 against 465 at 500),
+// unless the model is so small that those tiles, of its largest matrix, leave SMs without one (two
+// blocks of d 512, F 1408: 76 against 102 us at 500 tokens, equal at 2048).  int4: while decoding the
+// weights once per token tile is cheaper than the fp16 copies (72B-shaped block: 785 against 1026
+// us at 256 tokens, 1389 against 1517 at 512, 2014 against 1948 at 700).
+int pf_narrow_most(const kfl_stage *st) {
+  if (st->cfg.weight_fmt != KFL_BF16) return N4_MAX_TOKENS;
+  const int n_tiles = (2 * st->P.F + PG_N - 1) / PG_N;
+  return std::max(NW_MAX_TP, std::min(PF_PASS, (st->P.n_sm - 1) / n_tiles * PG_M));
 }
+bool pf_narrow(const kfl_stage *st, int n, bool precise = false) { return precise || n <= pf_narrow_most(st); }
 
 // Workspace for passes of up to `tokens` tokens (grown, never shrunk) and the weight maps.
 int ensure_prefill(kfl_stage *st, int tokens) {
@@ -831,7 +838,7 @@ int ensure_prefill(kfl_stage *st, int tokens) {
     if (st->cfg.qk_norm) ok = ok && get((void **)&st->pf_raw, (size_t)cap * P.ld_raw * 4);
     // argmax partials: per 256-column tile, or (passes on the few-token GEMM) per 32 rows
     if (st->flags & KFL_LOGITS_OUT) {
-      const int most = st->cfg.weight_fmt != KFL_BF16 ? N4_MAX_TOKENS : st->cfg.qk_norm ? PF_PASS : NW_MAX_TP;
+      const int most = st->cfg.qk_norm ? PF_PASS : pf_narrow_most(st);
       const int narrow = std::min(cap, most);
       const size_t am = std::max((size_t)cap * ((P.V + PG_N - 1) / PG_N), (size_t)narrow * narrow_argmax_slots(P.V));
       ok = ok && get((void **)&st->pf_amax, am * 4) && get((void **)&st->pf_aidx, am * 4);
@@ -959,14 +966,12 @@ struct PfInput {
   }
 };
 
-// One prefill GEMM with matrix j of block l (j = 4: lm_head).  bf16 stages run passes of up to
-// NW_MAX_TP tokens on the few-token kernel, longer ones (and int4 stages) on 128-token tiles with
-// the split count chosen for the shape.  int4 stages read the matrix's fp16 copy, dequantized ahead on
+// One prefill GEMM with matrix j of block l (j = 4: lm_head): on the few-token kernel (pf_narrow) or on
+// 128-token tiles.  int4 stages then read the matrix's fp16 copy, dequantized ahead on
 // the side stream (the next one is started before this GEMM, so dequantization overlaps the products).
 cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, PrefillEpiParams e, cudaStream_t s) {
   const Mat &m = pf_mat(st, l, j);
   const bool i4 = st->cfg.weight_fmt == KFL_INT4_G64;
-  int n_kt = m.n_kt;
   const CUtensorMap *b;
   const int g = st->pf_seq++;
   e.T = x.n;
@@ -986,12 +991,10 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, st->pf_deq[g % 2], 0);
     if (err != cudaSuccess) return err;
     b = &st->pf_maps[(g % 2) * 5 + j];
-    n_kt = 2 * m.n_kt;  // K tiles of 128 fp16
   } else {
     b = &st->pf_maps[j == 4 ? 4 * st->P.nl : 4 * l + j];
   }
-  e.splits = mode == PE_ARGMAX ? 1 : prefill_splits(e.T, e.N, n_kt, st->P.n_sm);
-  cudaError_t err = launch_prefill_gemm(mode, x.term[0], x.term[1], *b, n_kt, e, s);
+  cudaError_t err = launch_prefill_gemm(mode, x.term[0], x.term[1], *b, m.K, st->pf_nw, e, s);
   if (err == cudaSuccess && i4) err = cudaEventRecord(st->pf_used[g % 2], s);
   return err;
 }
