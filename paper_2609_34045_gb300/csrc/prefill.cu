@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 
 #include "../../include/kafila_gemm.h"
 #include "prefill_tc.cuh"
@@ -162,8 +163,8 @@ __device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t da, uint64_t db,
 
 // ---------------------------------------------------------------------------- GEMM kernel
 // One CTA per SM walks its share of the tiles (TileShare).  The TMA ring runs on across tile
-// boundaries, and two accumulators (all 512 TMEM columns) let the MMAs of the next tile proceed while
-// four epilogue warps drain the previous one.  Warp 0 issues TMA, warp 1 MMAs, warps 2-5 run the
+// boundaries, and two accumulators (all 512 TMEM columns) let the MMAs proceed while
+// the epilogue warps read the previous one.  Warp 0 issues TMA, warp 1 MMAs, warps 2-5 (2-9) run the
 // epilogue (warp w reads TMEM lanes 32 (w % 4) ..).  Every wait is bounded; a CTA that gives up sets
 // ERR_TIMEOUT, lets its copies and MMAs in flight complete (bounded), frees its TMEM and returns.
 //
@@ -172,16 +173,25 @@ __device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t da, uint64_t db,
 // launch and distributed shared memory: the down projection of 500 tokens (56 tiles) took 173 us, now
 // 85 with the kernel that sums its parts.  Two 7B-shaped blocks: 931 -> 815 us at 500 tokens, 2620 -> 1951 at
 // 1500, 2608 at 2048 as before (its tiles fill their rounds).
-constexpr int PP_THREADS = 192;
+//
+// DRAIN (the plain product): each accumulator takes only PP_CHUNK K blocks, and eight epilogue warps add
+// the chunks up in registers: tensor-core accumulation truncates (prefill_narrow_kernel says how
+// much), and an unsplit K of 18944 leaves the product of 2048 tokens 3.8e-5 off, drained 3.3e-6.  A
+// stage's products go without: attention's bf16 softmax weights leave 1e-3 at these lengths, and
+// the sums' registers cost the fused epilogues spills.
+constexpr int PP_CHUNK = 16;
+__host__ __device__ constexpr int pp_epi_warps(bool drain) { return drain ? 8 : 4; }
+__host__ __device__ constexpr int pp_threads(bool drain) { return (2 + pp_epi_warps(drain)) * 32; }
 constexpr int PP_TMEM_COLS = 2 * PG_N;
 
 // Where (in float4, plus the token row) a partial holds columns 4 j .. of the tile.
 __device__ __forceinline__ size_t wide_partial(int part, int j) { return ((size_t)part * (PG_N / 4) + j) * PG_M; }
 
-template <int MODE>
-__global__ void __launch_bounds__(PP_THREADS, 1)
+template <int MODE, bool DRAIN>
+__global__ void __launch_bounds__(pp_threads(DRAIN), 1)
     prefill_gemm_persistent(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_a2,
-                            const __grid_constant__ CUtensorMap tm_b, TileShare share, float *ws, PrefillEpiParams ep) {
+                            const __grid_constant__ CUtensorMap tm_b, int w_rows, TileShare share, float *ws,
+                            PrefillEpiParams ep) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t s_full[PG_STAGES], s_empty[PG_STAGES], s_acc_full[2], s_acc_empty[2], s_drain;
   __shared__ uint32_t s_tmem;
@@ -198,7 +208,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_addr(&s_acc_full[b]), 1);
-      mbar_init(smem_addr(&s_acc_empty[b]), 4);  // one arrival per epilogue warp
+      mbar_init(smem_addr(&s_acc_empty[b]), pp_epi_warps(DRAIN));  // one arrival per epilogue warp
     }
     mbar_init(smem_addr(&s_drain), 1);
     s_abort = 0;
@@ -231,7 +241,10 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
           tma_load_2d(sa + s * 2 * PG_A_BYTES, &tm_a, kb * PG_K, t0, full);
           tma_load_2d(sa + s * 2 * PG_A_BYTES + PG_A_BYTES, &tm_a2, kb * PG_K, t0, full);
           // weight tiles: (column within the K tile, row within the row block, K tile, row block)
-          tma_load_4d(sb + s * PG_B_BYTES, &tm_b, (kb & 1) * PG_K, 0, kb >> 1, n0 / RB, full);
+          if (w_rows)
+            tma_load_2d(sb + s * PG_B_BYTES, &tm_b, kb * PG_K, n0, full);
+          else
+            tma_load_4d(sb + s * PG_B_BYTES, &tm_b, (kb & 1) * PG_K, 0, kb >> 1, n0 / RB, full);
         }
         __syncwarp();
         if (++s == PG_STAGES) s = 0, ++use;
@@ -249,25 +262,31 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    // ---- MMA issuer (the whole warp, one elected lane issuing): segment i of this CTA accumulates
-    // into TMEM columns (i % 2) * PG_N
+    // ---- MMA issuer (the whole warp, one elected lane issuing): segment i of this CTA (DRAIN:
+    // chunk i of its segments) accumulates into TMEM columns (i % 2) * PG_N
     const uint32_t idesc = ep.f16 ? idesc_kind_f16(PG_M, PG_N, false) : idesc_kind_f16(PG_M, PG_N, true);
-    int s = 0, i = 0;
+    TileWalk w(share);
+    int s = 0, left = 0;
     uint32_t use = 0;
     bool ok = true;
-    for (TileWalk w(share); ok && w.next(); ++i) {
-      const int buf = i & 1;
+    for (int i = 0; ok; ++i) {
+      if (left == 0) {
+        if (!w.next()) break;
+        left = w.kb1 - w.kb0;
+      }
+      const int n = DRAIN ? min(left, PP_CHUNK) : left, buf = i & 1;
+      left -= n;
       if (i >= 2) ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&s_acc_empty[buf]), ((i >> 1) - 1) & 1));
       if (!ok) break;
       tc_fence_after();
       const uint32_t d = tmem + (uint32_t)(buf * PG_N);
-      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+      for (int kb = 0; kb < n; ++kb) {
         ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_full[s]), use & 1));
         if (!ok) break;
         tc_fence_after();
         const uint64_t da = sdesc_k_sw128(sa + s * 2 * PG_A_BYTES), db = sdesc_k_sw128(sb + s * PG_B_BYTES);
         if (elect_one()) {
-          mma_kblock(d, da, db, idesc, kb != w.kb0);
+          mma_kblock(d, da, db, idesc, kb != 0);
           mma_commit(smem_addr(&s_empty[s]));
         }
         __syncwarp();
@@ -285,30 +304,34 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     __syncwarp();
     mbar_wait(smem_addr(&s_drain), 0);
   } else {
-    // ---- epilogue warps 2..5: TMEM lanes 32 q .. 32 q + 31 (q = warp % 4) are tokens t0 + 32 q + lane
+    // ---- epilogue warps: TMEM lanes 32 q .. 32 q + 31 (q = warp % 4) are tokens t0 + 32 q + lane
     const int q = warp & 3, row = 32 * q + lane;
+    const uint32_t lanes = tmem + ((uint32_t)(32 * q) << 16);
     int i = 0;
-    for (TileWalk w(share); w.next(); ++i) {
-      const int buf = i & 1;
-      const bool ready = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_acc_full[buf]), (i >> 1) & 1));
-      if (!ready) {
-        if (lane == 0) {
-          *abort_flag = 1;
-          atomicOr(ep.err, ERR_TIMEOUT);
-        }
-        break;
+    // accumulator i is complete; false: given up
+    auto wait_acc = [&]() {
+      const bool ready = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_addr(&s_acc_full[i & 1]), (i >> 1) & 1));
+      if (!ready && lane == 0) {
+        *abort_flag = 1;
+        atomicOr(ep.err, ERR_TIMEOUT);
       }
       tc_fence_after();
+      return ready;
+    };
+    auto release_acc = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_addr(&s_acc_empty[i & 1]));
+      ++i;
+    };
+    bool ok = true;
+    for (TileWalk w(share); ok && w.next();) {
       const int n_tile = w.tile / t_tiles, t = (w.tile % t_tiles) * PG_M + row, n0 = n_tile * PG_N;
       const bool whole = w.whole();
       EpiState<MODE> st;
-      for (int c = 0; c < PG_N / 32; ++c) {
-        const int n = n0 + 32 * c;
-        if (n >= ep.N) break;  // uniform across the warp
-        uint32_t r[32];
-        tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * PG_N + 32 * c), r);
+      auto finish = [&](int c, const uint32_t(&r)[32]) {
         if (whole) {
-          if (t < ep.T) epilogue32<MODE>(ep, t, n, r, st);
+          if (t < ep.T) epilogue32<MODE>(ep, t, n0 + 32 * c, r, st);
         } else {
           float4 *at = reinterpret_cast<float4 *>(ws) + wide_partial(w.part, 8 * c) + row;
 #pragma unroll
@@ -316,16 +339,47 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
             at[j * PG_M] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
                                        __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
         }
-      }
-      if constexpr (MODE == PE_ARGMAX) {
-        if (whole && t < ep.T) {
-          ep.amax[(size_t)t * ep.n_tiles + n_tile] = st.best;
-          ep.aidx[(size_t)t * ep.n_tiles + n_tile] = st.bidx;
+      };
+      if constexpr (DRAIN) {
+        // warps 2-5 take columns 0-127, warps 6-9 columns 128-255
+        const int c0 = (warp - 2) >> 2 << 2;
+        uint32_t sum[4][32];
+        for (int left = w.kb1 - w.kb0; left > 0; left -= PP_CHUNK) {
+          if (!(ok = wait_acc())) break;
+          const bool first = left == w.kb1 - w.kb0;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            uint32_t r[16];
+            tmem_ld16(lanes + (uint32_t)((i & 1) * PG_N + 32 * c0 + 16 * c), r);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              uint32_t &y = sum[c / 2][(c & 1) * 16 + j];
+              y = first ? r[j] : __float_as_uint(__uint_as_float(y) + __uint_as_float(r[j]));
+            }
+          }
+          release_acc();
         }
+        if (!ok) break;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (n0 + 32 * (c0 + c) < ep.N) finish(c0 + c, sum[c]);  // uniform across the warp
+      } else {
+        if (!(ok = wait_acc())) break;
+        for (int c = 0; c < PG_N / 32; ++c) {
+          if (n0 + 32 * c >= ep.N) break;  // uniform across the warp
+          uint32_t r[32];
+          tmem_ld32(lanes + (uint32_t)((i & 1) * PG_N + 32 * c), r);
+          finish(c, r);
+        }
+        if constexpr (MODE == PE_ARGMAX) {
+          if (whole && t < ep.T) {
+            ep.amax[(size_t)t * ep.n_tiles + n_tile] = st.best;
+            ep.aidx[(size_t)t * ep.n_tiles + n_tile] = st.bidx;
+          }
+        }
+        release_acc();
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_addr(&s_acc_empty[buf]));
     }
   }
   tc_fence_before();
@@ -850,11 +904,39 @@ __global__ void __launch_bounds__(128) dequant_int4_f16_kernel(const uint8_t *ti
   }
 }
 
-// fp32 rows [T][K] (stride ldx) -> hi and lo bf16 terms (stride ld).
-__global__ void split_rows_kernel(const float *x, int K, int ldx, uint16_t *hi, uint16_t *lo, int ld) {
-  const int t = blockIdx.x;
-  for (int i = threadIdx.x; i < K; i += blockDim.x)
-    split_bf16(x[(size_t)t * ldx + i], hi[(size_t)t * ld + i], lo[(size_t)t * ld + i]);
+// fp32 rows [T][K] (stride ldx) -> hi and lo bf16 terms (stride ld), 1024 columns to a block; *err = 0.
+__global__ void __launch_bounds__(256) split_rows_kernel(const float *x, int K, int ldx, uint16_t *hi, uint16_t *lo,
+                                                         int ld, unsigned *err) {
+  pdl_launch_dependents();
+  const int t = blockIdx.y, i0 = blockIdx.x * 1024 + threadIdx.x;
+  if (t == 0 && i0 == 0) *err = 0;
+  float v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = i0 + 256 * j < K ? x[(size_t)t * ldx + i0 + 256 * j] : 0.f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (i0 + 256 * j < K) split_bf16(v[j], hi[(size_t)t * ld + i0 + 256 * j], lo[(size_t)t * ld + i0 + 256 * j]);
+}
+
+// A row-major matrix [N][K] whose rows TMA cannot address as weight tiles [n_rb][n_kt][RB][KT]
+// (zero-padded), one block per tile: each thread has 32 two-byte loads in flight.  (The loaders' repack
+// kernel, a thread per 16 bytes over a fixed grid with 64-bit index arithmetic, took 110 us for 233 MB.)
+__global__ void __launch_bounds__(256) tile_rows_kernel(const uint16_t *w, int N, int K, int n_kt, uint8_t *dst) {
+  const int rb = blockIdx.x / n_kt, kt = blockIdx.x - rb * n_kt;
+  const int ch = threadIdx.x % (KT / 8), r0 = threadIdx.x / (KT / 8), k0 = kt * KT + ch * 8;
+  uint16_t v[4][8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = rb * RB + r0 + 16 * i;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[i][j] = r < N && k0 + j < K ? w[(size_t)r * K + k0 + j] : uint16_t(0);
+  }
+  uint4 *tile = reinterpret_cast<uint4 *>(dst + (size_t)blockIdx.x * TILE_BYTES);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    tile[(r0 + 16 * i) * (KT / 8) + ch] =
+        make_uint4(v[i][0] | (uint32_t)v[i][1] << 16, v[i][2] | (uint32_t)v[i][3] << 16, v[i][4] | (uint32_t)v[i][5] << 16,
+                   v[i][6] | (uint32_t)v[i][7] << 16);
 }
 
 // next_ids[t]: the lowest index among the largest logits, over the column tiles' partial maxima;
@@ -935,6 +1017,20 @@ int encode_terms_map(CUtensorMap *map, const uint16_t *base, int K, int rows, in
              : -1;
 }
 
+int encode_rows_map(CUtensorMap *map, const uint16_t *w, int K, int N, int box_rows) {
+  auto fn = encode_fn();
+  if (!fn || K % 8 != 0 || (reinterpret_cast<uintptr_t>(w) & 15) != 0) return -1;
+  const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)N};
+  const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
+  const cuuint32_t box[2] = {PG_K, (cuuint32_t)box_rows};
+  const cuuint32_t estr[2] = {1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t *>(w), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? 0
+             : -1;
+}
+
 // Weight tiles [n_rb][n_kt][RB][KT] bf16 as a 4-D tensor (column, row, K tile, row block):
 // boxes of 64 columns x RB rows x 1 K tile x box_rb row blocks; row blocks >= n_rb read as zero.
 int encode_tiles_map(CUtensorMap *map, const uint8_t *tiles, int n_kt, int n_rb, int box_rb) {
@@ -967,11 +1063,12 @@ static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int threads, size
 }
 
 template <int MODE>
-static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b, int n_kb,
+static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b, bool w_rows, int n_kb,
                                const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
+  constexpr bool DRAIN = MODE == PE_STORE;
   static bool smem_set = false;
   if (!smem_set) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_gemm_persistent<MODE>,
+    cudaError_t e = cudaFuncSetAttribute(prefill_gemm_persistent<MODE, DRAIN>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
     if (e != cudaSuccess) return e;
     smem_set = true;
@@ -980,23 +1077,24 @@ static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, cons
   const int tiles = (ep.T + PG_M - 1) / PG_M * ((ep.N + PG_N - 1) / PG_N);
   const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min(tiles, ws.n_sm), (long long)tiles * n_kb / 4));
   const TileShare share = share_tiles(tiles, n_kb, grid, false, NW_PARTS);
-  cudaError_t e = launch_pdl(prefill_gemm_persistent<MODE>, dim3(grid), PP_THREADS, PG_SMEM, s, a, a2, b, share, ws.partial, ep);
+  cudaError_t e = launch_pdl(prefill_gemm_persistent<MODE, DRAIN>, dim3(grid), pp_threads(DRAIN), PG_SMEM, s, a, a2, b, (int)w_rows, share,
+                             ws.partial, ep);
   if (e == cudaSuccess && share.cut())
     e = launch_pdl(wide_reduce_kernel<MODE>, dim3(share.tail * (MODE == PE_ARGMAX ? 1 : PG_N / 32)), PG_M, 0, s, share,
                    grid, ws.partial, ep);
   return e;
 }
 
-cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b, int K,
-                                const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
+cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b,
+                                bool w_rows, int K, const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
   if (ep.T <= 0 || ep.N <= 0) return cudaSuccess;
   const int n_kb = (K + PG_K - 1) / PG_K;
   switch (mode) {
-    case PE_STORE: return launch_mode<PE_STORE>(a, a2, b, n_kb, ws, ep, s);
-    case PE_RESID: return launch_mode<PE_RESID>(a, a2, b, n_kb, ws, ep, s);
-    case PE_SWIGLU: return launch_mode<PE_SWIGLU>(a, a2, b, n_kb, ws, ep, s);
-    case PE_QKV: return launch_mode<PE_QKV>(a, a2, b, n_kb, ws, ep, s);
-    case PE_ARGMAX: return launch_mode<PE_ARGMAX>(a, a2, b, n_kb, ws, ep, s);
+    case PE_STORE: return launch_mode<PE_STORE>(a, a2, b, w_rows, n_kb, ws, ep, s);
+    case PE_RESID: return launch_mode<PE_RESID>(a, a2, b, w_rows, n_kb, ws, ep, s);
+    case PE_SWIGLU: return launch_mode<PE_SWIGLU>(a, a2, b, w_rows, n_kb, ws, ep, s);
+    case PE_QKV: return launch_mode<PE_QKV>(a, a2, b, w_rows, n_kb, ws, ep, s);
+    case PE_ARGMAX: return launch_mode<PE_ARGMAX>(a, a2, b, w_rows, n_kb, ws, ep, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1054,9 +1152,13 @@ cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, u
   return cudaGetLastError();
 }
 
-cudaError_t launch_split_bf16(const float *x, int T, int K, int ldx, uint16_t *hi, uint16_t *lo, int ld,
+cudaError_t launch_split_bf16(const float *x, int T, int K, int ldx, uint16_t *hi, uint16_t *lo, int ld, unsigned *err,
                               cudaStream_t s) {
-  split_rows_kernel<<<T, 256, 0, s>>>(x, K, ldx, hi, lo, ld);
+  for (int t0 = 0; t0 < T; t0 += 65535) {  // the grid's y limit
+    const int n = std::min(65535, T - t0);
+    split_rows_kernel<<<dim3((K + 1023) / 1024, n), 256, 0, s>>>(x + (size_t)t0 * ldx, K, ldx, hi + (size_t)t0 * ld,
+                                                               lo + (size_t)t0 * ld, ld, err);
+  }
   return cudaGetLastError();
 }
 
@@ -1068,6 +1170,50 @@ cudaError_t launch_prefill_argmax(const float *amax, const int *aidx, int n_tile
 }  // namespace kfl
 
 // ---------------------------------------------------------------------------- C ABI
+namespace {
+
+// The device's memory pool for kfl_matmul_bf16w's temporary buffers, made at its first call there.  Of
+// what the calls free, the pool keeps up to MATMUL_KEEP_BYTES for the next and returns the rest at
+// their synchronisation; a cudaMalloc and cudaFree per call cost 80 to 250 us.  Calls on several
+// threads and streams each take buffers of their own from it.
+constexpr uint64_t MATMUL_KEEP_BYTES = 64ull << 20;
+constexpr int MATMUL_MAX_DEVICES = 64;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pool[MATMUL_MAX_DEVICES] = {};
+
+cudaMemPool_t matmul_pool(int dev) {
+  if (dev < 0 || dev >= MATMUL_MAX_DEVICES) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = MATMUL_KEEP_BYTES;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      if (pool) cudaMemPoolDestroy(pool);
+      return nullptr;
+    }
+    g_pool[dev] = pool;
+  }
+  return g_pool[dev];
+}
+
+}  // namespace
+
+namespace kfl {
+// Returns what the current device's pool keeps (a stage that finds no memory asks for it).
+bool release_matmul_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MATMUL_MAX_DEVICES) return false;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  return g_pool[dev] && cudaMemPoolTrimTo(g_pool[dev], 0) == cudaSuccess;
+}
+}  // namespace kfl
+
 extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uint16_t *w, int N, float *y, int ldy,
                                 void *cuda_stream) {
   using namespace kfl;
@@ -1081,13 +1227,15 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     cudaGetLastError();
     return KFL_ERR_CUDA;
   }
-  // few tokens: the few-token kernel
-  const bool narrow = T <= NW_MAX_TP;
+  // few tokens: the few-token kernel.  A matrix whose rows TMA can address is read where it is; others
+  // (K not a multiple of 8, or an unaligned start) are copied into weight tiles first
+  const bool narrow = T <= NW_MAX_TP, w_rows = K % 8 == 0 && (reinterpret_cast<uintptr_t>(w) & 15) == 0;
   const int rows = (T + 7) / 8 * 8;
-  const size_t tile_bytes = (size_t)n_rb * n_kt * TILE_BYTES, x_bytes = (size_t)rows * ld * 2;
+  const size_t tile_bytes = w_rows ? 0 : (size_t)n_rb * n_kt * TILE_BYTES, x_bytes = (size_t)rows * ld * 2;
   const size_t ws_bytes = narrow_ws_bytes(n_sm, T);
+  cudaMemPool_t pool = matmul_pool(dev);
   void *mem = nullptr;
-  if (cudaMalloc(&mem, tile_bytes + 2 * x_bytes + ws_bytes + 16) != cudaSuccess) {
+  if (!pool || cudaMallocFromPoolAsync(&mem, tile_bytes + 2 * x_bytes + ws_bytes + 16, pool, s) != cudaSuccess) {
     cudaGetLastError();
     return KFL_ERR_OOM;
   }
@@ -1098,14 +1246,14 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
   unsigned *err = reinterpret_cast<unsigned *>(reinterpret_cast<uint8_t *>(partial) + ws_bytes);
   int rc = KFL_OK;
   CUtensorMap mh, ml, mb;
-  if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess ||
-      launch_split_bf16(x, T, K, ldx, xhi, xlo, ld, s) != cudaSuccess ||
-      launch_repack_bf16(w, N, K, nullptr, N, n_rb, n_kt, tiles, s) != cudaSuccess) {
+  if (!w_rows) tile_rows_kernel<<<(unsigned)n_rb * n_kt, 256, 0, s>>>(w, N, K, n_kt, tiles);
+  if (cudaPeekAtLastError() != cudaSuccess ||
+      launch_split_bf16(x, T, K, ldx, xhi, xlo, ld, err, s) != cudaSuccess) {
     rc = KFL_ERR_CUDA;
-  } else if (narrow ? encode_terms_map(&mh, xhi, K, T, ld, 2, (size_t)rows * ld, narrow_tp(T, 2)) ||
-                          encode_tiles_map(&mb, tiles, n_kt, n_rb, 128 / RB)
-                    : encode_act_map(&mh, xhi, K, T, ld) || encode_act_map(&ml, xlo, K, T, ld) ||
-                          encode_tiles_map(&mb, tiles, n_kt, n_rb, PG_N / RB)) {
+  } else if ((narrow ? encode_terms_map(&mh, xhi, K, T, ld, 2, (size_t)rows * ld, narrow_tp(T, 2))
+                     : encode_act_map(&mh, xhi, K, T, ld) || encode_act_map(&ml, xlo, K, T, ld)) ||
+             (w_rows ? encode_rows_map(&mb, w, K, N, narrow ? 128 : PG_N)
+                     : encode_tiles_map(&mb, tiles, n_kt, n_rb, (narrow ? 128 : PG_N) / RB))) {
     rc = KFL_ERR_CUDA;
   } else {
     PrefillEpiParams e = {};
@@ -1115,18 +1263,17 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     e.ldo = ldy;
     e.err = err;
     unsigned h_err = 0;
-    cudaError_t ce;
     const NarrowWorkspace ws = {partial, n_sm};
-    ce = narrow ? launch_prefill_narrow(PE_STORE, mb, mh, K, 2, ws, e, s)
-                : launch_prefill_gemm(PE_STORE, mh, ml, mb, K, ws, e, s);
-    if (ce != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess ||
-        cudaMemcpy(&h_err, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
+    const cudaError_t ce = narrow ? launch_prefill_narrow(PE_STORE, mb, w_rows, mh, K, 2, ws, e, s)
+                                  : launch_prefill_gemm(PE_STORE, mh, ml, mb, w_rows, K, ws, e, s);
+    if (ce != cudaSuccess || cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
       rc = KFL_ERR_CUDA;
     else if (h_err & ERR_TIMEOUT)
       rc = KFL_ERR_TIMEOUT;
   }
-  cudaStreamSynchronize(s);
-  cudaFree(mem);
+  cudaFreeAsync(mem, s);
+  if (rc != KFL_OK) cudaStreamSynchronize(s);
   cudaGetLastError();
   return rc;
 }

@@ -53,7 +53,7 @@ struct PrefillEpiParams {
   const int *positions;    // [T], -1 for a refused token (nothing of it is stored)
   int slot, hd, hkv, qdim, kvdim, max_ctx;
   const float *rope_cos, *rope_sin;  // [max_ctx][hd / 2]
-  // PE_ARGMAX: [T][n_tiles] partial maxima and their indices
+  // PE_ARGMAX: [T][n_tiles] partial maxima (of 256 columns, or of 32 rows in the few-token GEMM) and their indices
   float *amax;
   int *aidx;
   int n_tiles;
@@ -88,8 +88,9 @@ struct NarrowWorkspace {
 size_t narrow_ws_bytes(int n_sm, int T);  // for passes of up to T tokens
 int narrow_argmax_slots(int N);  // PE_ARGMAX: partial maxima per token (n_tiles of PrefillEpiParams)
 int narrow_tp(int T, int terms);  // tokens of a tile
-// w: encode_tiles_map with 2 row blocks per box; x: encode_terms_map with narrow_tp rows per box.
-cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensorMap &x, int K, int terms,
+// w: encode_tiles_map with 2 row blocks per box, or (w_rows) encode_rows_map with 128 rows; x:
+// encode_terms_map with narrow_tp rows per box.
+cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, const CUtensorMap &x, int K, int terms,
                                   const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s);
 // The same over int4 tiles [n_rb][n_kt][TILE4_BYTES], decoded in the kernel (fp16 terms).
 cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int n_kt, const CUtensorMap &x, int K,
@@ -102,12 +103,16 @@ int encode_act_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int 
 int encode_terms_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int ld, int terms, size_t term_stride,
                      int box_rows);
 int encode_tiles_map(CUtensorMap *map, const uint8_t *tiles, int n_kt, int n_rb, int box_rb);
+// A row-major bf16 matrix [N][K] (K a multiple of 8, 16-byte aligned): boxes of 64 columns x box_rows rows.
+int encode_rows_map(CUtensorMap *map, const uint16_t *w, int K, int N, int box_rows);
 // The launch attribute of a kernel that waits (griddepcontrol.wait) for the kernel before it.
 inline void pdl_attribute(cudaLaunchAttribute &a) {
   a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   a.val.programmaticStreamSerializationAllowed = 1;
 }
-cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a_hi, const CUtensorMap &a_lo, const CUtensorMap &b, int K,
+// b: encode_tiles_map with PG_N / RB row blocks per box, or (w_rows) encode_rows_map with PG_N rows.
+cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a_hi, const CUtensorMap &a_lo, const CUtensorMap &b,
+                                bool w_rows, int K,
                                 const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s);
 cudaError_t launch_prefill_attention(const PrefillAttnParams &p, int hd, int n_sm, cudaStream_t s);
 cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const int *positions_in, int T,
@@ -117,7 +122,8 @@ cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const 
                                    size_t term_stride, int terms, int ldx, int f16, unsigned *err, cudaStream_t s);
 // int4 group-64 tiles [n_rb][n_kt][TILE4_BYTES] -> fp16 tiles [n_rb][2 n_kt][RB][KT] of code x scale.
 cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, cudaStream_t s);
-cudaError_t launch_split_bf16(const float *x, int T, int K, int ldx, uint16_t *hi, uint16_t *lo, int ld,
+// fp32 rows [T][K] (stride ldx) as hi and lo bf16 terms (stride ld); *err = 0.
+cudaError_t launch_split_bf16(const float *x, int T, int K, int ldx, uint16_t *hi, uint16_t *lo, int ld, unsigned *err,
                               cudaStream_t s);
 cudaError_t launch_prefill_argmax(const float *amax, const int *aidx, int n_tiles, int T, int *next_ids,
                                   cudaStream_t s);

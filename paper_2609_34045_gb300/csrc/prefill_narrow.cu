@@ -36,6 +36,7 @@ constexpr int NW_RING = 226 * 1024;      // shared memory of the rings: a block'
 struct NarrowParams {
   TileShare share;  // of row tiles (of 128 mb rows) x token tiles, in K blocks of 64 (int4: units of 128)
   int t_tiles;
+  int w_rows;       // the weight map is over a row-major matrix (encode_rows_map), not over weight tiles
   int tp, terms;    // tokens of a tile (a multiple of 16), terms per token: tp * terms columns
   int stages, stage_bytes;
   int acc_cols;     // TMEM columns of one 128-row accumulator (tp * terms rounded up to 32)
@@ -50,16 +51,6 @@ struct NarrowParams {
 __device__ __forceinline__ size_t narrow_partial(int part, int m, int gr, int mb, int tp) {
   return ((size_t)part * mb * (tp / 16) + (size_t)m * (tp / 16) + gr) * (4 * 128);
 }
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // The epilogue of 16 tokens t0 .. t0 + 15 of output row n (this lane's; the warp's lanes hold 32
 // consecutive rows starting at a multiple of 32): load() fetches what it needs besides the sums, all
@@ -387,9 +378,13 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
       if (elect_one()) {
         mbar_arrive_expect_tx(full, bytes);
 #pragma unroll
-        for (int m = 0; m < MB; ++m)
-          tma_load_4d_hint(dst + m * NW_W_BYTES, &tm_w, (w.kb & 1) * 64, 0, w.kb >> 1,
-                           (w.r_tile * MB + m) * (128 / RB), full, pol);
+        for (int m = 0; m < MB; ++m) {
+          if (p.w_rows)
+            tma_load_2d_hint(dst + m * NW_W_BYTES, &tm_w, w.kb * 64, (w.r_tile * MB + m) * 128, full, pol);
+          else
+            tma_load_4d_hint(dst + m * NW_W_BYTES, &tm_w, (w.kb & 1) * 64, 0, w.kb >> 1,
+                             (w.r_tile * MB + m) * (128 / RB), full, pol);
+        }
       }
       __syncwarp();
       w.next(p);
@@ -815,10 +810,11 @@ int narrow_tp(int T, int terms) {
   return ((T + tiles - 1) / tiles + 15) / 16 * 16;
 }
 
-cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, const CUtensorMap &x, int K, int terms,
+cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, const CUtensorMap &x, int K, int terms,
                                   const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
   if (ep.T <= 0 || ep.N <= 0) return cudaSuccess;
   NarrowParams p = {};
+  p.w_rows = w_rows;
   p.terms = terms;
   p.tp = narrow_tp(ep.T, terms);
   p.t_tiles = (ep.T + p.tp - 1) / p.tp;

@@ -212,6 +212,21 @@ void make_plan(const kfl_model_cfg *c, int l0, int l1, int flags, int n_sm, Plan
 
 }  // namespace
 
+namespace kfl {
+bool release_matmul_pool();  // prefill.cu
+}
+
+namespace {
+// cudaMalloc, once more without what kfl_matmul_bf16w keeps if there is no memory.
+bool device_alloc(void **p, size_t bytes) {
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  if (release_matmul_pool() && cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
+}
+}  // namespace
+
 struct kfl_stage {
   kfl_model_cfg cfg;
   int l0 = 0, l1 = 0, flags = 0;
@@ -289,8 +304,7 @@ struct kfl_stage {
     ++alloc_count;
     if (fault_at > 0 && alloc_count == fault_at) return KFL_ERR_OOM;
     if (bytes == 0) bytes = 16;
-    if (cudaMalloc(p, bytes) != cudaSuccess) {
-      cudaGetLastError();
+    if (!device_alloc(p, bytes)) {
       *p = nullptr;
       return KFL_ERR_OOM;
     }
@@ -821,10 +835,7 @@ int ensure_prefill(kfl_stage *st, int tokens) {
     st->pf_allocs.clear();
     st->pf_cap = 0;
     auto get = [&](void **p, size_t bytes) {
-      if (cudaMalloc(p, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-      }
+      if (!device_alloc(p, bytes)) return false;
       st->pf_allocs.push_back(*p);
       return true;
     };
@@ -985,7 +996,7 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
   if (i4 && pf_narrow(st, x.n))
     return launch_prefill_narrow4(mode, m.tiles, m.n_rb, m.n_kt, x.all, m.K, x.terms, st->pf_nw, e, s);
   if (!i4 && pf_narrow(st, x.n, x.terms == 3))
-    return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], x.all, m.K, x.terms, st->pf_nw, e, s);
+    return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], false, x.all, m.K, x.terms, st->pf_nw, e, s);
   if (i4) {
     cudaError_t err = pf_dequant(st, g + 1);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, st->pf_deq[g % 2], 0);
@@ -994,7 +1005,7 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
   } else {
     b = &st->pf_maps[j == 4 ? 4 * st->P.nl : 4 * l + j];
   }
-  cudaError_t err = launch_prefill_gemm(mode, x.term[0], x.term[1], *b, m.K, st->pf_nw, e, s);
+  cudaError_t err = launch_prefill_gemm(mode, x.term[0], x.term[1], *b, false, m.K, st->pf_nw, e, s);
   if (err == cudaSuccess && i4) err = cudaEventRecord(st->pf_used[g % 2], s);
   return err;
 }

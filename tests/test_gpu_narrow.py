@@ -30,7 +30,9 @@ def _built():
 
 
 @pytest.mark.parametrize("T,Kd,N", [(1, 64, 1), (16, 72, 129), (17, 128, 300), (48, 1000, 40), (64, 3584, 640),
-                                    (65, 200, 29300), (127, 520, 384), (128, 136, 29185), (128, 2048, 1000)])
+                                    (65, 200, 29300), (127, 520, 384), (128, 136, 29185), (128, 2048, 1000),
+                                    # weight rows that TMA cannot address (K % 8 != 0) are copied to tiles first
+                                    (5, 67, 130), (129, 203, 513), (130, 200, 513)])
 def test_product_matches_fp64(T, Kd, N):
     rng = np.random.default_rng(T * 31 + Kd * 7 + N)
     x = rng.standard_normal((T, Kd)).astype(np.float32)
