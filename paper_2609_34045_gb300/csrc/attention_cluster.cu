@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(ATC_THREADS, 2) attn_cluster_kernel(const __gr
   const int C = p.cluster;
   const int pair = blockIdx.x / C, r = blockIdx.x % C;  // r: the CTA's rank in its cluster
   const int b = pair / p.n_kv_heads, kvh = pair % p.n_kv_heads;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int G = p.n_heads / p.n_kv_heads;
   const int gid = lane >> 2, tig = lane & 3;
   // trace slots of an attention CTA: go (start), enter (consumers past the wait on Q/K/V), x_go
@@ -189,13 +189,14 @@ __global__ void __launch_bounds__(ATC_THREADS, 2) attn_cluster_kernel(const __gr
     const int nsub_all = (P + ATT_SUB) / ATT_SUB;
     // rounded up: the larger shares go to the first CTAs, so that the last one, which holds the
     // rows this step writes and loads them only after the wait on Q/K/V, has the fewest
-    start = static_cast<int>(((long long)r * nsub_all + C - 1) / C) * ATT_SUB;
-    end = min(P + 1, static_cast<int>(((long long)(r + 1) * nsub_all + C - 1) / C) * ATT_SUB);
+    // (32-bit: at most 16 CTAs times 2^14 sub-tiles)
+    start = static_cast<int>((unsigned)(r * nsub_all + C - 1) / (unsigned)C) * ATT_SUB;
+    end = min(P + 1, static_cast<int>((unsigned)((r + 1) * nsub_all + C - 1) / (unsigned)C) * ATT_SUB);
   }
   const int nsub = end > start ? (end - start + ATT_SUB - 1) / ATT_SUB : 0;
   // output chunks of XCHUNK elements of the pair's G x HD: CTA r merges [c0, c1)
   const int nch = G * HD / XCHUNK;
-  const int c0 = static_cast<int>((long long)r * nch / C), c1 = static_cast<int>((long long)(r + 1) * nch / C);
+  const int c0 = static_cast<int>((unsigned)(r * nch) / (unsigned)C), c1 = static_cast<int>((unsigned)((r + 1) * nch) / (unsigned)C);
   const int own = (nch + C - 1) / C;  // rows of s_recv per source CTA
   const uint32_t rbar = smem_addr(&s_rbar);
   if (tid == 0) {
@@ -220,34 +221,42 @@ __global__ void __launch_bounds__(ATC_THREADS, 2) attn_cluster_kernel(const __gr
     // ------------------------------------------------------------------ producer
     // The cached rows [0, lo) were written by earlier steps: sub-tiles below lo go out while the
     // Q/K/V projection may still run, the rest after the wait on it.
-    if (lane == 0 && nsub > 0) {
+    // (the whole warp, one elected lane issuing)
+    if (nsub > 0) {
+      slot = __shfl_sync(0xffffffffu, slot, 0);
+      lo = __shfl_sync(0xffffffffu, lo, 0);
       const int row0 = (slot * p.n_kv_heads + kvh) * p.max_ctx;
       bool waited = false;
-      int issued = 0;
+      int issued = 0, s = 0;
+      uint32_t use = 0;
       for (int t = 0; t < nsub; ++t) {
-        const int s = t % S;
-        if (t >= S && !mbar_wait(smem_addr(&empty[s]), ((t / S) - 1) & 1)) {
+        const bool free_stage = __all_sync(0xffffffffu, use == 0 || mbar_wait(smem_addr(&empty[s]), (use - 1) & 1));
+        if (!free_stage) {
           s_abort = 1;
-          atomicOr(p.err, ERR_TIMEOUT);
+          if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
           break;
         }
-        if (s_abort) break;
+        if (__any_sync(0xffffffffu, s_abort != 0)) break;
         const int p0 = start + t * ATT_SUB;
         if (!waited && p0 + ATT_SUB > lo) {
           pdl_wait();
           waited = true;
-          stamp_by(true, TR_E_SUMMED);
+          stamp_by(lane == 0, TR_E_SUMMED);
         }
         const uint32_t fb = smem_addr(&full[s]);
-        mbar_arrive_expect_tx(fb, L::STAGE_BYTES);
         const uint32_t kd = sm0 + s * L::STAGE_BYTES, vd = kd + L::KV_BYTES;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(fb, L::STAGE_BYTES);
 #pragma unroll
-        for (int hb = 0; hb < L::BOXES; ++hb) {
-          atc_tma_load(kd + hb * L::BOX_BYTES, &kmap, 64 * hb, row0 + p0, fb);
-          atc_tma_load(vd + hb * L::BOX_BYTES, &vmap, 64 * hb, row0 + p0, fb);
+          for (int hb = 0; hb < L::BOXES; ++hb) {
+            atc_tma_load(kd + hb * L::BOX_BYTES, &kmap, 64 * hb, row0 + p0, fb);
+            atc_tma_load(vd + hb * L::BOX_BYTES, &vmap, 64 * hb, row0 + p0, fb);
+          }
         }
+        __syncwarp();
         ++issued;
-        if (t == 0) stamp_by(true, TR_W_LAST);
+        if (t == 0) stamp_by(lane == 0, TR_W_LAST);
+        if (++s == S) s = 0, ++use;
       }
       if (p.launch_at == 1) pdl_launch_dependents();
       // copies still in flight land before the shared memory is reused (bounded)
@@ -462,7 +471,7 @@ __global__ void __launch_bounds__(ATC_THREADS, 2) attn_cluster_kernel(const __gr
       }
       const int j = e / XCHUNK;
       const int o = ((j + 1) * C - 1) / nch;
-      const int jl = j - static_cast<int>((long long)o * nch / C);
+      const int jl = j - static_cast<int>((unsigned)(o * nch) / (unsigned)C);
       st_async_f4(map_to_rank(smem_addr(s_recv + ((size_t)r * own + jl) * XCHUNK + e % XCHUNK), o), v,
                   map_to_rank(rbar, o));
     }

@@ -453,6 +453,21 @@ __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// One lane of the (converged) warp.  MMAs, commits and bulk or tensor copies are issued under it by warps whose
+// control flow is uniform: under a plain lane == 0 test the compiler cannot tell that their
+// operands are uniform and moves them through a loop over the active lanes, which alone cost 148
+// to 245 cycles per tcgen05.mma in place of 70 to 112 (an N = 256 MMA executes in 128), and a producer
+// of 8 KiB bulk copies its bandwidth.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
+
 __device__ __forceinline__ void named_bar_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }

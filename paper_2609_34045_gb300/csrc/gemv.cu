@@ -48,11 +48,11 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2) gemv_kernel(const __grid_cons
 
   constexpr int KTILE = FMT == 0 ? KT : KT4;
   constexpr uint32_t WBYTES = FMT == 0 ? TILE_BYTES : TILE4_BYTES;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long T = (long long)p.n_rb * p.n_kt;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const unsigned T = (unsigned)p.n_rb * p.n_kt;
   const int G = gridDim.x, c = blockIdx.x;
-  const long long t0 = (long long)c * T / G, t1 = (long long)(c + 1) * T / G;
-  const int n = static_cast<int>(t1 - t0);
+  const unsigned t0 = tile_of_cta(c, T, G);
+  const int n = static_cast<int>(tile_of_cta(c + 1, T, G) - t0);
   const SegRing sr = {red, seg_full, seg_empty, seg_slots(FMT), seg_subs(FMT)};
 
   if (tid == 0) {
@@ -84,55 +84,59 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2) gemv_kernel(const __grid_cons
 
   if (warp == CONSUMER_WARPS) {
     // ------------------------------------------------------------------ producer
-    if (lane == 0) {
-      const uint64_t pol_w = policy_evict_first();
-      const uint64_t pol_x = policy_evict_last();
-      // int4: the K tile's block of the Act16 input, one contiguous copy
-      const uint32_t xbytes = FMT == 0 ? B * (KTILE * 4) : act16_copy_bytes(B, p.xsplit);
-      const int pre = n < S ? n : S;
-      stamp(TR_W_FIRST);
-      for (int i = 0; i < pre; ++i) {
-        const uint32_t fb = smem_addr(&full[i]);
-        mbar_arrive_expect_tx(fb, WBYTES + xbytes);
-        bulk_g2s(smem_addr(smem + (size_t)i * SB), p.w + (size_t)(t0 + i) * WBYTES, WBYTES, fb, pol_w);
-        s_issued = i + 1;
-      }
-      pdl_wait();
-      stamp(TR_X_GO);
-      auto issue_x = [&](int kt, int s) {
-        const uint32_t fb = smem_addr(&full[s]);
-        const uint32_t dst = smem_addr(smem + (size_t)s * SB + WBYTES);
-        if constexpr (FMT == 0) {
+    // (the whole warp, one elected lane issuing)
+    const uint64_t pol_w = policy_evict_first();
+    const uint64_t pol_x = policy_evict_last();
+    // int4: the K tile's block of the Act16 input, one contiguous copy
+    const uint32_t xbytes = FMT == 0 ? B * (KTILE * 4) : act16_copy_bytes(B, p.xsplit);
+    const int pre = n < S ? n : S;
+    if (lane == 0) stamp(TR_W_FIRST);
+    auto issue_w = [&](int i, int s) {
+      const uint32_t fb = smem_addr(&full[s]);
+      mbar_arrive_expect_tx(fb, WBYTES + xbytes);
+      bulk_g2s(smem_addr(smem + (size_t)s * SB), p.w + (size_t)(t0 + i) * WBYTES, WBYTES, fb, pol_w);
+      s_issued = i + 1;
+    };
+    auto issue_x = [&](int kt, int s) {
+      const uint32_t fb = smem_addr(&full[s]);
+      const uint32_t dst = smem_addr(smem + (size_t)s * SB + WBYTES);
+      if constexpr (FMT == 0) {
 #pragma unroll
-          for (int b = 0; b < B; ++b)
-            bulk_g2s(dst + b * (KTILE * 4), p.x + (size_t)b * p.ldx + (size_t)kt * KTILE, KTILE * 4, fb, pol_x);
-        } else {
-          bulk_g2s(dst, act16_tile(p.xin, kt), xbytes, fb, pol_x);
-        }
-      };
-      int kt_x = static_cast<int>(t0 % p.n_kt);
-      for (int i = 0; i < pre; ++i) {
-        issue_x(kt_x, i);
-        if (++kt_x == p.n_kt) kt_x = 0;
+        for (int b = 0; b < B; ++b)
+          bulk_g2s(dst + b * (KTILE * 4), p.x + (size_t)b * p.ldx + (size_t)kt * KTILE, KTILE * 4, fb, pol_x);
+      } else {
+        bulk_g2s(dst, act16_tile(p.xin, kt), xbytes, fb, pol_x);
       }
-      int s = 0;
-      uint32_t eph = 0;
-      for (int i = pre; i < n; ++i) {
-        if (!consumer_wait(smem_addr(&empty[s]), eph, &s_abort, p.err)) break;
-        const uint32_t fb = smem_addr(&full[s]);
-        mbar_arrive_expect_tx(fb, WBYTES + xbytes);
-        bulk_g2s(smem_addr(smem + (size_t)s * SB), p.w + (size_t)(t0 + i) * WBYTES, WBYTES, fb, pol_w);
-        issue_x(kt_x, s);
-        s_issued = i + 1;
-        if (++kt_x == p.n_kt) kt_x = 0;
-        if (++s == S) {
-          s = 0;
-          eph ^= 1u;
-        }
-      }
-      stamp(TR_W_LAST);
-      if constexpr (FMT == 1) pdl_launch_dependents();
+    };
+    for (int i = 0; i < pre; ++i) {
+      if (elect_one()) issue_w(i, i);
+      __syncwarp();
     }
+    pdl_wait();
+    if (lane == 0) stamp(TR_X_GO);
+    int kt_x = static_cast<int>(t0 % (unsigned)p.n_kt);
+    for (int i = 0; i < pre; ++i) {
+      if (elect_one()) issue_x(kt_x, i);
+      __syncwarp();
+      if (++kt_x == p.n_kt) kt_x = 0;
+    }
+    int s = 0;
+    uint32_t eph = 0;
+    for (int i = pre; i < n; ++i) {
+      if (!__all_sync(0xffffffffu, consumer_wait(smem_addr(&empty[s]), eph, &s_abort, p.err))) break;
+      if (elect_one()) {
+        issue_w(i, s);
+        issue_x(kt_x, s);
+      }
+      __syncwarp();
+      if (++kt_x == p.n_kt) kt_x = 0;
+      if (++s == S) {
+        s = 0;
+        eph ^= 1u;
+      }
+    }
+    if (lane == 0) stamp(TR_W_LAST);
+    if constexpr (FMT == 1) pdl_launch_dependents();
     return;
   }
   if (warp == CONSUMER_WARPS + 1) {

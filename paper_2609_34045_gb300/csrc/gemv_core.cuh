@@ -53,9 +53,16 @@ __device__ __forceinline__ float int4_code(uint32_t word, int j) {
   return __uint_as_float(((word >> (4 * j)) & 0xFu) ^ 0x4B000008u) - 8388616.0f;
 }
 
-__device__ __forceinline__ int cta_of_tile(long long t, long long T, int G) {
+// The stream-K split of T tiles over G CTAs (at most 512): CTA c takes [tile_of_cta(c), tile_of_cta(c +
+// 1)).  In 32 bits up to 2^23 tiles (128 GiB of bf16): a 64-bit division takes some 500 cycles, and these
+// stand before a GEMV's first copy and in the combine that its last CTA ends with.
+__device__ __forceinline__ unsigned tile_of_cta(unsigned c, unsigned T, unsigned G) {
+  return T < (1u << 23) ? c * T / G : static_cast<unsigned>((unsigned long long)c * T / G);
+}
+__device__ __forceinline__ int cta_of_tile(unsigned t, unsigned T, unsigned G) {
   // the largest c with floor(c*T/G) <= t
-  return static_cast<int>(((t + 1) * G - 1) / T);
+  return T < (1u << 23) ? static_cast<int>(((t + 1) * G - 1) / T)
+                        : static_cast<int>((((unsigned long long)t + 1) * G - 1) / T);
 }
 
 // Bounded wait on an mbarrier phase that also ends when the CTA aborts.
@@ -277,7 +284,7 @@ __host__ __device__ constexpr int ring_empty_count(int fmt) { return fmt == 0 ? 
 // GEMVs that share the ring.
 template <int B, bool XSPLIT>
 __device__ __forceinline__ void gemv_consume_int4(int n_kt, uint8_t *ring, uint64_t *full, uint64_t *empty, int S,
-                                                  int &s, uint32_t &phase, long long t0, int n, const SegRing &sr,
+                                                  int &s, uint32_t &phase, unsigned t0, int n, const SegRing &sr,
                                                   int &segc, volatile int *abort_flag, unsigned *err, int tid) {
   constexpr uint32_t SB = stage_bytes(B, 1);
   const int warp = tid >> 5, lane = tid & 31, team = warp >> 2;
@@ -291,7 +298,7 @@ __device__ __forceinline__ void gemv_consume_int4(int n_kt, uint8_t *ring, uint6
     ms -= S;
     mph ^= 1u;
   }
-  int kt = static_cast<int>(t0 % n_kt);
+  int kt = static_cast<int>(t0 % (unsigned)n_kt);
   int i = 0;
   while (i < n) {
     const int seg = min(n_kt - kt, n - i);
@@ -346,7 +353,7 @@ __device__ __forceinline__ void gemv_consume_int4(int n_kt, uint8_t *ring, uint6
 // across calls when consecutive GEMVs share the rings.
 template <int B, int FMT>
 __device__ __forceinline__ void gemv_consume(int n_kt, uint8_t *ring, uint64_t *full, uint64_t *empty, int S, int &s,
-                                             uint32_t &phase, long long t0, int n, const SegRing &sr, int &segc,
+                                             uint32_t &phase, unsigned t0, int n, const SegRing &sr, int &segc,
                                              volatile int *abort_flag, unsigned *err, int tid, bool xsplit) {
   if constexpr (FMT == 1) {
     if (xsplit)
@@ -356,7 +363,7 @@ __device__ __forceinline__ void gemv_consume(int n_kt, uint8_t *ring, uint64_t *
   } else {
     const int warp = tid >> 5, lane = tid & 31, kc = lane & 15, rsub = lane >> 4;
     float acc[B][4][2];  // rows warp*8 + rsub + 2j, this lane's K chunk
-    int kt = static_cast<int>(t0 % n_kt);
+    int kt = static_cast<int>(t0 % (unsigned)n_kt);
     for (int i = 0; i < n; ++i) {
       if (i == 0 || kt == 0) {
 #pragma unroll
@@ -619,19 +626,29 @@ __device__ __forceinline__ void epilogue_warp(const GemvParams &p, int rb, float
 // its epilogue and (persistent kernel) is published on the readiness counters.
 // inv / inv_ready: the RMSNorm scale of this GEMV, computed once, when first needed.
 template <int B, int EPI>
-__device__ __forceinline__ void gemv_epilogues(const GemvParams &p, long long t0, int n, long long T, int G, int c,
+__device__ __forceinline__ void gemv_epilogues(const GemvParams &p, unsigned t0, int n, unsigned T, int G, int c,
                                                const SegRing &sr, int &segc, float *inv, bool &inv_ready,
                                                volatile int *abort_flag, int lane, float *rx = nullptr,
                                                uint64_t *rx_bar = nullptr) {
-  int i = 0;
-  while (i < n) {
-    const long long t = t0 + i;
-    const int rb = static_cast<int>(t / p.n_kt);
-    const int kt0 = static_cast<int>(t - (long long)rb * p.n_kt);
-    const int len = min(p.n_kt - kt0, n - i);
+  int rb = static_cast<int>(t0 / (unsigned)p.n_kt) - 1, kt_next = static_cast<int>(t0 - (unsigned)(rb + 1) * p.n_kt);
+  for (int i = 0; i < n;) {
+    ++rb;
+    const int kt0 = kt_next, len = min(p.n_kt - kt0, n - i);
+    const bool first_seg = i == 0;
+    kt_next = 0;
     i += len;
     const int slot = segc % sr.nslot, use = segc / sr.nslot;
     ++segc;
+    // a shared row block's CTAs c_lo .. c_hi; all but c_lo start inside it (partial slot 0), as c_lo does
+    // only at its very start.  Worked out while the consumers are still at the segment
+    const bool shared = !(kt0 == 0 && len == p.n_kt) && !rx;
+    int c_lo = 0, c_hi = 0, slot_lo = 0;
+    if (shared) {
+      const unsigned lo = (unsigned)rb * p.n_kt;
+      c_lo = cta_of_tile(lo, T, G);
+      c_hi = cta_of_tile(lo + p.n_kt - 1, T, G);
+      slot_lo = tile_of_cta(c_lo, T, G) == lo ? 0 : 1;
+    }
     consumer_wait(smem_addr(&sr.full[slot]), use & 1, abort_flag, p.err);
     unsigned long long *tr = p.trace && lane == 0 ? p.trace + (size_t)c * TRACE_SLOTS : nullptr;
     if (tr) {
@@ -695,11 +712,9 @@ __device__ __forceinline__ void gemv_epilogues(const GemvParams &p, long long t0
         do_epi = ok != 0;
       }
       if (tr) tr[TR_E_KIND] = do_epi ? 2 : 1;
-    } else if (!(kt0 == 0 && len == p.n_kt)) {
+    } else if (shared) {
       // this row block is shared with neighbouring CTAs: the ticket counts the CTAs that have
       // published their partial; the one that finds all the others there sums every partial
-      const int c_lo = cta_of_tile((long long)rb * p.n_kt, T, G);
-      const int c_hi = cta_of_tile((long long)(rb + 1) * p.n_kt - 1, T, G);
       const unsigned others = static_cast<unsigned>(c_hi - c_lo);
       unsigned *ticket = reinterpret_cast<unsigned *>(p.tickets + rb);
       unsigned seen = 0;
@@ -708,8 +723,7 @@ __device__ __forceinline__ void gemv_epilogues(const GemvParams &p, long long t0
       __syncwarp();
       do_epi = seen == others;
       if (!do_epi) {
-        const int first_rb = static_cast<int>(t0 / p.n_kt);
-        const int myslot = (rb == first_rb) ? 0 : 1;
+        const int myslot = first_seg ? 0 : 1;
         float4 *mine = reinterpret_cast<float4 *>(p.partial + (size_t)(c * 2 + myslot) * (RB * MAXB));
         const float4 *r4 = reinterpret_cast<const float4 *>(red);
         for (int e = lane; e < RB * MAXB / 4; e += 32) mine[e] = r4[e];
@@ -736,8 +750,8 @@ __device__ __forceinline__ void gemv_epilogues(const GemvParams &p, long long t0
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const int cc = c0 + j;
-            const int frb = static_cast<int>(((long long)cc * T / G) / p.n_kt);
-            const float4 *src = reinterpret_cast<const float4 *>(p.partial + (size_t)(cc * 2 + (rb == frb ? 0 : 1)) * (RB * MAXB));
+            const float4 *src =
+                reinterpret_cast<const float4 *>(p.partial + (size_t)(cc * 2 + (cc == c_lo ? slot_lo : 0)) * (RB * MAXB));
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
               const int e = lane + 32 * k;
@@ -805,7 +819,7 @@ __device__ __forceinline__ void gemv_epilogues(const GemvParams &p, long long t0
 }
 
 template <int B>
-__device__ __forceinline__ void gemv_epilogues_any(int epi, const GemvParams &p, long long t0, int n, long long T,
+__device__ __forceinline__ void gemv_epilogues_any(int epi, const GemvParams &p, unsigned t0, int n, unsigned T,
                                                    int G, int c, const SegRing &sr, int &segc, float *inv,
                                                    bool &inv_ready, volatile int *abort_flag, int lane) {
   switch (epi) {

@@ -53,20 +53,6 @@ __device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t da, uint64
       : "memory");
 }
 
-// One lane of the (converged) warp.  MMAs, commits and tensor copies are issued under it by warps whose
-// control flow is uniform: under a plain lane == 0 test the compiler cannot tell that their
-// operands are uniform and moves them through a loop over the active lanes, which alone cost 148
-// to 245 cycles per MMA in place of 70 to 112 (an N = 256 MMA executes in 128).
-__device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "elect.sync _|p, 0xffffffff;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r));
-  return r != 0;
-}
-
 // Arrive on an mbarrier of this CTA once every MMA this thread issued before has completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)

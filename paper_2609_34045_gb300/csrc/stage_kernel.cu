@@ -29,17 +29,17 @@ constexpr int MK_WARPS = CONSUMER_WARPS + 3;  // consumers, weight producer, act
 constexpr int MK_THREADS = MK_WARPS * 32;
 
 // Tile range of CTA c in a GEMV phase: stream-K over min(T, grid) CTAs; the rest get none.
-__device__ __forceinline__ void phase_range(const GemvParams &g, int c, int grid, long long &T, int &G,
-                                            long long &t0, int &n) {
-  T = (long long)g.n_rb * g.n_kt;
-  G = T < grid ? static_cast<int>(T) : grid;
+__device__ __forceinline__ void phase_range(const GemvParams &g, int c, int grid, unsigned &T, int &G,
+                                            unsigned &t0, int &n) {
+  T = (unsigned)g.n_rb * g.n_kt;
+  G = T < (unsigned)grid ? static_cast<int>(T) : grid;
   if (c >= G) {
     t0 = 0;
     n = 0;
     return;
   }
-  t0 = (long long)c * T / G;
-  n = static_cast<int>((long long)(c + 1) * T / G - t0);
+  t0 = tile_of_cta(c, T, G);
+  n = static_cast<int>(tile_of_cta(c + 1, T, G) - t0);
 }
 
 // Is activation chunk kt of a GEMV phase written?  (acquire loads of the producers' counters)
@@ -65,14 +65,14 @@ __device__ __forceinline__ bool chunk_ready(const GemvParams &g, int kt) {
 // widest one does not raise the pressure of the rest of the kernel.
 template <int B, int FMT>
 __device__ __noinline__ void gemv_consume_call(int n_kt, uint8_t *ring, uint64_t *full, uint64_t *empty, int S,
-                                               int &s, uint32_t &phase, long long t0, int n, const SegRing &sr,
+                                               int &s, uint32_t &phase, unsigned t0, int n, const SegRing &sr,
                                                int &segc, volatile int *abort_flag, unsigned *err, int tid,
                                                bool xsplit) {
   gemv_consume<B, FMT>(n_kt, ring, full, empty, S, s, phase, t0, n, sr, segc, abort_flag, err, tid, xsplit);
 }
 
 template <int B>
-__device__ __noinline__ void gemv_epilogues_call(int epi, const GemvParams &p, long long t0, int n, long long T, int G,
+__device__ __noinline__ void gemv_epilogues_call(int epi, const GemvParams &p, unsigned t0, int n, unsigned T, int G,
                                                  int c, const SegRing &sr, int &segc, float *inv, bool &inv_ready,
                                                  volatile int *abort_flag, int lane) {
   gemv_epilogues_any<B>(epi, p, t0, n, T, G, c, sr, segc, inv, inv_ready, abort_flag, lane);
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) stage_kernel(const __grid_const
     for (int k = 0; k < kp.n_phases && !s_abort; ++k) {
       const Phase *ph = kp.phases + k;
       if (ph->kind != PH_GEMV) continue;
-      long long T, t0;
+      unsigned T, t0;
       int G, n;
       phase_range(ph->g, c, grid, T, G, t0, n);
       if (n == 0) continue;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) stage_kernel(const __grid_const
       const uint64_t pol_l2 = policy_evict_normal();
       struct Cursor {
         int k, i, n;
-        long long t0;
+        unsigned t0;
         const uint8_t *w;
         uint32_t bytes;  // a stage's copies: the tile and its activations
       };
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) stage_kernel(const __grid_const
         for (int k = from; k < kp.n_phases; ++k) {
           const Phase *ph = kp.phases + k;
           if (ph->kind != PH_GEMV) continue;
-          long long T, t0;
+          unsigned T, t0;
           int G, n;
           phase_range(ph->g, c, grid, T, G, t0, n);
           if (n == 0) continue;
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) stage_kernel(const __grid_const
       const Phase *ph = kp.phases + k;
       if (ph->kind != PH_GEMV) continue;
       const GemvParams &g = ph->g;
-      long long T, t0;
+      unsigned T, t0;
       int G, n;
       phase_range(g, c, grid, T, G, t0, n);
       if (n == 0) continue;
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) stage_kernel(const __grid_const
     const Phase *ph = kp.phases + k;
     const int kind = ph->kind;
     if (kind == PH_GEMV) {
-      long long T, t0;
+      unsigned T, t0;
       int G, n;
       phase_range(ph->g, c, grid, T, G, t0, n);
       if (tid == 0) stamp(k, TR_CONS_GO);
