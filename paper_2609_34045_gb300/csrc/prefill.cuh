@@ -81,6 +81,19 @@ constexpr int NW_MAX_TP = 128;            // tokens of a tile (two terms: 256 MM
 constexpr int NW_PARTS = 3;               // partial sums per CTA in a GEMM's workspace
 constexpr int N4_MAX_TOKENS = 512;       // int4 stages: passes of up to this many tokens decode in the GEMM
 constexpr int NW_W_BYTES = 128 * 64 * 2;  // a 128-row weight slice of 64 K
+// How a GEMM's output tiles are shared out (share_tiles, TileWalk in prefill_tc.cuh).
+struct TileShare {
+  int n_kb, waves, tail, splits;
+  bool cut() const { return tail > 0 && splits != 1; }
+};
+// Partial sums of a residual GEMM's cut tiles that nothing has added to h yet: the RMSNorm behind it does
+// (launch_narrow_norm).
+struct NarrowPending {
+  bool any = false;
+  TileShare share = {};
+  int grid = 0, mb = 0, tp = 0, t_tiles = 0;
+  const float *ws = nullptr;
+};
 struct NarrowWorkspace {
   float *partial;  // narrow_ws_bytes
   int n_sm;
@@ -91,10 +104,17 @@ int narrow_tp(int T, int terms);  // tokens of a tile
 // w: encode_tiles_map with 2 row blocks per box, or (w_rows) encode_rows_map with 128 rows; x:
 // encode_terms_map with narrow_tp rows per box.
 cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, const CUtensorMap &x, int K, int terms,
-                                  const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s);
+                                  const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s,
+                                  NarrowPending *pending = nullptr);
 // The same over int4 tiles [n_rb][n_kt][TILE4_BYTES], decoded in the kernel (fp16 terms).
 cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int n_kt, const CUtensorMap &x, int K,
-                                   int terms, const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s);
+                                   int terms, const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s,
+                                   NarrowPending *pending = nullptr);
+// RMSNorm (as launch_prefill_rmsnorm) of h after adding the pending sums to it.  d up to NW_NORM_MAX_D.
+constexpr int NW_NORM_MAX_D = 32768;
+cudaError_t launch_narrow_norm(const NarrowPending &pend, float *h, int ldh, int T, int d, const float *g, float eps,
+                               uint16_t *x, size_t term_stride, int terms, int ldx, int f16, unsigned *err,
+                               cudaStream_t s);
 
 // Host side (prefill.cu).
 int encode_act_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int ld);

@@ -46,10 +46,10 @@ struct NarrowParams {
   float *ws;        // partial sums (narrow_partial)
 };
 
-// Where (in float4, plus the row) a partial holds the sums of 128-row block m and token group gr:
-// [part][m][gr][4 x 4 tokens][128 rows].
+// Where (in floats) a partial holds the sums of 128-row block m and token group gr: [part][m][gr][16
+// tokens][128 rows].
 __device__ __forceinline__ size_t narrow_partial(int part, int m, int gr, int mb, int tp) {
-  return ((size_t)part * mb * (tp / 16) + (size_t)m * (tp / 16) + gr) * (4 * 128);
+  return ((size_t)part * mb * (tp / 16) + (size_t)m * (tp / 16) + gr) * (16 * 128);
 }
 
 // The epilogue of 16 tokens t0 .. t0 + 15 of output row n (this lane's; the warp's lanes hold 32
@@ -215,9 +215,9 @@ __device__ __forceinline__ void narrow_epilogue_warps(const NarrowParams &p, con
       if (whole) {
         e.store(ep, n, tt0 + gr * 16, v, lane, (r_tile * MB + m) * 4 + q);
       } else {
-        float4 *at = reinterpret_cast<float4 *>(p.ws) + narrow_partial(w.part, m, gr, MB, p.tp) + row;
+        float *at = p.ws + narrow_partial(w.part, m, gr, MB, p.tp) + row;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) at[j * 128] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        for (int j = 0; j < 16; ++j) at[j * 128] = v[j];
       }
     };
     if constexpr (DRAIN) {
@@ -278,29 +278,93 @@ __global__ void __launch_bounds__(128) narrow_reduce_kernel(NarrowParams p, int 
   pdl_wait();
   if (parts.n == 1 || t0 >= ep.T) return;
   const int n = (r_tile * mb + m) * 128 + row;
-  const float4 *ws = reinterpret_cast<const float4 *>(p.ws) + row;
+  const float *ws = p.ws + row;
   NarrowEpilogue<MODE> e;
   e.load(ep, n, t0, lane);
   float v[16] = {};
   for (int k = 0; k < parts.n; k += 4) {
-    float4 x[4][4];
+    float x[4][16];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const float4 *w = ws + narrow_partial(parts.part(k + i), m, gr, mb, p.tp);
+      const float *w = ws + narrow_partial(parts.part(k + i), m, gr, mb, p.tp);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[i][j] = k + i < parts.n ? __ldcg(w + j * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int j = 0; j < 16; ++j) x[i][j] = k + i < parts.n ? __ldcg(w + j * 128) : 0.f;
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        v[4 * j] += x[i][j].x;
-        v[4 * j + 1] += x[i][j].y;
-        v[4 * j + 2] += x[i][j].z;
-        v[4 * j + 3] += x[i][j].w;
-      }
+      for (int j = 0; j < 16; ++j) v[j] += x[i][j];
   }
   e.store(ep, n, t0, v, lane, (r_tile * mb + m) * 4 + q);
+}
+
+// One token's residual stream after a residual GEMM: the partial sums of the cut tiles added to h (in K
+// order, then h: as narrow_reduce_kernel), and its RMSNorm, in place of two kernels of which
+// each was latency.  A thread has NW_NORM_V groups of four elements in flight (43 tokens x 3584: 7.0 us for
+// 8.6 + 6.3, cold; 100 x 8192: 10.2 for 8.5 + 9.0).
+constexpr int NW_NORM_THREADS = 1024, NW_NORM_V = 2;
+__global__ void __launch_bounds__(NW_NORM_THREADS) narrow_norm_kernel(NarrowPending p, float *h, int ldh, int d,
+                                                                       const float *g, float eps, uint16_t *x,
+                                                                       size_t term_stride, int terms, int ldx, int f16,
+                                                                       unsigned *err) {
+  __shared__ TileParts s_parts[NW_NORM_MAX_D / 128];
+  __shared__ float red[NW_NORM_THREADS / 32];
+  pdl_launch_dependents();
+  const int t = blockIdx.x, rows = 128 * p.mb, tt = t / p.tp, tl = t - tt * p.tp;
+  const int dp = p.share.waves * p.grid;  // tiles below it are whole, and in h already
+  for (int r = threadIdx.x; r * rows < d; r += blockDim.x) {
+    const int tile = r * p.t_tiles + tt;
+    s_parts[r] = TileParts(p.share, max(tile - dp, 0), p.grid);
+    if (tile < dp) s_parts[r].n = 1;
+  }
+  __syncthreads();
+  pdl_wait();
+  float *row = h + (size_t)t * ldh;
+  const float *ws = p.ws + (size_t)(tl & 15) * 128;
+  auto residual = [&](int n0) {
+    const TileParts parts = s_parts[n0 / rows];
+    float4 v = *reinterpret_cast<const float4 *>(row + n0), y = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (parts.n > 1) {
+      const float *at = ws + n0 % 128;
+      for (int k = 0; k < parts.n; k += 4) {
+        float4 a[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          a[i] = k + i < parts.n ? __ldcg(reinterpret_cast<const float4 *>(
+                                       at + narrow_partial(parts.part(k + i), n0 / 128 % p.mb, tl / 16, p.mb, p.tp)))
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y.x += a[i].x, y.y += a[i].y, y.z += a[i].z, y.w += a[i].w;
+      }
+      v = make_float4(v.x + y.x, v.y + y.y, v.z + y.z, v.w + y.w);
+      *reinterpret_cast<float4 *>(row + n0) = v;
+    }
+    return v;
+  };
+  float ss = 0.f;
+  float4 v[NW_NORM_V];
+#pragma unroll
+  for (int i = 0; i < NW_NORM_V; ++i) {  // d is a multiple of 8
+    const int n0 = 4 * (threadIdx.x + i * blockDim.x);
+    v[i] = n0 < d ? residual(n0) : make_float4(0.f, 0.f, 0.f, 0.f);
+    ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+  }
+  for (int n0 = 4 * (threadIdx.x + NW_NORM_V * blockDim.x); n0 < d; n0 += 4 * blockDim.x) {
+    const float4 a = residual(n0);
+    ss += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
+  }
+  const float inv = 1.0f / sqrtf(block_sum(ss, red) / d + eps);
+  auto put = [&](int n0, float4 a) {
+    store_normed(a, inv, *reinterpret_cast<const float4 *>(g + n0), x + (size_t)t * ldx + n0, term_stride, terms, f16,
+                 err);
+  };
+#pragma unroll
+  for (int i = 0; i < NW_NORM_V; ++i) {
+    const int n0 = 4 * (threadIdx.x + i * blockDim.x);
+    if (n0 < d) put(n0, v[i]);
+  }
+  for (int n0 = 4 * (threadIdx.x + NW_NORM_V * blockDim.x); n0 < d; n0 += 4 * blockDim.x)
+    put(n0, *reinterpret_cast<const float4 *>(row + n0));  // this thread's own h
 }
 
 // A producer's place in its CTA's segments: the K block it loads next, of row tile r_tile and the tokens
@@ -773,8 +837,13 @@ static int ring_smem(const void *kernel) {
 
 template <int MODE>
 static cudaError_t launch_narrow_reduce(const NarrowParams &p, int mb, int grid, const PrefillEpiParams &ep,
-                                        cudaStream_t s) {
+                                        cudaStream_t s, NarrowPending *pending) {
+  if (pending) pending->any = false;
   if (!p.share.cut()) return cudaSuccess;
+  if (pending && MODE == PE_RESID && ep.N <= NW_NORM_MAX_D) {
+    *pending = NarrowPending{true, p.share, grid, mb, p.tp, p.t_tiles, p.ws};
+    return cudaSuccess;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(p.share.tail * mb * (p.tp / 16)));
   cfg.blockDim = dim3(128);
@@ -788,7 +857,7 @@ static cudaError_t launch_narrow_reduce(const NarrowParams &p, int mb, int grid,
 
 template <int MODE, int MB, bool DRAIN>
 static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x, const NarrowParams &p, int grid,
-                                      const PrefillEpiParams &ep, cudaStream_t s) {
+                                      const PrefillEpiParams &ep, cudaStream_t s, NarrowPending *pending) {
   static const int smem = ring_smem(reinterpret_cast<const void *>(prefill_narrow_kernel<MODE, MB, DRAIN>));
   if (smem < 0) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
@@ -801,7 +870,7 @@ static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_narrow_kernel<MODE, MB, DRAIN>, w, x, p, ep);
-  return e == cudaSuccess ? launch_narrow_reduce<MODE>(p, MB, grid, ep, s) : e;
+  return e == cudaSuccess ? launch_narrow_reduce<MODE>(p, MB, grid, ep, s, pending) : e;
 }
 
 int narrow_tp(int T, int terms) {
@@ -811,7 +880,8 @@ int narrow_tp(int T, int terms) {
 }
 
 cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, const CUtensorMap &x, int K, int terms,
-                                  const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
+                                  const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s,
+                                  NarrowPending *pending) {
   if (ep.T <= 0 || ep.N <= 0) return cudaSuccess;
   NarrowParams p = {};
   p.w_rows = w_rows;
@@ -838,9 +908,9 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, c
   p.share = share_tiles(n_tiles, n_kb, grid, p.t_tiles == 1, NW_PARTS);
   auto go = [&](auto m) {
     constexpr int MODE = decltype(m)::value;
-    if (terms == 3) return launch_narrow_mode<MODE, 1, true>(w, x, p, grid, ep, s);
-    return mb == 2 ? launch_narrow_mode<MODE, 2, false>(w, x, p, grid, ep, s)
-                   : launch_narrow_mode<MODE, 1, false>(w, x, p, grid, ep, s);
+    if (terms == 3) return launch_narrow_mode<MODE, 1, true>(w, x, p, grid, ep, s, pending);
+    return mb == 2 ? launch_narrow_mode<MODE, 2, false>(w, x, p, grid, ep, s, pending)
+                   : launch_narrow_mode<MODE, 1, false>(w, x, p, grid, ep, s, pending);
   };
   switch (mode) {
     case PE_STORE: return go(std::integral_constant<int, PE_STORE>());
@@ -854,7 +924,7 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, c
 
 template <int MODE>
 static cudaError_t launch_narrow4_mode(const Narrow4Params &r, const CUtensorMap &x, const NarrowParams &p, int grid,
-                                       const PrefillEpiParams &ep, cudaStream_t s) {
+                                       const PrefillEpiParams &ep, cudaStream_t s, NarrowPending *pending) {
   static const int smem = ring_smem(reinterpret_cast<const void *>(prefill_narrow4_kernel<MODE>));
   if (smem < 0) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
@@ -867,11 +937,12 @@ static cudaError_t launch_narrow4_mode(const Narrow4Params &r, const CUtensorMap
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_narrow4_kernel<MODE>, r, x, p, ep);
-  return e == cudaSuccess ? launch_narrow_reduce<MODE>(p, 2, grid, ep, s) : e;
+  return e == cudaSuccess ? launch_narrow_reduce<MODE>(p, 2, grid, ep, s, pending) : e;
 }
 
 cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int n_kt, const CUtensorMap &x, int K,
-                                   int terms, const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
+                                   int terms, const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s,
+                                  NarrowPending *pending) {
   if (ep.T <= 0 || ep.N <= 0) return cudaSuccess;
   NarrowParams p = {};
   p.terms = terms;
@@ -895,7 +966,7 @@ cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int
   const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min<long long>(n_tiles, ws.n_sm), U / 2));
   p.share = share_tiles(n_tiles, n_kb, grid, p.t_tiles == 1, NW_PARTS);
   auto go = [&](auto m) {
-    return launch_narrow4_mode<decltype(m)::value>(r, x, p, grid, ep, s);
+    return launch_narrow4_mode<decltype(m)::value>(r, x, p, grid, ep, s, pending);
   };
   switch (mode) {
     case PE_RESID: return go(std::integral_constant<int, PE_RESID>());
@@ -904,6 +975,20 @@ cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int
     case PE_ARGMAX: return go(std::integral_constant<int, PE_ARGMAX>());
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_narrow_norm(const NarrowPending &pend, float *h, int ldh, int T, int d, const float *g, float eps,
+                               uint16_t *x, size_t term_stride, int terms, int ldx, int f16, unsigned *err,
+                               cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(T);
+  cfg.blockDim = dim3(std::min(NW_NORM_THREADS, (d / 4 + 31) / 32 * 32));
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  pdl_attribute(attr[0]);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, narrow_norm_kernel, pend, h, ldh, d, g, eps, x, term_stride, terms, ldx, f16, err);
 }
 
 }  // namespace kfl

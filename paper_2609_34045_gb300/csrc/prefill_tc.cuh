@@ -227,10 +227,6 @@ struct ScalePair {
 //    CTAs at work together still read the same K (the sequence had each at a K of its own: 2048
 //    tokens' down projection, 290 MB of weights and tokens, went from 201 to 281 us).
 // A cut tile is summed from its partial sums, in K order, by a kernel behind the GEMM.
-struct TileShare {
-  int n_kb, waves, tail, splits;
-  bool cut() const { return tail > 0 && splits != 1; }
-};
 // parts_per_cta: how many partial sums per CTA the workspace holds (2 for the sequence).
 inline TileShare share_tiles(int tiles, int n_kb, int grid, bool sequence, int parts_per_cta) {
   TileShare s = {n_kb, tiles / grid, tiles % grid, 1};
@@ -290,6 +286,7 @@ struct TileWalk {
 // The partial sums of tail tile k, in K order.
 struct TileParts {
   int n, at, step, rest;  // part i: i == 0 ? at : rest + i * step
+  TileParts() = default;
   __device__ __forceinline__ TileParts(const TileShare &s, int k, int grid) {
     if (s.splits > 0) {
       n = s.splits;
@@ -318,6 +315,40 @@ __device__ __forceinline__ void split_pack(float x0, float x1, uint32_t &hi, uin
   split_term(x1, h1, l1, f16);
   hi = (uint32_t)h0 | ((uint32_t)h1 << 16);
   lo = (uint32_t)l0 | ((uint32_t)l1 << 16);
+}
+
+// What rounding leaves out of the fp32 product a * b * c (to first order).
+__device__ __forceinline__ float product3_rest(float a, float b, float c) {
+  const float p = a * b;
+  return fmaf(fmaf(a, b, -p), c, fmaf(p, c, -(p * c)));
+}
+
+// The block's sum of v (whole warps; red: a float per warp).
+__device__ __forceinline__ float block_sum(float v, float *red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
+  __syncthreads();
+  v = threadIdx.x % 32 < blockDim.x / 32 ? red[threadIdx.x % 32] : 0.f;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Four consecutive normalised values v * inv * g as 16-bit terms, term_stride elements apart (x 8-byte
+// aligned).
+__device__ __forceinline__ void store_normed(float4 v, float inv, float4 g, uint16_t *x, size_t term_stride, int terms,
+                                             int f16, unsigned *err) {
+  uint2 hi, lo;
+  const float y0 = v.x * inv * g.x, y1 = v.y * inv * g.y, y2 = v.z * inv * g.z, y3 = v.w * inv * g.w;
+  split_pack(y0, y1, hi.x, lo.x, f16, err);
+  split_pack(y2, y3, hi.y, lo.y, f16, err);
+  *reinterpret_cast<uint2 *>(x) = hi;
+  *reinterpret_cast<uint2 *>(x + term_stride) = lo;
+  if (terms == 3)  // bf16 terms: what the first two, and the products' roundings, leave
+    *reinterpret_cast<uint2 *>(x + 2 * term_stride) =
+        make_uint2(pack_bf16(y0 - bf16_lo(hi.x) - bf16_lo(lo.x) + product3_rest(v.x, inv, g.x),
+                             y1 - bf16_hi(hi.x) - bf16_hi(lo.x) + product3_rest(v.y, inv, g.y)),
+                   pack_bf16(y2 - bf16_lo(hi.y) - bf16_lo(lo.y) + product3_rest(v.z, inv, g.z),
+                             y3 - bf16_hi(hi.y) - bf16_hi(lo.y) + product3_rest(v.w, inv, g.w)));
 }
 
 }  // namespace kfl

@@ -980,7 +980,9 @@ struct PfInput {
 // One prefill GEMM with matrix j of block l (j = 4: lm_head): on the few-token kernel (pf_narrow) or on
 // 128-token tiles.  int4 stages then read the matrix's fp16 copy, dequantized ahead on
 // the side stream (the next one is started before this GEMM, so dequantization overlaps the products).
-cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, PrefillEpiParams e, cudaStream_t s) {
+// pending: a residual GEMM may leave the sums of its cut tiles to the norm behind it.
+cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, PrefillEpiParams e, cudaStream_t s,
+                    NarrowPending *pending = nullptr) {
   const Mat &m = pf_mat(st, l, j);
   const bool i4 = st->cfg.weight_fmt == KFL_INT4_G64;
   const CUtensorMap *b;
@@ -994,9 +996,9 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
     e.n_tiles = st->pf_amax_cols;
   }
   if (i4 && pf_narrow(st, x.n))
-    return launch_prefill_narrow4(mode, m.tiles, m.n_rb, m.n_kt, x.all, m.K, x.terms, st->pf_nw, e, s);
+    return launch_prefill_narrow4(mode, m.tiles, m.n_rb, m.n_kt, x.all, m.K, x.terms, st->pf_nw, e, s, pending);
   if (!i4 && pf_narrow(st, x.n, x.terms == 3))
-    return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], false, x.all, m.K, x.terms, st->pf_nw, e, s);
+    return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], false, x.all, m.K, x.terms, st->pf_nw, e, s, pending);
   if (i4) {
     cudaError_t err = pf_dequant(st, g + 1);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, st->pf_deq[g % 2], 0);
@@ -1039,7 +1041,12 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
         a.encode(st->pf_a, P.F, n, terms, narrow))
       return KFL_ERR_CUDA;
     st->pf_amax_cols = narrow ? narrow_argmax_slots(P.V) : (P.V + PG_N - 1) / PG_N;
+    NarrowPending pend;
     auto norm = [&](const float *g) {
+      if (pend.any) {
+        pend.any = false;
+        return launch_narrow_norm(pend, st->pf_h, P.ldh, n, P.d, g, eps, x.base, x.stride, terms, x.ld, i4, st->err, s);
+      }
       return launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, g, eps, x.base, x.stride, terms, x.ld, i4, st->err, s);
     };
     PrefillEpiParams r = {};  // O and down: into the residual stream
@@ -1122,7 +1129,7 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       t.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)P.hd));
       t.err = st->err;
       CK(launch_prefill_attention(t, P.hd, P.n_sm, s));
-      CK(pf_gemm(st, PE_RESID, o, l, 1, r, s));
+      CK(pf_gemm(st, PE_RESID, o, l, 1, r, s, &pend));
       CK(norm(L.g_ffn));
       PrefillEpiParams g = {};
       g.err = st->err;
@@ -1132,7 +1139,8 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       g.term_stride = a.stride;
       g.ldo16 = lda;
       CK(pf_gemm(st, PE_SWIGLU, x, l, 2, g, s));
-      CK(pf_gemm(st, PE_RESID, a, l, 3, r, s));
+      // (the last block of a body stage has no norm behind it)
+      CK(pf_gemm(st, PE_RESID, a, l, 3, r, s, l + 1 < P.nl || (st->flags & KFL_LOGITS_OUT) ? &pend : nullptr));
     }
     if (st->flags & KFL_LOGITS_OUT) {
       CK(norm(st->g_final));

@@ -64,6 +64,32 @@ def test_prefill_matches_the_oracle(model, n, monkeypatch):
     p.close()
 
 
+@pytest.mark.parametrize("model,d,n", [(RAGGED, 8320, 18),  # past what the norm's threads hold in registers
+                                       (RAGGED128, 8320, 130), (dataclasses.replace(RAGGED, qk_norm=True), 8264, 100),
+                                       (RAGGED_INT4, 16640, 33),
+                                       (RAGGED, 16648, 200),  # the same of the norm behind the 128-token tiles
+                                       (RAGGED, 32776, 17)])  # too many row tiles for the residual sums' norm
+def test_long_rows_match_the_oracle(model, d, n, monkeypatch):
+    """Residual sums and RMSNorm of rows at the edges of their kernels' ranges.  The attention norm's gain is
+    scaled by about (320 / d)^(1/2), so q and k keep the size they have at d_model 320, where the bar
+    comes from.  Unscaled (weights of 0.02), scores at d_model 16648 spread by (0.02^2 d) sqrt(64) / 8 =
+    6.7 and a softmax picks single keys: a K element a bf16 step (2^-8 of 2.6) over then moves a
+    score by 2.6 * 2^-8 * 2.6 / 8, a weight by 0.3 % of itself, and several of them a row by 1e-2."""
+    monkeypatch.setenv("KFL_PREFILL_DENSE_MIN", "1")
+    plain, scale = wl.layer_weights, np.float32(2.0 ** -round(np.log2(d / 320) / 2))
+
+    def layer_weights(*a):
+        w = plain(*a)
+        w["attn_norm"] = wl.f32_to_bf16_bits(wl.bf16_bits_to_f32(w["attn_norm"]) * scale)
+        return w
+
+    monkeypatch.setattr(wl, "layer_weights", layer_weights)
+    p = Pair(dataclasses.replace(model, d_model=d, vocab=300), 0, 2, K.KFL_IS_HEAD, 2, (5, 30), 256, seed=59, max_batch=2)
+    _prefill(p, 1, 30, n, 59, True)
+    p.compare_kv()
+    p.close()
+
+
 def test_int4_scales_below_the_fp16_normals():
     """Scales that fp16 cannot hold exactly (2^-14 and below, bf16 significands) take the fp32 product
     of code and scale.  The down projection's are set to 2^-16 and below: fp16 weights of 2^-24
