@@ -9,7 +9,7 @@
 //   * the grid is persistent (one CTA per SM) and split "stream-K" style: CTA c streams the
 //     contiguous tile range [c*T/G, (c+1)*T/G) of the flattened tile sequence, so every SM
 //     moves the same number of bytes whatever the matrix shape;
-//   * one producer thread per CTA feeds a ring of shared-memory stages with 1-D TMA bulk
+//   * one producer warp per CTA (its elected lane) feeds a ring of shared-memory stages with 1-D TMA bulk
 //     copies (cp.async.bulk + mbarrier complete_tx); eight consumer warps read tiles and the
 //     matching fp32 activation chunks from shared memory and accumulate in fp32;
 //   * under programmatic dependent launch the producer starts streaming weights, which do not

@@ -6,7 +6,8 @@
 // byte and term: at T = 128 the MMAs of a 16 KiB weight slice take about 512 cycles, its share of
 // the HBM bandwidth about 750).  So every SM streams an equal share of the matrix, whatever its
 // shape (TileShare), and a row tile that several CTAs share is summed from their partial sums in CTA
-// order by a small kernel behind it (narrow_reduce_kernel).
+// order by a small kernel behind it (narrow_reduce_kernel; a residual's by the next norm,
+// narrow_norm_kernel).
 // The tokens' terms share each MMA: 128 weight rows x (terms x tokens) columns, so a token count
 // of 16 costs an eighth of the 128-token tile of prefill_gemm_persistent, and the epilogue's lanes
 // hold consecutive output columns of one token.
@@ -14,7 +15,7 @@
 // Measured (7B-shaped blocks, 43 tokens): the gate/up loop streams its 272 MB in 36 us (7.0 TB/s
 // after the first ring fill).  Clusters of up to 8 CTAs per 128-token tile, reducing through
 // distributed shared memory, took 51 us for Q/K/V, 39 for O and down on average and 58 for gate/up
-// (four blocks with everything between: 954 us, now 614).
+// (four blocks with everything between: 954 us, now 522).
 #include <algorithm>
 #include <type_traits>
 

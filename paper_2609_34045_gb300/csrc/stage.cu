@@ -273,7 +273,7 @@ struct kfl_stage {
   std::vector<cudaEvent_t> ev;
   double prof_ms[KFL_KERNEL_KINDS] = {};
   int64_t prof_n[KFL_KERNEL_KINDS] = {};
-  // dense prefill (bf16 stages): the workspace of one pass of up to pf_cap tokens, allocated at
+  // dense prefill: the workspace of one pass of up to pf_cap tokens, allocated at
   // the first dense prefill, and the tensor maps of the weight tiles (per layer: Q/K/V, O,
   // gate/up, down; then lm_head)
   int pf_cap = 0;
@@ -806,7 +806,7 @@ int run_step(kfl_stage *st, const int32_t *ids, const float *hidden_in, const in
   return KFL_OK;
 }
 
-// ---- dense prefill (bf16 weights) ---------------------------------------------------------
+// ---- dense prefill ------------------------------------------------------------------------
 constexpr int PF_PASS = 2048;        // tokens per pass of the dense prefill
 constexpr int PF_PAIR_TOKENS = 512;  // passes of up to this many tokens carry q and the softmax weights as pairs
 
