@@ -537,9 +537,9 @@ __device__ __forceinline__ void act16_put_consts(const Act16 &a, int b, int ch, 
 // Chunk ch of user b of an Act16, one element per lane (x = 0 past the vector's end); the whole
 // warp calls it.
 __device__ __forceinline__ void act16_put_warp(const Act16 &a, int b, int ch, float x, int lane) {
-  float mx = fabsf(x);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  // the largest |x| (NaN aside): magnitudes order as their bits, so one reduction in place of five
+  // shuffles (72B-shaped int4, four users, four blocks and head: 706 -> 702 us per step)
+  const float mx = __uint_as_float(__reduce_max_sync(0xffffffffu, x == x ? __float_as_uint(fabsf(x)) : 0u));
   float iv;
   const float m = xchunk_scale(mx, &iv);
   const bool upper = (lane & 15) >= 8;
