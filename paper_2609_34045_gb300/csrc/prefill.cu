@@ -841,10 +841,10 @@ __global__ void prefill_input_kernel(const int *ids, const float *hidden_in, con
   }
 }
 
-// x[t] = h[t] / rms(h[t]) * g as two or three 16-bit terms (term_stride elements apart), one block per token, four elements per
-// thread step (d a multiple of 8; h, g and x rows 16-byte aligned).  Bound by latency: a thread's
-// first RN_V groups of h and g are loaded at once and kept (2048 x 3584: 13.9 us, 4.2 TB/s; 17.8 one group at a time, read
-// twice).
+// x[t] = h[t] / rms(h[t]) * g as two or three 16-bit terms (term_stride elements apart), one block per
+// token, four elements per thread step (d a multiple of 8; h, g and x rows 16-byte aligned).  Bound
+// by latency: a thread's first RN_V groups of h and g are loaded at once and kept (2048 x 3584:
+// 13.9 us, 4.2 TB/s; 17.8 one group at a time, read twice).
 constexpr int RN_V = 4;
 __global__ void prefill_rmsnorm_kernel(const float *h, int ldh, int d, const float *g, float eps, uint16_t *x,
                                        size_t term_stride, int terms, int ldx, int f16, unsigned *err) {
