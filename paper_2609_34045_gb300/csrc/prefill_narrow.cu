@@ -780,6 +780,7 @@ __global__ void __launch_bounds__(N4_THREADS, 1)
 #pragma unroll
         for (int g = 0; g < 2; ++g) exact = exact && ScalePair(sc[half][g]).exact();
       exact = __all_sync(0xffffffffu, exact);
+      __syncwarp();  // every lane's reads, before lane 0 gives the stage back (a vote orders no memory)
       if (lane == 0) mbar_arrive(smem_addr(&s_cempty[cs]));
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
