@@ -991,14 +991,15 @@ __global__ void prefill_argmax_kernel(const float *amax, const int *aidx, int n_
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+  static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> found{nullptr};
+  PFN_cuTensorMapEncodeTiled_v12000 fn = found.load();
   if (!fn) {
     void *p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
             cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+      found = fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
     else
       cudaGetLastError();
   }
@@ -1088,19 +1089,15 @@ template <int MODE>
 static cudaError_t launch_mode(const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b, bool w_rows, int n_kb,
                                const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s) {
   constexpr bool DRAIN = MODE == PE_STORE;
-  static bool smem_set = false;
-  if (!smem_set) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_gemm_persistent<MODE, DRAIN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
-    if (e != cudaSuccess) return e;
-    smem_set = true;
-  }
+  static SmemOptIn opt_in;
+  cudaError_t e = opt_in(reinterpret_cast<const void *>(prefill_gemm_persistent<MODE, DRAIN>), (int)PG_SMEM);
+  if (e != cudaSuccess) return e;
   // one persistent CTA per SM (fewer if there are not four K blocks for each)
   const int tiles = (ep.T + PG_M - 1) / PG_M * ((ep.N + PG_N - 1) / PG_N);
   const int grid = (int)std::min<long long>(ws.n_sm, std::max<long long>(std::min(tiles, ws.n_sm), (long long)tiles * n_kb / 4));
   const TileShare share = share_tiles(tiles, n_kb, grid, false, NW_PARTS);
-  cudaError_t e = launch_pdl(prefill_gemm_persistent<MODE, DRAIN>, dim3(grid), pp_threads(DRAIN), PG_SMEM, s, a, a2, b, (int)w_rows, share,
-                             ws.partial, ep);
+  e = launch_pdl(prefill_gemm_persistent<MODE, DRAIN>, dim3(grid), pp_threads(DRAIN), PG_SMEM, s, a, a2, b, (int)w_rows,
+                 share, ws.partial, ep);
   if (e == cudaSuccess && share.cut())
     e = launch_pdl(wide_reduce_kernel<MODE>, dim3(share.tail * (MODE == PE_ARGMAX ? 1 : PG_N / 32)), PG_M, 0, s, share,
                    grid, ws.partial, ep);
@@ -1123,13 +1120,10 @@ cudaError_t launch_prefill_gemm(int mode, const CUtensorMap &a, const CUtensorMa
 
 template <int HD, bool PRECISE>
 static cudaError_t launch_attn_hd(const PrefillAttnParams &p, int n_sm, cudaStream_t s) {
-  static bool attr = false;
+  static SmemOptIn opt_in;
   const int bytes = PaLayout<HD>::BYTES;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_attn_kernel<HD, PRECISE>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  const cudaError_t e = opt_in(reinterpret_cast<const void *>(prefill_attn_kernel<HD, PRECISE>), bytes);
+  if (e != cudaSuccess) return e;
   // split the keys until about two CTAs per SM (as many as fit) have work
   const int blocks = (p.T + PA_ROWS - 1) / PA_ROWS * p.n_heads;
   int split = 1;

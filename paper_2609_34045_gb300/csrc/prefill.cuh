@@ -4,6 +4,8 @@
 
 #include <cuda.h>  // CUtensorMap (the type only; maps are encoded through the runtime's entry point)
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace kfl {
@@ -125,6 +127,24 @@ int encode_terms_map(CUtensorMap *map, const uint16_t *base, int K, int rows, in
 int encode_tiles_map(CUtensorMap *map, const uint8_t *tiles, int n_kt, int n_rb, int box_rb);
 // A row-major bf16 matrix [N][K] (K a multiple of 8, 16-byte aligned): boxes of 64 columns x box_rows rows.
 int encode_rows_map(CUtensorMap *map, const uint16_t *w, int K, int N, int box_rows);
+// Opts a kernel in to its dynamic shared memory before a launch.  The attribute holds for the device it
+// was set on, so it is set once on each (a bit per device; beyond 64, at every launch); a failure is not
+// remembered.  One per kernel, shared by every thread.
+class SmemOptIn {
+  std::atomic<uint64_t> done_{0};
+
+ public:
+  cudaError_t operator()(const void *kernel, int bytes) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (done_.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+  }
+};
 // The launch attribute of a kernel that waits (griddepcontrol.wait) for the kernel before it.
 inline void pdl_attribute(cudaLaunchAttribute &a) {
   a.id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -830,12 +830,22 @@ int narrow_argmax_slots(int N) { return (N + 127) / 128 * 4; }
 
 // Opts a kernel in to a block's whole shared memory; returns its dynamic part (the rings start on
 // the KiB boundary after the kernel's own barriers), or -1.
-static int ring_smem(const void *kernel) {
-  cudaFuncAttributes a;
-  if (cudaFuncGetAttributes(&a, kernel) != cudaSuccess || a.sharedSizeBytes > 1024) return -1;
-  const int dyn = NW_RING + 1024 - (int)a.sharedSizeBytes;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) == cudaSuccess ? dyn : -1;
-}
+class RingOptIn {
+  SmemOptIn opt_in_;
+  std::atomic<int> own_{-1};  // the kernel's static shared memory
+
+ public:
+  int operator()(const void *kernel) {
+    int own = own_.load(std::memory_order_relaxed);
+    if (own < 0) {
+      cudaFuncAttributes a;
+      if (cudaFuncGetAttributes(&a, kernel) != cudaSuccess || a.sharedSizeBytes > 1024) return -1;
+      own_.store(own = (int)a.sharedSizeBytes, std::memory_order_relaxed);
+    }
+    const int dyn = NW_RING + 1024 - own;
+    return opt_in_(kernel, dyn) == cudaSuccess ? dyn : -1;
+  }
+};
 
 template <int MODE>
 static cudaError_t launch_narrow_reduce(const NarrowParams &p, int mb, int grid, const PrefillEpiParams &ep,
@@ -860,7 +870,8 @@ static cudaError_t launch_narrow_reduce(const NarrowParams &p, int mb, int grid,
 template <int MODE, int MB, bool DRAIN>
 static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x, const NarrowParams &p, int grid,
                                       const PrefillEpiParams &ep, cudaStream_t s, NarrowPending *pending) {
-  static const int smem = ring_smem(reinterpret_cast<const void *>(prefill_narrow_kernel<MODE, MB, DRAIN>));
+  static RingOptIn opt_in;
+  const int smem = opt_in(reinterpret_cast<const void *>(prefill_narrow_kernel<MODE, MB, DRAIN>));
   if (smem < 0) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
@@ -927,7 +938,8 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, c
 template <int MODE>
 static cudaError_t launch_narrow4_mode(const Narrow4Params &r, const CUtensorMap &x, const NarrowParams &p, int grid,
                                        const PrefillEpiParams &ep, cudaStream_t s, NarrowPending *pending) {
-  static const int smem = ring_smem(reinterpret_cast<const void *>(prefill_narrow4_kernel<MODE>));
+  static RingOptIn opt_in;
+  const int smem = opt_in(reinterpret_cast<const void *>(prefill_narrow4_kernel<MODE>));
   if (smem < 0) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);

@@ -1,0 +1,103 @@
+"""The library's host code on a CUDA runtime without a GPU (fake_cudart.cpp): what the prefill's launches
+and workspace do on a second device, when an allocation fails and under stream capture."""
+import ctypes as C
+import dataclasses
+import importlib
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2609_34045_gb300 import stage as K
+from paper_2609_34045_gb300 import workload as wl
+
+B = importlib.import_module("paper_2609_34045_gb300.build")  # (the package binds the name to its function)
+HERE = os.path.dirname(os.path.abspath(__file__))
+# weight tiles of 128 tokens from 129 tokens on (F large enough for every SM), few layers
+WIDE = wl.ModelShape(n_layers_total=1, d_model=128, n_heads=2, n_kv_heads=1, head_dim=64, ffn=19456, vocab=300)
+SMALL = wl.ModelShape(n_layers_total=1, d_model=128, n_heads=2, n_kv_heads=1, head_dim=64, ffn=256, vocab=300)
+QK = dataclasses.replace(SMALL, qk_norm=True)
+INT4 = dataclasses.replace(SMALL, weight_fmt="int4_g64")
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    B.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    objs = [os.path.join(B.BUILD, f) for f in sorted(os.listdir(B.BUILD)) if f.endswith(".o")]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", cuda, "-o", out,
+                    os.path.join(HERE, "fake_cudart.cpp"), *objs], check=True)
+    return out
+
+
+@pytest.fixture
+def dev(fake_lib, tmp_path, monkeypatch):
+    """The library on a fake device of its own, behind the package's binding."""
+    path = shutil.copy(fake_lib, tmp_path / "libkafila_fake.so")
+    monkeypatch.setattr(K, "LIB_PATH", str(path))
+    monkeypatch.setattr(K, "_lib", None)
+    monkeypatch.delenv("KFL_PREFILL_DENSE_MIN", raising=False)
+    lib = K.lib()
+    lib.fake_live.restype = lib.fake_pool_held.restype = C.c_size_t
+    lib.fake_launches.restype = lib.fake_mallocs.restype = lib.fake_marked.restype = C.c_long
+    lib.fake_budget.argtypes = [C.c_size_t]
+    return lib
+
+
+def _stage(model, max_batch=1):
+    d, hd, kv, f = model.d_model, model.head_dim, model.n_kv_heads * model.head_dim, model.ffn
+    w = {n: np.zeros(m, dtype=np.uint16) for n, m in (("attn_norm", d), ("ffn_norm", d), ("q_norm", hd), ("k_norm", hd))}
+    for n, rows, cols in (("wq", model.n_heads * hd, d), ("wk", kv, d), ("wv", kv, d), ("wo", d, model.n_heads * hd),
+                          ("wg", f, d), ("wu", f, d), ("wd", d, f)):
+        w[n] = (np.zeros((rows, cols), dtype=np.uint16) if model.weight_fmt == "bf16" else
+                (np.zeros((rows, cols // 8), dtype=np.uint32), np.zeros((rows, cols // 64), dtype=np.uint16)))
+    st = K.kfl_stage_create(K.model_cfg(model, 4096, max_batch), 0, 1, 0)
+    K.kfl_stage_load_layer(st, 0, w, on_device=False)
+    return st
+
+
+def _prefill(st, n):
+    """The return code of a prompt of n tokens (no kernel runs: the buffers are never read)."""
+    pos = np.arange(n, dtype=np.int32)
+    h = np.zeros(1, dtype=np.float32)
+    return K.lib().kfl_stage_prefill(st.handle, None, h.ctypes.data, pos.ctypes.data, 0, n, h.ctypes.data, None, None)
+
+
+def _matmul(T, k, n):
+    a = np.zeros(4, dtype=np.float32)
+    at = (a.ctypes.data + 15) // 16 * 16
+    return K.lib().kfl_matmul_bf16w(at, T, k, k, at, n, at, (n + 3) // 4 * 4, None)
+
+
+@pytest.mark.parametrize("model,n,kernel", [
+    (SMALL, 40, "prefill_narrow_kernel"), (SMALL, 9, "prefill_narrow_kernel"), (QK, 40, "prefill_narrow_kernel"),
+    (INT4, 40, "prefill_narrow4_kernel"), (WIDE, 200, "prefill_gemm_persistent"),
+    (WIDE, 600, "prefill_attn_kernel")])
+def test_prompts_on_a_second_device(dev, model, n, kernel):
+    """The kernels' shared memory is opted in on each device that launches them."""
+    for d in range(2):
+        dev.cudaSetDevice(d)
+        st = _stage(model)
+        before = dev.fake_launches(kernel.encode())
+        assert _prefill(st, n) == 0
+        assert dev.fake_launches(kernel.encode()) > before
+        K.kfl_stage_destroy(st)
+
+
+@pytest.mark.parametrize("T", [40, 300])
+def test_product_on_a_second_device(dev, T):
+    for d in range(2):
+        dev.cudaSetDevice(d)
+        assert _matmul(T, 64, 256) == 0
+
+
+@pytest.mark.parametrize("model,n", [(SMALL, 40), (INT4, 40), (WIDE, 200)])
+def test_a_failed_opt_in_is_tried_again(dev, model, n):
+    st = _stage(model)
+    dev.fake_fail_optin(1)
+    assert _prefill(st, n) < 0
+    assert _prefill(st, n) == 0
+    K.kfl_stage_destroy(st)
