@@ -166,7 +166,9 @@ int kfl_stage_decode_users(kfl_stage *st, const int32_t *token_ids, const float 
  * decode steps' precision (three bf16 terms per activation).  Other prompts, and those while a
  * capture, trace or profile is on or for which no workspace can be allocated, go as steps of up
  * to max_batch rows, in order, every row of a step addressing the user's slot (the decode step's
- * kernels).  Enqueued on cuda_stream, returns without waiting.
+ * kernels).  Enqueued on cuda_stream, returns without waiting.  Dense prompts can be captured once
+ * a call that was not has made the workspace for their size; what a capture used stays allocated
+ * until kfl_stage_destroy, also when longer prompts have outgrown it.
  *   token_ids  device int32[n_tokens] (KFL_EMBED_IN), else ignored
  *   hidden_in  device fp32[n_tokens][d_model] (without KFL_EMBED_IN)
  *   positions  device int32[n_tokens]: token t's position, distinct, normally start + t; the

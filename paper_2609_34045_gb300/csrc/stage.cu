@@ -286,6 +286,8 @@ struct kfl_stage {
   float *pf_raw = nullptr;  // QK-norm stages: the Q/K/V projection before the norm and RoPE [token][ld_raw]
   float *pf_amax = nullptr;
   std::vector<void *> pf_allocs;
+  bool pf_captured = false;         // a captured graph holds the workspace's addresses
+  std::vector<void *> pf_retired;   // workspaces outgrown since: kept for the graphs until the stage goes
   // bf16 stages: the maps of every layer's weight tiles [4 l + j] (Q/K/V, O, gate/up, down), then
   // lm_head.  int4 stages: one map per matrix kind [j] (then lm_head) over pf_w16, the fp16 tiles
   // of the matrix being multiplied (dequantized just before its GEMM)
@@ -831,8 +833,12 @@ int ensure_prefill(kfl_stage *st, int tokens) {
   const Plan &P = st->P;
   const int cap = std::min(PF_PASS, round_up(tokens, PG_M)), first = std::min(PF_PASS, tokens);
   if (cap > st->pf_cap) {
-    for (void *p : st->pf_allocs) cudaFree(p);
+    if (st->pf_captured)
+      st->pf_retired.insert(st->pf_retired.end(), st->pf_allocs.begin(), st->pf_allocs.end());
+    else
+      for (void *p : st->pf_allocs) cudaFree(p);
     st->pf_allocs.clear();
+    st->pf_captured = false;
     st->pf_cap = 0;
     auto get = [&](void **p, size_t bytes) {
       if (!device_alloc(p, bytes)) return false;
@@ -1012,6 +1018,15 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
   return err;
 }
 
+// Whether s is being captured (a stream that cannot say, such as the legacy one while another
+// captures, is taken to be).
+bool is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 // The prompt in passes of up to pf_cap tokens.  Per pass and block: RMSNorm -> Q/K/V GEMM (RoPE,
 // K/V appended to the user's slot) -> causal attention over the slot -> O GEMM + residual ->
 // RMSNorm -> gate/up GEMM (SwiGLU) -> down GEMM + residual; the head: final RMSNorm -> lm_head GEMM
@@ -1024,6 +1039,7 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
   const Plan &P = st->P;
   int rc = ensure_prefill(st, T);
   if (rc != KFL_OK) return rc;
+  if (is_capturing(s)) st->pf_captured = true;
   const bool embed = (st->flags & KFL_EMBED_IN) != 0;
   const int i4 = st->cfg.weight_fmt == KFL_INT4_G64 ? 1 : 0;
   const int ldq = pf_ld(P.qdim), lda = pf_ld(P.F);
@@ -1167,13 +1183,7 @@ bool prefill_precise(kfl_stage *st, int n_tokens, int dense_min, cudaStream_t s)
   // that would take more than one decode step
   if (st->cfg.qk_norm ? n_tokens < dense_min : n_tokens <= st->cfg.max_batch || std::getenv("KFL_PREFILL_DENSE_MIN"))
     return false;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  const int need = std::min(PF_PASS, round_up(n_tokens, PG_M));
-  if (cap != cudaStreamCaptureStatusNone) return st->pf_cap >= need && !st->pf_maps.empty();
+  if (is_capturing(s)) return st->pf_cap >= std::min(PF_PASS, round_up(n_tokens, PG_M)) && !st->pf_maps.empty();
   return ensure_prefill(st, n_tokens) == KFL_OK;
 }
 
@@ -1789,6 +1799,7 @@ extern "C" void kfl_stage_destroy(kfl_stage *st) {
   if (st->cap_stream) cudaStreamDestroy(st->cap_stream);
   for (void *p : st->allocs) cudaFree(p);
   for (void *p : st->pf_allocs) cudaFree(p);
+  for (void *p : st->pf_retired) cudaFree(p);
   for (int b = 0; b < 2; ++b) {
     if (st->pf_w16[b]) cudaFree(st->pf_w16[b]);
     if (st->pf_deq[b]) cudaEventDestroy(st->pf_deq[b]);

@@ -101,3 +101,20 @@ def test_a_failed_opt_in_is_tried_again(dev, model, n):
     assert _prefill(st, n) < 0
     assert _prefill(st, n) == 0
     K.kfl_stage_destroy(st)
+
+
+@pytest.mark.parametrize("model,n", [(QK, 40), (SMALL, 9), (SMALL, 40), (INT4, 40)])
+def test_a_captured_prompt_keeps_its_workspace(dev, model, n):
+    """A longer prompt after the capture leaves the memory that the captured graph uses alone; the
+    stage's end gives all of it back."""
+    st = _stage(model)
+    assert _prefill(st, n) == 0
+    dev.fake_capturing(1)
+    assert _prefill(st, n) == 0
+    dev.fake_capturing(0)
+    dev.fake_mark()
+    held = dev.fake_marked()
+    assert _prefill(st, 700) == 0
+    assert dev.fake_marked() == held
+    K.kfl_stage_destroy(st)
+    assert dev.fake_live() == 0
