@@ -182,7 +182,11 @@ int kfl_stage_decode_users(kfl_stage *st, const int32_t *token_ids, const float 
  * stage's dense prefill an activation beyond the fp16 range (|x| >= 65520, or not finite) is
  * found on the device too: kfl_stage_status then reports KFL_ERR_OVERFLOW and the call's
  * outputs and cache rows are not valid.
- * Errors returned here: KFL_ERR_ARG, KFL_ERR_RANGE (user), KFL_ERR_STATE, KFL_ERR_CUDA. */
+ * The dense workspace (about 60 MB of partial sums and the activations of the longest pass so far) is not
+ * part of kfl_stage_memory_bytes.  Where a longer prompt finds no memory for it, the workspace of the
+ * shorter ones stays.
+ * Errors returned here: KFL_ERR_ARG, KFL_ERR_RANGE (user), KFL_ERR_STATE, KFL_ERR_OOM (the workspace of
+ * a prompt that does not fall back to steps), KFL_ERR_CUDA. */
 int kfl_stage_prefill(kfl_stage *st, const int32_t *token_ids, const float *hidden_in,
                       const int32_t *positions, int user, int n_tokens, float *hidden_out,
                       int32_t *next_ids, void *cuda_stream);

@@ -227,6 +227,21 @@ bool device_alloc(void **p, size_t bytes) {
 }
 }  // namespace
 
+// The workspace of one dense prefill pass of up to `cap` tokens.
+struct PrefillWorkspace {
+  int cap = 0;
+  float *h = nullptr;
+  uint16_t *q = nullptr;
+  uint16_t *x = nullptr, *o = nullptr, *a = nullptr;  // GEMM inputs as terms [term][token][ld]
+  float *partial = nullptr;  // the GEMMs' partial sums
+  int *pos = nullptr, *slots = nullptr, *aidx = nullptr;
+  float *raw = nullptr;  // QK-norm stages: the Q/K/V projection before the norm and RoPE [token][ld_raw]
+  float *amax = nullptr;
+  std::vector<void *> allocs;
+  size_t bytes = 0;
+  bool captured = false;  // a captured graph holds its addresses
+};
+
 struct kfl_stage {
   kfl_model_cfg cfg;
   int l0 = 0, l1 = 0, flags = 0;
@@ -273,21 +288,12 @@ struct kfl_stage {
   std::vector<cudaEvent_t> ev;
   double prof_ms[KFL_KERNEL_KINDS] = {};
   int64_t prof_n[KFL_KERNEL_KINDS] = {};
-  // dense prefill: the workspace of one pass of up to pf_cap tokens, allocated at
-  // the first dense prefill, and the tensor maps of the weight tiles (per layer: Q/K/V, O,
-  // gate/up, down; then lm_head)
-  int pf_cap = 0;
-  float *pf_h = nullptr;
-  uint16_t *pf_q = nullptr;
-  uint16_t *pf_x = nullptr, *pf_o = nullptr, *pf_a = nullptr;  // GEMM inputs as terms [term][token][ld]
-  NarrowWorkspace pf_nw = {};  // the few-token GEMM's partial sums
+  // dense prefill: the workspace, allocated at the first dense prefill, and the tensor maps of the weight
+  // tiles (per layer: Q/K/V, O, gate/up, down; then lm_head)
+  PrefillWorkspace pf;
+  int pf_failed = 0;               // tokens of the last workspace there was no memory for (0: none since)
   int pf_amax_cols = 0;
-  int *pf_pos = nullptr, *pf_slots = nullptr, *pf_aidx = nullptr;
-  float *pf_raw = nullptr;  // QK-norm stages: the Q/K/V projection before the norm and RoPE [token][ld_raw]
-  float *pf_amax = nullptr;
-  std::vector<void *> pf_allocs;
-  bool pf_captured = false;         // a captured graph holds the workspace's addresses
-  std::vector<void *> pf_retired;   // workspaces outgrown since: kept for the graphs until the stage goes
+  std::vector<void *> pf_retired;  // workspaces outgrown since a graph captured them: kept until the stage goes
   // bf16 stages: the maps of every layer's weight tiles [4 l + j] (Q/K/V, O, gate/up, down), then
   // lm_head.  int4 stages: one map per matrix kind [j] (then lm_head) over pf_w16, the fp16 tiles
   // of the matrix being multiplied (dequantized just before its GEMM)
@@ -828,42 +834,80 @@ int pf_narrow_most(const kfl_stage *st) {
 }
 bool pf_narrow(const kfl_stage *st, int n, bool precise = false) { return precise || n <= pf_narrow_most(st); }
 
+// Calls block(pointer, bytes) for every buffer of a workspace for passes of up to `cap` tokens.
+template <typename F>
+void pf_blocks(const kfl_stage *st, int cap, PrefillWorkspace &w, F block) {
+  const Plan &P = st->P;
+  // two terms per input, and q in bf16; QK-norm stages three, and q in fp32 (so do passes of fewer
+  // than 16 tokens, which need less than the room of 128 with two)
+  const size_t rows = (size_t)cap * (st->cfg.qk_norm ? 3 : 2);
+  block((void **)&w.h, (size_t)cap * P.ldh * 4);
+  block((void **)&w.q, rows * pf_ld(P.qdim) * 2);
+  block((void **)&w.x, rows * pf_ld(P.d) * 2);
+  block((void **)&w.o, rows * pf_ld(P.qdim) * 2);
+  block((void **)&w.a, rows * pf_ld(P.F) * 2);
+  block((void **)&w.pos, (size_t)cap * 4);
+  block((void **)&w.slots, (size_t)cap * 4);
+  if (st->cfg.qk_norm) block((void **)&w.raw, (size_t)cap * P.ld_raw * 4);
+  // argmax partials: per 256-column tile, or (passes on the few-token GEMM) per 32 rows
+  if (st->flags & KFL_LOGITS_OUT) {
+    const int narrow = std::min(cap, st->cfg.qk_norm ? PF_PASS : pf_narrow_most(st));
+    const size_t am = std::max((size_t)cap * ((P.V + PG_N - 1) / PG_N), (size_t)narrow * narrow_argmax_slots(P.V));
+    block((void **)&w.amax, am * 4);
+    block((void **)&w.aidx, am * 4);
+  }
+  block((void **)&w.partial, narrow_ws_bytes(P.n_sm, cap));
+}
+
+void pf_free(PrefillWorkspace &w) {
+  for (void *p : w.allocs) cudaFree(p);
+  w = PrefillWorkspace();
+}
+
+// A workspace for `cap` tokens, or nothing.
+bool pf_alloc(const kfl_stage *st, int cap, PrefillWorkspace &w) {
+  bool ok = true;
+  pf_blocks(st, cap, w, [&](void **p, size_t bytes) {
+    ok = ok && device_alloc(p, bytes);
+    if (ok) w.allocs.push_back(*p), w.bytes += bytes;
+  });
+  if (!ok) return pf_free(w), false;
+  w.cap = cap;
+  return true;
+}
+
+// The workspace for `cap` tokens in place of the smaller one there is.  Without the memory for it the
+// smaller one stays (made again if it had to go first), and the size is not tried again until the
+// device has as much free.
+int pf_grow(kfl_stage *st, int cap) {
+  if (st->pf_failed && cap >= st->pf_failed) {
+    PrefillWorkspace w;
+    size_t need = 0, free_bytes = 0, total = 0;
+    pf_blocks(st, cap, w, [&](void **, size_t bytes) { need += bytes; });
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) cudaGetLastError();
+    if (free_bytes + (st->pf.captured ? 0 : st->pf.bytes) < need) return KFL_ERR_OOM;
+  }
+  PrefillWorkspace w;
+  const int before = st->pf.cap;
+  if (!st->pf.captured) pf_free(st->pf);
+  if (!pf_alloc(st, cap, w)) {
+    st->pf_failed = cap;
+    if (!st->pf.captured && before > 0) pf_alloc(st, before, st->pf);
+    return KFL_ERR_OOM;
+  }
+  st->pf_retired.insert(st->pf_retired.end(), st->pf.allocs.begin(), st->pf.allocs.end());
+  st->pf = std::move(w);
+  st->pf_failed = 0;
+  return KFL_OK;
+}
+
 // Workspace for passes of up to `tokens` tokens (grown, never shrunk) and the weight maps.
 int ensure_prefill(kfl_stage *st, int tokens) {
   const Plan &P = st->P;
   const int cap = std::min(PF_PASS, round_up(tokens, PG_M)), first = std::min(PF_PASS, tokens);
-  if (cap > st->pf_cap) {
-    if (st->pf_captured)
-      st->pf_retired.insert(st->pf_retired.end(), st->pf_allocs.begin(), st->pf_allocs.end());
-    else
-      for (void *p : st->pf_allocs) cudaFree(p);
-    st->pf_allocs.clear();
-    st->pf_captured = false;
-    st->pf_cap = 0;
-    auto get = [&](void **p, size_t bytes) {
-      if (!device_alloc(p, bytes)) return false;
-      st->pf_allocs.push_back(*p);
-      return true;
-    };
-    // two terms per input, and q in bf16; QK-norm stages three, and q in fp32 (so do passes of fewer
-    // than 16 tokens, which need less than the room of 128 with two)
-    const size_t rows = (size_t)cap * (st->cfg.qk_norm ? 3 : 2);
-    bool ok = get((void **)&st->pf_h, (size_t)cap * P.ldh * 4) && get((void **)&st->pf_q, rows * pf_ld(P.qdim) * 2) &&
-              get((void **)&st->pf_x, rows * pf_ld(P.d) * 2) && get((void **)&st->pf_o, rows * pf_ld(P.qdim) * 2) &&
-              get((void **)&st->pf_a, rows * pf_ld(P.F) * 2) && get((void **)&st->pf_pos, (size_t)cap * 4) &&
-              get((void **)&st->pf_slots, (size_t)cap * 4);
-    if (st->cfg.qk_norm) ok = ok && get((void **)&st->pf_raw, (size_t)cap * P.ld_raw * 4);
-    // argmax partials: per 256-column tile, or (passes on the few-token GEMM) per 32 rows
-    if (st->flags & KFL_LOGITS_OUT) {
-      const int most = st->cfg.qk_norm ? PF_PASS : pf_narrow_most(st);
-      const int narrow = std::min(cap, most);
-      const size_t am = std::max((size_t)cap * ((P.V + PG_N - 1) / PG_N), (size_t)narrow * narrow_argmax_slots(P.V));
-      ok = ok && get((void **)&st->pf_amax, am * 4) && get((void **)&st->pf_aidx, am * 4);
-    }
-    st->pf_nw.n_sm = P.n_sm;
-    ok = ok && get((void **)&st->pf_nw.partial, narrow_ws_bytes(P.n_sm, cap));
-    if (!ok) return KFL_ERR_OOM;
-    st->pf_cap = cap;
+  if (cap > st->pf.cap) {
+    const int rc = pf_grow(st, cap);
+    if (rc != KFL_OK) return rc;
   }
   if (st->pf_maps.empty() && st->cfg.weight_fmt == KFL_INT4_G64 && !pf_narrow(st, first)) {
     // the fp16 scratch holds the largest matrix; its maps are per matrix kind
@@ -997,14 +1041,16 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
   e.terms = x.terms;
   e.f16 = i4 ? 1 : 0;
   if (mode == PE_ARGMAX) {
-    e.amax = st->pf_amax;
-    e.aidx = st->pf_aidx;
+    e.amax = st->pf.amax;
+    e.aidx = st->pf.aidx;
     e.n_tiles = st->pf_amax_cols;
   }
+  const NarrowWorkspace ws = {st->pf.partial, st->P.n_sm};
   if (i4 && pf_narrow(st, x.n))
-    return launch_prefill_narrow4(mode, m.tiles, m.n_rb, m.n_kt, x.all, m.K, x.terms, st->pf_nw, e, s, pending);
+    return launch_prefill_narrow4(mode, m.tiles, m.n_rb, m.n_kt, x.all, m.K, x.terms, ws, e, s, pending);
   if (!i4 && pf_narrow(st, x.n, x.terms == 3))
-    return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], false, x.all, m.K, x.terms, st->pf_nw, e, s, pending);
+    return launch_prefill_narrow(mode, st->pf_maps_nw[j == 4 ? 4 * st->P.nl : 4 * l + j], false, x.all, m.K, x.terms,
+                                 ws, e, s, pending);
   if (i4) {
     cudaError_t err = pf_dequant(st, g + 1);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, st->pf_deq[g % 2], 0);
@@ -1013,7 +1059,7 @@ cudaError_t pf_gemm(kfl_stage *st, int mode, const PfInput &x, int l, int j, Pre
   } else {
     b = &st->pf_maps[j == 4 ? 4 * st->P.nl : 4 * l + j];
   }
-  cudaError_t err = launch_prefill_gemm(mode, x.term[0], x.term[1], *b, false, m.K, st->pf_nw, e, s);
+  cudaError_t err = launch_prefill_gemm(mode, x.term[0], x.term[1], *b, false, m.K, ws, e, s);
   if (err == cudaSuccess && i4) err = cudaEventRecord(st->pf_used[g % 2], s);
   return err;
 }
@@ -1027,7 +1073,7 @@ bool is_capturing(cudaStream_t s) {
   return true;
 }
 
-// The prompt in passes of up to pf_cap tokens.  Per pass and block: RMSNorm -> Q/K/V GEMM (RoPE,
+// The prompt in passes of up to pf.cap tokens.  Per pass and block: RMSNorm -> Q/K/V GEMM (RoPE,
 // K/V appended to the user's slot) -> causal attention over the slot -> O GEMM + residual ->
 // RMSNorm -> gate/up GEMM (SwiGLU) -> down GEMM + residual; the head: final RMSNorm -> lm_head GEMM
 // with the greedy argmax.
@@ -1039,36 +1085,36 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
   const Plan &P = st->P;
   int rc = ensure_prefill(st, T);
   if (rc != KFL_OK) return rc;
-  if (is_capturing(s)) st->pf_captured = true;
+  if (is_capturing(s)) st->pf.captured = true;
   const bool embed = (st->flags & KFL_EMBED_IN) != 0;
   const int i4 = st->cfg.weight_fmt == KFL_INT4_G64 ? 1 : 0;
   const int ldq = pf_ld(P.qdim), lda = pf_ld(P.F);
   const float eps = st->cfg.rms_eps;
-  for (int t0 = 0; t0 < T; t0 += st->pf_cap) {
-    const int n = std::min(st->pf_cap, T - t0);
+  for (int t0 = 0; t0 < T; t0 += st->pf.cap) {
+    const int n = std::min(st->pf.cap, T - t0);
     const bool narrow = pf_narrow(st, n, precise);
     const int terms = precise ? 3 : 2;
     CK(launch_prefill_input(ids ? ids + t0 : nullptr, hidden_in ? hidden_in + (size_t)t0 * P.d : nullptr,
-                            positions + t0, n, embed ? st->embed : nullptr, P.V, P.d, P.ldh, st->pf_h, st->pf_pos,
-                            st->cfg.max_ctx, user, st->pf_slots, st->err, s));
+                            positions + t0, n, embed ? st->embed : nullptr, P.V, P.d, P.ldh, st->pf.h, st->pf.pos,
+                            st->cfg.max_ctx, user, st->pf.slots, st->err, s));
     if (!narrow) CK(pf_pass_begin(st, s));
     PfInput x, o, a;
-    if (x.encode(st->pf_x, P.d, n, terms, narrow) || o.encode(st->pf_o, P.qdim, n, terms, narrow) ||
-        a.encode(st->pf_a, P.F, n, terms, narrow))
+    if (x.encode(st->pf.x, P.d, n, terms, narrow) || o.encode(st->pf.o, P.qdim, n, terms, narrow) ||
+        a.encode(st->pf.a, P.F, n, terms, narrow))
       return KFL_ERR_CUDA;
     st->pf_amax_cols = narrow ? narrow_argmax_slots(P.V) : (P.V + PG_N - 1) / PG_N;
     NarrowPending pend;
     auto norm = [&](const float *g) {
       if (pend.any) {
         pend.any = false;
-        return launch_narrow_norm(pend, st->pf_h, P.ldh, n, P.d, g, eps, x.base, x.stride, terms, x.ld, i4, st->err, s);
+        return launch_narrow_norm(pend, st->pf.h, P.ldh, n, P.d, g, eps, x.base, x.stride, terms, x.ld, i4, st->err, s);
       }
-      return launch_prefill_rmsnorm(st->pf_h, P.ldh, n, P.d, g, eps, x.base, x.stride, terms, x.ld, i4, st->err, s);
+      return launch_prefill_rmsnorm(st->pf.h, P.ldh, n, P.d, g, eps, x.base, x.stride, terms, x.ld, i4, st->err, s);
     };
     PrefillEpiParams r = {};  // O and down: into the residual stream
     r.err = st->err;
     r.N = P.d;
-    r.out = st->pf_h;
+    r.out = st->pf.h;
     r.ldo = P.ldh;
     for (int l = 0; l < P.nl; ++l) {
       const LayerDev &L = st->layers[l];
@@ -1078,11 +1124,11 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       PrefillEpiParams e = {};
       e.err = st->err;
       e.N = L.qkv.N;
-      e.out16 = st->pf_q;
+      e.out16 = st->pf.q;
       e.ldo16 = ldq;
       e.kcache = kcl;
       e.vcache = vcl;
-      e.positions = st->pf_pos;
+      e.positions = st->pf.pos;
       e.slot = user;
       e.hd = P.hd;
       e.hkv = P.hkv;
@@ -1093,24 +1139,24 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       e.rope_sin = st->rope_sin;
       // q in fp32, and q and the softmax weights as bf16 pairs in attention, wherever attention is
       // bound by latency rather than by its MMAs (which this doubles)
-      float *q32 = narrow || n <= PF_PAIR_TOKENS ? reinterpret_cast<float *>(st->pf_q) : nullptr;
+      float *q32 = narrow || n <= PF_PAIR_TOKENS ? reinterpret_cast<float *>(st->pf.q) : nullptr;
       if (st->cfg.qk_norm) {
         PrefillEpiParams raw = {};
         raw.err = st->err;
         raw.N = L.qkv.N;
-        raw.out = st->pf_raw;
+        raw.out = st->pf.raw;
         raw.ldo = P.ld_raw;
         CK(pf_gemm(st, PE_STORE, x, l, 0, raw, s));
         QkNormParams qn = {};
-        qn.raw = st->pf_raw;
+        qn.raw = st->pf.raw;
         qn.ld_raw = P.ld_raw;
         qn.g_q = L.g_q;
         qn.g_k = L.g_k;
         qn.q = q32;
         qn.kcache = kcl;
         qn.vcache = vcl;
-        qn.positions = st->pf_pos;
-        qn.slots = st->pf_slots;
+        qn.positions = st->pf.pos;
+        qn.slots = st->pf.slots;
         qn.rope_cos = st->rope_cos;
         qn.rope_sin = st->rope_sin;
         qn.batch = n;
@@ -1126,7 +1172,7 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
         CK(pf_gemm(st, PE_QKV, x, l, 0, e, s));
       }
       PrefillAttnParams t = {};
-      t.q = st->pf_q;
+      t.q = st->pf.q;
       t.q32 = q32;
       t.ldq = q32 ? P.qdim : ldq;
       t.o = o.base;
@@ -1136,7 +1182,7 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       t.f16 = i4;
       t.kcache = kcl;
       t.vcache = vcl;
-      t.positions = st->pf_pos;
+      t.positions = st->pf.pos;
       t.slot = user;
       t.T = n;
       t.n_heads = P.hq;
@@ -1164,10 +1210,10 @@ int run_prefill_dense(kfl_stage *st, const int32_t *ids, const float *hidden_in,
       z.err = st->err;
       z.N = P.V;
       CK(pf_gemm(st, PE_ARGMAX, x, -1, 4, z, s));
-      CK(launch_prefill_argmax(st->pf_amax, st->pf_aidx, st->pf_amax_cols, n, next_ids + t0, s));
+      CK(launch_prefill_argmax(st->pf.amax, st->pf.aidx, st->pf_amax_cols, n, next_ids + t0, s));
     }
     if (hidden_out)
-      CK(cudaMemcpy2DAsync(hidden_out + (size_t)t0 * P.d, (size_t)P.d * 4, st->pf_h, (size_t)P.ldh * 4,
+      CK(cudaMemcpy2DAsync(hidden_out + (size_t)t0 * P.d, (size_t)P.d * 4, st->pf.h, (size_t)P.ldh * 4,
                            (size_t)P.d * 4, n, cudaMemcpyDeviceToDevice, s));
   }
   return KFL_OK;
@@ -1183,7 +1229,7 @@ bool prefill_precise(kfl_stage *st, int n_tokens, int dense_min, cudaStream_t s)
   // that would take more than one decode step
   if (st->cfg.qk_norm ? n_tokens < dense_min : n_tokens <= st->cfg.max_batch || std::getenv("KFL_PREFILL_DENSE_MIN"))
     return false;
-  if (is_capturing(s)) return st->pf_cap >= std::min(PF_PASS, round_up(n_tokens, PG_M)) && !st->pf_maps.empty();
+  if (is_capturing(s)) return st->pf.cap >= std::min(PF_PASS, round_up(n_tokens, PG_M)) && !st->pf_maps.empty();
   return ensure_prefill(st, n_tokens) == KFL_OK;
 }
 
@@ -1798,7 +1844,7 @@ extern "C" void kfl_stage_destroy(kfl_stage *st) {
   for (cudaEvent_t e : st->ev) cudaEventDestroy(e);
   if (st->cap_stream) cudaStreamDestroy(st->cap_stream);
   for (void *p : st->allocs) cudaFree(p);
-  for (void *p : st->pf_allocs) cudaFree(p);
+  pf_free(st->pf);
   for (void *p : st->pf_retired) cudaFree(p);
   for (int b = 0; b < 2; ++b) {
     if (st->pf_w16[b]) cudaFree(st->pf_w16[b]);

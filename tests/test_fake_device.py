@@ -118,3 +118,34 @@ def test_a_captured_prompt_keeps_its_workspace(dev, model, n):
     assert dev.fake_marked() == held
     K.kfl_stage_destroy(st)
     assert dev.fake_live() == 0
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("model", [QK, SMALL])
+def test_no_memory_for_a_larger_workspace(dev, model, captured):
+    """A prompt whose workspace finds no memory leaves the smaller one in use and nothing else behind, does
+    not try again while there is no more memory, and runs once there is."""
+    st = _stage(model)
+    assert _prefill(st, 40) == 0
+    if captured:
+        dev.fake_capturing(1)
+        assert _prefill(st, 40) == 0
+        dev.fake_capturing(0)
+    held, kernel = dev.fake_live(), b"prefill_narrow_kernel"
+    dev.fake_budget(held + (1 << 20))
+    # a QK-norm stage's prompt goes as decode steps then, another's is refused
+    dense, steps = dev.fake_launches(kernel), dev.fake_launches(b"decode graph")
+    assert _prefill(st, 1500) == (0 if model.qk_norm else -3)
+    assert dev.fake_launches(kernel) == dense
+    assert (dev.fake_launches(b"decode graph") > steps) == model.qk_norm
+    assert dev.fake_live() == held
+    assert _prefill(st, 40) == 0
+    assert dev.fake_launches(kernel) > dense  # densely again, on the workspace it had
+    calls = dev.fake_mallocs()
+    _prefill(st, 1500)
+    assert dev.fake_mallocs() == calls and dev.fake_live() == held
+    dev.fake_budget(1 << 40)
+    dense = dev.fake_launches(kernel)
+    assert _prefill(st, 1500) == 0 and dev.fake_launches(kernel) > dense
+    K.kfl_stage_destroy(st)
+    assert dev.fake_live() == 0
