@@ -697,10 +697,7 @@ int upload_phases(kfl_stage *st, int batch) {
   if (st->phases_dev[batch]) return KFL_OK;
   const std::vector<Phase> phases = build_phases(st, batch, true);
   void *d = nullptr;
-  if (cudaMalloc(&d, phases.size() * sizeof(Phase)) != cudaSuccess) {
-    cudaGetLastError();
-    return KFL_ERR_OOM;
-  }
+  if (!device_alloc(&d, phases.size() * sizeof(Phase))) return KFL_ERR_OOM;
   st->phases_dev[batch] = static_cast<Phase *>(d);
   st->n_phases = (int)phases.size();
   CK(cudaMemcpy(d, phases.data(), phases.size() * sizeof(Phase), cudaMemcpyHostToDevice));
@@ -918,9 +915,9 @@ int ensure_prefill(kfl_stage *st, int tokens) {
     // each resource is made once (a call that failed part way keeps what it made, and the next
     // call completes the set; kfl_stage_destroy frees them)
     for (int b = 0; b < 2; ++b) {
-      if (!st->pf_w16[b] && cudaMalloc((void **)&st->pf_w16[b], most) != cudaSuccess) {
-        cudaGetLastError();
+      if (!st->pf_w16[b] && !device_alloc((void **)&st->pf_w16[b], most)) {
         st->pf_w16[b] = nullptr;
+        if (b == 1) cudaFree(st->pf_w16[0]), st->pf_w16[0] = nullptr;
         return KFL_ERR_OOM;
       }
       if ((!st->pf_deq[b] && cudaEventCreateWithFlags(&st->pf_deq[b], cudaEventDisableTiming) != cudaSuccess) ||
@@ -1240,10 +1237,7 @@ int to_device(kfl_stage *st, const void *src, size_t bytes, int on_device, void 
     return KFL_OK;
   }
   void *d = nullptr;
-  if (cudaMalloc(&d, bytes ? bytes : 16) != cudaSuccess) {
-    cudaGetLastError();
-    return KFL_ERR_OOM;
-  }
+  if (!device_alloc(&d, bytes ? bytes : 16)) return KFL_ERR_OOM;
   tmp.push_back(d);
   CK(cudaMemcpy(d, src, bytes, cudaMemcpyHostToDevice));
   *out = d;
@@ -1280,16 +1274,10 @@ int load_matrix(kfl_stage *st, Mat &m, const std::vector<std::pair<const kfl_mat
     wcat = const_cast<void *>(parts[0].first->w);
     scat = const_cast<void *>(parts[0].first->scales);
   } else {
-    if (cudaMalloc(&wcat, n_src * row_w) != cudaSuccess) {
-      cudaGetLastError();
-      return KFL_ERR_OOM;
-    }
+    if (!device_alloc(&wcat, n_src * row_w)) return KFL_ERR_OOM;
     tmp.push_back(wcat);
     if (!bf) {
-      if (cudaMalloc(&scat, n_src * row_s) != cudaSuccess) {
-        cudaGetLastError();
-        return KFL_ERR_OOM;
-      }
+      if (!device_alloc(&scat, n_src * row_s)) return KFL_ERR_OOM;
       tmp.push_back(scat);
     }
     size_t off = 0;
@@ -1303,10 +1291,7 @@ int load_matrix(kfl_stage *st, Mat &m, const std::vector<std::pair<const kfl_mat
   }
   int *dmap = nullptr;
   if (!row_map.empty()) {
-    if (cudaMalloc(&dmap, row_map.size() * sizeof(int)) != cudaSuccess) {
-      cudaGetLastError();
-      return KFL_ERR_OOM;
-    }
+    if (!device_alloc((void **)&dmap, row_map.size() * sizeof(int))) return KFL_ERR_OOM;
     tmp.push_back(dmap);
     CK(cudaMemcpy(dmap, row_map.data(), row_map.size() * sizeof(int), cudaMemcpyHostToDevice));
   }

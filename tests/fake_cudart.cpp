@@ -25,7 +25,7 @@ std::set<void *> g_pool_blocks;
 std::map<const void *, std::string> g_names;                    // host function -> kernel name
 std::map<std::string, long> g_launches;
 std::map<std::pair<const void *, int>, size_t> g_optin;         // (function, device) -> shared memory
-size_t g_live = 0, g_budget = ~size_t(0);
+size_t g_live = 0, g_peak = 0, g_budget = ~size_t(0);
 size_t g_pool_used = 0, g_pool_held = 0, g_pool_keep = 0;       // of the one pool: blocks out, memory reserved
 long g_mallocs = 0, g_fail_optin = 0;
 bool g_capturing = false;
@@ -57,6 +57,11 @@ extern "C" {
 // ---- what the tests set and read
 void fake_budget(size_t bytes) { g_budget = bytes; }
 size_t fake_live() { return g_live; }
+size_t fake_peak() {  // the most that was live since the last call
+  const size_t peak = g_peak;
+  g_peak = g_live;
+  return peak;
+}
 long fake_mallocs() { return g_mallocs; }
 void fake_mark() {
   for (auto &b : g_blocks) b.second.marked = true;
@@ -160,6 +165,7 @@ cudaError_t cudaMalloc(void **p, size_t bytes) {
   std::memset(*p, 0, bytes < (1u << 22) ? bytes : (1u << 22));
   g_blocks[*p] = {bytes, false};
   g_live += bytes;
+  if (g_live > g_peak) g_peak = g_live;
   return cudaSuccess;
 }
 cudaError_t cudaFree(void *p) {

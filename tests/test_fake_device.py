@@ -41,21 +41,25 @@ def dev(fake_lib, tmp_path, monkeypatch):
     monkeypatch.setattr(K, "_lib", None)
     monkeypatch.delenv("KFL_PREFILL_DENSE_MIN", raising=False)
     lib = K.lib()
-    lib.fake_live.restype = lib.fake_pool_held.restype = C.c_size_t
+    lib.fake_live.restype = lib.fake_peak.restype = lib.fake_pool_held.restype = C.c_size_t
     lib.fake_launches.restype = lib.fake_mallocs.restype = lib.fake_marked.restype = C.c_long
     lib.fake_budget.argtypes = [C.c_size_t]
     return lib
 
 
-def _stage(model, max_batch=1):
+def _load(st, model):
     d, hd, kv, f = model.d_model, model.head_dim, model.n_kv_heads * model.head_dim, model.ffn
     w = {n: np.zeros(m, dtype=np.uint16) for n, m in (("attn_norm", d), ("ffn_norm", d), ("q_norm", hd), ("k_norm", hd))}
     for n, rows, cols in (("wq", model.n_heads * hd, d), ("wk", kv, d), ("wv", kv, d), ("wo", d, model.n_heads * hd),
                           ("wg", f, d), ("wu", f, d), ("wd", d, f)):
         w[n] = (np.zeros((rows, cols), dtype=np.uint16) if model.weight_fmt == "bf16" else
                 (np.zeros((rows, cols // 8), dtype=np.uint32), np.zeros((rows, cols // 64), dtype=np.uint16)))
-    st = K.kfl_stage_create(K.model_cfg(model, 4096, max_batch), 0, 1, 0)
     K.kfl_stage_load_layer(st, 0, w, on_device=False)
+
+
+def _stage(model, max_batch=1):
+    st = K.kfl_stage_create(K.model_cfg(model, 4096, max_batch), 0, 1, 0)
+    _load(st, model)
     return st
 
 
@@ -149,3 +153,20 @@ def test_no_memory_for_a_larger_workspace(dev, model, captured):
     assert _prefill(st, 1500) == 0 and dev.fake_launches(kernel) > dense
     K.kfl_stage_destroy(st)
     assert dev.fake_live() == 0
+
+
+@pytest.mark.parametrize("call", ["load", "long prompt"])
+def test_memory_kept_by_the_product_is_given_back(dev, call):
+    """What kfl_matmul_bf16w's pool keeps stands in no other allocation's way: host weights' copies while they
+    load, the fp16 copies of an int4 stage's long prompts."""
+    model = dataclasses.replace(WIDE, weight_fmt="int4_g64")
+    for known in (False, True):
+        st = _stage(model)
+        run = {"load": lambda: _load(st, model), "long prompt": lambda: _prefill(st, 600)}[call]
+        if known:
+            assert _matmul(2048, 8192, 8192) == 0 and dev.fake_pool_held() >= 32 << 20
+            dev.fake_budget(peak)
+        dev.fake_peak()
+        assert not run()
+        peak = dev.fake_peak()
+        K.kfl_stage_destroy(st)
