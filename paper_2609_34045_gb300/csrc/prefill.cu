@@ -1262,6 +1262,7 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
   float *partial = reinterpret_cast<float *>(xlo + (size_t)rows * ld);
   unsigned *err = reinterpret_cast<unsigned *>(reinterpret_cast<uint8_t *>(partial) + ws_bytes);
   int rc = KFL_OK;
+  unsigned h_err = 0;
   CUtensorMap mh, ml, mb;
   if (!w_rows) tile_rows_kernel<<<(unsigned)n_rb * n_kt, 256, 0, s>>>(w, N, K, n_kt, tiles);
   if (cudaPeekAtLastError() != cudaSuccess ||
@@ -1279,18 +1280,15 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
     e.out = y;
     e.ldo = ldy;
     e.err = err;
-    unsigned h_err = 0;
     const NarrowWorkspace ws = {partial, n_sm};
     const cudaError_t ce = narrow ? launch_prefill_narrow(PE_STORE, mb, w_rows, mh, K, 2, ws, e, s)
                                   : launch_prefill_gemm(PE_STORE, mh, ml, mb, w_rows, K, ws, e, s);
-    if (ce != cudaSuccess || cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      rc = KFL_ERR_CUDA;
-    else if (h_err & ERR_TIMEOUT)
-      rc = KFL_ERR_TIMEOUT;
+    if (ce != cudaSuccess || cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess) rc = KFL_ERR_CUDA;
   }
+  // freed before the synchronisation: there the pool returns what it holds beyond its threshold
   cudaFreeAsync(mem, s);
-  if (rc != KFL_OK) cudaStreamSynchronize(s);
+  if (cudaStreamSynchronize(s) != cudaSuccess && rc == KFL_OK) rc = KFL_ERR_CUDA;
+  if (rc == KFL_OK && (h_err & ERR_TIMEOUT)) rc = KFL_ERR_TIMEOUT;
   cudaGetLastError();
   return rc;
 }

@@ -170,3 +170,11 @@ def test_memory_kept_by_the_product_is_given_back(dev, call):
         assert not run()
         peak = dev.fake_peak()
         K.kfl_stage_destroy(st)
+
+
+@pytest.mark.parametrize("T,k,n", [(300, 8191, 8191), (40, 8191, 8191), (40, 64, 64)])
+def test_the_product_keeps_no_more_than_its_threshold(dev, T, k, n):
+    """Of its temporary buffers (here up to 134 MB of weight tiles) the call leaves the pool 64 MiB."""
+    for _ in range(2):
+        assert _matmul(T, k, n) == 0
+        assert dev.fake_pool_held() <= 64 << 20
