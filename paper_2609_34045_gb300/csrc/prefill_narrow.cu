@@ -29,7 +29,10 @@ constexpr int NW_WARPS = 10;             // TMA, MMA, 8 epilogue warps
 constexpr int NW_THREADS = NW_WARPS * 32;
 constexpr int NW_EPI_THREADS = 256;
 constexpr int NW_DRAIN_TP = 80;          // tokens of a tile of three terms
-constexpr int NW_DRAIN_KB = 2;           // K blocks per drained accumulator
+constexpr int NW_DRAIN_KB = 2;           // K blocks per drained accumulator of three-term passes
+constexpr int NW_PRODUCT_KB = 16;        // and of the plain product's two terms
+// the most tokens of a drained tile
+__host__ __device__ constexpr int narrow_drain_tp(int mode) { return mode == PE_STORE ? NW_MAX_TP : NW_DRAIN_TP; }
 constexpr int NW_EPI_WARP = 2;            // the first epilogue warp
 constexpr int NW_MAX_STAGES = 12;
 constexpr int NW_RING = 226 * 1024;      // shared memory of the rings: a block's 227 KiB less the barriers' KiB
@@ -222,7 +225,7 @@ __device__ __forceinline__ void narrow_epilogue_warps(const NarrowParams &p, con
       }
     };
     if constexpr (DRAIN) {
-      constexpr int OWN = (NW_DRAIN_TP / 16 + 1) / 2;  // groups of this warp
+      constexpr int OWN = (narrow_drain_tp(MODE) / 16 + 1) / 2;  // groups of this warp
       float sum[OWN][16] = {};
       for (int left = w.kb1 - w.kb0; left > 0; left -= p.chunk) {
         if (!wait_acc()) return;
@@ -902,11 +905,13 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, c
   p.tp = narrow_tp(ep.T, terms);
   p.t_tiles = (ep.T + p.tp - 1) / p.tp;
   const int cols = p.tp * terms;
+  // Q/K/V (and its plain form): K and V are rounded to bf16 next, and every error before that moves some
+  // across a rounding
+  p.chunk = terms == 2 ? NW_PRODUCT_KB : mode == PE_QKV || mode == PE_STORE ? 1 : NW_DRAIN_KB;
   // wide tiles of many rows share their tokens' slices between two 128-row blocks: the slices (2 x
   // 16 KiB of terms at 128 tokens) then cost no more L2 reads than the weights
-  // Q/K/V: K and V are rounded to bf16 next, and every error before that moves some across a rounding
-  p.chunk = mode == PE_QKV || mode == PE_STORE ? 1 : NW_DRAIN_KB;
-  const int mb = terms == 2 && cols > 128 && (ep.N + 255) / 256 * p.t_tiles >= ws.n_sm * 3 / 4 ? 2 : 1;
+  const bool drain = terms == 3 || mode == PE_STORE;
+  const int mb = !drain && cols > 128 && (ep.N + 255) / 256 * p.t_tiles >= ws.n_sm * 3 / 4 ? 2 : 1;
   const int n_kb = (K + 63) / 64, n_tiles = (ep.N + 128 * mb - 1) / (128 * mb) * p.t_tiles;
   p.acc_cols = (cols + 31) / 32 * 32;
   p.bufs = 2 * mb * p.acc_cols <= 512 ? 2 : 1;
@@ -921,9 +926,12 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, c
   p.share = share_tiles(n_tiles, n_kb, grid, p.t_tiles == 1, NW_PARTS);
   auto go = [&](auto m) {
     constexpr int MODE = decltype(m)::value;
-    if (terms == 3) return launch_narrow_mode<MODE, 1, true>(w, x, p, grid, ep, s, pending);
-    return mb == 2 ? launch_narrow_mode<MODE, 2, false>(w, x, p, grid, ep, s, pending)
-                   : launch_narrow_mode<MODE, 1, false>(w, x, p, grid, ep, s, pending);
+    if constexpr (MODE != PE_STORE) {
+      if (!drain)
+        return mb == 2 ? launch_narrow_mode<MODE, 2, false>(w, x, p, grid, ep, s, pending)
+                       : launch_narrow_mode<MODE, 1, false>(w, x, p, grid, ep, s, pending);
+    }
+    return launch_narrow_mode<MODE, 1, true>(w, x, p, grid, ep, s, pending);
   };
   switch (mode) {
     case PE_STORE: return go(std::integral_constant<int, PE_STORE>());

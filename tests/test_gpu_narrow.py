@@ -50,6 +50,22 @@ def test_product_matches_fp64(T, Kd, N):
     assert np.all(got[:, N:] == 7.0)
 
 
+@pytest.mark.parametrize("T", [1, 64, 128, 129])
+def test_product_error_of_a_long_k(T):
+    """Both forms of the plain product at K = 18944: x's two terms leave 2^-18 of it (rms 2e-6), and the sums
+    are fp32 ones, so 1e-5 of the result (2-norm).  Left in the tensor core's accumulator, which truncates
+    (3e-8 per 16 products), they were up to 3.5e-5 off."""
+    k = n = 18944
+    g = torch.Generator(device="cuda").manual_seed(T)
+    x = torch.randn((T, k), generator=g, device="cuda")
+    w = torch.randn((n, k), generator=g, device="cuda", dtype=torch.bfloat16).mul_(0.02)
+    y = torch.zeros((T, n), device="cuda")
+    K.kfl_matmul_bf16w(x, T, k, k, w.view(torch.int16), n, y, n, torch.cuda.current_stream().cuda_stream)
+    ref = torch.cat([x.double() @ w[r:r + 2048].double().t() for r in range(0, n, 2048)], dim=1)
+    err = float((y.double() - ref).norm() / ref.norm())
+    assert err <= 1e-5, err
+
+
 @pytest.mark.parametrize("model,n", [(RAGGED, 16), (RAGGED, 65), (RAGGED, 128), (RAGGED128, 33),
                                      (dataclasses.replace(RAGGED, vocab=30000), 70), (RAGGED_INT4, 16),
                                      (RAGGED_INT4, 65), (RAGGED_INT4, 100), (RAGGED_INT4, 129)])
