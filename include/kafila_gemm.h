@@ -29,10 +29,10 @@ extern "C" {
  *   w  device bf16 [N][K] row-major (the nn.Linear convention); read only
  *   y  device fp32 [T][ldy], ldy >= N and a multiple of 4, 16-byte aligned; columns >= N untouched
  * Rows that TMA can address (K a multiple of 8, w 16-byte aligned) are read where they are; others are
- * copied into the decode path's tile layout first, and x into its two terms.  The temporaries come
- * from a memory pool of the device that keeps up to 64 MiB between calls.  Synchronous on cuda_stream.  Errors: KFL_ERR_ARG (sizes,
- * strides, alignment, NULL pointers), KFL_ERR_OOM, KFL_ERR_CUDA, KFL_ERR_TIMEOUT (a bounded wait
- * of the kernel's pipeline gave up). */
+ * copied into the decode path's tile layout first, some hundred MiB at a time, and x into its two terms.
+ * The temporaries come from a memory pool of the device that keeps up to 512 MiB between calls (a stage's
+ * allocations take it back); more than that is allocated by the call.  Synchronous on cuda_stream.  Errors: KFL_ERR_ARG (sizes, strides, alignment, NULL
+ * pointers), KFL_ERR_OOM, KFL_ERR_CUDA, KFL_ERR_TIMEOUT (a bounded wait of the kernel's pipeline gave up). */
 int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uint16_t *w, int N, float *y, int ldy,
                      void *cuda_stream);
 

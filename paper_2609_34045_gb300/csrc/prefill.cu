@@ -1191,9 +1191,12 @@ namespace {
 
 // The device's memory pool for kfl_matmul_bf16w's temporary buffers, made at its first call there.  Of
 // what the calls free, the pool keeps up to MATMUL_KEEP_BYTES for the next and returns the rest at
-// their synchronisation; a cudaMalloc and cudaFree per call cost 80 to 250 us.  Calls on several
-// threads and streams each take buffers of their own from it.
-constexpr uint64_t MATMUL_KEEP_BYTES = 64ull << 20;
+// their synchronisation.  A cudaMalloc and cudaFree per call cost 80 to 250 us, and what the pool has to
+// return at once costs more (613 MB: 1.2 ms of a 1.8 ms call), so that buffers beyond its bound, which only
+// more than some 4000 tokens of a K of 18944 need, are allocated by themselves.
+// Calls on several threads and streams each take buffers of their own from it.
+constexpr uint64_t MATMUL_KEEP_BYTES = 512ull << 20;
+constexpr uint64_t MATMUL_SLAB_BYTES = 128ull << 20;  // a copy of weight tiles may always have this much
 constexpr int MATMUL_MAX_DEVICES = 64;
 std::mutex g_pool_mutex;
 cudaMemPool_t g_pool[MATMUL_MAX_DEVICES] = {};
@@ -1222,12 +1225,20 @@ cudaMemPool_t matmul_pool(int dev) {
 }  // namespace
 
 namespace kfl {
-// Returns what the current device's pool keeps (a stage that finds no memory asks for it).
-bool release_matmul_pool() {
+// Returns what the current device's pool keeps.
+static bool release_matmul_pool() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MATMUL_MAX_DEVICES) return false;
   std::lock_guard<std::mutex> lock(g_pool_mutex);
   return g_pool[dev] && cudaMemPoolTrimTo(g_pool[dev], 0) == cudaSuccess;
+}
+
+bool device_alloc(void **p, size_t bytes) {
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  if (release_matmul_pool() && cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
 }
 }  // namespace kfl
 
@@ -1238,7 +1249,7 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
       (reinterpret_cast<uintptr_t>(y) & 15) != 0)
     return KFL_ERR_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  const int n_rb = (N + RB - 1) / RB, n_kt = (K + KT - 1) / KT, ld = (K + 63) / 64 * 64;
+  const int n_kt = (K + KT - 1) / KT, ld = (K + 63) / 64 * 64;
   int dev = 0, n_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
@@ -1248,12 +1259,24 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
   // (K not a multiple of 8, or an unaligned start) are copied into weight tiles first
   const bool narrow = T <= NW_MAX_TP, w_rows = K % 8 == 0 && (reinterpret_cast<uintptr_t>(w) & 15) == 0;
   const int rows = (T + 7) / 8 * 8;
-  const size_t tile_bytes = w_rows ? 0 : (size_t)n_rb * n_kt * TILE_BYTES, x_bytes = (size_t)rows * ld * 2;
-  const size_t ws_bytes = narrow_ws_bytes(n_sm, T);
-  cudaMemPool_t pool = matmul_pool(dev);
+  const size_t x_bytes = (size_t)rows * ld * 2, ws_bytes = narrow_ws_bytes(n_sm, T), fixed = 2 * x_bytes + ws_bytes + 16;
+  // a copied matrix goes a slab of rows at a time through what the pool may keep
+  int slab = N;
+  if (!w_rows) {
+    const size_t room = fixed + MATMUL_SLAB_BYTES <= MATMUL_KEEP_BYTES ? MATMUL_KEEP_BYTES - fixed : MATMUL_SLAB_BYTES;
+    const size_t most = std::max<size_t>(room / ((size_t)n_kt * KT * 2) / PG_N, 1) * PG_N;
+    slab = (int)std::min<size_t>(N, most);
+  }
+  const size_t tile_bytes = w_rows ? 0 : (size_t)((slab + RB - 1) / RB) * n_kt * TILE_BYTES, bytes = tile_bytes + fixed;
+  const bool pooled = bytes <= MATMUL_KEEP_BYTES;
   void *mem = nullptr;
-  if (!pool || cudaMallocFromPoolAsync(&mem, tile_bytes + 2 * x_bytes + ws_bytes + 16, pool, s) != cudaSuccess) {
-    cudaGetLastError();
+  if (pooled) {
+    cudaMemPool_t pool = matmul_pool(dev);
+    if (!pool || cudaMallocFromPoolAsync(&mem, bytes, pool, s) != cudaSuccess) {
+      cudaGetLastError();
+      return KFL_ERR_OOM;
+    }
+  } else if (!device_alloc(&mem, bytes)) {
     return KFL_ERR_OOM;
   }
   uint8_t *tiles = static_cast<uint8_t *>(mem);
@@ -1264,30 +1287,37 @@ extern "C" int kfl_matmul_bf16w(const float *x, int T, int K, int ldx, const uin
   int rc = KFL_OK;
   unsigned h_err = 0;
   CUtensorMap mh, ml, mb;
-  if (!w_rows) tile_rows_kernel<<<(unsigned)n_rb * n_kt, 256, 0, s>>>(w, N, K, n_kt, tiles);
-  if (cudaPeekAtLastError() != cudaSuccess ||
-      launch_split_bf16(x, T, K, ldx, xhi, xlo, ld, err, s) != cudaSuccess) {
+  if (narrow ? encode_terms_map(&mh, xhi, K, T, ld, 2, (size_t)rows * ld, narrow_tp(T, 2))
+             : encode_act_map(&mh, xhi, K, T, ld) || encode_act_map(&ml, xlo, K, T, ld))
     rc = KFL_ERR_CUDA;
-  } else if ((narrow ? encode_terms_map(&mh, xhi, K, T, ld, 2, (size_t)rows * ld, narrow_tp(T, 2))
-                     : encode_act_map(&mh, xhi, K, T, ld) || encode_act_map(&ml, xlo, K, T, ld)) ||
-             (w_rows ? encode_rows_map(&mb, w, K, N, narrow ? 128 : PG_N)
-                     : encode_tiles_map(&mb, tiles, n_kt, n_rb, (narrow ? 128 : PG_N) / RB))) {
-    rc = KFL_ERR_CUDA;
-  } else {
+  for (int n0 = 0; n0 < N && rc == KFL_OK; n0 += slab) {
     PrefillEpiParams e = {};
     e.T = T;
-    e.N = N;
-    e.out = y;
+    e.N = std::min(slab, N - n0);
+    e.out = y + n0;
     e.ldo = ldy;
     e.err = err;
+    const int n_rb = (e.N + RB - 1) / RB;
+    // (these two are launched when all before them is done, and so is what follows a slab's copy: the
+    // few-token kernel reads weights before it waits for the kernel before it)
+    if (!w_rows) tile_rows_kernel<<<(unsigned)n_rb * n_kt, 256, 0, s>>>(w + (size_t)n0 * K, e.N, K, n_kt, tiles);
+    if (cudaPeekAtLastError() != cudaSuccess ||
+        (n0 == 0 && launch_split_bf16(x, T, K, ldx, xhi, xlo, ld, err, s) != cudaSuccess) ||
+        (w_rows ? encode_rows_map(&mb, w, K, N, narrow ? 128 : PG_N)
+                : encode_tiles_map(&mb, tiles, n_kt, n_rb, (narrow ? 128 : PG_N) / RB))) {
+      rc = KFL_ERR_CUDA;
+      break;
+    }
     const NarrowWorkspace ws = {partial, n_sm};
-    const cudaError_t ce = narrow ? launch_prefill_narrow(PE_STORE, mb, w_rows, mh, K, 2, ws, e, s)
-                                  : launch_prefill_gemm(PE_STORE, mh, ml, mb, w_rows, K, ws, e, s);
-    if (ce != cudaSuccess || cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess) rc = KFL_ERR_CUDA;
+    if ((narrow ? launch_prefill_narrow(PE_STORE, mb, w_rows, mh, K, 2, ws, e, s, nullptr, n0 == 0)
+                : launch_prefill_gemm(PE_STORE, mh, ml, mb, w_rows, K, ws, e, s)) != cudaSuccess)
+      rc = KFL_ERR_CUDA;
   }
+  if (rc == KFL_OK && cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess) rc = KFL_ERR_CUDA;
   // freed before the synchronisation: there the pool returns what it holds beyond its threshold
-  cudaFreeAsync(mem, s);
+  if (pooled) cudaFreeAsync(mem, s);
   if (cudaStreamSynchronize(s) != cudaSuccess && rc == KFL_OK) rc = KFL_ERR_CUDA;
+  if (!pooled) cudaFree(mem);
   if (rc == KFL_OK && (h_err & ERR_TIMEOUT)) rc = KFL_ERR_TIMEOUT;
   cudaGetLastError();
   return rc;

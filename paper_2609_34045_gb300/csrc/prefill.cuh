@@ -104,10 +104,11 @@ size_t narrow_ws_bytes(int n_sm, int T);  // for passes of up to T tokens
 int narrow_argmax_slots(int N);  // PE_ARGMAX: partial maxima per token (n_tiles of PrefillEpiParams)
 int narrow_tp(int T, int terms);  // tokens of a tile
 // w: encode_tiles_map with 2 row blocks per box, or (w_rows) encode_rows_map with 128 rows; x:
-// encode_terms_map with narrow_tp rows per box.
+// encode_terms_map with narrow_tp rows per box.  early: w was written by nothing later than the kernel
+// before the last, so that the kernel may read it before it waits for the last.
 cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, const CUtensorMap &x, int K, int terms,
                                   const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s,
-                                  NarrowPending *pending = nullptr);
+                                  NarrowPending *pending = nullptr, bool early = true);
 // The same over int4 tiles [n_rb][n_kt][TILE4_BYTES], decoded in the kernel (fp16 terms).
 cudaError_t launch_prefill_narrow4(int mode, const uint8_t *tiles, int n_rb, int n_kt, const CUtensorMap &x, int K,
                                    int terms, const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s,
@@ -119,6 +120,8 @@ cudaError_t launch_narrow_norm(const NarrowPending &pend, float *h, int ldh, int
                                cudaStream_t s);
 
 // Host side (prefill.cu).
+// cudaMalloc, once more without what kfl_matmul_bf16w keeps if there is no memory.
+bool device_alloc(void **p, size_t bytes);
 int encode_act_map(CUtensorMap *map, const uint16_t *base, int K, int rows, int ld);
 // The terms of activation rows [term][rows][K] (row stride ld, term stride term_stride elements):
 // boxes of 64 columns x box_rows rows x every term.

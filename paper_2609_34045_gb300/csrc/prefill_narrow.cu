@@ -872,7 +872,7 @@ static cudaError_t launch_narrow_reduce(const NarrowParams &p, int mb, int grid,
 
 template <int MODE, int MB, bool DRAIN>
 static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x, const NarrowParams &p, int grid,
-                                      const PrefillEpiParams &ep, cudaStream_t s, NarrowPending *pending) {
+                                      const PrefillEpiParams &ep, cudaStream_t s, NarrowPending *pending, bool early) {
   static RingOptIn opt_in;
   const int smem = opt_in(reinterpret_cast<const void *>(prefill_narrow_kernel<MODE, MB, DRAIN>));
   if (smem < 0) return cudaErrorInvalidValue;
@@ -884,7 +884,7 @@ static cudaError_t launch_narrow_mode(const CUtensorMap &w, const CUtensorMap &x
   cudaLaunchAttribute attr[1];
   pdl_attribute(attr[0]);
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_narrow_kernel<MODE, MB, DRAIN>, w, x, p, ep);
   return e == cudaSuccess ? launch_narrow_reduce<MODE>(p, MB, grid, ep, s, pending) : e;
 }
@@ -897,7 +897,7 @@ int narrow_tp(int T, int terms) {
 
 cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, const CUtensorMap &x, int K, int terms,
                                   const NarrowWorkspace &ws, const PrefillEpiParams &ep, cudaStream_t s,
-                                  NarrowPending *pending) {
+                                  NarrowPending *pending, bool early) {
   if (ep.T <= 0 || ep.N <= 0) return cudaSuccess;
   NarrowParams p = {};
   p.w_rows = w_rows;
@@ -928,10 +928,10 @@ cudaError_t launch_prefill_narrow(int mode, const CUtensorMap &w, bool w_rows, c
     constexpr int MODE = decltype(m)::value;
     if constexpr (MODE != PE_STORE) {
       if (!drain)
-        return mb == 2 ? launch_narrow_mode<MODE, 2, false>(w, x, p, grid, ep, s, pending)
-                       : launch_narrow_mode<MODE, 1, false>(w, x, p, grid, ep, s, pending);
+        return mb == 2 ? launch_narrow_mode<MODE, 2, false>(w, x, p, grid, ep, s, pending, early)
+                       : launch_narrow_mode<MODE, 1, false>(w, x, p, grid, ep, s, pending, early);
     }
-    return launch_narrow_mode<MODE, 1, true>(w, x, p, grid, ep, s, pending);
+    return launch_narrow_mode<MODE, 1, true>(w, x, p, grid, ep, s, pending, early);
   };
   switch (mode) {
     case PE_STORE: return go(std::integral_constant<int, PE_STORE>());

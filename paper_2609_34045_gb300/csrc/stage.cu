@@ -212,21 +212,6 @@ void make_plan(const kfl_model_cfg *c, int l0, int l1, int flags, int n_sm, Plan
 
 }  // namespace
 
-namespace kfl {
-bool release_matmul_pool();  // prefill.cu
-}
-
-namespace {
-// cudaMalloc, once more without what kfl_matmul_bf16w keeps if there is no memory.
-bool device_alloc(void **p, size_t bytes) {
-  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
-  cudaGetLastError();
-  if (release_matmul_pool() && cudaMalloc(p, bytes) == cudaSuccess) return true;
-  cudaGetLastError();
-  return false;
-}
-}  // namespace
-
 // The workspace of one dense prefill pass of up to `cap` tokens.
 struct PrefillWorkspace {
   int cap = 0;
