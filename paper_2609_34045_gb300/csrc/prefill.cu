@@ -177,9 +177,23 @@ __device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t da, uint64_t db,
 // DRAIN (the plain product): each accumulator takes only PP_CHUNK K blocks, and eight epilogue warps add
 // the chunks up in registers: tensor-core accumulation truncates (prefill_narrow_kernel says how
 // much), and an unsplit K of 18944 leaves the product of 2048 tokens 3.8e-5 off, drained 3.3e-6.  A
-// stage's products go without: attention's bf16 softmax weights leave 1e-3 at these lengths, and
-// the sums' registers cost the fused epilogues spills.
-constexpr int PP_CHUNK = 16;
+// stage's products, of K = d_model mostly, go without: the sums' registers cost the fused epilogues
+// spills.
+//
+// A residual product takes a long K in equal chunks of at most PR_CHUNK K blocks (K = 4096: truncation
+// takes 8e-6 at most) and adds each to the residual stream, or to its partial sums, while the next
+// multiplies.  Unchunked, a whole tile of K = 18944 or 29568 lost 3.8e-5 or 5.9e-5.  Every chunk reads and writes
+// the tile once more: four 7B-shaped blocks of 2048 tokens take 5215 us for 5120 (chunks of 148: 5150, and
+// 1.9e-5), two 72B-shaped int4 ones of 900 tokens 5060 for 4960.
+constexpr int PP_CHUNK = 16, PR_CHUNK = 64;
+// K blocks of one accumulation of a segment of n.
+template <int MODE>
+__device__ __forceinline__ int pp_chunk(int n) {
+  if (MODE == PE_STORE) return PP_CHUNK;
+  if (MODE != PE_RESID || n <= PR_CHUNK) return n;
+  const int parts = (n + PR_CHUNK - 1) / PR_CHUNK;
+  return (n + parts - 1) / parts;
+}
 __host__ __device__ constexpr int pp_epi_warps(bool drain) { return drain ? 8 : 4; }
 __host__ __device__ constexpr int pp_threads(bool drain) { return (2 + pp_epi_warps(drain)) * 32; }
 constexpr int PP_TMEM_COLS = 2 * PG_N;
@@ -262,19 +276,20 @@ __global__ void __launch_bounds__(pp_threads(DRAIN), 1)
       }
     }
   } else if (warp == 1) {
-    // ---- MMA issuer (the whole warp, one elected lane issuing): segment i of this CTA (DRAIN:
-    // chunk i of its segments) accumulates into TMEM columns (i % 2) * PG_N
+    // ---- MMA issuer (the whole warp, one elected lane issuing): chunk i of this CTA's segments
+    // accumulates into TMEM columns (i % 2) * PG_N
     const uint32_t idesc = ep.f16 ? idesc_kind_f16(PG_M, PG_N, false) : idesc_kind_f16(PG_M, PG_N, true);
     TileWalk w(share);
-    int s = 0, left = 0;
+    int s = 0, left = 0, chunk = 0;
     uint32_t use = 0;
     bool ok = true;
     for (int i = 0; ok; ++i) {
       if (left == 0) {
         if (!w.next()) break;
         left = w.kb1 - w.kb0;
+        chunk = pp_chunk<MODE>(left);
       }
-      const int n = DRAIN ? min(left, PP_CHUNK) : left, buf = i & 1;
+      const int n = min(left, chunk), buf = i & 1;
       left -= n;
       if (i >= 2) ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&s_acc_empty[buf]), ((i >> 1) - 1) & 1));
       if (!ok) break;
@@ -329,15 +344,22 @@ __global__ void __launch_bounds__(pp_threads(DRAIN), 1)
       const int n_tile = w.tile / t_tiles, t = (w.tile % t_tiles) * PG_M + row, n0 = n_tile * PG_N;
       const bool whole = w.whole();
       EpiState<MODE> st;
-      auto finish = [&](int c, const uint32_t(&r)[32]) {
+      // `more`: a further chunk of the same sums
+      auto finish = [&](int c, const uint32_t(&r)[32], bool more = false) {
         if (whole) {
           if (t < ep.T) epilogue32<MODE>(ep, t, n0 + 32 * c, r, st);
         } else {
           float4 *at = reinterpret_cast<float4 *>(ws) + wide_partial(w.part, 8 * c) + row;
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            at[j * PG_M] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                       __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
+          for (int j = 0; j < 8; ++j) {
+            float4 y = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                                   __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
+            if constexpr (MODE == PE_RESID) {
+              const float4 x = more ? at[j * PG_M] : make_float4(0.f, 0.f, 0.f, 0.f);
+              y = make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
+            }
+            at[j * PG_M] = y;
+          }
         }
       };
       if constexpr (DRAIN) {
@@ -365,20 +387,24 @@ __global__ void __launch_bounds__(pp_threads(DRAIN), 1)
         for (int c = 0; c < 4; ++c)
           if (n0 + 32 * (c0 + c) < ep.N) finish(c0 + c, sum[c]);  // uniform across the warp
       } else {
-        if (!(ok = wait_acc())) break;
-        for (int c = 0; c < PG_N / 32; ++c) {
-          if (n0 + 32 * c >= ep.N) break;  // uniform across the warp
-          uint32_t r[32];
-          tmem_ld32(lanes + (uint32_t)((i & 1) * PG_N + 32 * c), r);
-          finish(c, r);
+        const int chunk = pp_chunk<MODE>(w.kb1 - w.kb0);
+        for (int left = w.kb1 - w.kb0, done = 0; left > 0; left -= chunk, ++done) {
+          if (!(ok = wait_acc())) break;
+          for (int c = 0; c < PG_N / 32; ++c) {
+            if (n0 + 32 * c >= ep.N) break;  // uniform across the warp
+            uint32_t r[32];
+            tmem_ld32(lanes + (uint32_t)((i & 1) * PG_N + 32 * c), r);
+            finish(c, r, done > 0);
+          }
+          release_acc();
         }
+        if (!ok) break;
         if constexpr (MODE == PE_ARGMAX) {
           if (whole && t < ep.T) {
             ep.amax[(size_t)t * ep.n_tiles + n_tile] = st.best;
             ep.aidx[(size_t)t * ep.n_tiles + n_tile] = st.bidx;
           }
         }
-        release_acc();
       }
     }
   }
