@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(PA_THREADS) prefill_attn_kernel(PrefillAttnPar
       float l = 0.f, y[4] = {};
 #pragma unroll
       for (int k = 0; k < PA_MAX_SPLIT; ++k)
-        if (k < n_split && ml[k].x > -INFINITY) {
+        if (k < n_split && ml[k].y != 0.f) {  // (a CTA that saw a key: m stays -inf, l is NaN where all were NaN)
           const float w = exp2f(ml[k].x - m);
           l += ml[k].y * w;
           y[0] += o[k].x * w;

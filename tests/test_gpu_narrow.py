@@ -162,3 +162,21 @@ def test_dense_at_decode_precision(model, n, start, max_batch, monkeypatch):
     rms = np.sqrt(np.mean(steps * steps, axis=1, keepdims=True))
     assert np.all(np.abs(dense - steps) <= 1e-3 * rms)
     p.close()
+
+
+@pytest.mark.parametrize("n", [9, 40])
+def test_nan_keys_reach_the_output(n):
+    """A key block of NaN alone is one CTA's whole share of the split keys: its rows' scores have no largest one,
+    and the merge takes them in all the same."""
+    m = wl.ModelShape(n_layers_total=1, d_model=128, n_heads=2, n_kv_heads=1, head_dim=64, ffn=256, vocab=300)
+    st = K.kfl_stage_create(K.model_cfg(m, 512, 4), 0, 1, 0)
+    K.kfl_stage_load_layer(st, 0, wl.layer_weights(m, 0, 3), on_device=False)
+    k, v = (torch.randn(1, 200, 64, device="cuda").to(torch.bfloat16) for _ in range(2))
+    k[:, 64:128] = float("nan")
+    K.kfl_kv_write(st, 0, 0, k, v, 200, True)
+    out = torch.zeros(n, m.d_model, device="cuda")
+    K.kfl_stage_prefill(st, None, torch.randn(n, m.d_model, device="cuda"),
+                        torch.arange(200, 200 + n, dtype=torch.int32, device="cuda"), 0, n, out, None,
+                        torch.cuda.current_stream().cuda_stream)
+    assert torch.isnan(out).all()
+    K.kfl_stage_destroy(st)
