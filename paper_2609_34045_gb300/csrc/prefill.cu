@@ -870,7 +870,9 @@ __global__ void prefill_input_kernel(const int *ids, const float *hidden_in, con
 // x[t] = h[t] / rms(h[t]) * g as two or three 16-bit terms (term_stride elements apart), one block per
 // token, four elements per thread step (d a multiple of 8; h, g and x rows 16-byte aligned).  Bound
 // by latency: a thread's first RN_V groups of h and g are loaded at once and kept (2048 x 3584:
-// 13.9 us, 4.2 TB/s; 17.8 one group at a time, read twice).
+// 13.9 us, 4.2 TB/s; 17.8 one group at a time, read twice).  A block has no more threads than those
+// groups need, but 64: at d 320, 256 threads with their registers for all four made 2048 tokens' two norms
+// of a block 13 us longer.
 constexpr int RN_V = 4;
 __global__ void prefill_rmsnorm_kernel(const float *h, int ldh, int d, const float *g, float eps, uint16_t *x,
                                        size_t term_stride, int terms, int ldx, int f16, unsigned *err) {
@@ -1186,7 +1188,8 @@ cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const i
 
 cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const float *g, float eps, uint16_t *x,
                                    size_t term_stride, int terms, int ldx, int f16, unsigned *err, cudaStream_t s) {
-  const int threads = d <= 256 * 4 * RN_V ? 256 : d <= 512 * 4 * RN_V ? 512 : 1024;
+  int threads = 64;
+  while (threads < 1024 && threads * 4 * RN_V < d) threads *= 2;
   return launch_pdl(prefill_rmsnorm_kernel, dim3(T), threads, 0, s, h, ldh, d, g, eps, x, term_stride, terms, ldx, f16, err);
 }
 
