@@ -160,8 +160,8 @@ int kfl_stage_decode_users(kfl_stage *st, const int32_t *token_ids, const float 
  * (environment, default 16) the prompt runs densely: passes of up to 2048 tokens through
  * tensor-core matrix products (tcgen05) and causal attention, each activation carried as two
  * 16-bit terms (bf16 with bf16 weights; fp16 with int4 weights, decoded in the products or, for
- * passes of more than 512 tokens, dequantized to fp16 tiles first; the workspace is allocated at
- * the stage's first dense prefill).  bf16 stages run a qk_norm stage's prompts, and prompts that
+ * passes of more than 128 tokens (small models) to 512 (large ones), dequantized to fp16 tiles first; the
+ * workspace is allocated at the stage's first dense prefill).  bf16 stages run a qk_norm stage's prompts, and prompts that
  * are shorter (while KFL_PREFILL_DENSE_MIN is not set) but longer than one step, densely at the
  * decode steps' precision (three bf16 terms per activation).  Other prompts, and those while a
  * capture, trace or profile is on or for which no workspace can be allocated, go as steps of up

@@ -81,7 +81,7 @@ struct PrefillAttnParams {
 // side by side as N, split stream-K over one CTA per SM
 constexpr int NW_MAX_TP = 128;            // tokens of a tile (two terms: 256 MMA columns)
 constexpr int NW_PARTS = 3;               // partial sums per CTA in a GEMM's workspace
-constexpr int N4_MAX_TOKENS = 512;       // int4 stages: passes of up to this many tokens decode in the GEMM
+constexpr int N4_MAX_TOKENS = 512;        // int4 stages: the longest passes that decode in the GEMM
 constexpr int NW_W_BYTES = 128 * 64 * 2;  // a 128-row weight slice of 64 K
 // How a GEMM's output tiles are shared out (share_tiles, TileWalk in prefill_tc.cuh).
 struct TileShare {

@@ -276,6 +276,7 @@ struct kfl_stage {
   // dense prefill: the workspace, allocated at the first dense prefill, and the tensor maps of the weight
   // tiles (per layer: Q/K/V, O, gate/up, down; then lm_head)
   PrefillWorkspace pf;
+  bool pf_no_copies = false;       // int4: there was no memory for the fp16 copies
   int pf_failed = 0;               // tokens of the last workspace there was no memory for (0: none since)
   int pf_amax_cols = 0;
   std::vector<void *> pf_retired;  // workspaces outgrown since a graph captured them: kept until the stage goes
@@ -807,10 +808,14 @@ int pf_ld(int n) { return round_up(n, 64); }
 // tokens x 256 rows (one 7B-shaped block: 240 us at 128 tokens either way, 408 against 465 at 500),
 // unless the model is so small that those tiles, of its largest matrix, leave SMs without one (two
 // blocks of d 512, F 1408: 76 against 102 us at 500 tokens, equal at 2048).  int4: while decoding the
-// weights once per token tile is cheaper than the fp16 copies (72B-shaped block: 785 against 1026
-// us at 256 tokens, 1389 against 1517 at 512, 2014 against 1948 at 700).
+// weights once per token tile is cheaper than the fp16 copies, which depends on how many they are.  One
+// block, decoded in the GEMM against fp16 copies, in us: d 512, F 1408: 114 to 116 at 129 tokens, 136 to
+// 125 at 200; 7B-shaped: 393 to 409 at 300, 504 to 485 at 400; 32B-shaped: 971 to 989 at 512, 1109
+// to 1089 at 600; 72B-shaped: 1685 to 1747 at 600, 2011 to 1974 at 700.
 int pf_narrow_most(const kfl_stage *st) {
-  if (st->cfg.weight_fmt != KFL_BF16) return N4_MAX_TOKENS;
+  if (st->cfg.weight_fmt != KFL_BF16 && st->pf_no_copies) return N4_MAX_TOKENS;
+  if (st->cfg.weight_fmt != KFL_BF16)
+    return (int)std::min<long long>(N4_MAX_TOKENS, NW_MAX_TP + 2LL * st->P.F * st->P.d / 600000);
   const int n_tiles = (2 * st->P.F + PG_N - 1) / PG_N;
   return std::max(NW_MAX_TP, std::min(PF_PASS, (st->P.n_sm - 1) / n_tiles * PG_M));
 }
@@ -833,7 +838,8 @@ void pf_blocks(const kfl_stage *st, int cap, PrefillWorkspace &w, F block) {
   if (st->cfg.qk_norm) block((void **)&w.raw, (size_t)cap * P.ld_raw * 4);
   // argmax partials: per 256-column tile, or (passes on the few-token GEMM) per 32 rows
   if (st->flags & KFL_LOGITS_OUT) {
-    const int narrow = std::min(cap, st->cfg.qk_norm ? PF_PASS : pf_narrow_most(st));
+    const int most = st->cfg.qk_norm ? PF_PASS : st->cfg.weight_fmt == KFL_BF16 ? pf_narrow_most(st) : N4_MAX_TOKENS;
+    const int narrow = std::min(cap, most);
     const size_t am = std::max((size_t)cap * ((P.V + PG_N - 1) / PG_N), (size_t)narrow * narrow_argmax_slots(P.V));
     block((void **)&w.amax, am * 4);
     block((void **)&w.aidx, am * 4);
@@ -903,7 +909,8 @@ int ensure_prefill(kfl_stage *st, int tokens) {
       if (!st->pf_w16[b] && !device_alloc((void **)&st->pf_w16[b], most)) {
         st->pf_w16[b] = nullptr;
         if (b == 1) cudaFree(st->pf_w16[0]), st->pf_w16[0] = nullptr;
-        return KFL_ERR_OOM;
+        st->pf_no_copies = true;  // prompts of up to N4_MAX_TOKENS decode in the products then
+        return pf_narrow(st, first) ? KFL_OK : KFL_ERR_OOM;
       }
       if ((!st->pf_deq[b] && cudaEventCreateWithFlags(&st->pf_deq[b], cudaEventDisableTiming) != cudaSuccess) ||
           (!st->pf_used[b] && cudaEventCreateWithFlags(&st->pf_used[b], cudaEventDisableTiming) != cudaSuccess)) {
@@ -923,6 +930,7 @@ int ensure_prefill(kfl_stage *st, int tokens) {
                              kinds[j]->n_rb, PG_N / RB))
           return KFL_ERR_CUDA;
     st->pf_maps = std::move(maps);
+    st->pf_no_copies = false;
   }
   if (st->pf_maps.empty() && st->cfg.weight_fmt == KFL_BF16) {
     std::vector<CUtensorMap> maps(4 * P.nl + 1), narrow(4 * P.nl + 1);

@@ -181,3 +181,26 @@ def test_the_product_keeps_no_more_than_its_threshold(dev, T, k, n):
         assert dev.fake_pool_held() <= 512 << 20 and dev.fake_live() == 0
     if n > 8192:
         assert dev.fake_launches(b"tile_rows_kernel") > 2
+
+
+@pytest.mark.parametrize("d,f,n,decoded", [(128, 256, 128, True), (128, 256, 129, False), (3584, 18944, 300, True),
+                                           (3584, 18944, 400, False), (5120, 27648, 512, True), (5120, 27648, 513, False)])
+def test_int4_prompts_decode_in_the_product_while_that_is_cheaper(dev, d, f, n, decoded):
+    st = _stage(dataclasses.replace(INT4, d_model=d, ffn=f))
+    assert _prefill(st, n) == 0
+    assert (dev.fake_launches(b"prefill_narrow4_kernel") > 0) == decoded
+    assert (dev.fake_launches(b"dequant_int4_f16_kernel") > 0) != decoded
+    K.kfl_stage_destroy(st)
+
+
+def test_int4_prompts_without_memory_for_the_copies(dev):
+    """Up to 512 tokens then decode in the products; longer ones are refused until there is memory."""
+    st = _stage(dataclasses.replace(INT4, d_model=3584, ffn=18944))
+    assert _prefill(st, 300) == 0
+    dev.fake_budget(dev.fake_live() + (400 << 20))  # the longer workspace, but no two copies of 272 MB
+    assert _prefill(st, 400) == 0 and dev.fake_launches(b"dequant_int4_f16_kernel") == 0
+    assert _prefill(st, 520) == -3
+    dev.fake_budget(1 << 40)
+    assert _prefill(st, 520) == 0 and dev.fake_launches(b"dequant_int4_f16_kernel") > 0
+    K.kfl_stage_destroy(st)
+    assert dev.fake_live() == 0
