@@ -12,6 +12,7 @@ import pytest
 
 from paper_2609_34045_gb300 import stage as K
 from paper_2609_34045_gb300 import workload as wl
+from test_gpu_wide import CASES
 
 B = importlib.import_module("paper_2609_34045_gb300.build")  # (the package binds the name to its function)
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -55,10 +56,15 @@ def _load(st, model):
         w[n] = (np.zeros((rows, cols), dtype=np.uint16) if model.weight_fmt == "bf16" else
                 (np.zeros((rows, cols // 8), dtype=np.uint32), np.zeros((rows, cols // 64), dtype=np.uint16)))
     K.kfl_stage_load_layer(st, 0, w, on_device=False)
+    if st.flags:
+        head = {"embed": np.zeros((model.vocab, d), dtype=np.uint16), "final_norm": w["attn_norm"]}
+        head["lm_head"] = head["embed"] if model.weight_fmt == "bf16" else (
+            np.zeros((model.vocab, d // 8), dtype=np.uint32), np.zeros((model.vocab, d // 64), dtype=np.uint16))
+        K.kfl_stage_load_head(st, head, on_device=False)
 
 
-def _stage(model, max_batch=1):
-    st = K.kfl_stage_create(K.model_cfg(model, 4096, max_batch), 0, 1, 0)
+def _stage(model, max_batch=1, flags=0):
+    st = K.kfl_stage_create(K.model_cfg(model, 4096, max_batch), 0, 1, flags)
     _load(st, model)
     return st
 
@@ -67,7 +73,8 @@ def _prefill(st, n):
     """The return code of a prompt of n tokens (no kernel runs: the buffers are never read)."""
     pos = np.arange(n, dtype=np.int32)
     h = np.zeros(1, dtype=np.float32)
-    return K.lib().kfl_stage_prefill(st.handle, None, h.ctypes.data, pos.ctypes.data, 0, n, h.ctypes.data, None, None)
+    return K.lib().kfl_stage_prefill(st.handle, pos.ctypes.data, h.ctypes.data, pos.ctypes.data, 0, n, h.ctypes.data,
+                                     pos.ctypes.data, None)
 
 
 def _matmul(T, k, n):
@@ -204,3 +211,12 @@ def test_int4_prompts_without_memory_for_the_copies(dev):
     assert _prefill(st, 520) == 0 and dev.fake_launches(b"dequant_int4_f16_kernel") > 0
     K.kfl_stage_destroy(st)
     assert dev.fake_live() == 0
+
+
+@pytest.mark.parametrize("model,n,kernels", [c[1:] for c in CASES], ids=[c[0] for c in CASES])
+def test_the_long_prompts_tests_reach_their_kernels(dev, model, n, kernels):
+    st = _stage(model, 2, K.KFL_IS_HEAD)
+    assert _prefill(st, n) == 0
+    missing = [k for k in kernels if dev.fake_launches(k.encode()) == 0]
+    assert not missing
+    K.kfl_stage_destroy(st)

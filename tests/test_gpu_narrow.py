@@ -83,7 +83,7 @@ def test_prefill_matches_the_oracle(model, n, monkeypatch):
 @pytest.mark.parametrize("model,d,n", [(RAGGED, 8320, 18),  # past what the norm's threads hold in registers
                                        (RAGGED128, 8320, 130), (dataclasses.replace(RAGGED, qk_norm=True), 8264, 100),
                                        (RAGGED_INT4, 16640, 33),
-                                       (RAGGED, 16648, 200),  # the same of the norm behind the 128-token tiles
+                                       (RAGGED, 16648, 200),
                                        (RAGGED, 32776, 17)])  # too many row tiles for the residual sums' norm
 def test_long_rows_match_the_oracle(model, d, n, monkeypatch):
     """Residual sums and RMSNorm of rows at the edges of their kernels' ranges.  The attention norm's gain is
