@@ -184,14 +184,18 @@ __device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t da, uint64_t db,
 // takes 8e-6 at most) and adds each to the residual stream, or to its partial sums, while the next
 // multiplies.  Unchunked, a whole tile of K = 18944 or 29568 lost 3.8e-5 or 5.9e-5.  Every chunk reads and writes
 // the tile once more: four 7B-shaped blocks of 2048 tokens take 5215 us for 5120 (chunks of 148: 5150, and
-// 1.9e-5), two 72B-shaped int4 ones of 900 tokens 5060 for 4960.
-constexpr int PP_CHUNK = 16, PR_CHUNK = 64;
+// 1.9e-5), two 72B-shaped int4 ones of 900 tokens 5060 for 4960.  Q/K/V of more than 2 PQ_CHUNK K blocks go in
+// chunks of PQ_CHUNK (K = 2048), added up in the workspace: a softmax of large scores feels every relative
+// error of q and k (those int4 blocks, against 64 bits: 6.23e-3 unchunked, 6.17e-3 in chunks of 4096 and
+// 6.13e-3 so, in the same time); K = 3584 in two of them took 2048 tokens 1 % for 1.075e-3 -> 1.071e-3.
+constexpr int PP_CHUNK = 16, PR_CHUNK = 64, PQ_CHUNK = 32;
 // K blocks of one accumulation of a segment of n.
 template <int MODE>
 __device__ __forceinline__ int pp_chunk(int n) {
   if (MODE == PE_STORE) return PP_CHUNK;
-  if (MODE != PE_RESID || n <= PR_CHUNK) return n;
-  const int parts = (n + PR_CHUNK - 1) / PR_CHUNK;
+  if ((MODE != PE_RESID && MODE != PE_QKV) || (MODE == PE_QKV && n <= 2 * PQ_CHUNK)) return n;
+  constexpr int MOST = MODE == PE_RESID ? PR_CHUNK : PQ_CHUNK;
+  const int parts = (n + MOST - 1) / MOST;
   return (n + parts - 1) / parts;
 }
 __host__ __device__ constexpr int pp_epi_warps(bool drain) { return drain ? 8 : 4; }
@@ -344,22 +348,31 @@ __global__ void __launch_bounds__(pp_threads(DRAIN), 1)
       const int n_tile = w.tile / t_tiles, t = (w.tile % t_tiles) * PG_M + row, n0 = n_tile * PG_N;
       const bool whole = w.whole();
       EpiState<MODE> st;
-      // `more`: a further chunk of the same sums
-      auto finish = [&](int c, const uint32_t(&r)[32], bool more = false) {
-        if (whole) {
+      // 32 columns' sums; of a segment in chunks: a chunk's, `more` after the first, `last` the last
+      auto finish = [&](int c, uint32_t(&r)[32], bool more, bool last) {
+        if (whole && (MODE == PE_RESID || (last && !more))) {
           if (t < ep.T) epilogue32<MODE>(ep, t, n0 + 32 * c, r, st);
-        } else {
-          float4 *at = reinterpret_cast<float4 *>(ws) + wide_partial(w.part, 8 * c) + row;
+          return;
+        }
+        // a whole tile's chunks meet where this CTA's first part goes later
+        float4 *at = reinterpret_cast<float4 *>(ws) + wide_partial(whole ? blockIdx.x : w.part, 8 * c) + row;
+        if (more) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            float4 y = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                   __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
-            if constexpr (MODE == PE_RESID) {
-              const float4 x = more ? at[j * PG_M] : make_float4(0.f, 0.f, 0.f, 0.f);
-              y = make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
-            }
-            at[j * PG_M] = y;
+            const float4 x = at[j * PG_M];
+            r[4 * j] = __float_as_uint(x.x + __uint_as_float(r[4 * j]));
+            r[4 * j + 1] = __float_as_uint(x.y + __uint_as_float(r[4 * j + 1]));
+            r[4 * j + 2] = __float_as_uint(x.z + __uint_as_float(r[4 * j + 2]));
+            r[4 * j + 3] = __float_as_uint(x.w + __uint_as_float(r[4 * j + 3]));
           }
+        }
+        if (whole && last) {
+          if (t < ep.T) epilogue32<MODE>(ep, t, n0 + 32 * c, r, st);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            at[j * PG_M] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                                       __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
         }
       };
       if constexpr (DRAIN) {
@@ -385,7 +398,7 @@ __global__ void __launch_bounds__(pp_threads(DRAIN), 1)
         if (!ok) break;
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-          if (n0 + 32 * (c0 + c) < ep.N) finish(c0 + c, sum[c]);  // uniform across the warp
+          if (n0 + 32 * (c0 + c) < ep.N) finish(c0 + c, sum[c], false, true);  // uniform across the warp
       } else {
         const int chunk = pp_chunk<MODE>(w.kb1 - w.kb0);
         for (int left = w.kb1 - w.kb0, done = 0; left > 0; left -= chunk, ++done) {
@@ -394,7 +407,7 @@ __global__ void __launch_bounds__(pp_threads(DRAIN), 1)
             if (n0 + 32 * c >= ep.N) break;  // uniform across the warp
             uint32_t r[32];
             tmem_ld32(lanes + (uint32_t)((i & 1) * PG_N + 32 * c), r);
-            finish(c, r, done > 0);
+            finish(c, r, done > 0, left <= chunk);
           }
           release_acc();
         }

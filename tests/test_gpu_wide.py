@@ -128,3 +128,37 @@ def test_error_of_a_long_mlp(fmt, d, f, n):
     err = float((out.double() - h.double() - y).norm() / y.norm())
     K.kfl_stage_destroy(st)
     assert err <= bar, err
+
+
+def test_rounding_of_a_long_value_projection():
+    """V rows of a product with more than a round of tiles and K = 8192, against 64 bits rounded to bf16: those
+    that land beside it.  Truncation of chunks of K = 2048 takes 4.1e-6 of a value's size, of the whole K 1.6e-5;
+    a bf16 step is 5.4e-3 (1 / 185) of the value on average, so 0.076 % and 0.30 % would land a step lower.
+    Twice that for values that are normal around zero: what they lose goes by their partial sums, of the
+    RMS's size, and their steps by their own.  (x's terms, 2^-22, add 0.01 %.)  The bar is between the two."""
+    d, n, kv = 8192, 900, 1024
+    g = torch.Generator(device="cuda").manual_seed(5)
+    m = wl.ModelShape(n_layers_total=1, d_model=d, n_heads=24, n_kv_heads=8, head_dim=128, ffn=256, vocab=300,
+                      weight_fmt="int4_g64")
+    w = {k: torch.ones(128 if k in ("q_norm", "k_norm") else d, device="cuda", dtype=torch.bfloat16)
+         for k in ("attn_norm", "ffn_norm", "q_norm", "k_norm")}
+    for name, rows, cols in (("wq", 3072, d), ("wk", kv, d), ("wv", kv, d), ("wo", d, 3072), ("wg", 256, d), ("wu", 256, d),
+                             ("wd", d, 256)):
+        w[name], codes = _codes(g, rows, cols)
+        if name == "wv":
+            wv = codes.double().mul_(2.0 ** -6)
+    st = K.kfl_stage_create(K.model_cfg(m, 960, 1), 0, 1, 0)
+    torch.cuda.synchronize()
+    K.kfl_stage_load_layer(st, 0, w, on_device=True)
+    h = _gaussian(g, n, d, std=1.0).float()
+    out = torch.zeros(n, d, device="cuda")
+    K.kfl_stage_prefill(st, None, h, torch.arange(n, dtype=torch.int32, device="cuda"), 0, n, out, None,
+                        torch.cuda.current_stream().cuda_stream)
+    k, v = (torch.zeros(8, 960, 128, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    K.kfl_kv_read(st, 0, 0, k, v, True)
+    x = h.double()
+    x = x / torch.sqrt((x * x).mean(-1, keepdim=True) + m.rms_eps)
+    ref = (x @ wv.t()).float().bfloat16().view(n, 8, 128).transpose(0, 1)
+    K.kfl_stage_destroy(st)
+    beside = float((v[:, :n] != ref).double().mean())
+    assert beside <= 2.5e-3, beside
