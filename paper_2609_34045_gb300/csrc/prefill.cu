@@ -1206,8 +1206,9 @@ cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const 
   return launch_pdl(prefill_rmsnorm_kernel, dim3(T), threads, 0, s, h, ldh, d, g, eps, x, term_stride, terms, ldx, f16, err);
 }
 
-cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, cudaStream_t s) {
-  dequant_int4_f16_kernel<<<8 * 152, 128, 0, s>>>(tiles4, n_rb * n_kt, dst);
+cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, int n_sm,
+                                    cudaStream_t s) {
+  dequant_int4_f16_kernel<<<8 * n_sm, 128, 0, s>>>(tiles4, n_rb * n_kt, dst);
   return cudaGetLastError();
 }
 

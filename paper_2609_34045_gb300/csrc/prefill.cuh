@@ -17,11 +17,11 @@ namespace kfl {
 // the int4 ones, with fp16 terms of X).  An output tile is PG_M tokens x PG_N weight rows,
 // computed with tcgen05.mma (M = PG_M, N = PG_N, K = 16 per instruction; each K slice once with
 // Xhi and once with Xlo against the same W slice), the fp32 accumulator in tensor memory, by a
-// persistent CTA per SM with two accumulators (prefill_gemm_persistent).  Operands reach shared memory by TMA with the 128-byte swizzle, PG_K = 64 bf16 (one
-// swizzle row) per pipeline stage: Xhi and Xlo through 2-D maps of the activation rows, W through
-// a 4-D map of the decode path's weight tiles [N/RB][K/KT][RB][KT] (one box = PG_N / RB row
-// blocks x 64 columns of one K tile), so the prefill streams the weights from where the decode
-// step reads them.
+// persistent CTA per SM with two accumulators (prefill_gemm_persistent).  Operands reach shared memory
+// by TMA with the 128-byte swizzle, PG_K = 64 bf16 (one swizzle row) per pipeline stage: Xhi and Xlo
+// through 2-D maps of the activation rows, W through a 4-D map of the decode path's weight tiles
+// [N/RB][K/KT][RB][KT] (one box = PG_N / RB row blocks x 64 columns of one K tile), so the prefill
+// streams the weights from where the decode step reads them.
 constexpr int PG_M = 128;
 constexpr int PG_N = 256;
 constexpr int PG_K = 64;
@@ -48,14 +48,15 @@ struct PrefillEpiParams {
   int ldo16;
   int terms;               // PE_SWIGLU: terms stored, term_stride elements apart
   size_t term_stride;
-  // PE_QKV (out not NULL: q in fp32 to out [T][ldo] instead of out16): rows [0, qdim) q, [qdim, qdim + kvdim) k (pairs (i, i + hd/2) adjacent per head, as
-  // the weights were loaded), then v in natural order; K/V stored at the token's position of
+  // PE_QKV (out not NULL: q in fp32 to out [T][ldo] instead of out16): rows [0, qdim) q, [qdim, qdim +
+  // kvdim) k (pairs (i, i + hd/2) adjacent per head, as the weights were loaded), then v in natural order; K/V stored at the token's position of
   // KV slot `slot` of this layer's caches [max_batch][Hkv][max_ctx][hd]
   uint16_t *kcache, *vcache;
   const int *positions;    // [T], -1 for a refused token (nothing of it is stored)
   int slot, hd, hkv, qdim, kvdim, max_ctx;
   const float *rope_cos, *rope_sin;  // [max_ctx][hd / 2]
-  // PE_ARGMAX: [T][n_tiles] partial maxima (of 256 columns, or of 32 rows in the few-token GEMM) and their indices
+  // PE_ARGMAX: [T][n_tiles] partial maxima (of 256 columns, or of 32 rows in the few-token GEMM) and
+  // their indices
   float *amax;
   int *aidx;
   int n_tiles;
@@ -164,7 +165,8 @@ cudaError_t launch_prefill_input(const int *ids, const float *hidden_in, const i
 cudaError_t launch_prefill_rmsnorm(const float *h, int ldh, int T, int d, const float *g, float eps, uint16_t *x,
                                    size_t term_stride, int terms, int ldx, int f16, unsigned *err, cudaStream_t s);
 // int4 group-64 tiles [n_rb][n_kt][TILE4_BYTES] -> fp16 tiles [n_rb][2 n_kt][RB][KT] of code x scale.
-cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, cudaStream_t s);
+cudaError_t launch_dequant_int4_f16(const uint8_t *tiles4, int n_rb, int n_kt, uint16_t *dst, int n_sm,
+                                    cudaStream_t s);
 // fp32 rows [T][K] (stride ldx) as hi and lo bf16 terms (stride ld); *err = 0.
 cudaError_t launch_split_bf16(const float *x, int T, int K, int ldx, uint16_t *hi, uint16_t *lo, int ld, unsigned *err,
                               cudaStream_t s);

@@ -175,7 +175,8 @@ __device__ __forceinline__ uint32_t hfma2(uint32_t a, uint32_t b, uint32_t c) {
 
 // The eight codes of an A-fragment word as exact fp16 pairs: rows gid and gid + 8 of columns 2 tig,
 // 2 tig + 1 (c0, c1) and of columns 2 tig + 8, 2 tig + 9 (c2, c3).  The nibbles, top bit flipped, become
-// 1024 + u or 1024 + 16 u (u = code + 8).
+// 1024 + u or 1024 + 16 u (u = code + 8): integers placed in the mantissa of fp16 1024, as published by
+// Kim, Henry, Fahim and Awadalla, "Who Says Elephants Can't Run" (arXiv 2211.10017).
 __device__ __forceinline__ void decode_word(uint32_t w, uint32_t &c0, uint32_t &c1, uint32_t &c2, uint32_t &c3) {
   const uint32_t w8 = w >> 8;
   asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(c0) : "r"(w), "r"(0x000F000Fu), "r"(0x64086408u));
@@ -293,11 +294,12 @@ struct TileParts {
       at = rest = k;
       step = s.tail;
     } else {
-      // the CTAs first .. last meet the tile; every one but the first starts inside it
+      // the CTAs first .. last meet the tile; every one but the first starts inside it (partial 0), the
+      // first comes to its start (partial 1)
       const unsigned U = s.tail * s.n_kb, G = grid, lo = k * s.n_kb;
       const int first = (int)(((lo + 1) * G - 1) / U), last = (int)(((lo + s.n_kb) * G - 1) / U);
       n = last - first + 1;
-      at = first * 2 + (first * U / G > lo ? 0 : 1);
+      at = first * 2 + 1;
       rest = first * 2;
       step = 2;
     }

@@ -282,7 +282,7 @@ struct kfl_stage {
   std::vector<void *> pf_retired;  // workspaces outgrown since a graph captured them: kept until the stage goes
   // bf16 stages: the maps of every layer's weight tiles [4 l + j] (Q/K/V, O, gate/up, down), then
   // lm_head.  int4 stages: one map per matrix kind [j] (then lm_head) over pf_w16, the fp16 tiles
-  // of the matrix being multiplied (dequantized just before its GEMM)
+  // of the matrix being multiplied (dequantized just before its GEMM; passes that pf_narrow does not take)
   std::vector<CUtensorMap> pf_maps;  // int4: [buffer * 5 + kind]
   std::vector<CUtensorMap> pf_maps_nw;  // bf16 stages: the same tiles in the few-token GEMM's boxes
   std::vector<CUtensorMap> kv_maps;  // attention clusters: layer l's K cache [2 l] and V cache [2 l + 1]
@@ -980,7 +980,8 @@ cudaError_t pf_dequant(kfl_stage *st, int g) {
   if (!pf_seq_matrix(st, g, &l, &j)) return cudaSuccess;
   const Mat &m = pf_mat(st, l, j);
   cudaError_t err = cudaStreamWaitEvent(st->pf_side, st->pf_used[g % 2], 0);
-  if (err == cudaSuccess) err = launch_dequant_int4_f16(m.tiles, m.n_rb, m.n_kt, st->pf_w16[g % 2], st->pf_side);
+  if (err == cudaSuccess)
+    err = launch_dequant_int4_f16(m.tiles, m.n_rb, m.n_kt, st->pf_w16[g % 2], st->P.n_sm, st->pf_side);
   if (err == cudaSuccess) err = cudaEventRecord(st->pf_deq[g % 2], st->pf_side);
   return err;
 }

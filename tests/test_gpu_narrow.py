@@ -1,6 +1,6 @@
 """GPU parity of the prefill's few-token matrix product (stream-K over the SMs, weight rows as the MMA's
-rows) at the edges of its tiles: token groups of 16 up to 128, row tiles of 128 and (many rows, more
-than 64 tokens) 256, one K block of 64 up to several per CTA, with ragged tails; and its int4 form,
+rows) at the edges of its tiles: token groups of 16 up to 128, row tiles of 128 and (a stage's many rows,
+more than 64 tokens) 256, one K block of 64 up to several per CTA, with ragged tails; and its int4 form,
 which decodes the weights on the way (256-row tiles, K units of 128).
 
 The plain product against fp64: x carried to about 2^-16 relative by its two terms, fp32
@@ -40,9 +40,11 @@ def test_product_matches_fp64(T, Kd, N):
     ldy = (N + 3) // 4 * 4
     y = torch.full((T, ldy), 7.0, dtype=torch.float32, device="cuda")
     wd = w.view(torch.int16).cuda().contiguous()
-    for _ in range(2):  # the second call finds whatever the first left in the tickets
-        K.kfl_matmul_bf16w(torch.from_numpy(x).cuda(), T, Kd, Kd, wd, N, y, ldy,
-                           torch.cuda.current_stream().cuda_stream)
+    # what the call finds in the pool's memory: another shape's terms and partial sums, far from these
+    big = torch.full((T + 3, Kd + 64), 3e38, device="cuda")
+    K.kfl_matmul_bf16w(big, T + 3, Kd + 64, Kd + 64, torch.full((N + 5, Kd + 64), 0x7F00, dtype=torch.int16, device="cuda"),
+                       N + 5, torch.zeros((T + 3, ldy + 8), device="cuda"), ldy + 8, torch.cuda.current_stream().cuda_stream)
+    K.kfl_matmul_bf16w(torch.from_numpy(x).cuda(), T, Kd, Kd, wd, N, y, ldy, torch.cuda.current_stream().cuda_stream)
     got = y.cpu().numpy()
     ref = x.astype(np.float64) @ w.to(torch.float64).numpy().T
     rms = np.sqrt(np.mean(ref * ref, axis=1, keepdims=True))
@@ -54,7 +56,7 @@ def test_product_matches_fp64(T, Kd, N):
 def test_product_error_of_a_long_k(T):
     """Both forms of the plain product at K = 18944: x's two terms leave 2^-18 of it (rms 2e-6), and the sums
     are fp32 ones, so 1e-5 of the result (2-norm).  Left in the tensor core's accumulator, which truncates
-    (3e-8 per 16 products), they were up to 3.5e-5 off."""
+    (3e-8 per 16 products), they were 1.5e-5 off."""
     k = n = 18944
     g = torch.Generator(device="cuda").manual_seed(T)
     x = torch.randn((T, k), generator=g, device="cuda")

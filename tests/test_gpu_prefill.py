@@ -2,9 +2,8 @@
 
 A prompt of one user goes through the stage either as steps of up to max_batch rows on the user's
 KV slot (the decode kernels) or densely (tensor-core matrix products over all its tokens, causal
-attention over the slot; int4 weights dequantized to fp16 first); the oracle runs the whole prompt
-in one pass.  Bar as
-for decode: every token's output within max-abs 1e-2 of the oracle's RMS, greedy ids equal where
+attention over the slot; int4 weights decoded to fp16 in the products or ahead of them); the oracle
+runs the whole prompt in one pass.  Bar as for decode: every token's output within max-abs 1e-2 of the oracle's RMS, greedy ids equal where
 the oracle's top-2 margin exceeds 1e-2, the user's written cache rows within tolerance and every
 other row of every slot bit-identical.
 """
