@@ -180,14 +180,14 @@ __device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t da, uint64_t db,
 // stage's products, of K = d_model mostly, go without: the sums' registers cost the fused epilogues
 // spills.
 //
-// A residual product takes a long K in equal chunks of at most PR_CHUNK K blocks (K = 4096: truncation
-// takes 8e-6 at most) and adds each to the residual stream, or to its partial sums, while the next
-// multiplies.  Unchunked, a whole tile of K = 18944 or 29568 lost 3.8e-5 or 5.9e-5.  Every chunk reads and writes
-// the tile once more: four 7B-shaped blocks of 2048 tokens take 5215 us for 5120 (chunks of 148: 5150, and
-// 1.9e-5), two 72B-shaped int4 ones of 900 tokens 5060 for 4960.  Q/K/V of more than 2 PQ_CHUNK K blocks go in
-// chunks of PQ_CHUNK (K = 2048), added up in the workspace: a softmax of large scores feels every relative
-// error of q and k (those int4 blocks, against 64 bits: 6.23e-3 unchunked, 6.17e-3 in chunks of 4096 and
-// 6.13e-3 so, in the same time); K = 3584 in two of them took 2048 tokens 1 % for 1.075e-3 -> 1.071e-3.
+// Residual products and Q/K/V take a long K in equal chunks, whose sums meet in the workspace while the
+// next chunk multiplies (coalesced, loaded a step ahead: adding each to the rows of the residual stream
+// took 2 to 13 % of a pass, as it stalled the MMAs).  O and down: at most PR_CHUNK K blocks (K = 4096:
+// truncation takes 8e-6), where a whole tile of K = 18944 or 29568 lost 3.8e-5 or 5.9e-5.  Q/K/V of more
+// than 2 PQ_CHUNK: at most PQ_CHUNK (K = 2048), because a softmax of large scores feels every relative
+// error of q and k: two 72B-shaped int4 blocks of 900 tokens are 6.23e-3 from 64 bits unchunked, 6.17e-3 in
+// chunks of 4096 and 6.14e-3 so.  Those two take 4985 us for 4890 unchunked, four 7B-shaped blocks of 2048
+// tokens 5165 for 5098.
 constexpr int PP_CHUNK = 16, PR_CHUNK = 64, PQ_CHUNK = 32;
 // K blocks of one accumulation of a segment of n.
 template <int MODE>
@@ -348,31 +348,17 @@ __global__ void __launch_bounds__(pp_threads(DRAIN), 1)
       const int n_tile = w.tile / t_tiles, t = (w.tile % t_tiles) * PG_M + row, n0 = n_tile * PG_N;
       const bool whole = w.whole();
       EpiState<MODE> st;
-      // 32 columns' sums; of a segment in chunks: a chunk's, `more` after the first, `last` the last
-      auto finish = [&](int c, uint32_t(&r)[32], bool more, bool last) {
-        if (whole && (MODE == PE_RESID || (last && !more))) {
-          if (t < ep.T) epilogue32<MODE>(ep, t, n0 + 32 * c, r, st);
-          return;
-        }
-        // a whole tile's chunks meet where this CTA's first part goes later
-        float4 *at = reinterpret_cast<float4 *>(ws) + wide_partial(whole ? blockIdx.x : w.part, 8 * c) + row;
-        if (more) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float4 x = at[j * PG_M];
-            r[4 * j] = __float_as_uint(x.x + __uint_as_float(r[4 * j]));
-            r[4 * j + 1] = __float_as_uint(x.y + __uint_as_float(r[4 * j + 1]));
-            r[4 * j + 2] = __float_as_uint(x.z + __uint_as_float(r[4 * j + 2]));
-            r[4 * j + 3] = __float_as_uint(x.w + __uint_as_float(r[4 * j + 3]));
-          }
-        }
+      // where this row's partial sums are; a whole tile's chunks meet where this CTA's first part goes later
+      float4 *part = reinterpret_cast<float4 *>(ws) + wide_partial(whole ? blockIdx.x : w.part, 0) + row;
+      // 32 columns' sums, `last` if no chunk of them follows
+      auto finish = [&](int c, const uint32_t(&r)[32], bool last) {
         if (whole && last) {
           if (t < ep.T) epilogue32<MODE>(ep, t, n0 + 32 * c, r, st);
         } else {
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            at[j * PG_M] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                       __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
+            part[(8 * c + j) * PG_M] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                                                   __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
         }
       };
       if constexpr (DRAIN) {
@@ -398,16 +384,40 @@ __global__ void __launch_bounds__(pp_threads(DRAIN), 1)
         if (!ok) break;
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-          if (n0 + 32 * (c0 + c) < ep.N) finish(c0 + c, sum[c], false, true);  // uniform across the warp
+          if (n0 + 32 * (c0 + c) < ep.N) finish(c0 + c, sum[c], true);  // uniform across the warp
       } else {
+        constexpr bool CHUNKS = MODE == PE_RESID || MODE == PE_QKV;
         const int chunk = pp_chunk<MODE>(w.kb1 - w.kb0);
         for (int left = w.kb1 - w.kb0, done = 0; left > 0; left -= chunk, ++done) {
+          // the earlier chunks' sums of 32 columns, loaded one step ahead
+          float4 x[2][8];
+          auto fetch = [&](int c, float4(&y)[8]) {
+            if (CHUNKS && done > 0 && n0 + 32 * c < ep.N)
+#pragma unroll
+              for (int j = 0; j < 8; ++j) y[j] = part[(8 * c + j) * PG_M];
+          };
+          fetch(0, x[0]);
           if (!(ok = wait_acc())) break;
-          for (int c = 0; c < PG_N / 32; ++c) {
-            if (n0 + 32 * c >= ep.N) break;  // uniform across the warp
+          auto step = [&](int c, const float4(&y)[8]) {
+            if (n0 + 32 * c >= ep.N) return;  // uniform across the warp
             uint32_t r[32];
             tmem_ld32(lanes + (uint32_t)((i & 1) * PG_N + 32 * c), r);
-            finish(c, r, done > 0, left <= chunk);
+            if (CHUNKS && done > 0) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                r[4 * j] = __float_as_uint(y[j].x + __uint_as_float(r[4 * j]));
+                r[4 * j + 1] = __float_as_uint(y[j].y + __uint_as_float(r[4 * j + 1]));
+                r[4 * j + 2] = __float_as_uint(y[j].z + __uint_as_float(r[4 * j + 2]));
+                r[4 * j + 3] = __float_as_uint(y[j].w + __uint_as_float(r[4 * j + 3]));
+              }
+            }
+            finish(c, r, left <= chunk);
+          };
+          for (int c = 0; c < PG_N / 32; c += 2) {
+            fetch(c + 1, x[1]);
+            step(c, x[0]);
+            if (c + 2 < PG_N / 32) fetch(c + 2, x[0]);
+            step(c + 1, x[1]);
           }
           release_acc();
         }
