@@ -182,3 +182,31 @@ def test_nan_keys_reach_the_output(n):
                         torch.cuda.current_stream().cuda_stream)
     assert torch.isnan(out).all()
     K.kfl_stage_destroy(st)
+
+
+@pytest.mark.parametrize("model,n", [(RAGGED, 9), (RAGGED, 40), (dataclasses.replace(RAGGED, qk_norm=True), 40),
+                                     (RAGGED_INT4, 40), (RAGGED_INT4, 200)])
+def test_captured_prompt_after_a_longer_one(model, n):
+    """A captured prompt replayed after a longer prompt has outgrown its workspace gives what it gave."""
+    st = K.kfl_stage_create(K.model_cfg(model, 1024, 4), 0, 1, 0)
+    K.kfl_stage_load_layer(st, 0, wl.layer_weights(model, 0, 3), on_device=False)
+    hidden = torch.randn(700, model.d_model, device="cuda")
+    pos = torch.arange(700, dtype=torch.int32, device="cuda")
+    out = torch.zeros(700, model.d_model, device="cuda")
+    run = lambda t: K.kfl_stage_prefill(st, None, hidden, pos, 1, t, out, None, torch.cuda.current_stream().cuda_stream)
+    run(n)
+    first = out[:n].clone()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run(n)
+    run(700)
+    # (what the longer prompt would have freed is likely to be given to these)
+    filler = [torch.full((1 << 20,), float("nan"), device="cuda") for _ in range(64)]
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert K.kfl_stage_status(st) == 0
+    assert torch.equal(out[:n], first)
+    del filler, graph
+    K.kfl_stage_destroy(st)
